@@ -219,12 +219,19 @@ struct ras_data {
   // shared-memory apply: one factor stream per subdomain (see ras.cu)
   bool smem_path = false;
   bool built = false;           // a setup has run (level sets exportable)
-  size_t smem_bytes = 0;        // ring + largest local vector
-  int m_max = 0;                // most extended rows in a subdomain
+  size_t smem_bytes = 0;        // largest local vector and its zero element
   dbuf<long long> blob_off;     // nsub + 1 byte offsets (stream bounds)
   dbuf<unsigned char> blob;     // the streams
-  dbuf<int> gidx;               // per subdomain and position: 2 * global row + owned flag
-  dbuf<int4> gdesc;             // group descriptors (packing scratch)
+  size_t lvl_smem[2] = {0, 0};  // k_ras_levels' shared memory, without and with the pruned lists
+  size_t pack_smem = 0;         // k_ras_pack's tables
+  bool symmetric = false;       // the pattern has (c, i) for every (i, c)
+  bool pruned = false;          // the last setup left unneeded rows out of the apply's lists
+  dbuf<int> gidx, gord;         // gather order (owned rows first): global row, ext index
+  dbuf<int> nown;               // owned rows per subdomain
+  dbuf<uint16_t> gpos;          // gather order: position of each row (per setup)
+  dbuf<int> alvl_rows, alvl_ptr;   // as lvl_rows, lvl_ptr, without the rows no owned row depends on
+  dbuf<uint2> gdesc;            // group descriptors
+  dbuf<int> ngrp;               // groups per subdomain
 };
 
 // ---------------------------------------------------------- linear system --

@@ -1152,7 +1152,7 @@ static int ls_solve_bicgstab(sim_ls_s *ls, double tol, int *its_out, double *rel
   }
   if (rn <= tol * bn) { *its_out = 0; *relres = rn / bn; return 0; }
   auto check = [&]() {
-    if (ls->errw[0]) RS_FAIL(SIM_ERR_TIMEOUT, "RAS apply: bulk copy wait gave up (code %d)", ls->errw[0]);
+    if (ls->errw[0]) RS_FAIL(SIM_ERR_TIMEOUT, "RAS setup gave up (code %d)", ls->errw[0]);
   };
   for (;;) {
     RS_CUDA(cudaMemcpyAsync(rh, r, nu * sizeof(double), cudaMemcpyDeviceToDevice, st));
@@ -1489,7 +1489,7 @@ int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
       k_loop_params<<<1, 1, 0, s>>>(ls->loopd.p, tol * bn, (double)std::min(m, maxit - its));
       RS_CUDA(cudaGraphLaunch(ls->loop_exec, s));
       std::vector<double> lo = d2h(ls->loopd.p + 2, 2, s);
-      if (ls->errw[0]) RS_FAIL(SIM_ERR_TIMEOUT, "RAS apply: bulk copy wait gave up (code %d)", ls->errw[0]);
+      if (ls->errw[0]) RS_FAIL(SIM_ERR_TIMEOUT, "RAS setup gave up (code %d)", ls->errw[0]);
       jend = (int)lo[0];
       its += jend;
       RS_LAUNCHED(1 + (long long)jend * (ls->it_launches + 1));
@@ -1504,7 +1504,7 @@ int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
       }
       RS_CUDA(cudaStreamSynchronize(s));
       if (use_graph) ls->graph_timers();
-      if (ls->errw[0]) RS_FAIL(SIM_ERR_TIMEOUT, "RAS apply: bulk copy wait gave up (code %d)", ls->errw[0]);
+      if (ls->errw[0]) RS_FAIL(SIM_ERR_TIMEOUT, "RAS setup gave up (code %d)", ls->errw[0]);
       double est = hp[4 * j], hnv = hp[4 * j + 1];
       its++;
       jend = j + 1;

@@ -13,43 +13,50 @@
 #include <algorithm>
 #include <cfloat>
 #include <climits>
+#include <type_traits>
 
-// Streamed per-subdomain factors for the shared-memory apply.  One warp
-// solves one subdomain: its local vector y lives in shared
-// memory, and the factors, which each application reads exactly once and in
-// a fixed order, flow through a small shared-memory ring filled by bulk
-// copies (cp.async.bulk + mbarrier) a few chunks ahead of the sweep.  The
-// stream of a subdomain (16-byte aligned pieces):
-//   header  {m, L groups, U groups, stream bytes, first group's start and
-//           bytes} 32 B
-//   groups  the rows of the L sweep (L levels 1.., level 0 has no entries),
-//           then the rows of the U sweep (U levels 0..), level by level;
-//           a level is split into groups of at most 32 rows (one per lane)
-//           and at most one chunk of bytes; a group never straddles the
-//           end of the ring (the stream is padded to the next ring period
-//           instead), so its pieces are contiguous in shared memory
-// A group:
-//   {nrows | nent << 16, bytes, next group's start, next group's bytes} 16 B
-//   row records: local row, first and end entry   8 B (L) or RREC_U (U, with
-//               (group-relative), U: the inverse  the 2x2 block, 4 values)
-//               diagonal block
-//   cols  u16[nent] | vals [nent][4]   (the row records, the columns and
-//   the values each start on a 16-byte boundary)
-// The global row of each local row (bit 0: owned) is a separate array
-// (gidx), read by the gather and the scatter.
+// Streamed per-subdomain factors for the shared-memory apply.  One block
+// solves one subdomain (one warp in FP32 / BF16, two in FP64): its local
+// vector y lives in shared memory, and the factors, which each application
+// reads exactly once and in a fixed order, stream through registers, a few
+// groups ahead of the sweep.  A subdomain's stream is a list of groups: the
+// rows of the L sweep (L levels 1.., level 0 has no entries), then the rows
+// of the U sweep (U levels 0..), level by level, without the rows no owned
+// row depends on (k_ras_levels); a level is split into groups of at most 32
+// rows, in descending order of their entry counts.  A group is a sequence of
+// pieces of 16 bytes per row (per row and component in FP64), each piece
+// stored for the first n[p] rows only:
+//   header    {row, col[0..5]} u16 (a missing column names the zero element
+//             behind y)
+//   blocks    U groups: the inverse diagonal block, then the entries; L
+//             groups: the entries.  A piece holds two BF16 blocks, one FP32
+//             block, or one component's half of an FP64 block
+// Piece by piece the reads of a warp are contiguous, and there is little
+// padding.  A row of more than RAS_K entries (a well's, a wide stencil's)
+// takes part in several groups, with the identity for the inverse diagonal
+// in all but the last.  The groups of each sweep are filled up to a multiple
+// of ras_ahead with empty ones (one row, behind the zero element).
+// A group's descriptor (64 bit): start / 16 (20 bits) | rows (6) | n[6] (6),
+// n[1..5] (6 bits each); n[0] = rows.
 #define RAS_SMEM_BUDGET (200 * 1024)
-#define RAS_GROUP_ROWS 32
-template <class TB> struct ring_cfg;                       // ring bytes, chunk bytes per stored type
-template <> struct ring_cfg<__nv_bfloat16> { static const int R = 4096, C = 1024; };
-template <> struct ring_cfg<float> { static const int R = 16384, C = 4096; };
-template <> struct ring_cfg<double> { static const int R = 32768, C = 8192; };
-// U row record: 8 bytes of indices, then the inverse diagonal block at DOFF
-template <class TB> __host__ __device__ constexpr int rrec_doff() { return 4 * (int)sizeof(TB) <= 8 ? 8 : 16; }
-template <class TB> __host__ __device__ constexpr int rrec_u() { return (rrec_doff<TB>() + 4 * (int)sizeof(TB) + 15) & ~15; }
-// a group's byte cap: one chunk (a group then touches at most two chunks,
-// and padding to the next ring period wastes at most a quarter of it)
-template <class TB> __host__ __device__ constexpr int group_cap() { return ring_cfg<TB>::C; }
+#define RAS_K 6                                  // entries of a row per group
+#define RAS_START_MAX (1LL << 24)                // a stream's bytes: 20-bit starts in units of 16
+// groups held in registers ahead of the sweep
+template <class TB> __host__ __device__ constexpr int ras_ahead() { return sizeof(TB) == 2 ? 3 : 2; }
+// stored bytes per 2x2 block
+static int ras_block_bytes(int prec) { return prec == SIM_PREC_FP64 ? 32 : prec == SIM_PREC_MIXED_BF16 ? 8 : 16; }
 __host__ __device__ inline int al16(int x) { return (x + 15) & ~15; }
+
+// flag = 1 when some entry (i, c) of the pattern has no entry (c, i)
+__global__ void k_pattern_asym(int nb, const int *rp, const int *ci, int *flag) {
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nb) return;
+  for (int q = rp[i]; q < rp[i + 1]; q++) {
+    int c = ci[q], lo = rp[c], hi = rp[c + 1];
+    while (lo < hi) { int mid = (lo + hi) >> 1; if (ci[mid] < i) lo = mid + 1; else hi = mid; }
+    if (lo >= rp[c + 1] || ci[lo] != i) *flag = 1;
+  }
+}
 
 // ------------------------------------------------- static partition (host)
 void ras_build_static(sim_ls_s *ls) {
@@ -110,7 +117,12 @@ void ras_build_static(sim_ls_s *ls) {
     sub_ptr[s + 1] = base + m;
     lrp_ptr[s + 1] = (int)lci.size();
     R.max_ext = std::max(R.max_ext, m);
-    R.max_nnz = std::max(R.max_nnz, (int)lci.size() - nnz0);
+    const int nz = (int)lci.size() - nnz0;
+    R.max_nnz = std::max(R.max_nnz, nz);
+    for (int k = 0; k < 2; k++) {               // k_ras_levels' shared memory, without and with the pruned lists
+      int cnt = (k ? 4 : 2) * (m + 1);
+      R.lvl_smem[k] = std::max(R.lvl_smem[k], sizeof(int) * ((size_t)3 * m + 1 + nz + (nz >= cnt ? 0 : cnt)));
+    }
   }
   cudaStream_t st = ls->st;
   h2d(R.sub_ptr, sub_ptr, st); h2d(R.ext, ext, st);
@@ -129,37 +141,50 @@ void ras_build_static(sim_ls_s *ls) {
   while (m < maxcells) m <<= 1;
   R.max_lvl_ptr = m;   // sort width (power of two >= most cells in a subdomain)
   // shared-memory apply: a bound on each subdomain's stream (the grouping
-  // follows the level sets of each setup, the bound only rows and entries:
-  // at most one group per walked row, each with its header and padding)
+  // follows the level sets of each setup, the bound only rows and entries: a
+  // row's parts have a header, an inverse diagonal block and a rounding each)
   {
-    int vb = ls->o.precision == SIM_PREC_FP64 ? 32 : (ls->o.precision == SIM_PREC_MIXED_BF16 ? 8 : 16);
-    int ru = ls->o.precision == SIM_PREC_FP64 ? rrec_u<double>()
-                                              : (ls->o.precision == SIM_PREC_MIXED_BF16 ? rrec_u<__nv_bfloat16>()
-                                                                                        : rrec_u<float>());
-    int ring = ls->o.precision == SIM_PREC_FP64 ? ring_cfg<double>::R
-                                                : (ls->o.precision == SIM_PREC_MIXED_BF16 ? ring_cfg<__nv_bfloat16>::R
-                                                                                          : ring_cfg<float>::R);
-    int yb = ls->o.precision == SIM_PREC_FP64 ? 16 : 8;   // local vector: double2 or float2 per row
+    const int prec = ls->o.precision, vb = ras_block_bytes(prec);
+    int yb = prec == SIM_PREC_FP64 ? 16 : 8;               // local vector: double2 or float2 per row
     std::vector<long long> boff(nsub + 1, 0);
     int mmax = 0;
-    bool fits16 = true;
+    bool fits = true;
     for (int s2 = 0; s2 < nsub; s2++) {
       long long ms = sub_ptr[s2 + 1] - sub_ptr[s2], nz = lrp_ptr[s2 + 1] - lrp_ptr[s2], e = nz - ms;
-      if (ms >= 65535) fits16 = false;
-      long long bound = 16 + 2 * ms * (16 + 48) + ms * (8 + ru) + e * (2 + vb);   // header + 3 paddings per group
-      bound = bound + bound / 3 + ring;                     // ring-period padding: <= one chunk per ring
+      if (ms >= 65534) fits = false;                       // 16-bit rows, the zero element and one more
+      long long bound = (2 * ms + e / RAS_K + 5) * (32 + vb) + e * vb;   // (up to two empty groups per sweep)
+      if (bound >= RAS_START_MAX) fits = false;
       boff[s2 + 1] = boff[s2] + ((bound + 15) & ~15LL);
       mmax = std::max(mmax, (int)ms);
     }
-    R.m_max = mmax;
-    // the ring, then the local vector, then one product per entry of a group
-    // (a group holds at most a chunk: 16-bit column + block per entry)
-    int chunk = ring / 4, pmax = chunk / (2 + vb) + 1;
-    R.smem_bytes = ((size_t)mmax * yb + 15) / 16 * 16 + ring + (size_t)pmax * yb;
-    R.smem_path = fits16 && R.smem_bytes <= RAS_SMEM_BUDGET;
+    R.smem_bytes = ((size_t)mmax + 2) * yb;
+    // k_ras_pack's tables: groups per level, then the groups' sizes
+    R.pack_smem = (4 * (size_t)mmax + (size_t)R.max_nnz / RAS_K + 24) * sizeof(int);
+    R.smem_path = fits && R.smem_bytes <= RAS_SMEM_BUDGET && R.pack_smem <= RAS_SMEM_BUDGET;
     if (R.smem_path) {
+      // gather / scatter order: the owned rows first, each part in natural
+      // order (runs of neighbouring cells share their sectors)
+      std::vector<int> gidx(ext.size()), gord(ext.size()), nown(nsub, 0);
+      for (int s2 = 0; s2 < nsub; s2++) {
+        int at = sub_ptr[s2];
+        for (int pass = 0; pass < 2; pass++)
+          for (int a = sub_ptr[s2]; a < sub_ptr[s2 + 1]; a++)
+            if ((owned[a] != 0) == (pass == 0)) { gidx[at] = ext[a]; gord[at] = a - sub_ptr[s2]; at++; nown[s2] += pass == 0; }
+      }
       h2d(R.blob_off, boff, st); R.blob.alloc(boff[nsub]);
-      R.gidx.alloc(ext.size()); R.gdesc.alloc(2 * ext.size() + 2 * (size_t)nsub);
+      h2d(R.gidx, gidx, st); h2d(R.gord, gord, st); h2d(R.nown, nown, st);
+      R.gpos.alloc(ext.size()); R.ngrp.alloc(2 * (size_t)nsub);
+      // the lists without unneeded rows rely on a symmetric pattern (which the
+      // interface asks for); one that is not keeps every row
+      dbuf<int> asym;
+      asym.alloc(1);
+      RS_CUDA(cudaMemsetAsync(asym.p, 0, sizeof(int), st));
+      k_pattern_asym<<<grid_for(nb, 256), 256, 0, st>>>(nb, ls->rp.p, ls->ci.p, asym.p);
+      RS_LAUNCHED(1);
+      R.symmetric = d2h(asym.p, 1, st)[0] == 0;
+      R.alvl_rows.alloc(2 * next_tot); R.alvl_ptr.alloc(2 * (next_tot + nsub));
+      R.gdesc.alloc(2 * ext.size() + 8 * (size_t)nsub + nnz_tot / RAS_K + 1);
+      RS_CUDA(cudaStreamSynchronize(st));                  // the host vectors above go out of scope
     }
   }
   if ((size_t)m * 12 > 200 * 1024) RS_FAIL(SIM_ERR_ARG, "RAS: %d cells per subdomain is too many (reduce tile_x/tile_y)", maxcells);
@@ -260,71 +285,95 @@ __global__ void k_ras_pattern(const int *sub_ptr, const int *lrp_ptr, const int 
 // within a chunk of 32 rows by matching levels, so the fill keeps the
 // ascending order).  Blocks
 // whose pattern does not fit in shared memory take k_ras_levels_serial.
+//
+// The apply's own row lists (alvl_rows, alvl_ptr) leave out the rows whose
+// solution no owned row depends on: only owned rows are written back, and
+// row i of the U sweep is needed when i is owned or some needed row c < i
+// has it in its U part (c's entry i; the pattern is symmetric, so i's entry
+// c), row i of the L sweep when the U sweep needs it or some needed row
+// c > i does.  Both closures follow the level recurrences, so the flags ride
+// along with the levels (bit 0 of the stored value).
 __global__ void __launch_bounds__(128) k_ras_levels(const int *sub_ptr, const int *lrp_ptr, const int *frp,
-                                                    const int *fci, int *lvl, int *lvl_rows, int *nlev,
-                                                    int *lvl_ptr, int *err) {
+                                                    const int *fci, const int *perm, const uint8_t *owned, int *lvl,
+                                                    int *lvl_rows, int *nlev, int *lvl_ptr, int *alvl_rows,
+                                                    int *alvl_ptr, int *err) {   // alvl_rows NULL: no pruned lists
   extern __shared__ int lsm[];
   int s = blockIdx.x, base = sub_ptr[s], m = sub_ptr[s + 1] - base, pbase = lrp_ptr[s], fbase = base + s;
   int nnz = frp[fbase + m] - frp[fbase];
   const int *rpg = frp + fbase, *cig = fci + pbase + frp[fbase];
-  int *srp = lsm, *sci = srp + (m + 1), *LvL = sci + nnz, *LvU = LvL + m, *cnt = LvU + m;   // cnt: 2 (m + 1)
+  // cnt (2 or 4 arrays of m + 1) takes the columns' place once the levels
+  // are known, or the space behind them where the columns are fewer
+  const int sets = alvl_rows ? 4 : 2;
+  int *srp = lsm, *LvL = srp + (m + 1), *LvU = LvL + m, *sci = LvU + m;
+  int *cnt = nnz >= sets * (m + 1) ? sci : sci + nnz;
   for (int k = threadIdx.x; k <= m; k += blockDim.x) srp[k] = rpg[k] - rpg[0];
   for (int k = threadIdx.x; k < nnz; k += blockDim.x) sci[k] = cig[k];
   for (int k = threadIdx.x; k < m; k += blockDim.x) { LvL[k] = -1; LvU[k] = -1; }
-  for (int k = threadIdx.x; k < 2 * (m + 1); k += blockDim.x) cnt[k] = 0;
   __syncthreads();
   // L levels: thread t takes rows t, t + nt, ... ascending and waits (in
   // shared memory) for each column c < i to have its level; every wait is
   // on a lower row, taken earlier by its thread, so the waits end.  U levels
   // the same from the last row down.  Each wait is bounded: past the limit
-  // the kernel records code 5 and takes 0 for that level.
+  // the kernel records code 5 and takes 0 for that level.  Stored: 2 level +
+  // needed (L pass: by the U sweep; U pass: by the L sweep).
   volatile int *vL = LvL, *vU = LvU;
   const int LIMIT = 1 << 22;
   bool bad = false;
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    int l = 0;
+    int l = 0, need = owned[base + perm[base + i]] ? 1 : 0;
     for (int q = srp[i]; q < srp[i + 1]; q++) {
       int c = sci[q];
       if (c >= i) break;                            // columns ascending
       int v, spins = 0;
       while ((v = vL[c]) < 0 && ++spins < LIMIT) {}
-      if (v < 0) { bad = true; v = 0; }
-      l = max(l, v + 1);
+      if (v < 0) { bad = true; v = 1; }
+      l = max(l, (v >> 1) + 1);
+      need |= v & 1;
     }
-    vL[i] = l;
+    vL[i] = 2 * l + need;
   }
+  __syncthreads();
   for (int i = m - 1 - (int)threadIdx.x; i >= 0; i -= blockDim.x) {
-    int u = 0;
+    int u = 0, need = LvL[i] & 1;
     for (int q = srp[i + 1] - 1; q >= srp[i]; q--) {
       int c = sci[q];
       if (c <= i) break;
       int v, spins = 0;
       while ((v = vU[c]) < 0 && ++spins < LIMIT) {}
-      if (v < 0) { bad = true; v = 0; }
-      u = max(u, v + 1);
+      if (v < 0) { bad = true; v = 1; }
+      u = max(u, (v >> 1) + 1);
+      need |= v & 1;
     }
-    vU[i] = u;
+    vU[i] = 2 * u + need;
   }
   if (bad) atomicExch(err, 5);
   __syncthreads();
-  // counts per level, then per warp (0: L, 1: U) the scan and the fill
+  for (int k = threadIdx.x; k < sets * (m + 1); k += blockDim.x) cnt[k] = 0;
+  __syncthreads();
+  // counts per level, then per warp (0: L, 1: U, 2 and 3: L and U with the
+  // needed rows only) the scan and the fill
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    atomicAdd(&cnt[LvL[i]], 1);
-    atomicAdd(&cnt[(m + 1) + LvU[i]], 1);
+    int l = LvL[i], u = LvU[i];
+    atomicAdd(&cnt[l >> 1], 1);
+    atomicAdd(&cnt[(m + 1) + (u >> 1)], 1);
+    if (sets == 4 && (u & 1)) atomicAdd(&cnt[2 * (m + 1) + (l >> 1)], 1);
+    if (sets == 4 && (l & 1)) atomicAdd(&cnt[3 * (m + 1) + (u >> 1)], 1);
+    lvl[2 * base + i] = l >> 1; lvl[2 * base + m + i] = u >> 1;
   }
   __syncthreads();
   int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int k = threadIdx.x; k < m; k += blockDim.x) { lvl[2 * base + k] = LvL[k]; lvl[2 * base + m + k] = LvU[k]; }
-  if (wid > 1) return;
-  bool upper = wid == 1;
-  const int *Lv = upper ? LvU : LvL;
-  int *c = cnt + (upper ? m + 1 : 0);
-  int *pp = lvl_ptr + 2 * (base + s) + (upper ? m + 1 : 0);
-  int *rr = lvl_rows + 2 * base + (upper ? m : 0);
-  // number of levels: one past the last non-empty count
+  if (wid > 1 && !alvl_rows) return;
+  const bool upper = wid & 1, some = wid > 1;
+  const int *Lv = upper ? LvU : LvL, *Nd = upper ? LvL : LvU;   // a row's flag sits with the other level
+  int *c = cnt + wid * (m + 1), *c0 = cnt + (upper ? m + 1 : 0);
+  int *pp = (some ? alvl_ptr : lvl_ptr) + 2 * (base + s) + (upper ? m + 1 : 0);
+  int *rr = (some ? alvl_rows : lvl_rows) + 2 * base + (upper ? m : 0);
+  // number of levels: one past the last non-empty count (of all rows: the
+  // counts become cursors below, so both warps of a triangle look first)
   int nl = 0;
-  for (int k = lane; k < m; k += 32) if (c[k]) nl = max(nl, k + 1);
+  for (int k = lane; k < m; k += 32) if (c0[k]) nl = max(nl, k + 1);
   for (int o = 16; o > 0; o >>= 1) nl = max(nl, __shfl_xor_sync(0xffffffffu, nl, o));
+  if (alvl_rows) __syncthreads(); else asm volatile("bar.sync 1, 64;" ::: "memory");
   // exclusive scan of the counts into pp[0..nl] and the cursors c[0..nl)
   int run = 0;
   for (int k0 = 0; k0 <= nl; k0 += 32) {
@@ -336,14 +385,16 @@ __global__ void __launch_bounds__(128) k_ras_levels(const int *sub_ptr, const in
   }
   __syncwarp();
   for (int i0 = 0; i0 < m; i0 += 32) {
-    int i = i0 + lane, lv = i < m ? Lv[i] : -1 - lane;
+    int i = i0 + lane;
+    bool in = i < m && (!some || (Nd[i] & 1));
+    int lv = in ? Lv[i] >> 1 : -1 - lane;
     unsigned grp = __match_any_sync(0xffffffffu, lv);
-    if (i < m) rr[c[lv] + __popc(grp & ((1u << lane) - 1u))] = i;
+    if (in) rr[c[lv] + __popc(grp & ((1u << lane) - 1u))] = i;
     __syncwarp();
-    if (i < m && lane == __ffs(grp) - 1) c[lv] += __popc(grp);
+    if (in && lane == __ffs(grp) - 1) c[lv] += __popc(grp);
     __syncwarp();
   }
-  if (lane == 0) nlev[2 * s + (upper ? 1 : 0)] = nl;
+  if (lane == 0 && !some) nlev[2 * s + (upper ? 1 : 0)] = nl;
 }
 
 // the same, one thread per triangle walking the rows serially from global
@@ -474,15 +525,18 @@ void ras_setup(sim_ls_s *ls) {
   k_ras_pattern<<<R.nsub, 256, 0, s>>>(R.sub_ptr.p, R.lrp_ptr.p, R.lrp.p, R.lrlen.p, R.lci.p, R.lsrc.p, R.perm.p,
                                        R.ipos.p, R.frp.p, R.fci.p, R.fdiag.p, fsrc.p);
   // level sets from shared memory when the largest pattern fits
-  size_t lsmem = (5 * (size_t)R.max_ext + 3 + (size_t)R.max_nnz) * sizeof(int);
+  size_t lsmem = R.lvl_smem[1];
   static bool lattr = false;
   if (!lattr) {
     RS_CUDA(cudaFuncSetAttribute(k_ras_levels, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     lattr = true;
   }
+  R.pruned = R.smem_path && R.symmetric && lsmem <= 200 * 1024;   // the apply's lists leave unneeded rows out
+  if (!R.pruned) lsmem = R.lvl_smem[0];
   if (lsmem <= 200 * 1024)
-    k_ras_levels<<<R.nsub, 128, lsmem, s>>>(R.sub_ptr.p, R.lrp_ptr.p, R.frp.p, R.fci.p, R.lvl.p, R.lvl_rows.p,
-                                            R.nlev.p, R.lvl_ptr.p, ls->errw_dev);
+    k_ras_levels<<<R.nsub, 128, lsmem, s>>>(R.sub_ptr.p, R.lrp_ptr.p, R.frp.p, R.fci.p, R.perm.p, R.owned.p, R.lvl.p,
+                                            R.lvl_rows.p, R.nlev.p, R.lvl_ptr.p, R.pruned ? R.alvl_rows.p : nullptr,
+                                            R.pruned ? R.alvl_ptr.p : nullptr, ls->errw_dev);
   else
     k_ras_levels_serial<<<R.nsub, 64, 0, s>>>(R.sub_ptr.p, R.lrp_ptr.p, R.frp.p, R.fci.p, R.lvl.p, R.lvl_rows.p,
                                               R.nlev.p, R.lvl_ptr.p);
@@ -562,410 +616,418 @@ __global__ void k_ras_apply(const int *sub_ptr, const int *ext, const uint8_t *o
   }
 }
 
-// pack the factors of each subdomain into its blob (one block per subdomain)
+// values as they are stored in the streams
 template <class TB> __device__ __forceinline__ TB to_blob(float v);
 template <> __device__ __forceinline__ float to_blob<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 to_blob<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 template <class TB> __device__ __forceinline__ TB to_blob_d(double v) { return to_blob<TB>((float)v); }
 template <> __device__ __forceinline__ double to_blob_d<double>(double v) { return v; }
-__device__ __forceinline__ float from_blob(float v) { return v; }
-__device__ __forceinline__ double from_blob(double v) { return v; }
-__device__ __forceinline__ float from_blob(__nv_bfloat16 v) { return __bfloat162float(v); }
-// one 2x2 block of the packed factors in a single shared-memory load
-__device__ __forceinline__ void blk4(const __nv_bfloat16 *B, float &b0, float &b1, float &b2, float &b3) {
-  uint2 u = *reinterpret_cast<const uint2 *>(B);
-  __nv_bfloat162 lo = *reinterpret_cast<__nv_bfloat162 *>(&u.x), hi = *reinterpret_cast<__nv_bfloat162 *>(&u.y);
-  b0 = __low2float(lo); b1 = __high2float(lo); b2 = __low2float(hi); b3 = __high2float(hi);
-}
-__device__ __forceinline__ void blk4(const float *B, float &b0, float &b1, float &b2, float &b3) {
-  float4 v = *reinterpret_cast<const float4 *>(B);
-  b0 = v.x; b1 = v.y; b2 = v.z; b3 = v.w;
-}
-__device__ __forceinline__ void blk4(const double *B, double &b0, double &b1, double &b2, double &b3) {
-  double2 u = reinterpret_cast<const double2 *>(B)[0], v = reinterpret_cast<const double2 *>(B)[1];
-  b0 = u.x; b1 = u.y; b2 = v.x; b3 = v.y;
-}
-// a -= sum over q in [q0, q1) of B_q y[cols[q]], in the order of q; the
-// entries are taken four at a time so that their column and block loads,
-// then their y loads, are in flight together
-template <class T, class T2, class TB>
-__device__ __forceinline__ void row_sub(T2 &a, int q0, int q1, const uint16_t *cols, const TB *vals, const T2 *y) {
-  for (int q = q0; q < q1; q += 4) {
-    int c[4];
-    T bb[4][4];
-#pragma unroll
-    for (int u = 0; u < 4; u++)
-      if (q + u < q1) { c[u] = cols[q + u]; blk4(vals + 4 * (q + u), bb[u][0], bb[u][1], bb[u][2], bb[u][3]); }
-    T2 yc[4];
-#pragma unroll
-    for (int u = 0; u < 4; u++)
-      if (q + u < q1) yc[u] = y[c[u]];
-#pragma unroll
-    for (int u = 0; u < 4; u++)
-      if (q + u < q1) { a.x -= bb[u][0] * yc[u].x + bb[u][1] * yc[u].y; a.y -= bb[u][2] * yc[u].x + bb[u][3] * yc[u].y; }
-  }
+// BF16 pairs of a stored block
+__device__ __forceinline__ void blk4(unsigned u, unsigned w, float &b0, float &b1, float &b2, float &b3) {
+  b0 = __uint_as_float(u << 16); b1 = __uint_as_float(u & 0xffff0000u);
+  b2 = __uint_as_float(w << 16); b3 = __uint_as_float(w & 0xffff0000u);
 }
 
-// T: factor type (FP32 or FP64), TB: stored value type (T, or BF16).
-// One block per subdomain.  Thread 0 splits the levels into groups (at most
-// 32 rows and group_cap bytes each) and lays them out; then each warp fills
-// whole groups: row records (with the inverse diagonal block for U rows),
-// columns and values in the row's entry order.
+// The groups of one subdomain are numbered from this entry of gdesc on.
+__device__ __forceinline__ size_t ras_group0(int s, int base, int pbase) {
+  return 2 * (size_t)base + 8 * (size_t)s + (size_t)(pbase / RAS_K);
+}
+
+// Packs the factors of each subdomain into its stream (one block of four
+// warps per subdomain; T: factor type, TB: stored type).  A warp takes a
+// level at a time, its lanes the next 32 rows of the level's list, which
+// become one group, or several when a row has more than RAS_K entries.  The
+// groups are counted, numbered, sized and placed, then filled one warp each.
+// (The first version split each level with one thread walking its rows: 0.47
+// ms per setup on the 1M-cell case, bound by that thread's dependent loads.)
 template <class T, class TB>
-__global__ void k_ras_pack(const int *sub_ptr, const int *lrp_ptr, const int *ext, const uint8_t *owned,
-                           const int *perm, const int *frp, const int *fci, const int *fdiag, const T *fv,
-                           const T *dinv, const int *lvl_rows, const int *nlev, const int *lvl_ptr,
-                           const long long *blob_off, unsigned char *blobs, int *gidx, int4 *gdesc,
-                           const int *order, int *err) {
-  int s = order[blockIdx.x], base = sub_ptr[s], m = sub_ptr[s + 1] - base, pbase = lrp_ptr[s], fbase = base + s;
+__global__ void __launch_bounds__(128) k_ras_pack(const int *sub_ptr, const int *lrp_ptr, const int *frp,
+                                                  const int *fci, const int *fdiag, const int *ipos, const int *gord,
+                                                  uint16_t *gpos, const T *fv, const T *dinv, const int *lvl_rows,
+                                                  const int *nlev, const int *lvl_ptr, const long long *blob_off,
+                                                  unsigned char *blobs, uint2 *gdesc, int *ngrp, const int *order,
+                                                  int *err) {
+  const int s = order[blockIdx.x], base = sub_ptr[s], m = sub_ptr[s + 1] - base, pbase = lrp_ptr[s], fbase = base + s;
   const int *pL = lvl_ptr + 2 * (base + s), *pU = pL + (m + 1);
   const int *rL = lvl_rows + 2 * base, *rU = rL + m;
-  int nL = nlev[2 * s], nU = nlev[2 * s + 1];
+  const int nL = nlev[2 * s], nU = nlev[2 * s + 1];
   unsigned char *b = blobs + blob_off[s];
-  int4 *gd = gdesc + 2 * (base + s);                 // room for 2 (m + 1) groups
-  const int VB = 4 * (int)sizeof(TB), RU = rrec_u<TB>(), CAP = group_cap<TB>(), RB = ring_cfg<TB>::R;
-  __shared__ int ngr[3];
+  uint2 *gd = gdesc + ras_group0(s, base, pbase);
+  constexpr int BPP = sizeof(TB) == 2 ? 2 : 1;              // blocks per piece
+  constexpr int PB = sizeof(TB) == 8 ? 32 : 16;             // bytes per row of a piece
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  constexpr int AH = ras_ahead<TB>();
+  __shared__ int ngr, ngl, pad0, pad1;                      // groups, those of the L sweep, the empty ones' starts
   // dynamic shared memory: per level its group count (then the first group's
-  // index), per group its bytes
+  // index), per group its bytes (then its start)
   extern __shared__ int psm[];
-  const int nlevels = (nL > 1 ? nL - 1 : 0) + nU;
+  const int nLw = nL > 1 ? nL - 1 : 0, nlevels = nLw + nU;
   int *lgc = psm, *gby = psm + nlevels + 1;
-  // row i's entries in the factor: [frp, diag) lower, (diag, frp next) upper
-  auto nlo = [&](int i) { return fdiag[base + i] - pbase - frp[fbase + i]; };
-  auto nup = [&](int i) { return frp[fbase + i + 1] - (fdiag[base + i] - pbase) - 1; };
-  // level lv of the sweep order: L levels 1..nL-1, then U levels 0..nU-1
-  auto level_of = [&](int lv, int &sweep, int &a, int &a1) {
-    int nLw = nL > 1 ? nL - 1 : 0;
-    sweep = lv >= nLw;
-    int l = sweep ? lv - nLw : lv + 1;
-    const int *pp = sweep ? pU : pL;
-    a = pp[l]; a1 = pp[l + 1];
-  };
-  // split one level into groups of at most RAS_GROUP_ROWS rows and CAP bytes;
-  // emit(first, rows, entries) for each group in order
+  // positions in gather order
+  for (int k = threadIdx.x; k < m; k += blockDim.x) gpos[base + k] = (uint16_t)ipos[base + gord[base + k]];
+  // groups of one level of the sweep order (L levels 1..nL-1, then U levels):
+  // emit(up, row, entries of the row, first entry, part) in every lane, lanes
+  // beyond the level with entries -1
   auto split = [&](int lv, auto emit) {
-    int sweep, a, a1;
-    level_of(lv, sweep, a, a1);
-    const int *rr = sweep ? rU : rL;
-    int rrec = sweep ? RU : 8;
-    while (a < a1) {
-      int rows = 0, ent = 0;
-      for (;;) {
-        if (a + rows >= a1 || rows == RAS_GROUP_ROWS) break;
-        int i = rr[a + rows], ne = sweep ? nup(i) : nlo(i);
-        int nb = 16 + al16((rows + 1) * rrec) + al16(2 * (ent + ne)) + (ent + ne) * VB;
-        if (rows > 0 && nb > CAP) break;
-        rows++; ent += ne;
+    const bool up = lv >= nLw;
+    const int l = up ? lv - nLw : lv + 1;
+    const int *pp = up ? pU : pL, *rr = up ? rU : rL;
+    const int a1 = pp[l + 1];
+    for (int a = pp[l]; a < a1; a += 32) {
+      int i = 0, ne = -1, q0 = 0;
+      if (a + lane < a1) {
+        i = rr[a + lane];
+        const int d = fdiag[base + i] - pbase;
+        if (up) { q0 = d + 1; ne = frp[fbase + i + 1] - d - 1; }
+        else { q0 = frp[fbase + i]; ne = d - q0; }
       }
-      emit(a, rows, ent, sweep);
-      a += rows;
+      const int kmax = __reduce_max_sync(0xffffffffu, ne);
+      for (int p = 0; p == 0 || p * RAS_K < kmax; p++) emit(up, i, ne, q0, p);
     }
   };
-  for (int lv = threadIdx.x; lv < nlevels; lv += blockDim.x) {       // groups per level
+  for (int lv = wid; lv < nlevels; lv += nwarps) {                   // groups per level
     int c = 0;
-    split(lv, [&](int, int, int, int) { c++; });
-    lgc[lv] = c;
+    split(lv, [&](bool, int, int, int, int) { c++; });
+    if (lane == 0) lgc[lv] = c;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {                                            // first group of each level
-    int acc = 0, nLw = nL > 1 ? nL - 1 : 0, ngL = 0;
-    for (int lv = 0; lv < nlevels; lv++) { int c = lgc[lv]; lgc[lv] = acc; acc += c; if (lv == nLw - 1) ngL = acc; }
-    lgc[nlevels] = acc;
-    ngr[0] = nLw > 0 ? ngL : 0; ngr[1] = acc - ngr[0];
+  auto scan = [&](int *v, int n) {                                   // exclusive, one warp; returns the total
+    int run = 0;
+    for (int k0 = 0; k0 < n; k0 += 32) {
+      int k = k0 + lane, t = k < n ? v[k] : 0, x = t;
+      for (int o = 1; o < 32; o <<= 1) { int y = __shfl_up_sync(0xffffffffu, x, o); if (lane >= o) x += y; }
+      if (k < n) v[k] = run + x - t;
+      run += __shfl_sync(0xffffffffu, x, 31);
+    }
+    return run;
+  };
+  // first group of each level; the L sweep's groups, then the U sweep's, are
+  // filled up to a multiple of AH
+  if (wid == 0) {
+    const int nl = scan(lgc, nLw), padl = (AH - nl % AH) % AH;
+    const int nu = scan(lgc + nLw, nU), padu = (AH - nu % AH) % AH;
+    for (int k = nLw + lane; k < nlevels; k += 32) lgc[k] += nl + padl;
+    if (lane == 0) {
+      ngl = nl + padl; ngr = nl + padl + nu + padu;
+      for (int k = 0; k < padl; k++) gby[nl + k] = 16 + PB;
+      for (int k = 0; k < padu; k++) gby[nl + padl + nu + k] = 16 + PB;
+      pad0 = nl; pad1 = nl + padl + nu;                      // where the empty ones start
+    }
   }
   __syncthreads();
-  for (int lv = threadIdx.x; lv < nlevels; lv += blockDim.x) {       // descriptors and bytes
+  // blocks of a row in part p: its entries from p RAS_K on (at most RAS_K),
+  // after the inverse diagonal block of a U row
+  auto blocks = [&](bool up, int ne, int p) { return ne < 0 || (p > 0 && ne <= p * RAS_K) ? 0 : min(ne - p * RAS_K, RAS_K) + (up ? 1 : 0); };
+  for (int lv = wid; lv < nlevels; lv += nwarps) {                   // bytes of each group
     int g = lgc[lv];
-    split(lv, [&](int a, int rows, int ent, int sweep) {
-      int rrec = sweep ? RU : 8;
-      gd[g] = make_int4(a, rows, ent, sweep);
-      gby[g] = al16(16 + al16(rows * rrec) + al16(2 * ent) + ent * VB);
+    split(lv, [&](bool up, int, int ne, int, int p) {
+      const int nb = blocks(up, ne, p);
+      const bool in = p == 0 ? ne >= 0 : ne > p * RAS_K;
+      const int by = __reduce_add_sync(0xffffffffu, in ? 16 + (nb + BPP - 1) / BPP * PB : 0);
+      if (lane == 0) gby[g] = by;
       g++;
     });
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // offsets: groups in order after a 32-byte stream header, none across the
-    // end of a ring period (moved to the next period instead)
-    int ng = ngr[0] + ngr[1], off = 32;
-    for (int g = 0; g < ng; g++) {
-      int gb = gby[g];
-      if ((off & (RB - 1)) + gb > RB) off = (off + RB - 1) & ~(RB - 1);
-      gd[g].w = (off << 1) | gd[g].w;
-      off += gb;
-    }
-    // the stream must fit its bound (rows and entries only); never true by
+  const int ng = ngr;
+  if (wid == 0) {
+    const int total = scan(gby, ng);
+    // the stream must fit its bound (rows and entries only); never false by
     // construction, checked so that a violation is an error, not an overrun
-    if ((long long)off > blob_off[s + 1] - blob_off[s]) { atomicExch(err, 4); ngr[0] = 0; ngr[1] = 0; off = 32; ng = 0; }
-    ngr[2] = off;
-    int *hdr = (int *)b;
-    hdr[0] = m; hdr[1] = ngr[0]; hdr[2] = ngr[1]; hdr[3] = off;
-    // each group records the next one's start and size: the stream header the first's
-    hdr[4] = ng ? (gd[0].w >> 1) : 0;
-    hdr[5] = ng ? gby[0] : 0;
+    if (lane == 0) {
+      const bool fits = total <= blob_off[s + 1] - blob_off[s];
+      if (!fits) { atomicExch(err, 4); ngr = 0; gd[0] = make_uint2(0, 0); }
+      ngrp[2 * s] = fits ? ngl : 0; ngrp[2 * s + 1] = fits ? ng : 0;
+    }
   }
   __syncthreads();
-  int ng = ngr[0] + ngr[1];
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  for (int g = wid; g < ng; g += nwarps) {
-    int4 d = gd[g];
-    int sweep = d.w & 1, goff = d.w >> 1, rows = d.y, ent = d.z, rrec = sweep ? RU : 8;
-    const int *rr = sweep ? rU : rL;
-    unsigned char *G = b + goff;
-    uint16_t *cols = (uint16_t *)(G + 16 + al16(rows * rrec));
-    TB *vals = (TB *)(G + 16 + al16(rows * rrec) + al16(2 * ent));
-    int i = lane < rows ? rr[d.x + lane] : 0;
-    int ne = lane < rows ? (sweep ? nup(i) : nlo(i)) : 0;
-    int e0 = ne;                                      // exclusive prefix of the entry counts
-    for (int o = 1; o < 32; o <<= 1) { int y = __shfl_up_sync(0xffffffffu, e0, o); if (lane >= o) e0 += y; }
-    e0 -= ne;
-    if (lane == 0) {
-      int *h = (int *)G;
-      h[0] = rows | (ent << 16); h[1] = al16(16 + al16(rows * rrec) + al16(2 * ent) + ent * VB);
-      h[2] = g + 1 < ng ? (gd[g + 1].w >> 1) : 0;                    // where the next group starts
-      h[3] = g + 1 < ng ? gby[g + 1] : 0;                              // and its bytes
-    }
-    if (lane < rows) {
-      uint16_t *rec = (uint16_t *)(G + 16 + lane * rrec);
-      rec[0] = (uint16_t)i; rec[1] = (uint16_t)e0; rec[2] = (uint16_t)(e0 + ne); rec[3] = 0;
-      if (sweep) {
-        TB *dv = (TB *)((unsigned char *)rec + rrec_doff<TB>());
-        const T *dsrc = dinv + 4 * (size_t)(base + i);
-        for (int u = 0; u < 4; u++) dv[u] = to_blob_d<TB>(dsrc[u]);
-      }
-      int q0 = sweep ? fdiag[base + i] - pbase + 1 : frp[fbase + i];
-      for (int k = 0; k < ne; k++) {
-        int q = q0 + k;
-        cols[e0 + k] = (uint16_t)fci[pbase + q];
-        const T *src = fv + 4 * (size_t)(pbase + q);
-        for (int u = 0; u < 4; u++) vals[4 * (e0 + k) + u] = to_blob_d<TB>(src[u]);
-      }
+  if (ngr == 0) return;
+  if (wid == 0 && lane < 2 * (AH - 1)) {                             // empty groups: row m + 1, columns m
+    const int g = lane < AH - 1 ? pad0 + lane : pad1 + lane - (AH - 1);
+    if (g < (lane < AH - 1 ? ngl : ng)) {
+      const unsigned mm = (unsigned)m | (unsigned)m << 16;
+      uint4 *G = reinterpret_cast<uint4 *>(b + gby[g]);
+      G[0] = make_uint4((unsigned)(m + 1) | (unsigned)m << 16, mm, mm, (unsigned)m);
+      for (int k = 0; k < PB / 16; k++) G[1 + k] = make_uint4(0, 0, 0, 0);
+      gd[g] = make_uint2((unsigned)(gby[g] >> 4) | 1u << 20, 0);
     }
   }
-  for (int pos = threadIdx.x; pos < m; pos += blockDim.x) {
-    int x = perm[base + pos];
-    gidx[base + pos] = (ext[base + x] << 1) | (owned[base + x] ? 1 : 0);
+  for (int lv = wid; lv < nlevels; lv += nwarps) {
+    int g = lgc[lv];
+    split(lv, [&](bool up, int i, int ne, int q0, int p) {
+      const bool in = p == 0 ? ne >= 0 : ne > p * RAS_K;
+      const int nb = blocks(up, ne, p), key = in ? nb : -1;
+      // rows by descending block count (equal counts in list order)
+      int rank = 0, before = 0;
+      for (int c = RAS_K + 1; c >= 0; c--) {
+        const unsigned eq = __ballot_sync(0xffffffffu, key == c);
+        if (key == c) rank = before + __popc(eq & ((1u << lane) - 1u));
+        before += __popc(eq);
+      }
+      const int rows = before;
+      unsigned char *G = b + gby[g];
+      // header: the row and its columns, missing ones naming the zero element
+      const int qe = pbase + q0 + p * RAS_K, n = in ? nb - (up ? 1 : 0) : 0;
+      if (in) {
+        unsigned c[RAS_K + 2];
+        c[0] = (unsigned)i; c[RAS_K + 1] = 0;
+#pragma unroll
+        for (int k = 0; k < RAS_K; k++) c[k + 1] = k < n ? (unsigned)fci[qe + k] : (unsigned)m;
+        reinterpret_cast<uint4 *>(G)[rank] = make_uint4(c[0] | c[1] << 16, c[2] | c[3] << 16, c[4] | c[5] << 16, c[6] | c[7] << 16);
+      }
+      unsigned char *at = G + 16 * rows;
+      unsigned nlo = 0, nhi = 0;                         // n[6], n[1..5]
+      const bool fin = ne <= (p + 1) * RAS_K;
+#pragma unroll
+      for (int q = 0; q * BPP <= RAS_K; q++) {
+        const int cnt = __popc(__ballot_sync(0xffffffffu, key > q * BPP));
+        if (key > q * BPP) {
+          TB *dst = reinterpret_cast<TB *>(at + (size_t)PB * rank);
+#pragma unroll
+          for (int u = 0; u < BPP; u++) {
+            const int k = q * BPP + u - (up ? 1 : 0);    // -1: the inverse diagonal block
+            T v[4] = {0, 0, 0, 0};
+            if (k < 0) {
+              if (fin) for (int w = 0; w < 4; w++) v[w] = dinv[4 * (size_t)(base + i) + w];
+              else v[0] = v[3] = T(1);
+            } else if (k < n) {
+              for (int w = 0; w < 4; w++) v[w] = fv[4 * (size_t)(qe + k) + w];
+            }
+            for (int w = 0; w < 4; w++) dst[4 * u + w] = to_blob_d<TB>(v[w]);
+          }
+        }
+        at += PB * cnt;
+        if (q >= 1 && q <= 5) nhi |= (unsigned)cnt << (6 * (q - 1));
+        if (q == 6) nlo = (unsigned)cnt;
+      }
+      if (lane == 0) gd[g] = make_uint2((unsigned)(gby[g] >> 4) | (unsigned)rows << 20 | nlo << 26, nhi);
+      g++;
+    });
   }
 }
-
-// one 2x2 block from the ring at stream offset off: a 32-byte FP64 block
-// may wrap around the ring's end, so its two 16-byte halves are addressed
-// separately (16-byte alignment keeps every other element whole)
-template <int RB> __device__ __forceinline__ void ring_blk4(const unsigned char *ring, int off, const __nv_bfloat16 *,
-                                                           float &b0, float &b1, float &b2, float &b3) {
-  blk4(reinterpret_cast<const __nv_bfloat16 *>(ring + (off & (RB - 1))), b0, b1, b2, b3);
-}
-template <int RB> __device__ __forceinline__ void ring_blk4(const unsigned char *ring, int off, const float *,
-                                                           float &b0, float &b1, float &b2, float &b3) {
-  blk4(reinterpret_cast<const float *>(ring + (off & (RB - 1))), b0, b1, b2, b3);
-}
-template <int RB> __device__ __forceinline__ void ring_blk4(const unsigned char *ring, int off, const double *,
-                                                           double &b0, double &b1, double &b2, double &b3) {
-  double2 u = *reinterpret_cast<const double2 *>(ring + (off & (RB - 1)));
-  double2 v = *reinterpret_cast<const double2 *>(ring + ((off + 16) & (RB - 1)));
-  b0 = u.x; b1 = u.y; b2 = v.x; b3 = v.y;
-}
-
-// explicit round-to-nearest products and sums (no contraction): the
-// entry-parallel sweep forms B_e y_c = fma(b0, y0, b1 y1) and subtracts it
-__device__ __forceinline__ float r_mul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double r_mul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float r_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double r_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ float r_sub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ double r_sub(double a, double b) { return __dsub_rn(a, b); }
 
 template <class T> struct v2_t;
 template <> struct v2_t<float> { typedef float2 type; };
 template <> struct v2_t<double> { typedef double2 type; };
 
-// ------------------------------------------------ bulk copies (TMA) ------
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_fence_init() {
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, uint64_t *bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// bounded wait: gives up after `limit` polls, records `code` in *err and
-// returns false (the hardware copies themselves cannot stall forever; the
-// bound only turns a fault into an error status instead of a hang)
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, unsigned parity, int *err, int code) {
-  for (int it = 0; it < (1 << 22); it++)
-    if (mbar_try_wait(bar, parity)) return true;
-  atomicExch(err, code);
-  return false;
-}
-
-// x = R(A)^{-1} f, one warp per subdomain (one warp per block).  Lane 0
-// keeps the ring NSLOT chunks ahead of the sweep with bulk copies; every lane
-// waits on a chunk's mbarrier before reading it (bounded waits).  The sweep
-// takes one group at a time: lane r solves row r of the group (its entries
-// in stored order), then the warp synchronises; at the end the owned rows
-// are written (or added).
+// x = R(A)^{-1} f, one block per subdomain.  The right-hand side is gathered
+// into y; then group after group, each lane subtracts its row's products in
+// stored order, a = f_i - sum_k B_k y_{c_k} (U rows: times the inverse
+// diagonal block), and stores y_i; at the end the owned rows are written (or
+// added).  Groups depend on earlier ones, so a block's time is its group
+// count (70 to 150 on the 1M-cell case) times one group's latency, which is
+// mostly one warp's own instructions.  They are kept few and free of
+// branches, so that the loads of a later group fill the waits of the current
+// one (a uniform branch costs about as much as a block's product; the same
+// sweep with a test per entry took 108 us per launch on the 1M-cell case): a group's pieces come straight from global memory into registers,
+// ras_ahead groups early (every lane its own row; no ring, no waits), missing
+// entries multiply the zero element, and what a lane or a group does not
+// have keeps an earlier group's values, which only ever multiply that zero
+// or are not stored.  A bulk prefetch into L2 runs RAS_PF_BYTES ahead of the
+// loads.  20 blocks per SM (at most 96 registers): with 113 the 2500
+// subdomains of the 1M-cell case needed a second wave.
+//
+// Per launch in the solver, against the sweep it replaces (factors through a
+// shared-memory ring, products by entry, then sums by row): 1M cells, BF16,
+// 137 -> 84 us; 200k, FP32, 74 -> 44 us; 65k, BF16, 75 -> 36 us; 207k, FP64,
+// 190 -> 98 us; 2,000 cells, FP64, 54 -> 34 us.
+//
+// FP64: the pipe takes 64 cycles per warp instruction whatever the number of
+// active lanes (measured), so two lanes share a row, one component each, and
+// a block has two warps: half the FP64 instructions in each warp's chain,
+// and the four sub-partitions' pipes evenly used; slots that none of a warp's
+// rows has are skipped.
+#define RAS_PF_BYTES 8192
+#define RAS_PF_STEP 2048
+template <class T> __host__ __device__ constexpr int ras_threads() { return sizeof(T) == 8 ? 64 : 32; }
+template <int NP> struct ras_group { uint2 d; uint4 h; uint4 p[NP]; };
 template <class T, class Tin, bool ACC, class TB>
-__global__ void __launch_bounds__(32) k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs,
-                                                        const int *gidx_all, const int *sub_ptr, const int *order,
-                                                        const Tin *__restrict__ f, T *__restrict__ x, int *err,
-                                                        int m_max_all) {
-  constexpr int RB = ring_cfg<TB>::R, CB = ring_cfg<TB>::C, NSLOT = RB / CB, RU = rrec_u<TB>();
-  extern __shared__ uint4 sm4[];
-  __shared__ uint64_t bar[NSLOT];
+__global__ void __launch_bounds__(ras_threads<T>(), sizeof(TB) == 2 ? 20 : sizeof(T) == 4 ? 16 : 8)
+k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const int *gidx_all, const uint16_t *gpos_all,
+                   const int *nown, const uint2 *gdesc, const int *ngrp, const int *lrp_ptr, const int *sub_ptr,
+                   const int *order, const Tin *__restrict__ f, T *__restrict__ x) {
+  constexpr bool D = sizeof(T) == 8;                   // FP64: two lanes per row
+  constexpr int BS = ras_threads<T>(), BPP = sizeof(TB) == 2 ? 2 : 1, NP = RAS_K / BPP + 1, AHEAD = ras_ahead<TB>();
   typedef typename v2_t<T>::type T2;
   typedef typename v2_t<Tin>::type Tin2;
-  const int lane = threadIdx.x;
-  const int s = order[blockIdx.x];
+  extern __shared__ uint4 sm4[];
+  T2 *y = reinterpret_cast<T2 *>(sm4);
+  const int tid = threadIdx.x, row_of = D ? tid >> 1 : tid, comp = tid & 1;
+  const int s = order[blockIdx.x], base = sub_ptr[s], m = sub_ptr[s + 1] - base, no = nown[s];
+  const int ngl = ngrp[2 * s], ng = ngrp[2 * s + 1];
+  const int *gidx = gidx_all + base;
+  const uint16_t *gpos = gpos_all + base;
   const unsigned char *st = blobs + blob_off[s];
-  const int *gidx = gidx_all + sub_ptr[s];
-  unsigned char *ring = reinterpret_cast<unsigned char *>(sm4);
-  T2 *y = reinterpret_cast<T2 *>(ring + RB);
-  const int m = sub_ptr[s + 1] - sub_ptr[s];
-  T2 *P = reinterpret_cast<T2 *>(reinterpret_cast<unsigned char *>(y) + (((size_t)m_max_all * sizeof(T2) + 15) & ~(size_t)15));
-  // header: m, L groups, U groups, stream bytes, first group's start and bytes
-  const int4 hd = *reinterpret_cast<const int4 *>(st);
-  const int ngL = hd.y, ng = hd.y + hd.z, total = hd.w;
-  int cons = reinterpret_cast<const int *>(st)[4];
-  int cur = reinterpret_cast<const int *>(st)[5];   // the group's bytes (each header names the next one's)
-  const int nchunk = (total + CB - 1) / CB;
-  if (lane == 0) {
-    for (int k = 0; k < NSLOT; k++) mbar_init(&bar[k], 1);
-    mbar_fence_init();
+  const uint4 *st_h = reinterpret_cast<const uint4 *>(st) + row_of, *st_b = reinterpret_cast<const uint4 *>(st) + tid;
+  const uint2 *gd = gdesc + ras_group0(s, base, lrp_ptr[s]);
+  const int bound = (int)(blob_off[s + 1] - blob_off[s]), glast = max(ng - 1, 0);
+  auto sync = [&]() { if (D) __syncthreads(); else __syncwarp(); };
+  int pf = min(bound, RAS_PF_BYTES);                   // the stream is prefetched into L2 up to here
+  if (tid == 0)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(st), "r"(pf) : "memory");
+  ras_group<NP> S[AHEAD];
+  const unsigned mm = (unsigned)m | (unsigned)m << 16;
+#pragma unroll
+  for (int k = 0; k < AHEAD; k++) {
+    S[k].h = make_uint4(mm, mm, mm, mm);
+#pragma unroll
+    for (int q = 0; q < NP; q++) S[k].p[q] = make_uint4(0, 0, 0, 0);
   }
-  __syncwarp();
-  int issued = 0;                                    // lane 0: chunks issued
-  auto issue_upto = [&](int lim) {
-    for (; issued < lim && issued < nchunk; issued++) {
-      int len = total - issued * CB < CB ? total - issued * CB : CB;
-      uint64_t *bk = &bar[issued % NSLOT];
-      mbar_arrive_expect_tx(bk, (unsigned)len);
-      bulk_g2s(ring + (issued % NSLOT) * CB, st + (size_t)issued * CB, (unsigned)len, bk);
+  // descriptors of the next groups to load, fetched two groups before their use
+  int gq = 0;
+  auto fetch_desc = [&]() { const uint2 d = __ldg(gd + min(gq, glast)); gq++; return d; };
+  uint2 dq0 = fetch_desc(), dq1 = fetch_desc();
+  // the next group into a register set
+  auto load = [&](ras_group<NP> &G) {
+    const uint2 d = dq0;
+    dq0 = dq1;
+    dq1 = fetch_desc();
+    const int rows = (d.x >> 20) & 63, start = d.x & 0xfffff;
+    G.d = d;
+    if (row_of < rows) {
+      G.h = __ldg(st_h + start);
+      G.p[0] = __ldg(st_b + (start + rows));
+    }
+    int q = start + (D ? 3 : 2) * rows;                // in units of 16 bytes
+#pragma unroll
+    for (int k = 1; k < NP; k++) {
+      const int n = k < 6 ? (d.y >> (6 * (k - 1))) & 63 : d.x >> 26;
+      if (row_of < n) G.p[k] = __ldg(st_b + q);
+      q += (D ? 2 : 1) * n;
+    }
+    // prefetch (thread 0) when the loads come within RAS_PF_BYTES of it
+    const bool go = 16 * start + RAS_PF_BYTES > pf && pf < bound;
+    const int len = min(bound - pf, RAS_PF_STEP);
+    asm volatile("{\n .reg .pred p;\n setp.ne.s32 p, %2, 0;\n @p cp.async.bulk.prefetch.L2.global [%0], %1;\n}\n" ::"l"(
+                     st + pf), "r"(len), "r"((int)(go && tid == 0)) : "memory");
+    pf += go ? len : 0;
+  };
+  // gather the extended right-hand side
+  const Tin2 *f2 = reinterpret_cast<const Tin2 *>(f);
+  constexpr int GU = D ? 8 : 16;
+  for (int p0 = tid; p0 < m; p0 += GU * BS) {
+    Tin2 v[GU];
+    int pos[GU];
+#pragma unroll
+    for (int u = 0; u < GU; u++)
+      if (p0 + u * BS < m) { v[u] = f2[gidx[p0 + u * BS]]; pos[u] = gpos[p0 + u * BS]; }
+#pragma unroll
+    for (int u = 0; u < GU; u++)
+      if (p0 + u * BS < m) { T2 t; t.x = (T)v[u].x; t.y = (T)v[u].y; y[pos[u]] = t; }
+  }
+#pragma unroll
+  for (int k = 0; k < AHEAD; k++) load(S[k]);
+  if (tid < 2) { T2 z; z.x = 0; z.y = 0; y[m + tid] = z; }
+  sync();
+  // one group: blocks of piece k are k BPP .. ; in a U group block 0 is the
+  // inverse diagonal and block b entry b - 1, in an L group block b entry b
+  auto solve = [&](const ras_group<NP> &G, auto up_) {
+    constexpr int UP = decltype(up_)::value;
+    constexpr int NB = RAS_K + UP;                      // blocks at most
+    const int rows = (G.d.x >> 20) & 63;
+    auto n_of = [&](int k) { return k == 0 ? rows : (int)(k < 6 ? (G.d.y >> (6 * (k - 1))) & 63 : G.d.x >> 26); };
+    auto col = [&](int e) {                             // entry e's column
+      const unsigned w = e == 0 ? G.h.x : e <= 2 ? G.h.y : e <= 4 ? G.h.z : G.h.w;
+      return (e & 1) == 0 ? w >> 16 : w & 0xffffu;
+    };
+    const int row = G.h.x & 0xffffu;
+    const int wfirst = D ? (tid >> 5) * 16 : 0;         // FP64: the warp's first row
+    T2 yc[RAS_K];
+    T a0;
+    [[maybe_unused]] T a1 = 0;
+    if constexpr (D) a0 = reinterpret_cast<const double *>(y + row)[comp];
+    else { const T2 t = y[row]; a0 = t.x; a1 = t.y; }
+#pragma unroll
+    for (int e = 0; e < RAS_K; e++) yc[e] = y[col(e)];
+#pragma unroll
+    for (int k = 0; k * BPP < NB; k++) {
+      if (D && n_of(k) <= wfirst) break;
+#pragma unroll
+      for (int u = 0; u < BPP; u++) {
+        const int e = k * BPP + u - UP;
+        if (e < 0 || e >= RAS_K) continue;
+        if constexpr (D) {
+          const double bx = __hiloint2double(G.p[k].y, G.p[k].x), by = __hiloint2double(G.p[k].w, G.p[k].z);
+          a0 = __fma_rn(-bx, yc[e].x, a0);
+          a0 = __fma_rn(-by, yc[e].y, a0);
+        } else {
+          float b0, b1, b2, b3;
+          if constexpr (BPP == 2) blk4(u ? G.p[k].z : G.p[k].x, u ? G.p[k].w : G.p[k].y, b0, b1, b2, b3);
+          else { b0 = __uint_as_float(G.p[k].x); b1 = __uint_as_float(G.p[k].y); b2 = __uint_as_float(G.p[k].z); b3 = __uint_as_float(G.p[k].w); }
+          // product first, then the subtraction: the same FP32 values as the
+          // sweeps have always had, and a shorter chain than two FMAs per entry
+          a0 = __fsub_rn(a0, __fmaf_rn(b0, yc[e].x, __fmul_rn(b1, yc[e].y)));
+          a1 = __fsub_rn(a1, __fmaf_rn(b2, yc[e].x, __fmul_rn(b3, yc[e].y)));
+        }
+      }
+    }
+    if constexpr (UP) {
+      if constexpr (D) {
+        const double dx = __hiloint2double(G.p[0].y, G.p[0].x), dy = __hiloint2double(G.p[0].w, G.p[0].z);
+        if (rows > wfirst) {
+          const double o = __shfl_xor_sync(0xffffffffu, a0, 1);
+          a0 = __fma_rn(comp ? dy : dx, a0, (comp ? dx : dy) * o);
+        }
+      } else {
+        float d0, d1, d2, d3;
+        if constexpr (BPP == 2) blk4(G.p[0].x, G.p[0].y, d0, d1, d2, d3);
+        else { d0 = __uint_as_float(G.p[0].x); d1 = __uint_as_float(G.p[0].y); d2 = __uint_as_float(G.p[0].z); d3 = __uint_as_float(G.p[0].w); }
+        const float t = d0 * a0 + d1 * a1;
+        a1 = d2 * a0 + d3 * a1;
+        a0 = t;
+      }
+    }
+    if (row_of < rows) {
+      if constexpr (D) reinterpret_cast<double *>(y + row)[comp] = a0;
+      else { T2 t; t.x = a0; t.y = a1; y[row] = t; }
     }
   };
-  if (lane == 0) issue_upto(NSLOT);
-  // gather the extended right-hand side (overlaps the first bulk copies)
-  const Tin2 *f2 = reinterpret_cast<const Tin2 *>(f);
-  for (int p0 = lane; p0 < m; p0 += 8 * 32) {
-    Tin2 v[8];
+  auto sweep = [&](int n, auto up_) {                    // n groups, a multiple of AHEAD
+    for (int g = 0; g < n; g += AHEAD) {
 #pragma unroll
-    for (int u = 0; u < 8; u++) { int pos = p0 + u * 32; if (pos < m) v[u] = f2[gidx[pos] >> 1]; }
+      for (int k = 0; k < AHEAD; k++) { solve(S[k], up_); load(S[k]); sync(); }
+    }
+  };
+  sweep(ngl, std::integral_constant<int, 0>());
+  sweep(ng - ngl, std::integral_constant<int, 1>());
+  for (int p0 = tid; p0 < no; p0 += 8 * BS) {            // the owned rows come first in gather order
+    T2 v[8], w[8];
+    int gi[8];
 #pragma unroll
-    for (int u = 0; u < 8; u++) {
-      int pos = p0 + u * 32;
-      if (pos < m) { T2 t; t.x = (T)v[u].x; t.y = (T)v[u].y; y[pos] = t; }
-    }
-  }
-  __syncwarp();
-  int landed = 0, freed = 0;                         // chunks waited for; chunks behind the sweep
-  bool ok = true;
-  for (int g = 0; g < ng; g++) {
-    // the whole group, its size known from the previous header
-    int need = (cons + cur + CB - 1) / CB;
-    for (; landed < need && ok; landed++) ok = mbar_wait_bounded(&bar[landed % NSLOT], (landed / NSLOT) & 1, err, 3);
-    if (!__all_sync(0xffffffffu, ok)) return;
-    const unsigned char *G = ring + (cons & (RB - 1));         // the group is contiguous in the ring
-    const int4 h4 = *reinterpret_cast<const int4 *>(G);
-    const int rows = h4.x & 0xffff, ent = h4.x >> 16;
-    const bool up = g >= ngL;
-    const int rrec = up ? RU : 8;
-    const uint16_t *cols = reinterpret_cast<const uint16_t *>(G + 16 + al16(rows * rrec));
-    const TB *vals = reinterpret_cast<const TB *>(G + 16 + al16(rows * rrec) + al16(2 * ent));
-    // every entry's product B_e y_c with all lanes (the columns belong to
-    // earlier levels, final already), then each row subtracts its own
-    // products in stored order
-    for (int e = lane; e < ent; e += 32) {
-      T b0, b1, b2, b3;
-      blk4(vals + 4 * e, b0, b1, b2, b3);
-      T2 yc = y[cols[e]], pe;
-      pe.x = r_fma(b0, yc.x, r_mul(b1, yc.y));
-      pe.y = r_fma(b2, yc.x, r_mul(b3, yc.y));
-      P[e] = pe;
-    }
-    __syncwarp();
-    if (lane < rows) {
-      const unsigned char *rec = G + 16 + lane * rrec;
-      const uint2 ri = *reinterpret_cast<const uint2 *>(rec);
-      const int i = ri.x & 0xffff, e0 = ri.x >> 16, e1 = ri.y & 0xffff;
-      T2 a = y[i];
-      for (int e = e0; e < e1; e++) {
-        T2 pe = P[e];
-        a.x = r_sub(a.x, pe.x);
-        a.y = r_sub(a.y, pe.y);
+    for (int u = 0; u < 8; u++)
+      if (p0 + u * BS < no) {
+        gi[u] = gidx[p0 + u * BS];
+        v[u] = y[gpos[p0 + u * BS]];
+        if (ACC) w[u] = reinterpret_cast<const T2 *>(x)[gi[u]];
       }
-      if (up) {
-        T d0, d1, d2, d3;
-        blk4(reinterpret_cast<const TB *>(rec + rrec_doff<TB>()), d0, d1, d2, d3);
-        T2 o;
-        o.x = d0 * a.x + d1 * a.y; o.y = d2 * a.x + d3 * a.y;
-        y[i] = o;
-      } else {
-        y[i] = a;
+#pragma unroll
+    for (int u = 0; u < 8; u++)
+      if (p0 + u * BS < no) {
+        if (ACC) { v[u].x += w[u].x; v[u].y += w[u].y; }
+        reinterpret_cast<T2 *>(x)[gi[u]] = v[u];
       }
-    }
-    cons = h4.z;                                     // the next group's start
-    cur = h4.w;                                      // and bytes
-    __syncwarp();
-    // chunks wholly behind the sweep are free: refill them
-    if (lane == 0 && cons / CB > freed) {
-      freed = cons / CB;
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue_upto(freed + NSLOT);
-    }
-  }
-  for (int pos = lane; pos < m; pos += 32) {
-    int gi = gidx[pos];
-    if (gi & 1) {
-      size_t gg = (size_t)(gi >> 1);
-      T2 v = y[pos];
-      if (ACC) { x[2 * gg] += v.x; x[2 * gg + 1] += v.y; }
-      else { x[2 * gg] = v.x; x[2 * gg + 1] = v.y; }
-    }
   }
 }
 
 void ras_pack(sim_ls_s *ls) {
   ras_data &R = ls->ras;
   if (!R.smem_path) return;
-  size_t psmem = (4 * (size_t)R.m_max + 8) * sizeof(int);      // level group counts and group bytes
   static bool pattr = false;
   if (!pattr) {
-    RS_CUDA(cudaFuncSetAttribute(k_ras_pack<float, __nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    RS_CUDA(cudaFuncSetAttribute(k_ras_pack<float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    RS_CUDA(cudaFuncSetAttribute(k_ras_pack<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    RS_CUDA(cudaFuncSetAttribute(k_ras_pack<float, __nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, RAS_SMEM_BUDGET));
+    RS_CUDA(cudaFuncSetAttribute(k_ras_pack<float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, RAS_SMEM_BUDGET));
+    RS_CUDA(cudaFuncSetAttribute(k_ras_pack<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, RAS_SMEM_BUDGET));
     pattr = true;
   }
-#define RAS_PACK_ARGS R.sub_ptr.p, R.lrp_ptr.p, R.ext.p, R.owned.p, R.perm.p, R.frp.p, R.fci.p, R.fdiag.p
-  if (ls->o.precision == SIM_PREC_MIXED_BF16)
-    k_ras_pack<float, __nv_bfloat16><<<R.nsub, 128, psmem, ls->st>>>(RAS_PACK_ARGS, R.fval32.p, R.dinv32.p, R.lvl_rows.p,
-                                                                R.nlev.p, R.lvl_ptr.p, R.blob_off.p, R.blob.p,
-                                                                R.gidx.p, R.gdesc.p, R.order.p, ls->errw_dev);
-  else if (ls->o.precision != SIM_PREC_FP64)
-    k_ras_pack<float, float><<<R.nsub, 128, psmem, ls->st>>>(RAS_PACK_ARGS, R.fval32.p, R.dinv32.p, R.lvl_rows.p, R.nlev.p,
-                                                        R.lvl_ptr.p, R.blob_off.p, R.blob.p, R.gidx.p, R.gdesc.p,
-                                                        R.order.p, ls->errw_dev);
-  else
-    k_ras_pack<double, double><<<R.nsub, 128, psmem, ls->st>>>(RAS_PACK_ARGS, R.fval.p, R.dinv.p, R.lvl_rows.p, R.nlev.p,
-                                                          R.lvl_ptr.p, R.blob_off.p, R.blob.p, R.gidx.p, R.gdesc.p,
-                                                          R.order.p, ls->errw_dev);
-#undef RAS_PACK_ARGS
+#define RAS_PACK(T, TB, FV, DI)                                                                                      \
+  k_ras_pack<T, TB><<<R.nsub, 128, R.pack_smem, ls->st>>>(                                                           \
+      R.sub_ptr.p, R.lrp_ptr.p, R.frp.p, R.fci.p, R.fdiag.p, R.ipos.p, R.gord.p, R.gpos.p, FV, DI,                  \
+      R.pruned ? R.alvl_rows.p : R.lvl_rows.p, R.nlev.p, R.pruned ? R.alvl_ptr.p : R.lvl_ptr.p, R.blob_off.p,       \
+      R.blob.p, R.gdesc.p, R.ngrp.p, R.order.p, ls->errw_dev)
+  if (ls->o.precision == SIM_PREC_MIXED_BF16) RAS_PACK(float, __nv_bfloat16, R.fval32.p, R.dinv32.p);
+  else if (ls->o.precision != SIM_PREC_FP64) RAS_PACK(float, float, R.fval32.p, R.dinv32.p);
+  else RAS_PACK(double, double, R.fval.p, R.dinv.p);
+#undef RAS_PACK
   RS_LAUNCHED(1);
 }
 
@@ -978,14 +1040,11 @@ __global__ void k_cast_acc(size_t m, const Tin *a, T *b, bool acc) {
 template <class T, class Tin, class TB>
 static void ras_apply_go(sim_ls_s *ls, const Tin *f, T *x, bool acc) {
   ras_data &R = ls->ras;
-  if (acc)
-    k_ras_apply_stream<T, Tin, true, TB><<<R.nsub, 32, R.smem_bytes, ls->st>>>(R.blob_off.p, R.blob.p, R.gidx.p,
-                                                                              R.sub_ptr.p, R.order.p, f, x, ls->errw_dev,
-                                                                              R.m_max);
-  else
-    k_ras_apply_stream<T, Tin, false, TB><<<R.nsub, 32, R.smem_bytes, ls->st>>>(R.blob_off.p, R.blob.p, R.gidx.p,
-                                                                               R.sub_ptr.p, R.order.p, f, x, ls->errw_dev,
-                                                                               R.m_max);
+#define RAS_APPLY_ARGS R.blob_off.p, R.blob.p, R.gidx.p, R.gpos.p, R.nown.p, R.gdesc.p, R.ngrp.p, R.lrp_ptr.p, R.sub_ptr.p, R.order.p, f, x
+  const int bs = ras_threads<T>();
+  if (acc) k_ras_apply_stream<T, Tin, true, TB><<<R.nsub, bs, R.smem_bytes, ls->st>>>(RAS_APPLY_ARGS);
+  else k_ras_apply_stream<T, Tin, false, TB><<<R.nsub, bs, R.smem_bytes, ls->st>>>(RAS_APPLY_ARGS);
+#undef RAS_APPLY_ARGS
 }
 template <class T, class Tin> static void ras_apply_launch(sim_ls_s *ls, const Tin *f, T *x, bool acc);
 template <> void ras_apply_launch<double, double>(sim_ls_s *ls, const double *f, double *x, bool acc) {
