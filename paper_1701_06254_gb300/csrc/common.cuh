@@ -76,15 +76,20 @@ inline thread_local bool rs_pdl_off = false;
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... KArgs, typename... Args>
-inline void launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                       Args... args) {
+inline void launch_pdl_if(bool pdl, void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                          Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid); cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at; cfg.numAttrs = rs_pdl_off ? 0 : 1;
+  cfg.attrs = at; cfg.numAttrs = pdl && !rs_pdl_off ? 1 : 0;
   RS_CUDA(cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...));
+}
+template <typename... KArgs, typename... Args>
+inline void launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                       Args... args) {
+  launch_pdl_if(true, kern, grid, block, smem, s, args...);
 }
 
 // ------------------------------------------------------- device helpers --
@@ -267,7 +272,7 @@ struct sim_ls_s {
   // need only the decoupled matrix): fork after the decoupling, join after both
   cudaStream_t st2 = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  dbuf<int> jd;                 // the step index the graph's kernels read
+  dbuf<int> jd;                 // the step index the graph's kernels read, and its copy for k_scale
   dbuf<double> vcur, zcur64;
   dbuf<float> zcur32, vcur32;
   dbuf<float> w2, isp;          // double-float w planes; split 1 / h_{j+1,j}

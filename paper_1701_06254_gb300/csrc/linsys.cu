@@ -240,7 +240,8 @@ template <> struct vec2_t<float> { typedef float2 type; };
 // y = A x  (f == nullptr) or y = f - A x.  Optional, for CPR: with e, x's
 // pressure components of the first np rows read as x_p + e (the pressure
 // correction added on the fly, the same FP32 sum as a separate pass), and
-// the corrected x written to xout for the warp's own rows; with pout, the
+// the corrected x written to xout for the warp's own rows (with jd, to the
+// *jd-th vector of 2 nb at xout); with pout, the
 // pressure components of y of the first np rows also written there.  One
 // warp owns 32 consecutive block rows: the warp reads its contiguous range of blocks coalesced
 // (lane t takes block q0 + t + 32k), stages the 2-vectors A_q x_{c(q)} in
@@ -251,15 +252,20 @@ template <> struct vec2_t<float> { typedef float2 type; };
 template <class Tv, class Tx, class Tf, class Ty>
 __global__ void __launch_bounds__(SPMV_WARPS * 32)
 k_bsr_spmv(int nb, const int *__restrict__ rp, const int *__restrict__ ci, const Tv *__restrict__ val,
-           const Tx *__restrict__ x, const Tf *__restrict__ f, Ty *__restrict__ y, int np = 0,
-           const Tx *__restrict__ e = nullptr, Tx *__restrict__ xout = nullptr, Ty *__restrict__ pout = nullptr) {
+           const Tx *x, const Tf *f, Ty *y, int np, const Tx *e, Tx *xout, Ty *pout, const int *jd,
+           int pdl) {
+  // (x, f and e come from the kernel before: no __restrict__, so that no load
+  // of them can move above pdl_wait)
   __shared__ Ty prod[SPMV_WARPS][SPMV_CHUNK][2];
   int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int r0 = (blockIdx.x * SPMV_WARPS + wid) * 32;
+  if (pdl) pdl_trigger();
   if (r0 >= nb) return;
   int r = r0 + lane, rend = min(r0 + 32, nb);
   int q0 = rp[r0], q1 = rp[rend];
   int myq0 = r < nb ? rp[r] : q1, myq1 = r < nb ? rp[r + 1] : q1;
+  if (pdl) pdl_wait();                         // the pattern is fixed; everything else is the previous kernels'
+  if (jd) xout += (size_t)*jd * 2 * nb;
   Ty a0 = 0, a1 = 0;
   typedef typename vec2_t<Tx>::type X2;
   for (int c0 = q0; c0 < q1; c0 += SPMV_CHUNK) {
@@ -301,12 +307,19 @@ k_bsr_spmv(int nb, const int *__restrict__ rp, const int *__restrict__ ci, const
   }
 }
 
+// Programmatic dependent launch for the kernels of an Arnoldi step where they
+// run in one wave of blocks (the SpMV: 8 blocks of 256 rows per SM): there a
+// launch's latency weighs (2,000 cells: 38 -> 23 us of Gram-Schmidt per step,
+// with the fewer launches of ortho_tail).  Beyond, the wait in every block
+// costs more than the overlap gives.
+static int arnoldi_pdl(int nb) { return nb <= 152 * 8 * SPMV_WARPS * 32; }
+
 template <class Tv, class Tx, class Tf, class Ty>
 static void spmv(const sim_ls_s *ls, const Tv *val, const Tx *x, const Tf *f, Ty *y, cudaStream_t s,
-                 const Tx *e = nullptr, Tx *xout = nullptr, Ty *pout = nullptr) {
-  unsigned g = grid_for(ls->nb, SPMV_WARPS * 32);
-  k_bsr_spmv<Tv, Tx, Tf, Ty><<<g, SPMV_WARPS * 32, 0, s>>>(ls->nb, ls->rp.p, ls->ci.p, val, x, f, y, ls->n, e, xout,
-                                                           pout);
+                 const Tx *e = nullptr, Tx *xout = nullptr, Ty *pout = nullptr, const int *jd = nullptr) {
+  const int pdl = arnoldi_pdl(ls->nb);
+  launch_pdl_if(pdl, k_bsr_spmv<Tv, Tx, Tf, Ty>, grid_for(ls->nb, SPMV_WARPS * 32), SPMV_WARPS * 32, 0, s, ls->nb,
+                ls->rp.p, ls->ci.p, val, x, f, y, ls->n, e, xout, pout, jd, pdl);
   RS_LAUNCHED(1);
 }
 
@@ -314,17 +327,21 @@ static void spmv(const sim_ls_s *ls, const Tv *val, const Tx *x, const Tf *f, Ty
 // lo (vallo) FP32 planes, z FP32 (exact), each block's products and each
 // row's sum carried as double-float on the FP32 pipes (the FP64 SpMV above is
 // bound by the FP64 rate).  Same traversal as k_bsr_spmv; w goes straight into
-// its hi / lo planes (w, w + 2 nb).
+// its hi / lo planes (w, w + 2 nb).  With jd, z is also copied into the *jd-th
+// vector of zout (its own rows, just read: no pass of its own).
 __global__ void __launch_bounds__(SPMV_WARPS * 32)
 k_bsr_spmv_df(int nb, const int *__restrict__ rp, const int *__restrict__ ci, const float *__restrict__ vh,
-              const float *__restrict__ vl, const float *__restrict__ x, float *__restrict__ w) {
+              const float *__restrict__ vl, const float *x, float *w, float *zout, const int *jd,
+              int pdl) {
   __shared__ float2 prod[SPMV_WARPS][SPMV_CHUNK][2];
   int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int r0 = (blockIdx.x * SPMV_WARPS + wid) * 32;
+  if (pdl) pdl_trigger();
   if (r0 >= nb) return;
   int r = r0 + lane, rend = min(r0 + 32, nb);
   int q0 = rp[r0], q1 = rp[rend];
   int myq0 = r < nb ? rp[r] : q1, myq1 = r < nb ? rp[r + 1] : q1;
+  if (pdl) pdl_wait();
   float a0h = 0.0f, a0l = 0.0f, a1h = 0.0f, a1l = 0.0f;
   for (int c0 = q0; c0 < q1; c0 += SPMV_CHUNK) {
     int c1 = min(c0 + SPMV_CHUNK, q1);
@@ -359,11 +376,14 @@ k_bsr_spmv_df(int nb, const int *__restrict__ rp, const int *__restrict__ ci, co
     size_t nu = 2 * (size_t)nb;
     reinterpret_cast<float2 *>(w)[r] = make_float2(a0h, a1h);
     reinterpret_cast<float2 *>(w + nu)[r] = make_float2(a0l, a1l);
+    if (jd) reinterpret_cast<float2 *>(zout + (size_t)*jd * nu)[r] = reinterpret_cast<const float2 *>(x)[r];
   }
 }
-static void spmv_df(const sim_ls_s *ls, const float *x, float *w, cudaStream_t s) {
-  unsigned g = grid_for(ls->nb, SPMV_WARPS * 32);
-  k_bsr_spmv_df<<<g, SPMV_WARPS * 32, 0, s>>>(ls->nb, ls->rp.p, ls->ci.p, ls->val32.p, ls->vallo.p, x, w);
+static void spmv_df(const sim_ls_s *ls, const float *x, float *w, cudaStream_t s, float *zout = nullptr,
+                    const int *jd = nullptr) {
+  const int pdl = arnoldi_pdl(ls->nb);
+  launch_pdl_if(pdl, k_bsr_spmv_df, grid_for(ls->nb, SPMV_WARPS * 32), SPMV_WARPS * 32, 0, s, ls->nb, ls->rp.p,
+                ls->ci.p, ls->val32.p, ls->vallo.p, x, w, zout, jd, pdl);
   RS_LAUNCHED(1);
 }
 // lo plane of the decoupled matrix: val - (double)val32
@@ -381,17 +401,6 @@ void ls_spmv64_untimed(sim_ls_s *ls, const double *x, double *y) {
 }
 
 // ------------------------------------------------------- CPR pieces ------
-template <class Ti, class To>
-__global__ void k_gather_p(int n, const Ti *r, To *f) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) f[i] = (To)r[2 * (size_t)i];
-}
-template <class T>
-__global__ void k_add_p(int n, const T *e, T *x) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) x[2 * (size_t)i] += e[i];
-}
-
 // CPR-FPF (Algorithm 2): z = R^{-1} v; r = v - A z; z += Pi_p M(A_pp)^{-1} Pi_r r;
 // r = v - A z; z += R^{-1} r.  FP64 preconditioner: A is the decoupled FP64
 // matrix; mixed: FP32 matrix, factors, hierarchy and vectors (FP64 coarsest).
@@ -403,7 +412,6 @@ static float *cpr_scratch(sim_ls_s *ls) {
 
 void ls_cpr(sim_ls_s *ls, const double *v, double *z64, float *z32) {
   cudaStream_t s = ls->st;
-  int n = ls->n;
   amg_level &L0 = ls->amg.lev[0];
   if (ls->o.precision != SIM_PREC_FP64) {
     // the first RAS stage into a scratch vector; the second SpMV reads it
@@ -417,15 +425,11 @@ void ls_cpr(sim_ls_s *ls, const double *v, double *z64, float *z32) {
     { rs_timed tm(ls, SIM_T_SPMV_PREC); spmv<float, float, double, float>(ls, ls->val32.p, zt, v, r, s, L0.x32.p, z32); }  // z = z + P e, r = v - A z
     ls_ras_apply<float, float>(ls, r, z32, true);                                      // RAS, added
   } else {
-    double *z = z64, *r = ls->x64a.p;
-    ls_ras_apply<double, double>(ls, v, z, false);
-    { rs_timed tm(ls, SIM_T_SPMV_PREC); spmv<double, double, double, double>(ls, ls->val.p, z, v, r, s); }
-    k_gather_p<double, double><<<grid_for(n, 256), 256, 0, s>>>(n, r, L0.f.p);
-    RS_LAUNCHED(1);
+    double *z = z64, *r = ls->x64a.p, *zt = ls->x64b.p;
+    ls_ras_apply<double, double>(ls, v, zt, false);
+    { rs_timed tm(ls, SIM_T_SPMV_PREC); spmv<double, double, double, double>(ls, ls->val.p, zt, v, r, s, nullptr, nullptr, L0.f.p); }
     { rs_timed tm(ls, SIM_T_VCYCLE); if (ls->capturing) amg_vcycle<double>(ls->amg, 0, s); else amg_vcycle_graph<double>(ls->amg, s); }
-    k_add_p<double><<<grid_for(n, 256), 256, 0, s>>>(n, L0.x.p, z);
-    RS_LAUNCHED(1);
-    { rs_timed tm(ls, SIM_T_SPMV_PREC); spmv<double, double, double, double>(ls, ls->val.p, z, v, r, s); }
+    { rs_timed tm(ls, SIM_T_SPMV_PREC); spmv<double, double, double, double>(ls, ls->val.p, zt, v, r, s, L0.x.p, z); }
     ls_ras_apply<double, double>(ls, r, z, true);
   }
 }
@@ -435,7 +439,6 @@ void ls_cpr(sim_ls_s *ls, const double *v, double *z64, float *z32) {
 // as ls_cpr's mixed branch.
 void ls_cpr32(sim_ls_s *ls, const float *v, float *z) {
   cudaStream_t s = ls->st;
-  int n = ls->n;
   amg_level &L0 = ls->amg.lev[0];
   float *r = ls->x32b.p, *zt = cpr_scratch(ls);
   ls_ras_apply<float, float>(ls, v, zt, false);                                        // RAS
@@ -561,15 +564,15 @@ void ls_setup(sim_ls_s *ls) {
 // clear, so the host never waits on it.  Each pass is one sweep over the
 // rows: a block owns a fixed row range, threads accumulate their part of
 // each dot product, warps reduce with shuffles and the block writes one
-// partial per vector; a second kernel adds the partials in block order, so
-// results do not depend on scheduling.
+// partial per vector; the block that finishes last adds the partials in block
+// order, so results do not depend on scheduling.  In FP64 the dot products
+// walk the basis upwards and the update downwards, so that the update starts
+// on the vectors that are still in L2.
 #define ORTHO_BS 256
-// Each block owns a fixed chunk of ORTHO_CH rows and keeps its slice of w in
-// shared memory.  Basis vectors are streamed vector-outer, rows-inner, so
-// loads are coalesced and independent.
-#define ORTHO_CH 2048
-#define ORTHO_CH_DF 8192
-static int ortho_blocks(int nu) { return (nu + ORTHO_CH - 1) / ORTHO_CH; }
+// Each block owns a fixed chunk of at most ORTHO_CH rows and keeps its slice
+// of w in shared memory.  Basis vectors are streamed vector-outer, rows-inner,
+// so loads are coalesced and independent.
+#define ORTHO_CH 8192
 
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
@@ -612,87 +615,6 @@ __device__ __forceinline__ double warp_sum8_d(const double *a, int lane) {
   t += __shfl_xor_sync(0xffffffffu, t, 2);
   t += __shfl_xor_sync(0xffffffffu, t, 1);
   return t;
-}
-
-// part[k][b] = V_k . w over the block's rows (k < nv); with_norm: part[nv][b] = w . w
-__global__ void __launch_bounds__(ORTHO_BS) k_ortho_dots(int nu, int nv, const double *__restrict__ V,
-                                                         const double *__restrict__ w, double *part, int with_norm,
-                                                         const int *cond, const int *jd) {
-  if (cond && *cond == 0) return;
-  if (jd) nv = *jd + 1;                        // graph replay: the step index lives on the device
-  extern __shared__ double ws[];             // ORTHO_CH doubles (dynamic)
-  __shared__ double red[2][ORTHO_BS / 32][ORTHO_G];
-  int nblk = gridDim.x, i0 = blockIdx.x * ORTHO_CH, len = min(ORTHO_CH, nu - i0);
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int t = threadIdx.x; t < len; t += ORTHO_BS) ws[t] = w[i0 + t];
-  __syncthreads();
-  int nt = nv + (with_norm ? 1 : 0);
-  for (int k0 = 0, grp = 0; k0 < nt; k0 += ORTHO_G, grp ^= 1) {
-    const double *vp[ORTHO_G];
-    double acc[ORTHO_G];
-#pragma unroll
-    for (int g = 0; g < ORTHO_G; g++) {
-      int k = k0 + g;                          // vector nv is w itself (its squared norm)
-      vp[g] = k < nv ? V + (size_t)k * nu + i0 : (k == nv ? w + i0 : nullptr);
-      acc[g] = 0.0;
-    }
-    for (int t = threadIdx.x; t < len; t += ORTHO_BS) {
-      double wt = ws[t];
-#pragma unroll
-      for (int g = 0; g < ORTHO_G; g++)
-        if (vp[g]) acc[g] += __ldg(vp[g] + t) * wt;
-    }
-    double tot = warp_sum8_d(acc, lane);
-    if ((lane & 3) == 0) red[grp][warp][((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = tot;
-    __syncthreads();                           // red[grp] is rewritten two groups later, after another barrier
-    if (threadIdx.x < ORTHO_G && k0 + threadIdx.x < nt) {
-      double s = 0.0;
-      for (int q = 0; q < ORTHO_BS / 32; q++) s += red[grp][q][threadIdx.x];
-      part[(size_t)(k0 + threadIdx.x) * nblk + blockIdx.x] = s;
-    }
-  }
-}
-
-// w -= sum_k h_k V_k over the block's rows, then part[0][b] = ||w||^2
-__global__ void __launch_bounds__(ORTHO_BS) k_ortho_update(int nu, int nv, const double *__restrict__ V, double *w,
-                                                           const double *__restrict__ h, double *part,
-                                                           const int *cond, const int *jd) {
-  if (cond && *cond == 0) return;
-  if (jd) nv = *jd + 1;
-  extern __shared__ double ws[];
-  __shared__ double sred[ORTHO_BS / 32];
-  int i0 = blockIdx.x * ORTHO_CH, len = min(ORTHO_CH, nu - i0);
-  for (int t = threadIdx.x; t < len; t += ORTHO_BS) ws[t] = w[i0 + t];
-  for (int k0 = 0; k0 < nv; k0 += ORTHO_G) {   // each thread updates only its own rows: no barrier needed
-    const double *vp[ORTHO_G];
-    double hk[ORTHO_G];
-#pragma unroll
-    for (int g = 0; g < ORTHO_G; g++) {
-      int k = k0 + g;
-      vp[g] = k < nv ? V + (size_t)k * nu + i0 : nullptr;
-      hk[g] = k < nv ? h[k] : 0.0;
-    }
-    // two rows per thread per iteration: their 16 loads are in flight together
-    for (int t = threadIdx.x; t < len; t += 2 * ORTHO_BS) {
-      int t2 = t + ORTHO_BS;
-      bool two = t2 < len;
-      double v0[ORTHO_G], v1[ORTHO_G];
-#pragma unroll
-      for (int g = 0; g < ORTHO_G; g++) {
-        if (vp[g]) { v0[g] = __ldg(vp[g] + t); if (two) v1[g] = __ldg(vp[g] + t2); }
-      }
-      double s0 = ws[t], s1 = two ? ws[t2] : 0.0;
-#pragma unroll
-      for (int g = 0; g < ORTHO_G; g++)       // same order as one vector at a time: w - h_0 v_0 - h_1 v_1 ...
-        if (vp[g]) { s0 -= hk[g] * v0[g]; if (two) s1 -= hk[g] * v1[g]; }
-      ws[t] = s0;
-      if (two) ws[t2] = s1;
-    }
-  }
-  double n2 = 0.0;
-  for (int t = threadIdx.x; t < len; t += ORTHO_BS) { double v = ws[t]; w[i0 + t] = v; n2 += v * v; }
-  double tot = block_sum_d(n2, sred);
-  if (threadIdx.x == 0) part[blockIdx.x] = tot;
 }
 
 // ------------------------------------------------ double-float basis ----
@@ -769,6 +691,114 @@ __device__ __forceinline__ void reduce_tail(int nout, int nblk, const double *pa
   if (threadIdx.x == 0) *ticket = 0;
 }
 
+// After an update pass (thread 0 of its last block): h_{j+1,j} = ||w|| and its
+// reciprocal (isp: split into hi + lo), the flag for a second pass when the
+// first kept less than 1% of w (||w_1||^2 < 1e-4 ||w||^2, the latter behind
+// the dot products), and in graph replay the step index for k_scale's blocks
+// (jd[0] moves on while they run).
+__device__ __forceinline__ void norm_tail(int nv, const double *nrm, int *flag, const double *h1, double *hnorm,
+                                          float *isp, int *jd) {
+  if (threadIdx.x != 0) return;
+  __threadfence();
+  const double n2 = *(volatile const double *)nrm;
+  if (flag) *flag = n2 < 1e-4 * h1[nv] ? 1 : 0;
+  const double hn = sqrt(n2), inv = hn > 0.0 ? 1.0 / hn : 0.0;
+  hnorm[0] = hn;
+  hnorm[1] = inv;
+  if (isp) { float a, b; df_split(inv, a, b); isp[0] = a; isp[1] = b; }
+  if (jd) jd[1] = jd[0];
+}
+
+// part[k][b] = V_k . w over the block's rows (k < nv); with_norm: part[nv][b] = w . w
+__global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots(int nu, int ch, int nv, const double *__restrict__ V,
+                                                            const double *__restrict__ w, double *part, int with_norm,
+                                                            const int *cond, const int *jd, int *ticket, double *out,
+                                                            int pdl) {
+  if (pdl) { pdl_trigger(); pdl_wait(); }
+  if (cond && *cond == 0) return;
+  if (jd) nv = *jd + 1;                        // graph replay: the step index lives on the device
+  extern __shared__ double ws[];             // ch doubles (dynamic)
+  __shared__ double red[2][ORTHO_BS / 32][ORTHO_G];
+  int nblk = gridDim.x, i0 = blockIdx.x * ch, len = min(ch, nu - i0);
+  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int t = threadIdx.x; t < len; t += ORTHO_BS) ws[t] = w[i0 + t];
+  __syncthreads();
+  int nt = nv + (with_norm ? 1 : 0);
+  for (int k0 = 0, grp = 0; k0 < nt; k0 += ORTHO_G, grp ^= 1) {
+    const double *vp[ORTHO_G];
+    double acc[ORTHO_G];
+#pragma unroll
+    for (int g = 0; g < ORTHO_G; g++) {
+      int k = k0 + g;                          // vector nv is w itself (its squared norm)
+      vp[g] = k < nv ? V + (size_t)k * nu + i0 : (k == nv ? w + i0 : nullptr);
+      acc[g] = 0.0;
+    }
+    for (int t = threadIdx.x; t < len; t += ORTHO_BS) {
+      double wt = ws[t];
+#pragma unroll
+      for (int g = 0; g < ORTHO_G; g++)
+        if (vp[g]) acc[g] += __ldg(vp[g] + t) * wt;
+    }
+    double tot = warp_sum8_d(acc, lane);
+    if ((lane & 3) == 0) red[grp][warp][((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = tot;
+    __syncthreads();                           // red[grp] is rewritten two groups later, after another barrier
+    if (threadIdx.x < ORTHO_G && k0 + threadIdx.x < nt) {
+      double s = 0.0;
+      for (int q = 0; q < ORTHO_BS / 32; q++) s += red[grp][q][threadIdx.x];
+      part[(size_t)(k0 + threadIdx.x) * nblk + blockIdx.x] = s;
+    }
+  }
+  if (last_block(ticket)) reduce_tail(nt, nblk, part, out, ticket);   // out[k] = V_k . w (and ||w||^2)
+}
+
+// w -= sum_k h_k V_k over the block's rows, then part[0][b] = ||w||^2
+__global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update(int nu, int ch, int nv, const double *__restrict__ V,
+                                                              double *w, const double *__restrict__ h, double *part,
+                                                              const int *cond, int *jd, int *ticket, double *nrm,
+                                                              int *flag, const double *h1, double *hnorm, int pdl) {
+  if (pdl) { pdl_trigger(); pdl_wait(); }
+  if (cond && *cond == 0) return;
+  if (jd) nv = *jd + 1;
+  extern __shared__ double ws[];
+  __shared__ double sred[ORTHO_BS / 32];
+  int i0 = blockIdx.x * ch, len = min(ch, nu - i0);
+  for (int t = threadIdx.x; t < len; t += ORTHO_BS) ws[t] = w[i0 + t];
+  for (int k0 = (nv - 1) / ORTHO_G * ORTHO_G; k0 >= 0; k0 -= ORTHO_G) {   // each thread updates only its own rows
+    const double *vp[ORTHO_G];
+    double hk[ORTHO_G];
+#pragma unroll
+    for (int g = 0; g < ORTHO_G; g++) {
+      int k = k0 + g;
+      vp[g] = k < nv ? V + (size_t)k * nu + i0 : nullptr;
+      hk[g] = k < nv ? h[k] : 0.0;
+    }
+    // two rows per thread per iteration: their 16 loads are in flight together
+    for (int t = threadIdx.x; t < len; t += 2 * ORTHO_BS) {
+      int t2 = t + ORTHO_BS;
+      bool two = t2 < len;
+      double v0[ORTHO_G], v1[ORTHO_G];
+#pragma unroll
+      for (int g = 0; g < ORTHO_G; g++) {
+        if (vp[g]) { v0[g] = __ldg(vp[g] + t); if (two) v1[g] = __ldg(vp[g] + t2); }
+      }
+      double s0 = ws[t], s1 = two ? ws[t2] : 0.0;
+#pragma unroll
+      for (int g = 0; g < ORTHO_G; g++)       // one vector at a time
+        if (vp[g]) { s0 -= hk[g] * v0[g]; if (two) s1 -= hk[g] * v1[g]; }
+      ws[t] = s0;
+      if (two) ws[t2] = s1;
+    }
+  }
+  double n2 = 0.0;
+  for (int t = threadIdx.x; t < len; t += ORTHO_BS) { double v = ws[t]; w[i0 + t] = v; n2 += v * v; }
+  double tot = block_sum_d(n2, sred);
+  if (threadIdx.x == 0) part[blockIdx.x] = tot;
+  if (last_block(ticket)) {
+    reduce_tail(1, gridDim.x, part, nrm, ticket);
+    norm_tail(nv, nrm, flag, h1, hnorm, nullptr, jd);
+  }
+}
+
 // k_ortho_dots on pair planes: V vector k at V + 2k nu (hi) and + (2k+1) nu
 // (lo), w at w (hi) and w + nu (lo).  Vector offsets are 32-bit (the basis
 // holds at most 2 (ORTHO_MAXV + 1) nu < 2^31 floats) and each thread takes
@@ -776,10 +806,11 @@ __device__ __forceinline__ void reduce_tail(int nout, int nblk, const double *pa
 __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots_df(int nu, int ch, int nv, const float *__restrict__ V,
                                                                const float *__restrict__ w, double *part,
                                                                int with_norm, const int *cond, const int *jd,
-                                                               int *ticket, double *out) {
+                                                               int *ticket, double *out, int pdl) {
+  if (pdl) { pdl_trigger(); pdl_wait(); }
   if (cond && *cond == 0) return;
   if (jd) nv = *jd + 1;
-  extern __shared__ float2 wp[];               // ORTHO_CH pairs (dynamic)
+  extern __shared__ float2 wp[];               // ch pairs (dynamic)
   __shared__ double red[2][ORTHO_BS / 32][ORTHO_G];
   int nblk = gridDim.x, i0 = blockIdx.x * ch, len = min(ch, nu - i0);
   int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -838,8 +869,10 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots_df(int nu, int ch, i
 // thread per iteration
 __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update_df(int nu, int ch, int nv, const float *__restrict__ V,
                                                                  float *w, const double *__restrict__ h, double *part,
-                                                                 const int *cond, const int *jd, int *ticket,
-                                                                 double *nrm, int *flag, const double *h1) {
+                                                                 const int *cond, int *jd, int *ticket, double *nrm,
+                                                                 int *flag, const double *h1, double *hnorm,
+                                                                 float *isp, int pdl) {
+  if (pdl) { pdl_trigger(); pdl_wait(); }
   if (cond && *cond == 0) return;
   if (jd) nv = *jd + 1;
   extern __shared__ float2 wp[];
@@ -865,7 +898,7 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update_df(int nu, int ch,
         }
       float2 x = wp[t], y = two ? wp[t2] : make_float2(0.0f, 0.0f);
 #pragma unroll
-      for (int g = 0; g < ORTHO_G; g++)       // w - h_0 v_0 - h_1 v_1 ..., one vector at a time
+      for (int g = 0; g < ORTHO_G; g++)       // one vector at a time
         if (g < ng) {
           float2 hk = hs[k0 + g];
           float p, e, s2, err;
@@ -905,24 +938,100 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update_df(int nu, int ch,
   }
   if (last_block(ticket)) {
     reduce_tail(1, gridDim.x, part, nrm, ticket);        // nrm = ||w||^2 after the pass
-    // first pass: flag the second one when it kept less than 1% of w
-    // (||w_1||^2 < 1e-4 ||w||^2, as k_dgks); ||w||^2 sits after the dot products
-    if (flag && threadIdx.x == 0) { __threadfence(); *flag = (*(volatile double *)nrm < 1e-4 * h1[nv]) ? 1 : 0; }
+    norm_tail(nv, nrm, flag, h1, hnorm, isp, jd);
   }
 }
-// V_{j+1} = w / h_{j+1,j}, the reciprocal split once by k_arnoldi_col (isp)
-// v_{j+1} = w / h_{j+1,j} into the basis; with vcur, its hi plane also into
-// the fixed buffer the next graph-replayed step's CPR reads
-__global__ void k_scale_df(int nu, const float *w, const float *isp, float *V, int j1, const int *jd, float *vcur) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (jd) j1 = *jd + 1;
-  if (i >= nu) return;
-  float p, e, h, l;
-  df_mul(w[i], w[(size_t)nu + i], isp[0], isp[1], p, e);
-  df_fast(p, e, h, l);
-  V[(size_t)(2 * j1) * nu + i] = h;
-  V[(size_t)(2 * j1 + 1) * nu + i] = l;
-  if (vcur) vcur[i] = h;
+
+// Hessenberg column j: h = h1 + h2 (h1 without a second pass), h_{j+1,j} =
+// hnorm[0]; previous Givens rotations, a new one, and the residual estimate
+// |g_{j+1}| (host: the step's pinned slot).  One warp; the rotations are a
+// serial recurrence of four FP64 operations a step, which two lanes share
+// (each operation holds the FP64 pipe for 64 cycles).
+// G layout: [0..m*(m+1)) H column-major (m+1 per column), cs[m], sn[m], g[m+1]
+__device__ __forceinline__ void arnoldi_col(int j, int m, const double *h1, const double *h2, const int *flag,
+                                            const double *hnorm, double *G, volatile double *host) {
+  __shared__ double sc[ORTHO_MAXV + 1], scs[ORTHO_MAXV], ssn[ORTHO_MAXV];
+  double *H = G, *cs = G + (size_t)m * (m + 1), *sn = cs + m, *g = sn + m;
+  double *col = H + (size_t)j * (m + 1);
+  const int lane = threadIdx.x & 31;
+  const bool re = *flag != 0;
+  for (int k = lane; k <= j; k += 32) sc[k] = re ? h1[k] + h2[k] : h1[k];
+  for (int k = lane; k < j; k += 32) { scs[k] = cs[k]; ssn[k] = sn[k]; }
+  __syncwarp();
+  const double hn = hnorm[0];
+  double a = sc[0];
+  for (int k = 0; k < j; k++) {                  // lane 0: the rotated entry k, lane 1: what goes on to k + 1
+    const double x = (lane & 1) ? -ssn[k] : scs[k], y = (lane & 1) ? scs[k] : ssn[k];
+    const double t = x * a + y * sc[k + 1];
+    a = __shfl_sync(0xffffffffu, t, 1);
+    if (lane == 0) col[k] = t;
+  }
+  const double rr = sqrt(a * a + hn * hn), q = ((lane & 1) ? hn : a) / rr;
+  const double sj = __shfl_sync(0xffffffffu, q, 1);
+  if (lane != 0) return;
+  cs[j] = q; sn[j] = sj;
+  col[j] = rr; col[j + 1] = 0.0;
+  const double gj = g[j];
+  g[j + 1] = -sj * gj;
+  g[j] = q * gj;
+  host[0] = fabs(g[j + 1]);
+  host[1] = hn;
+  host[2] = re ? 1.0 : 0.0;
+}
+// The end of an Arnoldi step.  Block 0: the Hessenberg column, beside the
+// others' work instead of in front of it, and in graph replay the step
+// counter.  The other blocks: V_{j+1} = w / h_{j+1,j}, SCALE_PT pairs of rows
+// per thread; with vcur, what the next graph-replayed step's CPR reads (FP64:
+// the vector, double-float: its hi plane) also into that fixed buffer.
+#define SCALE_PT 4
+struct col_args { int m; const double *h1, *h2; const int *flag; const double *hnorm; double *G; double *host; };
+template <bool DF> struct scale_t { typedef double type; };
+template <> struct scale_t<true> { typedef float type; };
+template <bool DF>
+__global__ void __launch_bounds__(256) k_scale(int nu, const typename scale_t<DF>::type *w, const float *isp,
+                                               typename scale_t<DF>::type *V, int j, int *jd,
+                                               typename scale_t<DF>::type *vcur, col_args c, int pdl) {
+  if (pdl) { pdl_trigger(); pdl_wait(); }
+  if (blockIdx.x == 0) {
+    if (threadIdx.x >= 32) return;
+    if (jd) j = jd[0];
+    arnoldi_col(j, c.m, c.h1, c.h2, c.flag, c.hnorm, c.G, c.host + (jd ? 4 * j : 0));
+    if (jd && threadIdx.x == 0) jd[0] = j + 1;
+    return;
+  }
+  if (jd) j = jd[1];
+  const int np = nu / 2, b0 = (blockIdx.x - 1) * 256 * SCALE_PT + threadIdx.x;
+  if (DF) {
+    const float2 *wh = reinterpret_cast<const float2 *>(w), *wl = reinterpret_cast<const float2 *>(w + nu);
+    float2 *vh = reinterpret_cast<float2 *>(V + (size_t)(2 * j + 2) * nu);
+    float2 *vl = reinterpret_cast<float2 *>(V + (size_t)(2 * j + 3) * nu), *vc = reinterpret_cast<float2 *>(vcur);
+    const float sh = isp[0], sl = isp[1];
+#pragma unroll
+    for (int u = 0; u < SCALE_PT; u++) {
+      const int i = b0 + 256 * u;
+      if (i >= np) break;
+      const float2 a = wh[i], b = wl[i];
+      float p, e;
+      float2 h, l;
+      df_mul(a.x, b.x, sh, sl, p, e); df_fast(p, e, h.x, l.x);
+      df_mul(a.y, b.y, sh, sl, p, e); df_fast(p, e, h.y, l.y);
+      vh[i] = h; vl[i] = l;
+      if (vc) vc[i] = h;
+    }
+  } else {
+    const double2 *w2 = reinterpret_cast<const double2 *>(w);
+    double2 *v2 = reinterpret_cast<double2 *>(V + (size_t)(j + 1) * nu), *vc = reinterpret_cast<double2 *>(vcur);
+    const double inv = c.hnorm[1];
+#pragma unroll
+    for (int u = 0; u < SCALE_PT; u++) {
+      const int i = b0 + 256 * u;
+      if (i >= np) break;
+      double2 a = w2[i];
+      a.x *= inv; a.y *= inv;
+      v2[i] = a;
+      if (vc) vc[i] = a;
+    }
+  }
 }
 __global__ void k_start_df(int nu, const double *r, double beta, float *V, double *G, int m, float *vcur) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -940,129 +1049,28 @@ static void ortho_attr() {
   if (done) return;
   RS_CUDA(cudaFuncSetAttribute(k_ortho_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, ORTHO_CH * 8));
   RS_CUDA(cudaFuncSetAttribute(k_ortho_update, cudaFuncAttributeMaxDynamicSharedMemorySize, ORTHO_CH * 8));
-  RS_CUDA(cudaFuncSetAttribute(k_ortho_dots_df, cudaFuncAttributeMaxDynamicSharedMemorySize, ORTHO_CH_DF * 8));
-  RS_CUDA(cudaFuncSetAttribute(k_ortho_update_df, cudaFuncAttributeMaxDynamicSharedMemorySize, ORTHO_CH_DF * 8));
+  RS_CUDA(cudaFuncSetAttribute(k_ortho_dots_df, cudaFuncAttributeMaxDynamicSharedMemorySize, ORTHO_CH * 8));
+  RS_CUDA(cudaFuncSetAttribute(k_ortho_update_df, cudaFuncAttributeMaxDynamicSharedMemorySize, ORTHO_CH * 8));
   done = true;
 }
-static void ortho_dots(int nu, int nv, const double *V, const double *w, double *part, int with_norm, const int *cond,
-                       int nblk, cudaStream_t s, const int *jd = nullptr) {
-  ortho_attr();
-  k_ortho_dots<<<nblk, ORTHO_BS, ORTHO_CH * 8, s>>>(nu, nv, V, w, part, with_norm, cond, jd);
-}
-static void ortho_update(int nu, int nv, const double *V, double *w, const double *h, double *part, const int *cond,
-                         int nblk, cudaStream_t s, const int *jd = nullptr) {
-  ortho_attr();
-  k_ortho_update<<<nblk, ORTHO_BS, ORTHO_CH * 8, s>>>(nu, nv, V, w, h, part, cond, jd);
-}
 
-// double-float kernels: one wave of 4 blocks per SM, each owning an equal
-// chunk of rows (a multiple of 64, at most ORTHO_CH_DF), its slice of w in
-// shared memory
-static int ortho_blocks_df(int nu, int *ch) {
+// one wave of 4 blocks per SM, each owning an equal chunk of rows (a multiple
+// of 64, at most ORTHO_CH; in FP64 at least 256, one per thread), its slice of
+// w in shared memory
+static int ortho_blocks(int nu, bool df, int *ch) {
   int nblk = 152 * 4;
-  int c = ((nu + nblk - 1) / nblk + 63) & ~63;
-  if (c > ORTHO_CH_DF) { c = ORTHO_CH_DF; nblk = (nu + c - 1) / c; }
-  else nblk = (nu + c - 1) / c;
+  int c = std::min(std::max(((nu + nblk - 1) / nblk + 63) & ~63, df ? 64 : 256), ORTHO_CH);
   *ch = c;
-  return std::max(nblk, 1);
-}
-static void ortho_dots_df(int nu, int ch, int nv, const float *V, const float *w, double *part, int with_norm,
-                          const int *cond, int nblk, cudaStream_t s, const int *jd, int *ticket, double *out) {
-  ortho_attr();
-  k_ortho_dots_df<<<nblk, ORTHO_BS, (size_t)ch * 8, s>>>(nu, ch, nv, V, w, part, with_norm, cond, jd, ticket, out);
-}
-static void ortho_update_df(int nu, int ch, int nv, const float *V, float *w, const double *h, double *part,
-                            const int *cond, int nblk, cudaStream_t s, const int *jd, int *ticket, double *nrm,
-                            int *flag, const double *h1) {
-  ortho_attr();
-  k_ortho_update_df<<<nblk, ORTHO_BS, (size_t)ch * 8, s>>>(nu, ch, nv, V, w, h, part, cond, jd, ticket, nrm, flag, h1);
+  return std::max((nu + c - 1) / c, 1);
 }
 
-// out[k] = sum over blocks of part[k][*]: one warp per k, lanes add a fixed
-// stride of the partials, then a fixed shuffle tree (deterministic)
-__global__ void k_reduce_parts(int nv, int nblk, const double *part, double *out, const int *cond, const int *jd,
-                               int extra) {
-  if (cond && *cond == 0) return;
-  if (jd) nv = *jd + 1 + extra;
-  int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (k >= nv) return;
-  double t = 0;
-  for (int b = lane; b < nblk; b += 32) t += part[(size_t)k * nblk + b];
-  t = warp_sum_d(t);
-  if (lane == 0) out[k] = t;
-}
-static void reduce_parts(int nv, int nblk, const double *part, double *out, const int *cond, cudaStream_t s,
-                         const int *jd = nullptr, int extra = 0) {
-  int cover = jd ? ORTHO_MAXV + 1 : nv;        // graph replay: enough warps for any step
-  k_reduce_parts<<<(cover + 3) / 4, 128, 0, s>>>(nv, nblk, part, out, cond, jd, extra);
-}
-// flag = ||w_1||^2 < 1e-4 ||w||^2 (the first pass kept less than 1% of w)
-__global__ void k_dgks(const double *w2_before, const double *w2_after, int *flag, const double *h1, const int *jd) {
-  if (jd) w2_before = h1 + *jd + 1;            // ||w||^2 follows the step's dot products
-  *flag = (*w2_after < 1e-4 * *w2_before) ? 1 : 0;
-}
-
-// Hessenberg column j: h = h1 + h2, h_{j+1,j} = ||w||; previous Givens
-// rotations, a new one, and the residual estimate |g_{j+1}|.
-// G layout: [0..m*(m+1)) H column-major (m+1 per column), cs[m], sn[m], g[m+1]
-__global__ void k_arnoldi_col(int j, int m, const double *h1, const double *h2, const double *nrm_a,
-                              const double *nrm_b, const int *flag, double *G, double *hnorm, volatile double *host,
-                              const int *jd, float *isp) {
-  // one warp: the column's inputs and the previous rotations are loaded
-  // into shared memory in parallel, then lane 0 applies the rotations (a
-  // serial recurrence) from there
-  __shared__ double sc[ORTHO_MAXV + 1], scs[ORTHO_MAXV], ssn[ORTHO_MAXV];
-  if (jd) { j = *jd; host += 4 * j; }          // graph replay: pinned slot j
-  double *H = G, *cs = G + (size_t)m * (m + 1), *sn = cs + m, *g = sn + m;
-  double *col = H + (size_t)j * (m + 1);
-  const int lane = threadIdx.x;
-  bool re = *flag != 0;
-  for (int k = lane; k <= j; k += 32) sc[k] = re ? h1[k] + h2[k] : h1[k];
-  for (int k = lane; k < j; k += 32) { scs[k] = cs[k]; ssn[k] = sn[k]; }
-  __syncwarp();
-  if (lane != 0) return;
-  double hn = sqrt(re ? *nrm_b : *nrm_a);
-  hnorm[0] = hn;
-  hnorm[1] = hn > 0.0 ? 1.0 / hn : 0.0;
-  if (isp) { float a, b; df_split(hnorm[1], a, b); isp[0] = a; isp[1] = b; }
-  sc[j + 1] = 0.0;
-  for (int k = 0; k < j; k++) {
-    double t = scs[k] * sc[k] + ssn[k] * sc[k + 1];
-    sc[k + 1] = -ssn[k] * sc[k] + scs[k] * sc[k + 1];
-    sc[k] = t;
+__global__ void k_start(int nu, const double *r, double beta, double *v0, double *G, int m, double *vcur) {
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nu) {
+    const double v = r[i] * (1.0 / beta);
+    v0[i] = v;
+    if (vcur) vcur[i] = v;
   }
-  double rr = sqrt(sc[j] * sc[j] + hn * hn);
-  double cj = sc[j] / rr, sj = hn / rr;
-  cs[j] = cj; sn[j] = sj;
-  for (int k = 0; k < j; k++) col[k] = sc[k];
-  col[j] = rr; col[j + 1] = 0.0;
-  double gj = g[j];
-  g[j + 1] = -sj * gj;
-  g[j] = cj * gj;
-  host[0] = fabs(g[j + 1]);
-  host[1] = hn;
-  host[2] = re ? 1.0 : 0.0;
-}
-__global__ void k_scale(int nu, const double *w, const double *inv_hn, double *v, const int *jd) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (jd) v += (size_t)(*jd + 1) * nu;     // graph replay: v is the basis, the target is V_{j+1}
-  if (i < nu) v[i] = w[i] * *inv_hn;       // 1 / h_{j+1,j} formed once by k_arnoldi_col
-}
-// graph replay helpers: the step's basis vector in and preconditioned vector out
-// of fixed buffers, and the step counter
-__global__ void k_basis_get(int nu, const double *V, const int *jd, double *vcur) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nu) vcur[i] = V[(size_t)*jd * nu + i];
-}
-template <class T>
-__global__ void k_basis_put(int nu, const T *zcur, T *Z, const int *jd) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nu) Z[(size_t)*jd * nu + i] = zcur[i];
-}
-__global__ void k_step_inc(int *jd) { (*jd)++; }
-__global__ void k_start(int nu, const double *r, double beta, double *v0, double *G, int m) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nu) v0[i] = r[i] * (1.0 / beta);
   if (i == 0) { double *g = G + (size_t)m * (m + 1) + 2 * m; for (int k = 0; k <= m; k++) g[k] = 0.0; g[0] = beta; }
 }
 __global__ void k_hsolve(int jend, int m, const double *G, double *yk) {
@@ -1240,7 +1248,7 @@ int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
   bool df = mixed && !ls->o.fp64_basis && 2.0 * (m + 1) * (double)nu < 2147483647.0;
   ls->V.ensure((size_t)(m + 1) * nu);
   if (mixed) ls->Z32.ensure((size_t)m * nu); else ls->Z.ensure((size_t)m * nu);
-  int chd = 0, nblk = df ? ortho_blocks_df(nu, &chd) : ortho_blocks(nu);
+  int ch = 0, nblk = ortho_blocks(nu, df, &ch);
   ls->partial.ensure((size_t)(ORTHO_MAXV + 1) * nblk + 8);
   ls->hbuf.ensure((size_t)(m + 1) * (m + 1) + 4 * (m + 1) + 4 * ORTHO_MAXV + 16);
   double *G = ls->hbuf.p, *h1 = G + (size_t)(m + 1) * (m + 1) + 3 * (m + 1), *h2 = h1 + ORTHO_MAXV + 1,
@@ -1269,42 +1277,36 @@ int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
   // rotations, and V_{j+1}.  jdp: the step index is read on the device (graph
   // replay) instead of j.  Mixed precision: double-float planes.
   float *V32 = reinterpret_cast<float *>(ls->V.p);
-  if (df) {
-    ls->w2.ensure(2 * (size_t)nu); ls->isp.ensure(2);
-    if (!ls->ticket.p) { ls->ticket.ensure(1); RS_CUDA(cudaMemsetAsync(ls->ticket.p, 0, sizeof(int), s)); }
-  }
-  auto ortho_tail = [&](cudaStream_t c, int j, const int *jdp) {
-    int nv = jdp ? 0 : j + 1;
+  if (df) { ls->w2.ensure(2 * (size_t)nu); ls->isp.ensure(2); }
+  if (!ls->ticket.p) { ls->ticket.ensure(1); RS_CUDA(cudaMemsetAsync(ls->ticket.p, 0, sizeof(int), s)); }
+  ortho_attr();
+  auto ortho_tail = [&](cudaStream_t c, int j, int *jdp) {
+    // two passes of dot products and update (the second runs only when the
+    // first one's last block has set the flag), then the column and V_{j+1}
+    const int nv = jdp ? 0 : j + 1;
     double *part = ls->partial.p;
+    int *tk = ls->ticket.p;
+    const size_t sm = (size_t)ch * 8;
+    const unsigned gs = 1 + grid_for(nu / 2, 256 * SCALE_PT);
+    const int pdl = arnoldi_pdl(ls->nb);
+    const col_args ca = {m, h1, h2, flag, hn, G, jdp ? hp_dev : hp_dev + 4 * j};
+    auto ortho = [&](auto kern, auto... a) { launch_pdl_if(pdl, kern, nblk, ORTHO_BS, sm, c, nu, ch, nv, a..., pdl); };
     if (df) {
-      float *w2 = ls->w2.p;                    // written by the double-float SpMV
-      // the reductions, and the test for a second pass, run in the last
-      // block of each sweep
-      int *tk = ls->ticket.p;
-      ortho_dots_df(nu, chd, nv, V32, w2, part, 1, nullptr, nblk, c, jdp, tk, h1);   // h1[nv] = ||w||^2
-      ortho_update_df(nu, chd, nv, V32, w2, h1, part, nullptr, nblk, c, jdp, tk, nrm, flag, h1);
-      ortho_dots_df(nu, chd, nv, V32, w2, part, 0, flag, nblk, c, jdp, tk, h2);
-      ortho_update_df(nu, chd, nv, V32, w2, h2, part, flag, nblk, c, jdp, tk, nrm_b, nullptr, nullptr);
-      k_arnoldi_col<<<1, 32, 0, c>>>(j, m, h1, h2, nrm, nrm_b, flag, G, hn, jdp ? hp_dev : hp_dev + 4 * j, jdp,
-                                    ls->isp.p);
-      k_scale_df<<<grid_for(nu, 256), 256, 0, c>>>(nu, w2, ls->isp.p, V32, j + 1, jdp, jdp ? ls->vcur32.p : nullptr);
-      RS_LAUNCHED(6);
+      float *w2 = ls->w2.p, *isp = ls->isp.p;  // w2 written by the double-float SpMV
+      ortho(k_ortho_dots_df, V32, w2, part, 1, nullptr, jdp, tk, h1);
+      ortho(k_ortho_update_df, V32, w2, h1, part, nullptr, jdp, tk, nrm, flag, h1, hn, isp);
+      ortho(k_ortho_dots_df, V32, w2, part, 0, flag, jdp, tk, h2);
+      ortho(k_ortho_update_df, V32, w2, h2, part, flag, jdp, tk, nrm_b, nullptr, nullptr, hn, isp);
+      launch_pdl_if(pdl, k_scale<true>, gs, 256, 0, c, nu, w2, isp, V32, j, jdp, jdp ? ls->vcur32.p : nullptr, ca, pdl);
     } else {
-      ortho_dots(nu, nv, ls->V.p, ls->w.p, part, 1, nullptr, nblk, c, jdp);
-      reduce_parts(nv + 1, nblk, part, h1, nullptr, c, jdp, 1);
-      ortho_update(nu, nv, ls->V.p, ls->w.p, h1, part, nullptr, nblk, c, jdp);
-      reduce_parts(1, nblk, part, nrm, nullptr, c);
-      k_dgks<<<1, 1, 0, c>>>(h1 + nv, nrm, flag, h1, jdp);
-      ortho_dots(nu, nv, ls->V.p, ls->w.p, part, 0, flag, nblk, c, jdp);
-      reduce_parts(nv, nblk, part, h2, flag, c, jdp, 0);
-      ortho_update(nu, nv, ls->V.p, ls->w.p, h2, part, flag, nblk, c, jdp);
-      reduce_parts(1, nblk, part, nrm_b, flag, c);
-      k_arnoldi_col<<<1, 32, 0, c>>>(j, m, h1, h2, nrm, nrm_b, flag, G, hn, jdp ? hp_dev : hp_dev + 4 * j, jdp,
-                                    nullptr);
-      k_scale<<<grid_for(nu, 256), 256, 0, c>>>(nu, ls->w.p, hn + 1, jdp ? ls->V.p : ls->V.p + (size_t)(j + 1) * nu,
-                                                jdp);
-      RS_LAUNCHED(11);
+      double *w = ls->w.p, *V = ls->V.p;
+      ortho(k_ortho_dots, V, w, part, 1, nullptr, jdp, tk, h1);
+      ortho(k_ortho_update, V, w, h1, part, nullptr, jdp, tk, nrm, flag, h1, hn);
+      ortho(k_ortho_dots, V, w, part, 0, flag, jdp, tk, h2);
+      ortho(k_ortho_update, V, w, h2, part, flag, jdp, tk, nrm_b, nullptr, nullptr, hn);
+      launch_pdl_if(pdl, k_scale<false>, gs, 256, 0, c, nu, w, nullptr, V, j, jdp, jdp ? ls->vcur.p : nullptr, ca, pdl);
     }
+    RS_LAUNCHED(5);
   };
   // One Arnoldi step j (CPR, SpMV, orthogonalisation, Givens); its residual
   // estimate and h_{j+1,j} land in pinned slot j
@@ -1331,9 +1333,9 @@ int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
     RS_CHECK_LAUNCH();
   };
   // The same Arnoldi step as one CUDA graph, replayed for every j: the step
-  // index lives on the device (jd), the basis vector is copied into a fixed
-  // buffer and the preconditioned vector out of one, and the kernels that
-  // depend on j read it from jd.  Recorded once per setup (the hierarchy's
+  // index lives on the device (jd), the step's basis vector sits in a fixed
+  // buffer and its preconditioned vector goes through one, and the kernels
+  // that depend on j read it from jd.  Recorded once per setup (the hierarchy's
   // buffers may move at a setup); kernel timers become event nodes of the
   // graph, read after each replay.
   // The recording holds raw pointers: record again whenever one of the
@@ -1347,39 +1349,30 @@ int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
   if (use_graph && ls->it_exec && memcmp(sig, ls->it_sig, sizeof(sig)) != 0) ls->drop_graph();
   // one Arnoldi step recorded on stream c (the capture stream)
   auto record_step = [&](cudaStream_t c) {
-      const int *jd = ls->jd.p;
-      if (df) {                              // vcur32 holds v_j (k_start_df, k_scale_df)
+      int *jd = ls->jd.p;                    // vcur / vcur32 hold v_j (k_start, k_scale)
+      if (df) {
         ls_cpr32(ls, ls->vcur32.p, ls->zcur32.p);
-        {
-          rs_timed tm(ls, SIM_T_SPMV64);
-          spmv_df(ls, ls->zcur32.p, ls->w2.p, c);
-        }
-        k_basis_put<float><<<grid_for(nu, 256), 256, 0, c>>>(nu, ls->zcur32.p, ls->Z32.p, jd);
+        rs_timed tm(ls, SIM_T_SPMV64);
+        spmv_df(ls, ls->zcur32.p, ls->w2.p, c, ls->Z32.p, jd);
       } else if (mixed) {
-        k_basis_get<<<grid_for(nu, 256), 256, 0, c>>>(nu, ls->V.p, jd, ls->vcur.p);
         ls_cpr(ls, ls->vcur.p, nullptr, ls->zcur32.p);
-        {
-          rs_timed tm(ls, SIM_T_SPMV64);
-          spmv<double, float, double, double>(ls, ls->val.p, ls->zcur32.p, (const double *)nullptr, ls->w.p, c);
-        }
-        k_basis_put<float><<<grid_for(nu, 256), 256, 0, c>>>(nu, ls->zcur32.p, ls->Z32.p, jd);
+        rs_timed tm(ls, SIM_T_SPMV64);
+        spmv<double, float, double, double>(ls, ls->val.p, ls->zcur32.p, (const double *)nullptr, ls->w.p, c, nullptr,
+                                            ls->Z32.p, nullptr, jd);
       } else {
-        k_basis_get<<<grid_for(nu, 256), 256, 0, c>>>(nu, ls->V.p, jd, ls->vcur.p);
         ls_cpr(ls, ls->vcur.p, ls->zcur64.p, nullptr);
-        ls_spmv64(ls, ls->zcur64.p, ls->w.p);
-        k_basis_put<double><<<grid_for(nu, 256), 256, 0, c>>>(nu, ls->zcur64.p, ls->Z.p, jd);
+        rs_timed tm(ls, SIM_T_SPMV64);
+        spmv<double, double, double, double>(ls, ls->val.p, ls->zcur64.p, (const double *)nullptr, ls->w.p, c, nullptr,
+                                             ls->Z.p, nullptr, jd);
       }
       rs_timed tm(ls, SIM_T_ORTHO);
       ortho_tail(c, 0, jd);
       tm.stop();
-      k_step_inc<<<1, 1, 0, c>>>(ls->jd.p);
-      RS_LAUNCHED(df ? 2 : 3);
       RS_CHECK_LAUNCH();
   };
   if (use_graph && !ls->it_exec) {
     ls->drop_graph();
-    ortho_attr();
-    ls->jd.ensure(1);
+    ls->jd.ensure(2);
     if (df) ls->vcur32.ensure(nu); else ls->vcur.ensure(nu);
     if (mixed) ls->zcur32.ensure(nu); else ls->zcur64.ensure(nu);
     if (!ls->cap) RS_CUDA(cudaStreamCreateWithFlags(&ls->cap, cudaStreamNonBlocking));
@@ -1480,7 +1473,7 @@ int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
   ls->last_mode = use_loop ? 2 : use_graph ? 1 : 0;
   for (;;) {
     if (df) k_start_df<<<grid_for(nu, 256), 256, 0, s>>>(nu, ls->r.p, beta, V32, G, m, use_graph ? ls->vcur32.p : nullptr);
-    else k_start<<<grid_for(nu, 256), 256, 0, s>>>(nu, ls->r.p, beta, ls->V.p, G, m);
+    else k_start<<<grid_for(nu, 256), 256, 0, s>>>(nu, ls->r.p, beta, ls->V.p, G, m, use_graph ? ls->vcur.p : nullptr);
     RS_LAUNCHED(1);
     int jend = 0;
     if (use_graph) RS_CUDA(cudaMemsetAsync(ls->jd.p, 0, sizeof(int), s));

@@ -845,7 +845,7 @@ template <class T, class Tin, bool ACC, class TB>
 __global__ void __launch_bounds__(ras_threads<T>(), sizeof(TB) == 2 ? 20 : sizeof(T) == 4 ? 16 : 8)
 k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const int *gidx_all, const uint16_t *gpos_all,
                    const int *nown, const uint2 *gdesc, const int *ngrp, const int *lrp_ptr, const int *sub_ptr,
-                   const int *order, const Tin *__restrict__ f, T *__restrict__ x) {
+                   const int *order, const Tin *f, T *x) {
   constexpr bool D = sizeof(T) == 8;                   // FP64: two lanes per row
   constexpr int BS = ras_threads<T>(), BPP = sizeof(TB) == 2 ? 2 : 1, NP = RAS_K / BPP + 1, AHEAD = ras_ahead<TB>();
   typedef typename v2_t<T>::type T2;
@@ -862,6 +862,7 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
   const uint2 *gd = gdesc + ras_group0(s, base, lrp_ptr[s]);
   const int bound = (int)(blob_off[s + 1] - blob_off[s]), glast = max(ng - 1, 0);
   auto sync = [&]() { if (D) __syncthreads(); else __syncwarp(); };
+  pdl_trigger();
   int pf = min(bound, RAS_PF_BYTES);                   // the stream is prefetched into L2 up to here
   if (tid == 0)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(st), "r"(pf) : "memory");
@@ -902,15 +903,23 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
                      st + pf), "r"(len), "r"((int)(go && tid == 0)) : "memory");
     pf += go ? len : 0;
   };
-  // gather the extended right-hand side
+  // gather the extended right-hand side, the first indices ahead of the wait
+  // for the kernel that makes f (all other inputs are fixed between setups)
   const Tin2 *f2 = reinterpret_cast<const Tin2 *>(f);
   constexpr int GU = D ? 8 : 16;
-  for (int p0 = tid; p0 < m; p0 += GU * BS) {
-    Tin2 v[GU];
-    int pos[GU];
+  int gi[GU], pos[GU];
+  auto indices = [&](int p0) {
 #pragma unroll
     for (int u = 0; u < GU; u++)
-      if (p0 + u * BS < m) { v[u] = f2[gidx[p0 + u * BS]]; pos[u] = gpos[p0 + u * BS]; }
+      if (p0 + u * BS < m) { gi[u] = gidx[p0 + u * BS]; pos[u] = gpos[p0 + u * BS]; }
+  };
+  indices(tid);
+  pdl_wait();
+  for (int p0 = tid; p0 < m; p0 += GU * BS) {
+    Tin2 v[GU];
+    if (p0 != tid) indices(p0);
+#pragma unroll
+    for (int u = 0; u < GU; u++) if (p0 + u * BS < m) v[u] = f2[gi[u]];
 #pragma unroll
     for (int u = 0; u < GU; u++)
       if (p0 + u * BS < m) { T2 t; t.x = (T)v[u].x; t.y = (T)v[u].y; y[pos[u]] = t; }
@@ -992,7 +1001,6 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
   sweep(ng - ngl, std::integral_constant<int, 1>());
   for (int p0 = tid; p0 < no; p0 += 8 * BS) {            // the owned rows come first in gather order
     T2 v[8], w[8];
-    int gi[8];
 #pragma unroll
     for (int u = 0; u < 8; u++)
       if (p0 + u * BS < no) {
@@ -1042,8 +1050,8 @@ static void ras_apply_go(sim_ls_s *ls, const Tin *f, T *x, bool acc) {
   ras_data &R = ls->ras;
 #define RAS_APPLY_ARGS R.blob_off.p, R.blob.p, R.gidx.p, R.gpos.p, R.nown.p, R.gdesc.p, R.ngrp.p, R.lrp_ptr.p, R.sub_ptr.p, R.order.p, f, x
   const int bs = ras_threads<T>();
-  if (acc) k_ras_apply_stream<T, Tin, true, TB><<<R.nsub, bs, R.smem_bytes, ls->st>>>(RAS_APPLY_ARGS);
-  else k_ras_apply_stream<T, Tin, false, TB><<<R.nsub, bs, R.smem_bytes, ls->st>>>(RAS_APPLY_ARGS);
+  if (acc) launch_pdl(k_ras_apply_stream<T, Tin, true, TB>, R.nsub, bs, R.smem_bytes, ls->st, RAS_APPLY_ARGS);
+  else launch_pdl(k_ras_apply_stream<T, Tin, false, TB>, R.nsub, bs, R.smem_bytes, ls->st, RAS_APPLY_ARGS);
 #undef RAS_APPLY_ARGS
 }
 template <class T, class Tin> static void ras_apply_launch(sim_ls_s *ls, const Tin *f, T *x, bool acc);
