@@ -52,28 +52,52 @@ __global__ void k_tpos_warp(int n, const int *rp, const int *ci, int *tpos, int 
 
 // Strength of connection (S), and with dinv given the l1-Jacobi diagonal of
 // the same row (d_i = a_ii + sum_{j != i} |a_ij|; 1 / d_i, FP64 and FP32),
-// from one pass over the row.
-__global__ void k_strength(int n, const int *rp, const int *ci, const double *v, double theta, uint8_t *S,
-                           double *dinv, float *dinv32) {
+// from one pass over the row.  A thread per row; ROW_B entries' loads are
+// issued together (one entry at a time, a row of 36 entries was a chain of 36
+// L2 latencies, twice: 31 us on a level of 1,600 rows against 11 us), and a
+// row of at most ROW_B entries stays in registers for the second pass.
+#define ROW_B 8
+__global__ void k_strength(int n, const int *__restrict__ rp, const int *__restrict__ ci, const double *__restrict__ v,
+                           double theta, uint8_t *__restrict__ S, double *dinv, float *dinv32) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   bool have = false; double mx = 0.0; long long mxk = 0;
   double s = 0.0, aii = 0.0;
-  for (int q = rp[i]; q < rp[i + 1]; q++) {
-    const double a = v[q];
-    if (ci[q] == i) { aii = a; continue; }
-    s = add_rn(s, fabs(a));
-    long long tk = -dkey(a);                        // key of t = -a_iq
-    if (!have || tk > mxk) { mx = -a; mxk = tk; have = true; }
+  const int q0 = rp[i], q1 = rp[i + 1];
+  double a[ROW_B];
+  bool diag[ROW_B];
+  auto load = [&](int qb) {
+#pragma unroll
+    for (int u = 0; u < ROW_B; u++) {
+      const bool in = qb + u < q1;
+      a[u] = in ? v[qb + u] : 0.0;
+      diag[u] = in && ci[qb + u] == i;
+    }
+  };
+  for (int qb = q0; qb < q1; qb += ROW_B) {
+    load(qb);
+#pragma unroll
+    for (int u = 0; u < ROW_B; u++) {
+      if (qb + u >= q1) break;
+      if (diag[u]) { aii = a[u]; continue; }
+      s = add_rn(s, fabs(a[u]));
+      long long tk = -dkey(a[u]);                      // key of t = -a_iq
+      if (!have || tk > mxk) { mx = -a[u]; mxk = tk; have = true; }
+    }
   }
   long long thrk = dkey(mul_rn(theta, mx));
   bool any = have && mxk > 0;                       // max_k (-a_ik) > 0
-  for (int q = rp[i]; q < rp[i + 1]; q++)
-    S[q] = (uint8_t)(any && ci[q] != i && -dkey(v[q]) >= thrk);
+  for (int qb = q0; qb < q1; qb += ROW_B) {
+    if (q1 - q0 > ROW_B) load(qb);
+#pragma unroll
+    for (int u = 0; u < ROW_B; u++)
+      if (qb + u < q1) S[qb + u] = (uint8_t)(any && !diag[u] && -dkey(a[u]) >= thrk);
+  }
   if (dinv) {
     double d = add_rn(aii, s);
-    dinv[i] = 1.0 / d;
-    if (dinv32) dinv32[i] = (float)(1.0 / d);
+    const double r = 1.0 / d;
+    dinv[i] = r;
+    if (dinv32) dinv32[i] = (float)r;
   }
 }
 
@@ -269,55 +293,81 @@ __global__ void k_cflag(int n, const int8_t *cf, int *flag) {
 }
 
 // ------------------------------------------------------- interpolation ----
-__global__ void k_interp_count(int n, const int *rp, const int *ci, const uint8_t *S, const int8_t *cf, int *len) {
+// entries per row of P, and the C flag of each point
+__global__ void k_interp_count(int n, const int *__restrict__ rp, const int *__restrict__ ci,
+                               const uint8_t *__restrict__ S, const int8_t *__restrict__ cf, int *len, int *flag) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int c = 0;
-  if (cf[i] == 1) c = 1;
-  else for (int q = rp[i]; q < rp[i + 1]; q++) if (S[q] && cf[ci[q]] == 1) c++;
-  len[i] = c;
+  const bool cpt = cf[i] == 1;
+  if (!cpt)
+    for (int q0 = rp[i], q1 = rp[i + 1]; q0 < q1; q0 += ROW_B) {
+      int j[ROW_B]; bool st[ROW_B];
+#pragma unroll
+      for (int u = 0; u < ROW_B; u++) { const bool in = q0 + u < q1; j[u] = in ? ci[q0 + u] : i; st[u] = in && S[q0 + u]; }
+#pragma unroll
+      for (int u = 0; u < ROW_B; u++) c += st[u] && cf[j[u]] == 1;
+    }
+  len[i] = cpt ? 1 : c;
+  flag[i] = cpt;
 }
 
 // pcap: capacity of pci / pv (a row that would pass it sets *err and is
 // skipped; nnz(P) <= nnz(A) makes that impossible for direct interpolation)
-__global__ void k_interp_fill(int n, const int *rp, const int *ci, const double *v, const uint8_t *S,
-                              const int8_t *cf, const int *cidx, const int *prp, int *pci, double *pv, int pcap,
-                              int *err) {
+// pv32: the FP32 copy of pv (mixed precision) or nullptr
+__global__ void k_interp_fill(int n, const int *__restrict__ rp, const int *__restrict__ ci,
+                              const double *__restrict__ v, const uint8_t *__restrict__ S,
+                              const int8_t *__restrict__ cf, const int *__restrict__ cidx, const int *__restrict__ prp,
+                              int *pci, double *pv, float *pv32, int pcap, int *err) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int o = prp[i];
   if (prp[i + 1] > pcap) { atomicExch(err, 1); return; }
-  if (cf[i] == 1) { pci[o] = cidx[i]; pv[o] = 1.0; return; }
+  if (cf[i] == 1) { pci[o] = cidx[i]; pv[o] = 1.0; if (pv32) pv32[o] = 1.0f; return; }
   if (prp[i + 1] == o) return;
   // sums in the row's column order: sneg / spos (one FP64 add per entry,
   // its target chosen by the sign) while the strong C entries are listed;
-  // then snegc and the weights over that list only
+  // then snegc and the weights over that list only.  ROW_B entries' loads are
+  // in flight together.
   const int MAXC = 32;
   int m = prp[i + 1] - o, qs[MAXC], nq = 0;
   double sneg = 0.0, spos = 0.0, snegc = 0.0, aii = 0.0;
-  for (int q = rp[i]; q < rp[i + 1]; q++) {
-    double a = v[q];
-    int j = ci[q];
-    if (S[q] && cf[j] == 1 && nq < MAXC) qs[nq++] = q;
-    if (j == i) { aii = a; continue; }
-    bool neg = dkey(a) < 0;
-    double acc = add_rn(neg ? sneg : spos, a);
-    if (neg) sneg = acc; else spos = acc;
+  const int q1 = rp[i + 1];
+  for (int q0 = rp[i]; q0 < q1; q0 += ROW_B) {
+    double a[ROW_B]; int j[ROW_B]; bool st[ROW_B];
+#pragma unroll
+    for (int u = 0; u < ROW_B; u++) {
+      const bool in = q0 + u < q1;
+      a[u] = in ? v[q0 + u] : 0.0; j[u] = in ? ci[q0 + u] : i; st[u] = in && S[q0 + u];
+    }
+#pragma unroll
+    for (int u = 0; u < ROW_B; u++) st[u] = st[u] && cf[j[u]] == 1;
+#pragma unroll
+    for (int u = 0; u < ROW_B; u++) {
+      if (q0 + u >= q1) break;
+      if (st[u] && nq < MAXC) qs[nq++] = q0 + u;
+      if (j[u] == i) { aii = a[u]; continue; }
+      bool neg = dkey(a[u]) < 0;
+      double acc = add_rn(neg ? sneg : spos, a[u]);
+      if (neg) sneg = acc; else spos = acc;
+    }
   }
   if (m <= MAXC) {
     for (int t = 0; t < m; t++) snegc = add_rn(snegc, v[qs[t]]);
   } else {
-    for (int q = rp[i]; q < rp[i + 1]; q++) if (S[q] && cf[ci[q]] == 1) snegc = add_rn(snegc, v[q]);
+    for (int q = rp[i]; q < q1; q++) if (S[q] && cf[ci[q]] == 1) snegc = add_rn(snegc, v[q]);
   }
   double dg = add_rn(aii, spos), alpha = div_rn(sneg, snegc);
+  auto put = [&](int at, int q) {
+    const double w = div_rn(-mul_rn(alpha, v[q]), dg);
+    pci[at] = cidx[ci[q]]; pv[at] = w;
+    if (pv32) pv32[at] = (float)w;
+  };
   if (m <= MAXC) {
-    for (int t = 0; t < m; t++) {
-      int q = qs[t];
-      pci[o + t] = cidx[ci[q]]; pv[o + t] = div_rn(-mul_rn(alpha, v[q]), dg);
-    }
+    for (int t = 0; t < m; t++) put(o + t, qs[t]);
   } else {
-    for (int q = rp[i]; q < rp[i + 1]; q++)
-      if (S[q] && cf[ci[q]] == 1) { pci[o] = cidx[ci[q]]; pv[o++] = div_rn(-mul_rn(alpha, v[q]), dg); }
+    for (int q = rp[i]; q < q1; q++)
+      if (S[q] && cf[ci[q]] == 1) put(o++, q);
   }
 }
 
@@ -458,34 +508,56 @@ __global__ void k_transpose_fill(int n, const int *rp, const int *ci, const doub
     tci[o] = i; tv[o] = v[q];
   }
 }
-// one warp per row: rows of at most 32 entries by a bitonic network across
+// Bitonic network over a warp's two registers per lane (indices lane and
+// lane + 32; M = 32 uses the first only): ascending keys, values carried along
+__device__ __forceinline__ void warp_sort64(int M, int lane, int &k0, int &k1, double &v0, double &v1) {
+  for (int kk = 2; kk <= M; kk <<= 1)
+    for (int j = kk >> 1; j > 0; j >>= 1) {
+      if (j == 32) {                                // partners in the lane's two registers (kk = 64: ascending)
+        if (k0 > k1) { int x = k0; k0 = k1; k1 = x; double w = v0; v0 = v1; v1 = w; }
+        continue;
+      }
+#pragma unroll
+      for (int r = 0; r < 2; r++) {
+        if (r == 1 && M == 32) break;
+        int x = r ? k1 : k0;
+        double vx = r ? v1 : v0;
+        int y = __shfl_xor_sync(0xffffffffu, x, j);
+        double vy = __shfl_xor_sync(0xffffffffu, vx, j);
+        int i = lane + 32 * r;
+        bool keep_min = ((i & j) == 0) == ((i & kk) == 0);   // the lower index keeps the minimum when ascending
+        bool take = keep_min ? y < x : y > x;
+        if (take) { x = y; vx = vy; }
+        if (r) { k1 = x; v1 = vx; } else { k0 = x; v0 = vx; }
+      }
+    }
+}
+// one warp per row: rows of at most 64 entries by a bitonic network across
 // the lanes (columns within a row are distinct, so the order is unique),
-// longer rows by an insertion sort in the first lane
-__global__ void k_sort_rows_warp(int n, const int *rp, int *ci, double *v) {
+// longer rows by an insertion sort in the first lane (at 32 entries one long
+// row held up a whole level: 28 us on one of 1,600 rows).  v32: the FP32 copy
+// of v (mixed precision) or nullptr.
+__global__ void k_sort_rows_warp(int n, const int *rp, int *ci, double *v, float *v32) {
   int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (i >= n) return;
   int a0 = rp[i], len = rp[i + 1] - a0;
-  if (len <= 32) {
-    int c = lane < len ? ci[a0 + lane] : INT_MAX;
-    double x = lane < len ? v[a0 + lane] : 0.0;
-#pragma unroll
-    for (int k = 2; k <= 32; k <<= 1)
-#pragma unroll
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        int oc = __shfl_xor_sync(0xffffffffu, c, j);
-        double ox = __shfl_xor_sync(0xffffffffu, x, j);
-        bool up = (lane & k) == 0, lower = (lane & j) == 0;
-        bool take = lower == up ? oc < c : oc > c;     // keep the smaller key on the ascending side
-        if (take) { c = oc; x = ox; }
+  if (len <= 64) {
+    int k0 = lane < len ? ci[a0 + lane] : INT_MAX, k1 = lane + 32 < len ? ci[a0 + lane + 32] : INT_MAX;
+    double v0 = lane < len ? v[a0 + lane] : 0.0, v1 = lane + 32 < len ? v[a0 + lane + 32] : 0.0;
+    warp_sort64(len <= 32 ? 32 : 64, lane, k0, k1, v0, v1);
+    if (lane < len) { ci[a0 + lane] = k0; v[a0 + lane] = v0; if (v32) v32[a0 + lane] = (float)v0; }
+    if (lane + 32 < len) { ci[a0 + lane + 32] = k1; v[a0 + lane + 32] = v1; if (v32) v32[a0 + lane + 32] = (float)v1; }
+  } else {
+    if (lane == 0) {
+      int a1 = a0 + len;
+      for (int a = a0 + 1; a < a1; a++) {
+        int c = ci[a]; double x = v[a]; int b = a - 1;
+        while (b >= a0 && ci[b] > c) { ci[b + 1] = ci[b]; v[b + 1] = v[b]; b--; }
+        ci[b + 1] = c; v[b + 1] = x;
       }
-    if (lane < len) { ci[a0 + lane] = c; v[a0 + lane] = x; }
-  } else if (lane == 0) {
-    int a1 = a0 + len;
-    for (int a = a0 + 1; a < a1; a++) {
-      int c = ci[a]; double x = v[a]; int b = a - 1;
-      while (b >= a0 && ci[b] > c) { ci[b + 1] = ci[b]; v[b + 1] = v[b]; b--; }
-      ci[b + 1] = c; v[b + 1] = x;
     }
+    __syncwarp();
+    if (v32) for (int t = lane; t < len; t += 32) v32[a0 + t] = (float)v[a0 + t];
   }
 }
 
@@ -493,7 +565,7 @@ __global__ void k_sort_rows_warp(int n, const int *rp, int *ci, double *v) {
 // short: a bitonic network over the group's lanes (rows of at most G
 // entries), longer rows by an insertion sort in the group's first lane
 template <int G>
-__global__ void k_sort_rows_g(int n, const int *rp, int *ci, double *v) {
+__global__ void k_sort_rows_g(int n, const int *rp, int *ci, double *v, float *v32) {
   if (n <= 0) return;
   int gi = (blockIdx.x * blockDim.x + threadIdx.x) / G, k = threadIdx.x % G;
   bool valid = gi < n;
@@ -514,7 +586,7 @@ __global__ void k_sort_rows_g(int n, const int *rp, int *ci, double *v) {
     }
   if (!valid) return;
   if (small) {
-    if (k < len) { ci[a0 + k] = c; v[a0 + k] = x; }
+    if (k < len) { ci[a0 + k] = c; v[a0 + k] = x; if (v32) v32[a0 + k] = (float)x; }
   } else if (k == 0) {
     int a1 = a0 + len;
     for (int a = a0 + 1; a < a1; a++) {
@@ -522,6 +594,7 @@ __global__ void k_sort_rows_g(int n, const int *rp, int *ci, double *v) {
       while (b >= a0 && ci[b] > cc) { ci[b + 1] = ci[b]; v[b + 1] = v[b]; b--; }
       ci[b + 1] = cc; v[b + 1] = xx;
     }
+    if (v32) for (int a = a0; a < a1; a++) v32[a] = (float)v[a];
   }
 }
 
@@ -541,17 +614,29 @@ __global__ void k_row_products(int n, const int *arp, const int *aci, const int 
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int s = 0;
-  for (int q = arp[i]; q < arp[i + 1]; q++) { int k = aci[q]; s += brp[k + 1] - brp[k]; }
+  const int q1 = arp[i + 1];
+  for (int q0 = arp[i]; q0 < q1; q0 += ROW_B) {       // ROW_B entries' loads in flight together
+    int k[ROW_B];
+#pragma unroll
+    for (int u = 0; u < ROW_B; u++) k[u] = q0 + u < q1 ? aci[q0 + u] : -1;
+#pragma unroll
+    for (int u = 0; u < ROW_B; u++) if (k[u] >= 0) s += brp[k[u] + 1] - brp[k[u]];
+  }
   prod[i] = s;
   if (arp[i + 1] - arp[i] > SPG_KMAX || s > merge_p) atomicMax(mx, s + 1);   // + 1: "a hash row exists" even with 0 products
 }
 // C row i = scratch[toff[i] .. toff[i] + clen[i]), eight lanes per row
+// (cv32: the FP32 copy of cv or nullptr)
 __global__ void k_pack_rows(int n, const int *toff, const int *clen, const int *crp, const int *tci, const double *tv,
-                            int *cci, double *cv) {
+                            int *cci, double *cv, float *cv32) {
   int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, lane = threadIdx.x & 7;
   if (row >= n) return;
   int a = toff[row], b = crp[row], len = clen[row];
-  for (int t = lane; t < len; t += 8) { cci[b + t] = tci[a + t]; cv[b + t] = tv[a + t]; }
+  for (int t = lane; t < len; t += 8) {
+    const double x = tv[a + t];
+    cci[b + t] = tci[a + t]; cv[b + t] = x;
+    if (cv32) cv32[b + t] = (float)x;
+  }
 }
 
 // C = A B for the rows of A with at most K entries and at most merge_p
@@ -715,27 +800,7 @@ __global__ void __launch_bounds__(256) k_spgemm_hash(int n, const int *arp, cons
       // shuffles instead of shared-memory passes
       int k0 = lane < u ? keys[lane] : INT_MAX, k1 = lane + 32 < u ? keys[lane + 32] : INT_MAX;
       double v0 = lane < u ? vals[lane] : 0.0, v1 = lane + 32 < u ? vals[lane + 32] : 0.0;
-      const int M = u <= 32 ? 32 : 64;
-      for (int kk = 2; kk <= M; kk <<= 1)
-        for (int j = kk >> 1; j > 0; j >>= 1) {
-          if (j == 32) {                                // partners in the lane's two registers (kk = 64: ascending)
-            if (k0 > k1) { int x = k0; k0 = k1; k1 = x; double w = v0; v0 = v1; v1 = w; }
-            continue;
-          }
-#pragma unroll
-          for (int r = 0; r < 2; r++) {
-            if (r == 1 && M == 32) break;
-            int x = r ? k1 : k0;
-            double vx = r ? v1 : v0;
-            int y = __shfl_xor_sync(FULL, x, j);
-            double vy = __shfl_xor_sync(FULL, vx, j);
-            int i = lane + 32 * r;
-            bool keep_min = ((i & j) == 0) == ((i & kk) == 0);   // the lower index keeps the minimum when ascending
-            bool take = keep_min ? y < x : y > x;
-            if (take) { x = y; vx = vy; }
-            if (r) { k1 = x; v1 = vx; } else { k0 = x; v0 = vx; }
-          }
-        }
+      warp_sort64(u <= 32 ? 32 : 64, lane, k0, k1, v0, v1);
       if (lane < u) { cci[out + lane] = k0; cv[out + lane] = v0; }
       if (lane + 32 < u) { cci[out + lane + 32] = k1; cv[out + lane + 32] = v1; }
     } else {
@@ -792,8 +857,9 @@ static void spgemm_count(const csr_dev<double> &A, const csr_dev<double> &B, int
   rs_scan_dev(z.toff.p, z.toff.p, n, z.toff.p + n, tot, s);      // row offsets into the scratch arrays
 }
 
+// C32: C's FP32 values are written too (nullptr: FP64 only)
 static void spgemm_fill(const csr_dev<double> &A, const csr_dev<double> &B, csr_dev<double> &C, int total, int mx1,
-                        int *nnz, cudaStream_t s) {
+                        int *nnz, cudaStream_t s, csr_dev<float> *C32 = nullptr) {
   spg_scratch &z = spg();
   int n = A.n, mx = std::max(mx1 - 1, 0);
   // hash-table slots per warp: at least the products of the largest row in
@@ -835,8 +901,9 @@ static void spgemm_fill(const csr_dev<double> &A, const csr_dev<double> &B, csr_
   RS_CHECK_LAUNCH();
   rs_scan_dev(z.clen.p, C.rp.p, n, C.rp.p + n, nnz, s);
   C.ci.ensure(std::max(total, 1)); C.v.ensure(std::max(total, 1));
+  if (C32) C32->v.ensure(std::max(total, 1));
   k_pack_rows<<<grid_for((size_t)n * 8, 256), 256, 0, s>>>(n, z.toff.p, z.clen.p, C.rp.p, z.tci.p, z.tv.p, C.ci.p,
-                                                          C.v.p);
+                                                          C.v.p, C32 ? C32->v.p : nullptr);
   RS_LAUNCHED(1);
   RS_CHECK_LAUNCH();
 }
@@ -1006,7 +1073,8 @@ __global__ void __launch_bounds__(64) k_dense_inv_cols(int n, const double *lu, 
 }
 
 // ----------------------------------------------------------- host setup ---
-// FP32 values of an FP64 operator (the pattern stays the FP64 operator's)
+// FP32 values of an FP64 operator (the pattern stays the FP64 operator's);
+// the other copies are written by the kernels that make the FP64 values
 static void csr_cast(const csr_dev<double> &a, csr_dev<float> &b, cudaStream_t s) {
   b.n = a.n; b.m = a.m; b.nnz = a.nnz;
   b.v.ensure(a.nnz);
@@ -1019,15 +1087,15 @@ static void csr_cast(const csr_dev<double> &a, csr_dev<float> &b, cudaStream_t s
 // after the products of R (A P) are known (wait 2); nnz of the coarse
 // operators at the next wait 1 or at the end.
 enum {
-  AF_SYM = 0,        // pattern of A not structurally symmetric
-  AF_PCAP = 1,       // a row of P beyond its capacity
-  AF_NC = 2,         // C points (coarse size)
-  AF_PNNZ = 3,       // nnz(P)
-  AF_APTOT = 4, AF_APMX = 5, AF_APNNZ = 6,     // products, long-row marker and nnz of A P
-  AF_RAPTOT = 7, AF_RAPMX = 8,                 // the same for R (A P)
-  AF_PRND = 9,       // PMIS rounds taken (-1: not finished within the cap)
-  AF_SLOTS = 16,
-  AF_LNNZ = 16,      // [16 + l]: nnz of level l's operator (l >= 1)
+  AF_LNNZ = 0,       // [l]: nnz of level l's operator (l >= 1)
+  AF_ZERO = 32,      // the words from here on are zero at the start of a level
+  AF_SYM = 32,       // pattern of A not structurally symmetric
+  AF_PCAP = 33,      // a row of P beyond its capacity
+  AF_NC = 34,        // C points (coarse size)
+  AF_PNNZ = 35,      // nnz(P)
+  AF_APTOT = 36, AF_APMX = 37, AF_APNNZ = 38,  // products, long-row marker and nnz of A P
+  AF_RAPTOT = 39, AF_RAPMX = 40,               // the same for R (A P)
+  AF_PRND = 41,      // PMIS rounds taken (-1: not finished within the cap)
   AF_CNT = 48,       // [48 + r]: undecided points after PMIS round r - 1 (r = 0: after the initialisation)
   AF_ROUNDS_MAX = 1020,
   AF_WORDS = AF_CNT + AF_ROUNDS_MAX + 8
@@ -1090,13 +1158,14 @@ static void pmis_tail(amg_level &L, amg_hier &h, int n, int lanes, int r0, cudaS
 static int build_p(amg_level &L, amg_hier &h, const rs_opts &o, int n, size_t acap, dbuf<int> &cidx,
                    cudaStream_t s) {
   int *F = h.flag.p;
-  k_cflag<<<grid_for(n, 256), 256, 0, s>>>(n, L.cf.p, cidx.p);
-  RS_LAUNCHED(1);
-  rs_scan_dev(cidx.p, cidx.p, n, cidx.p + n, F + AF_NC, s);
+  const bool mixed = o.precision != SIM_PREC_FP64;
   L.P.n = n;
   L.P.rp.ensure(n + 1);
   int pnnz = -1;
   if (o.interp == SIM_INTERP_EXTI) {
+    k_cflag<<<grid_for(n, 256), 256, 0, s>>>(n, L.cf.p, cidx.p);
+    RS_LAUNCHED(1);
+    rs_scan_dev(cidx.p, cidx.p, n, cidx.p + n, F + AF_NC, s);
     static thread_local dbuf<int> uoff, cand;
     static thread_local dbuf<double> dk;
     uoff.ensure(n + 1);
@@ -1118,15 +1187,18 @@ static int build_p(amg_level &L, amg_hier &h, const rs_opts &o, int n, size_t ac
                                                  uoff.p, cand.p, dk.p, L.P.rp.p, L.P.ci.p, L.P.v.p);
     RS_LAUNCHED(2);
   } else {
-    k_interp_count<<<grid_for(n, 256), 256, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.strong.p, L.cf.p, L.P.rp.p);
+    k_interp_count<<<grid_for(n, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.strong.p, L.cf.p, L.P.rp.p, cidx.p);
     RS_LAUNCHED(1);
-    rs_scan_dev(L.P.rp.p, L.P.rp.p, n, L.P.rp.p + n, F + AF_PNNZ, s);
+    rs_scan_dev2(L.P.rp.p, L.P.rp.p + n, F + AF_PNNZ, cidx.p, cidx.p + n, F + AF_NC, n, s);
     L.P.ci.ensure(acap > 0 ? acap : 1); L.P.v.ensure(acap > 0 ? acap : 1);
+    if (mixed) L.P32.v.ensure(L.P.ci.n);
     k_interp_fill<<<grid_for(n, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.A.v.p, L.strong.p, L.cf.p, cidx.p,
-                                                   L.P.rp.p, L.P.ci.p, L.P.v.p, (int)L.P.ci.n, F + AF_PCAP);
+                                                   L.P.rp.p, L.P.ci.p, L.P.v.p, mixed ? L.P32.v.p : nullptr,
+                                                   (int)L.P.ci.n, F + AF_PCAP);
     RS_LAUNCHED(1);
   }
   RS_CHECK_LAUNCH();
+  RS_CUDA(cudaEventRecord(h.ev_p, s));
   spgemm_count(L.A, L.P, F + AF_APTOT, F + AF_APMX, s);
   return pnnz;
 }
@@ -1137,6 +1209,14 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
   if (!h.hflag) RS_CUDA(cudaMallocHost((void **)&h.hflag, AF_WORDS * sizeof(int)));
   int *F = h.flag.p;
   bool mixed = o.precision != SIM_PREC_FP64;
+  if (!h.st_r) {
+    // R = P^T is built on a stream of its own beside the products of A P
+    int least = 0, greatest = 0;
+    RS_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+    RS_CUDA(cudaStreamCreateWithPriority(&h.st_r, cudaStreamNonBlocking, greatest));
+    RS_CUDA(cudaEventCreateWithFlags(&h.ev_p, cudaEventDisableTiming));
+    RS_CUDA(cudaEventCreateWithFlags(&h.ev_r, cudaEventDisableTiming));
+  }
   int l = 0;
   for (;;) {
     amg_level &L = h.lev[l];
@@ -1159,9 +1239,9 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
       h.coarse_dense = 1;
       break;
     }
-    rs_fill_i(F, 0, AF_SLOTS, s);
-    rs_fill_i(F + AF_CNT, 0, AF_WORDS - AF_CNT, s);
-    if (nnz_hint > 8LL * n) k_tpos_warp<<<grid_for((size_t)n * 32, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.tpos.p, F + AF_SYM);
+    rs_fill_i(F + AF_ZERO, 0, AF_WORDS - AF_ZERO, s);
+    if (l == 0 && h.tpos0) {}                           // the finest pattern never changes: positions kept
+    else if (nnz_hint > 8LL * n) k_tpos_warp<<<grid_for((size_t)n * 32, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.tpos.p, F + AF_SYM);
     else k_tpos<<<grid_for(n, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.tpos.p, F + AF_SYM);
     k_strength<<<grid_for(n, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.A.v.p, o.theta, L.strong.p, L.dinv.p,
                                               mixed ? L.dinv32.p : nullptr);
@@ -1181,6 +1261,7 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
     int pnnz = build_p(L, h, o, n, acap, cidx, s);
     const int *hf = amg_read(h, 0, AF_CNT + PMIS_HINT_ROUNDS, s);   // wait 1
     if (hf[AF_SYM]) RS_FAIL(SIM_ERR_ARG, "AMG: level %d pattern is not structurally symmetric", l);
+    if (l == 0) h.tpos0 = true;
     if (hf[AF_PCAP]) RS_FAIL(SIM_ERR_ARG, "AMG: level %d interpolation beyond its capacity", l);
     if (hf[AF_PRND] < 0) RS_FAIL(SIM_ERR_TIMEOUT, "AMG: PMIS did not finish in %d rounds", (int)AF_ROUNDS_MAX);
     L.P.nnz = pnnz >= 0 ? pnnz : hf[AF_PNNZ];
@@ -1194,35 +1275,45 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
     if (nc == 0) { h.coarse_dense = 0; break; }
     L.P.m = nc;
     static thread_local csr_dev<double> AP;
-    spgemm_fill(L.A, L.P, AP, ap_tot, ap_mx, F + AF_APNNZ, s);
-    // R = P^T
+    // R = P^T, from the moment P is complete, beside A P
     L.R.n = nc; L.R.m = n; L.R.nnz = L.P.nnz;
     L.R.rp.ensure(nc + 1); L.R.ci.ensure(L.P.nnz > 0 ? L.P.nnz : 1); L.R.v.ensure(L.P.nnz > 0 ? L.P.nnz : 1);
+    if (mixed) L.R32.v.ensure(L.P.nnz > 0 ? L.P.nnz : 1);
     static thread_local dbuf<int> fill;
     fill.ensure(nc + 1);
-    rs_fill_i(L.R.rp.p, 0, nc + 1, s);
-    rs_fill_i(fill.p, 0, nc + 1, s);
-    k_col_count<<<grid_for(L.P.nnz, 256), 256, 0, s>>>(L.P.nnz, L.P.ci.p, L.R.rp.p);
-    RS_LAUNCHED(1);
-    rs_scan_dev(L.R.rp.p, L.R.rp.p, nc, L.R.rp.p + nc, nullptr, s);
-    k_transpose_fill<<<grid_for(n, 256), 256, 0, s>>>(n, L.P.rp.p, L.P.ci.p, L.P.v.p, L.R.rp.p, fill.p, L.R.ci.p,
-                                                      L.R.v.p);
-    {                                                  // rows of R: lanes per row by their mean length
+    {
+      cudaStream_t sr = h.st_r;
+      float *r32 = mixed ? L.R32.v.p : nullptr;
+      RS_CUDA(cudaStreamWaitEvent(sr, h.ev_p, 0));
+      rs_fill_i(L.R.rp.p, 0, nc + 1, sr);
+      rs_fill_i(fill.p, 0, nc + 1, sr);
+      k_col_count<<<grid_for(L.P.nnz, 256), 256, 0, sr>>>(L.P.nnz, L.P.ci.p, L.R.rp.p);
+      RS_LAUNCHED(1);
+      rs_scan_dev(L.R.rp.p, L.R.rp.p, nc, L.R.rp.p + nc, nullptr, sr, &h.scan_r);
+      k_transpose_fill<<<grid_for(n, 256), 256, 0, sr>>>(n, L.P.rp.p, L.P.ci.p, L.P.v.p, L.R.rp.p, fill.p, L.R.ci.p,
+                                                         L.R.v.p);
+      // rows of R: lanes per row by their mean length (a row longer than its
+      // group falls to one lane's insertion sort: groups of 16 only where
+      // rows average at most 8 entries)
       double avg = nc ? (double)L.P.nnz / nc : 0.0;
-      // (a row longer than its group falls to one lane's insertion sort:
-      // groups of 16 only where rows average at most 8 entries)
-      if (avg <= 4.0) k_sort_rows_g<8><<<grid_for((size_t)nc * 8, 128), 128, 0, s>>>(nc, L.R.rp.p, L.R.ci.p, L.R.v.p);
+      if (avg <= 4.0)
+        k_sort_rows_g<8><<<grid_for((size_t)nc * 8, 128), 128, 0, sr>>>(nc, L.R.rp.p, L.R.ci.p, L.R.v.p, r32);
       else if (avg <= 8.0)
-        k_sort_rows_g<16><<<grid_for((size_t)nc * 16, 128), 128, 0, s>>>(nc, L.R.rp.p, L.R.ci.p, L.R.v.p);
-      else k_sort_rows_warp<<<grid_for((size_t)nc * 32, 128), 128, 0, s>>>(nc, L.R.rp.p, L.R.ci.p, L.R.v.p);
+        k_sort_rows_g<16><<<grid_for((size_t)nc * 16, 128), 128, 0, sr>>>(nc, L.R.rp.p, L.R.ci.p, L.R.v.p, r32);
+      else k_sort_rows_warp<<<grid_for((size_t)nc * 32, 128), 128, 0, sr>>>(nc, L.R.rp.p, L.R.ci.p, L.R.v.p, r32);
+      RS_LAUNCHED(2);
+      RS_CHECK_LAUNCH();
+      RS_CUDA(cudaEventRecord(h.ev_r, sr));
     }
-    RS_LAUNCHED(2);
+    spgemm_fill(L.A, L.P, AP, ap_tot, ap_mx, F + AF_APNNZ, s);
+    RS_CUDA(cudaStreamWaitEvent(s, h.ev_r, 0));
     // A_{l+1} = R (A P)
     spgemm_count(L.R, AP, F + AF_RAPTOT, F + AF_RAPMX, s);
-    hf = amg_read(h, 0, AF_SLOTS, s);                   // wait 2
+    hf = amg_read(h, AF_ZERO, AF_CNT - AF_ZERO, s);     // wait 2
     AP.nnz = hf[AF_APNNZ];
-    spgemm_fill(L.R, AP, h.lev[l + 1].A, hf[AF_RAPTOT], hf[AF_RAPMX], F + AF_LNNZ + l + 1, s);
-    if (mixed) { csr_cast(L.P, L.P32, s); csr_cast(L.R, L.R32, s); }
+    spgemm_fill(L.R, AP, h.lev[l + 1].A, hf[AF_RAPTOT], hf[AF_RAPMX], F + AF_LNNZ + l + 1, s,
+                mixed ? &h.lev[l + 1].A32 : nullptr);
+    if (mixed && o.interp == SIM_INTERP_EXTI) csr_cast(L.P, L.P32, s);
     l++;
   }
   h.nlev = l + 1;
@@ -1234,7 +1325,6 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
     for (int k = 1; k < h.nlev; k++) if (h.lev[k].A.nnz < 0) h.lev[k].A.nnz = hf[AF_LNNZ + k];
   }
   for (int k = 0; k < h.nlev; k++) h.lev[k].nnz_prev = h.lev[k].A.nnz;
-  for (int k = 0; k < h.nlev && mixed; k++) csr_cast(h.lev[k].A, h.lev[k].A32, s);
   amg_level &C = h.lev[l];
   if (h.coarse_dense) {
     int n = C.A.n;

@@ -118,7 +118,9 @@ int rs_scan(const int *in, int *out, int n, cudaStream_t s);
 // the same without a host wait: the total goes to device memory, at tail
 // (e.g. out + n) and tot2 (either may be nullptr); in may alias out when
 // tail is not in[n] of a later use.  Stream-ordered, no synchronisation.
-void rs_scan_dev(const int *in, int *out, int n, int *tail, int *tot2, cudaStream_t s);
+void rs_scan_dev(const int *in, int *out, int n, int *tail, int *tot2, cudaStream_t s, dbuf<int> *part = nullptr);
+// two arrays of n in place, their totals at tail / tot2 each
+void rs_scan_dev2(int *a, int *tail_a, int *tot_a, int *b, int *tail_b, int *tot_b, int n, cudaStream_t s);
 // deterministic reductions (fixed association order for a given n)
 void rs_dot_partials(const double *x, const double *y, int n, double *partials, int nblk, cudaStream_t s);
 double rs_norm2(const double *x, int n, cudaStream_t s);   // syncs
@@ -176,6 +178,10 @@ struct amg_hier {
   dbuf<double> hashw;           // PMIS weights
   dbuf<int8_t> newc;
   dbuf<int> plist;              // PMIS undecided-point lists (two of n)
+  bool tpos0 = false;           // level 0's transposed positions are known (its pattern is fixed)
+  cudaStream_t st_r = nullptr;  // R = P^T, beside the products of A P
+  cudaEvent_t ev_p = nullptr, ev_r = nullptr;
+  dbuf<int> scan_r;             // scan scratch of that stream
   // the V-cycle of the current hierarchy as a CUDA graph ([0] FP64, [1] FP32),
   // captured on first use after a setup; the capture stream only records
   cudaGraphExec_t vc_exec[2] = {nullptr, nullptr};
@@ -184,7 +190,14 @@ struct amg_hier {
   void drop_graphs() {
     for (auto &e : vc_exec) if (e) { cudaGraphExecDestroy(e); e = nullptr; }
   }
-  ~amg_hier() { drop_graphs(); if (cap) cudaStreamDestroy(cap); if (hflag) cudaFreeHost(hflag); }
+  ~amg_hier() {
+    drop_graphs();
+    if (cap) cudaStreamDestroy(cap);
+    if (st_r) cudaStreamDestroy(st_r);
+    if (ev_p) cudaEventDestroy(ev_p);
+    if (ev_r) cudaEventDestroy(ev_r);
+    if (hflag) cudaFreeHost(hflag);
+  }
 };
 
 void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s);   // level 0 A must be filled

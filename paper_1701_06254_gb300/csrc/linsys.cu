@@ -189,9 +189,13 @@ __global__ void k_identity_d(int nb, double *dmat) {
 }
 
 // A_pp: entry [0][0] of every cell-cell block (Pi_r of eq. 34 keeps cell pressures)
-__global__ void k_extract_app(int nnz, const int *src, const double *val, double *v) {
+// (v32: the FP32 copy of the V-cycle's level 0, or nullptr)
+__global__ void k_extract_app(int nnz, const int *src, const double *val, double *v, float *v32) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < nnz) v[k] = val[4 * (size_t)src[k]];
+  if (k >= nnz) return;
+  const double x = val[4 * (size_t)src[k]];
+  v[k] = x;
+  if (v32) v32[k] = (float)x;
 }
 
 // ------------------------------------------------ double-float helpers ---
@@ -520,7 +524,9 @@ void ls_setup(sim_ls_s *ls) {
   }
   if (!(ls->o.decoupling == SIM_DEC_QI && v32)) RS_LAUNCHED(1);
   csr_dev<double> &A0 = ls->amg.lev[0].A;
-  k_extract_app<<<grid_for(A0.nnz, 256), 256, 0, s>>>(A0.nnz, ls->app_src.p, ls->val.p, A0.v.p);
+  if (v32) ls->amg.lev[0].A32.v.ensure(A0.nnz);
+  k_extract_app<<<grid_for(A0.nnz, 256), 256, 0, s>>>(A0.nnz, ls->app_src.p, ls->val.p, A0.v.p,
+                                                        v32 ? ls->amg.lev[0].A32.v.p : nullptr);
   RS_LAUNCHED(1);
   }
   RS_CHECK_LAUNCH();

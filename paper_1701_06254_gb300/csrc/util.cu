@@ -91,8 +91,8 @@ __global__ void k_scan_empty(int *tail, int *tot2) {
   if (tot2) *tot2 = 0;
 }
 // one block over the whole array, chunk after chunk (short arrays: one
-// launch instead of three)
-__global__ void k_scan_one(const int *in, int *out, int n, int *tail, int *tot2) {
+// launch instead of two)
+__device__ __forceinline__ void scan_one(const int *in, int *out, int n, int *tail, int *tot2) {
   __shared__ int sh[SCAN_BS / 32]; __shared__ int tot;
   int carry = 0;
   for (int c0 = 0; c0 < n; c0 += SCAN_CHUNK) {
@@ -109,24 +109,40 @@ __global__ void k_scan_one(const int *in, int *out, int n, int *tail, int *tot2)
     if (tot2) *tot2 = carry;
   }
 }
-void rs_scan_dev(const int *in, int *out, int n, int *tail, int *tot2, cudaStream_t s) {
+__global__ void k_scan_one(const int *in, int *out, int n, int *tail, int *tot2) { scan_one(in, out, n, tail, tot2); }
+__global__ void k_scan_one2(int *a, int *tail_a, int *tot_a, int *b, int *tail_b, int *tot_b, int n) {
+  if (blockIdx.x) scan_one(b, b, n, tail_b, tot_b); else scan_one(a, a, n, tail_a, tot_a);
+}
+static const int SCAN_ONE_MAX = 8 * SCAN_CHUNK;
+void rs_scan_dev(const int *in, int *out, int n, int *tail, int *tot2, cudaStream_t s, dbuf<int> *scratch) {
   if (n <= 0) {
     k_scan_empty<<<1, 1, 0, s>>>(tail, tot2);
     RS_LAUNCHED(1);
     return;
   }
-  if (n <= 8 * SCAN_CHUNK) {
+  if (n <= SCAN_ONE_MAX) {
     k_scan_one<<<1, SCAN_BS, 0, s>>>(in, out, n, tail, tot2);
     RS_LAUNCHED(1);
     RS_CHECK_LAUNCH();
     return;
   }
   int nblk = (n + SCAN_CHUNK - 1) / SCAN_CHUNK;
-  static thread_local dbuf<int> part;
+  static thread_local dbuf<int> own;
+  dbuf<int> &part = scratch ? *scratch : own;
   part.ensure(nblk + 1);
   k_scan_partials<<<nblk, SCAN_BS, 0, s>>>(in, n, part.p);
   k_scan_final<<<nblk, SCAN_BS, 0, s>>>(in, out, n, part.p, nblk, tail, tot2);
   RS_LAUNCHED(2);
+  RS_CHECK_LAUNCH();
+}
+void rs_scan_dev2(int *a, int *tail_a, int *tot_a, int *b, int *tail_b, int *tot_b, int n, cudaStream_t s) {
+  if (n <= 0 || n > SCAN_ONE_MAX) {
+    rs_scan_dev(a, a, n, tail_a, tot_a, s);
+    rs_scan_dev(b, b, n, tail_b, tot_b, s);
+    return;
+  }
+  k_scan_one2<<<2, SCAN_BS, 0, s>>>(a, tail_a, tot_a, b, tail_b, tot_b, n);
+  RS_LAUNCHED(1);
   RS_CHECK_LAUNCH();
 }
 
