@@ -18,10 +18,14 @@
 #include <climits>
 
 // ------------------------------------------------------------ pattern -----
-__global__ void k_tpos(int n, const int *rp, const int *ci, int *tpos, int *err) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+// tpos[q]: the position of (j, i) in row j for entry q = (i, j), by binary
+// search; L lanes per row (one for short rows, a warp for long ones: a thread
+// walking 40 searches one after another was latency-bound)
+template <int L>
+__device__ __forceinline__ void tpos_row(int g, int n, const int *rp, const int *ci, int *tpos, int *err) {
+  const int i = g / L;
   if (i >= n) return;
-  for (int q = rp[i]; q < rp[i + 1]; q++) {
+  for (int q = rp[i] + g % L; q < rp[i + 1]; q += L) {
     int j = ci[q], lo = rp[j], hi = rp[j + 1] - 1, pos = -1;
     while (lo <= hi) {
       int mid = (lo + hi) >> 1, c = ci[mid];
@@ -33,32 +37,23 @@ __global__ void k_tpos(int n, const int *rp, const int *ci, int *tpos, int *err)
   }
 }
 
-// the same with one warp per row (levels with long rows: a thread walking
-// 40 binary searches one after another was latency-bound)
-__global__ void k_tpos_warp(int n, const int *rp, const int *ci, int *tpos, int *err) {
-  int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (i >= n) return;
-  for (int q = rp[i] + lane; q < rp[i + 1]; q += 32) {
-    int j = ci[q], lo = rp[j], hi = rp[j + 1] - 1, pos = -1;
-    while (lo <= hi) {
-      int mid = (lo + hi) >> 1, c = ci[mid];
-      if (c == i) { pos = mid; break; }
-      if (c < i) lo = mid + 1; else hi = mid - 1;
-    }
-    if (pos < 0) atomicExch(err, 1);
-    tpos[q] = pos < 0 ? q : pos;
-  }
-}
-
 // Strength of connection (S), and with dinv given the l1-Jacobi diagonal of
 // the same row (d_i = a_ii + sum_{j != i} |a_ij|; 1 / d_i, FP64 and FP32),
 // from one pass over the row.  A thread per row; ROW_B entries' loads are
 // issued together (one entry at a time, a row of 36 entries was a chain of 36
 // L2 latencies, twice: 31 us on a level of 1,600 rows against 11 us), and a
 // row of at most ROW_B entries stays in registers for the second pass.
+// The blocks from nstr on find the transposed positions (L lanes per row)
+// beside it: both need only the level's operator.
 #define ROW_B 8
-__global__ void k_strength(int n, const int *__restrict__ rp, const int *__restrict__ ci, const double *__restrict__ v,
-                           double theta, uint8_t *__restrict__ S, double *dinv, float *dinv32) {
+template <int L>
+__global__ void __launch_bounds__(128) k_strength(int n, const int *__restrict__ rp, const int *__restrict__ ci,
+                                                  const double *__restrict__ v, double theta, uint8_t *__restrict__ S,
+                                                  double *dinv, float *dinv32, unsigned nstr, int *tpos, int *err) {
+  if (blockIdx.x >= nstr) {
+    tpos_row<L>((blockIdx.x - nstr) * blockDim.x + threadIdx.x, n, rp, ci, tpos, err);
+    return;
+  }
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   bool have = false; double mx = 0.0; long long mxk = 0;
@@ -292,6 +287,32 @@ __global__ void k_cflag(int n, const int8_t *cf, int *flag) {
   if (i < n) flag[i] = cf[i] == 1;
 }
 
+// ------------------------------------------------ products of a row ------
+// products per row of C; mx = 1 + the most products of a row that the
+// hash kernel handles, 0 if there is none
+#define SPG_KMAX 8                               // (see SpGEMM below)
+#define SPG_ROW_B 8
+#define SPG_MERGE_P 96
+__device__ __forceinline__ void row_products(int i, int n, const int *arp, const int *aci, const int *bbeg,
+                                             const int *bend, int *prod, int *mx, int merge_p) {
+  if (i >= n) return;
+  int s = 0;
+  const int q0 = arp[i], q1 = arp[i + 1];
+  for (int qb = q0; qb < q1; qb += SPG_ROW_B) {       // several entries' loads in flight together
+    int k[SPG_ROW_B];
+#pragma unroll
+    for (int u = 0; u < SPG_ROW_B; u++) k[u] = qb + u < q1 ? aci[qb + u] : -1;
+#pragma unroll
+    for (int u = 0; u < SPG_ROW_B; u++) if (k[u] >= 0) s += bend[k[u]] - bbeg[k[u]];
+  }
+  prod[i] = s;
+  if (q1 - q0 > SPG_KMAX || s > merge_p) atomicMax(mx, s + 1);   // + 1: "a hash row exists" even with 0 products
+}
+__global__ void k_row_products(int n, const int *arp, const int *aci, const int *bbeg, const int *bend, int *prod,
+                               int *mx, int merge_p) {
+  row_products(blockIdx.x * blockDim.x + threadIdx.x, n, arp, aci, bbeg, bend, prod, mx, merge_p);
+}
+
 // ------------------------------------------------------- interpolation ----
 // entries per row of P, and the C flag of each point
 __global__ void k_interp_count(int n, const int *__restrict__ rp, const int *__restrict__ ci,
@@ -314,11 +335,17 @@ __global__ void k_interp_count(int n, const int *__restrict__ rp, const int *__r
 
 // pcap: capacity of pci / pv (a row that would pass it sets *err and is
 // skipped; nnz(P) <= nnz(A) makes that impossible for direct interpolation)
-// pv32: the FP32 copy of pv (mixed precision) or nullptr
+// pv32: the FP32 copy of pv (mixed precision) or nullptr.  The blocks from
+// nfill on count the products of A P beside it (they need P's row lengths only).
 __global__ void k_interp_fill(int n, const int *__restrict__ rp, const int *__restrict__ ci,
                               const double *__restrict__ v, const uint8_t *__restrict__ S,
                               const int8_t *__restrict__ cf, const int *__restrict__ cidx, const int *__restrict__ prp,
-                              int *pci, double *pv, float *pv32, int pcap, int *err) {
+                              int *pci, double *pv, float *pv32, int pcap, int *err, unsigned nfill, int *prod,
+                              int *mx, int merge_p) {
+  if (blockIdx.x >= nfill) {
+    row_products((blockIdx.x - nfill) * blockDim.x + threadIdx.x, n, rp, ci, prp, prp + 1, prod, mx, merge_p);
+    return;
+  }
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int o = prp[i];
@@ -606,25 +633,6 @@ __global__ void k_sort_rows_g(int n, const int *rp, int *ci, double *v, float *v
 // others: k_spgemm_hash (one warp per row).  One pass: each row is written at the offset of its product
 // count (an upper bound of its length) into a scratch array, then the rows
 // are packed.
-// products per row of C; mx = 1 + the most products of a row that the
-// hash kernel handles, 0 if there is none
-#define SPG_KMAX 8
-#define SPG_MERGE_P 96
-__global__ void k_row_products(int n, const int *arp, const int *aci, const int *brp, int *prod, int *mx, int merge_p) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int s = 0;
-  const int q1 = arp[i + 1];
-  for (int q0 = arp[i]; q0 < q1; q0 += ROW_B) {       // ROW_B entries' loads in flight together
-    int k[ROW_B];
-#pragma unroll
-    for (int u = 0; u < ROW_B; u++) k[u] = q0 + u < q1 ? aci[q0 + u] : -1;
-#pragma unroll
-    for (int u = 0; u < ROW_B; u++) if (k[u] >= 0) s += brp[k[u] + 1] - brp[k[u]];
-  }
-  prod[i] = s;
-  if (arp[i + 1] - arp[i] > SPG_KMAX || s > merge_p) atomicMax(mx, s + 1);   // + 1: "a hash row exists" even with 0 products
-}
 // C row i = scratch[toff[i] .. toff[i] + clen[i]), eight lanes per row
 // (cv32: the FP32 copy of cv or nullptr)
 __global__ void k_pack_rows(int n, const int *toff, const int *clen, const int *crp, const int *tci, const double *tv,
@@ -650,8 +658,9 @@ __global__ void k_pack_rows(int n, const int *toff, const int *clen, const int *
 // (measured on the coarser levels of the 1M-cell hierarchy).
 template <int K>
 __global__ void __launch_bounds__(128) k_spgemm_merge(int n, const int *arp, const int *aci, const double *av,
-                                                      const int *brp, const int *bci, const double *bv,
-                                                      const int *toff, int *clen, int *cci, double *cv, int merge_p) {
+                                                      const int *bbeg, const int *bend, const int *bci,
+                                                      const double *bv, const int *toff, int *clen, int *cci,
+                                                      double *cv, int merge_p, int ends) {
   int row = blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= n) return;
   int a0 = arp[row], k = arp[row + 1] - a0;
@@ -663,7 +672,7 @@ __global__ void __launch_bounds__(128) k_spgemm_merge(int n, const int *arp, con
     col[q] = INT_MAX; pos[q] = 0; end[q] = 0; a[q] = 0.0;
     if (q < k) {
       int kk = aci[a0 + q];
-      pos[q] = brp[kk]; end[q] = brp[kk + 1]; a[q] = av[a0 + q];
+      pos[q] = bbeg[kk]; end[q] = bend[kk]; a[q] = av[a0 + q];
       if (pos[q] < end[q]) col[q] = bci[pos[q]];
     }
   }
@@ -699,7 +708,7 @@ __global__ void __launch_bounds__(128) k_spgemm_merge(int n, const int *arp, con
     cci[out + cnt] = c; cv[out + cnt] = s;
     cnt++;
   }
-  clen[row] = cnt;
+  clen[row] = ends ? out + cnt : cnt;
 }
 
 // Rows that the merge kernel leaves (more than SPG_KMAX entries in A, or
@@ -721,9 +730,10 @@ __host__ __device__ constexpr size_t spg_warp_doubles(int tcap) {
   return (size_t)tcap + 64 + ((size_t)tcap + 65 + 1) / 2;
 }
 __global__ void __launch_bounds__(256) k_spgemm_hash(int n, const int *arp, const int *aci, const double *av,
-                                                     const int *brp, const int *bci, const double *bv,
-                                                     const int *toff, int *clen, int *cci, double *cv, int tcap,
-                                                     int lo_p, double *gscratch, int merge_p) {
+                                                     const int *bbeg, const int *bend, const int *bci,
+                                                     const double *bv, const int *toff, int *clen, int *cci,
+                                                     double *cv, int tcap, int lo_p, double *gscratch, int merge_p,
+                                                     int ends) {
   extern __shared__ double sm_hash[];
   const int warps = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned FULL = 0xffffffffu;
@@ -743,7 +753,7 @@ __global__ void __launch_bounds__(256) k_spgemm_hash(int n, const int *arp, cons
     for (int q0 = a0; q0 < a1; q0 += 32) {
       int q = q0 + lane, len = 0, k = 0;
       double a = 0.0;
-      if (q < a1) { k = aci[q]; len = brp[k + 1] - brp[k]; a = av[q]; }
+      if (q < a1) { k = aci[q]; len = bend[k] - bbeg[k]; a = av[q]; }
       int incl = len;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) { int y = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += y; }
@@ -757,7 +767,7 @@ __global__ void __launch_bounds__(256) k_spgemm_hash(int n, const int *arp, cons
         if (t < tot) {
           int lo = 0, hi = nseg - 1;                          // last segment starting at or before t
           while (lo < hi) { int md = (lo + hi + 1) >> 1; if (seg_off[md] <= t) lo = md; else hi = md - 1; }
-          int b = brp[seg_k[lo]] + (t - seg_off[lo]), c = bci[b];
+          int b = bbeg[seg_k[lo]] + (t - seg_off[lo]), c = bci[b];
           prod = mul_rn(seg_a[lo], bv[b]);
           int h = (int)(((unsigned)c * 0x9E3779B1u) & (unsigned)(T - 1));
           for (int it = 0; it < T; it++) {
@@ -825,21 +835,30 @@ __global__ void __launch_bounds__(256) k_spgemm_hash(int n, const int *arp, cons
         }
       for (int i = lane; i < u; i += 32) { cci[out + i] = keys[i]; cv[out + i] = vals[i]; }
     }
-    if (lane == 0) clen[row] = u;
+    if (lane == 0) clen[row] = ends ? out + u : u;
     __syncwarp();
   }
 }
 
-// SpGEMM C = A B in two phases with one host wait between them.
+// SpGEMM C = A B in two phases with one host wait between them.  B's row k is
+// [beg[k], end[k]) of ci / v (a CSR matrix: rp and rp + 1).
 // spgemm_count: products per row of C (scratch offsets, toff) and their
 // total in *tot, the long-row marker (1 + the most products of a row that
 // the hash kernel handles, 0 if none) in *mx (which must be 0 before);
-// no host wait.  spgemm_fill: given those two values on the host, the
-// numeric product into scratch, the row pointers of C (C.rp[n] and *nnz =
-// nnz(C) on the device) and the packed rows; C's arrays are sized by the
-// product total, an upper bound of nnz(C), so no further wait is needed.
-struct spg_scratch { dbuf<int> toff, clen, tci; dbuf<double> tv, gs; };
-static spg_scratch &spg() { static thread_local spg_scratch z; return z; }
+// no host wait.  spgemm_numeric: given those two values on the host, the
+// numeric product into scratch, clen the rows' lengths (or, with ends, where
+// they end: A P of at most SPG_PACK_MIN products is read by the next product
+// straight from its scratch rows, which saves its row scan and a pass over
+// it; beyond, the gaps between the rows cost the next product more: on the
+// 1M-cell case's finest levels 100 us against 80 us of packing).  spgemm_pack: the row
+// pointers of C (C.rp[n] and *nnz = nnz(C) on the device) and the packed
+// rows; C's arrays are sized by the product total, an upper bound of nnz(C),
+// so no further wait is needed.
+#define SPG_PACK_MIN (4 << 20)
+struct spg_scratch { dbuf<int> toff, clen, tci; dbuf<double> tv; };
+static spg_scratch &spg(int k) { static thread_local spg_scratch z[2]; return z[k]; }   // [0] A P, [1] R (A P)
+struct row_ref { const int *beg, *end, *ci; const double *v; };
+static row_ref rows_of(const csr_dev<double> &B) { return {B.rp.p, B.rp.p + 1, B.ci.p, B.v.p}; }
 // Rows for the thread-per-row merge kernel (at most SPG_KMAX entries in A
 // and at most this many products): only when the product has enough rows to
 // fill the GPU with threads; on smaller products a thread's serial merge is
@@ -848,19 +867,21 @@ static spg_scratch &spg() { static thread_local spg_scratch z; return z; }
 // same bits, so the split changes no result.
 static int spg_merge_p(int n) { return n >= 65536 ? SPG_MERGE_P : -1; }
 
-static void spgemm_count(const csr_dev<double> &A, const csr_dev<double> &B, int *tot, int *mx, cudaStream_t s) {
-  spg_scratch &z = spg();
+// counted: k_interp_fill's launch has counted the products already
+static void spgemm_count(const csr_dev<double> &A, const row_ref &B, spg_scratch &z, int *tot, int *mx, bool counted,
+                         cudaStream_t s) {
   int n = A.n;
-  z.toff.ensure(n + 1); z.clen.ensure(n + 1);
-  k_row_products<<<grid_for(n, 256), 256, 0, s>>>(n, A.rp.p, A.ci.p, B.rp.p, z.toff.p, mx, spg_merge_p(n));
-  RS_LAUNCHED(1);
+  if (!counted) {
+    z.toff.ensure(n + 1); z.clen.ensure(n + 1);
+    k_row_products<<<grid_for(n, 128), 128, 0, s>>>(n, A.rp.p, A.ci.p, B.beg, B.end, z.toff.p, mx, spg_merge_p(n));
+    RS_LAUNCHED(1);
+  }
   rs_scan_dev(z.toff.p, z.toff.p, n, z.toff.p + n, tot, s);      // row offsets into the scratch arrays
 }
 
-// C32: C's FP32 values are written too (nullptr: FP64 only)
-static void spgemm_fill(const csr_dev<double> &A, const csr_dev<double> &B, csr_dev<double> &C, int total, int mx1,
-                        int *nnz, cudaStream_t s, csr_dev<float> *C32 = nullptr) {
-  spg_scratch &z = spg();
+static void spgemm_numeric(const csr_dev<double> &A, const row_ref &B, spg_scratch &z, int total, int mx1, int ends,
+                           cudaStream_t s) {
+  static thread_local dbuf<double> gs;
   int n = A.n, mx = std::max(mx1 - 1, 0);
   // hash-table slots per warp: at least the products of the largest row in
   // the launch; rows beyond 1024 products (above the 99.9th percentile on
@@ -877,28 +898,33 @@ static void spgemm_fill(const csr_dev<double> &A, const csr_dev<double> &B, csr_
     attr = true;
   }
   z.tci.ensure(std::max(total, 1)); z.tv.ensure(std::max(total, 1));
-  C.n = n; C.m = B.m; C.nnz = -1;                      // known on the host at the next wait
-  C.rp.ensure(n + 1);
   int mp = spg_merge_p(n);
   if (mp >= 0) {
-    k_spgemm_merge<SPG_KMAX><<<grid_for(n, 128), 128, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, B.rp.p, B.ci.p, B.v.p,
-                                                              z.toff.p, z.clen.p, z.tci.p, z.tv.p, mp);
+    k_spgemm_merge<SPG_KMAX><<<grid_for(n, 128), 128, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, B.beg, B.end, B.ci, B.v,
+                                                              z.toff.p, z.clen.p, z.tci.p, z.tv.p, mp, ends);
     RS_LAUNCHED(1);
   }
   if (mx1 > 0) {                                       // rows for the hash kernel
     unsigned grid = (unsigned)std::min<size_t>((n + warps - 1) / warps, 152 * 32);
-    k_spgemm_hash<<<grid, warps * 32, smem, s>>>(n, A.rp.p, A.ci.p, A.v.p, B.rp.p, B.ci.p, B.v.p, z.toff.p,
-                                                 z.clen.p, z.tci.p, z.tv.p, tcap, -1, nullptr, mp);
+    k_spgemm_hash<<<grid, warps * 32, smem, s>>>(n, A.rp.p, A.ci.p, A.v.p, B.beg, B.end, B.ci, B.v, z.toff.p,
+                                                 z.clen.p, z.tci.p, z.tv.p, tcap, -1, nullptr, mp, ends);
     RS_LAUNCHED(1);
     if (tall > tcap) {                                 // rows beyond the shared-memory capacity
       const int gw = 4, gblocks = 64;
-      z.gs.ensure((size_t)gblocks * gw * spg_warp_doubles(tall));
-      k_spgemm_hash<<<gblocks, gw * 32, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, B.rp.p, B.ci.p, B.v.p, z.toff.p, z.clen.p,
-                                                z.tci.p, z.tv.p, tall, tcap, z.gs.p, mp);
+      gs.ensure((size_t)gblocks * gw * spg_warp_doubles(tall));
+      k_spgemm_hash<<<gblocks, gw * 32, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, B.beg, B.end, B.ci, B.v, z.toff.p, z.clen.p,
+                                                z.tci.p, z.tv.p, tall, tcap, gs.p, mp, ends);
       RS_LAUNCHED(1);
     }
   }
   RS_CHECK_LAUNCH();
+}
+
+// C32: C's FP32 values are written too (nullptr: FP64 only)
+static void spgemm_pack(int n, int m, spg_scratch &z, csr_dev<double> &C, csr_dev<float> *C32, int total, int *nnz,
+                        cudaStream_t s) {
+  C.n = n; C.m = m; C.nnz = -1;                        // known on the host at the next wait
+  C.rp.ensure(n + 1);
   rs_scan_dev(z.clen.p, C.rp.p, n, C.rp.p + n, nnz, s);
   C.ci.ensure(std::max(total, 1)); C.v.ensure(std::max(total, 1));
   if (C32) C32->v.ensure(std::max(total, 1));
@@ -1093,9 +1119,9 @@ enum {
   AF_PCAP = 33,      // a row of P beyond its capacity
   AF_NC = 34,        // C points (coarse size)
   AF_PNNZ = 35,      // nnz(P)
-  AF_APTOT = 36, AF_APMX = 37, AF_APNNZ = 38,  // products, long-row marker and nnz of A P
-  AF_RAPTOT = 39, AF_RAPMX = 40,               // the same for R (A P)
-  AF_PRND = 41,      // PMIS rounds taken (-1: not finished within the cap)
+  AF_APTOT = 36, AF_APMX = 37,                 // products and long-row marker of A P
+  AF_RAPTOT = 38, AF_RAPMX = 39,               // the same for R (A P)
+  AF_PRND = 40,      // PMIS rounds taken (-1: not finished within the cap)
   AF_CNT = 48,       // [48 + r]: undecided points after PMIS round r - 1 (r = 0: after the initialisation)
   AF_ROUNDS_MAX = 1020,
   AF_WORDS = AF_CNT + AF_ROUNDS_MAX + 8
@@ -1159,6 +1185,7 @@ static int build_p(amg_level &L, amg_hier &h, const rs_opts &o, int n, size_t ac
                    cudaStream_t s) {
   int *F = h.flag.p;
   const bool mixed = o.precision != SIM_PREC_FP64;
+  spg_scratch &z = spg(0);
   L.P.n = n;
   L.P.rp.ensure(n + 1);
   int pnnz = -1;
@@ -1192,14 +1219,16 @@ static int build_p(amg_level &L, amg_hier &h, const rs_opts &o, int n, size_t ac
     rs_scan_dev2(L.P.rp.p, L.P.rp.p + n, F + AF_PNNZ, cidx.p, cidx.p + n, F + AF_NC, n, s);
     L.P.ci.ensure(acap > 0 ? acap : 1); L.P.v.ensure(acap > 0 ? acap : 1);
     if (mixed) L.P32.v.ensure(L.P.ci.n);
-    k_interp_fill<<<grid_for(n, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.A.v.p, L.strong.p, L.cf.p, cidx.p,
-                                                   L.P.rp.p, L.P.ci.p, L.P.v.p, mixed ? L.P32.v.p : nullptr,
-                                                   (int)L.P.ci.n, F + AF_PCAP);
+    z.toff.ensure(n + 1); z.clen.ensure(n + 1);
+    const unsigned g = grid_for(n, 128);
+    k_interp_fill<<<2 * g, 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.A.v.p, L.strong.p, L.cf.p, cidx.p, L.P.rp.p, L.P.ci.p,
+                                        L.P.v.p, mixed ? L.P32.v.p : nullptr, (int)L.P.ci.n, F + AF_PCAP, g, z.toff.p,
+                                        F + AF_APMX, spg_merge_p(n));
     RS_LAUNCHED(1);
   }
   RS_CHECK_LAUNCH();
   RS_CUDA(cudaEventRecord(h.ev_p, s));
-  spgemm_count(L.A, L.P, F + AF_APTOT, F + AF_APMX, s);
+  spgemm_count(L.A, rows_of(L.P), z, F + AF_APTOT, F + AF_APMX, o.interp != SIM_INTERP_EXTI, s);
   return pnnz;
 }
 
@@ -1240,15 +1269,21 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
       break;
     }
     rs_fill_i(F + AF_ZERO, 0, AF_WORDS - AF_ZERO, s);
-    if (l == 0 && h.tpos0) {}                           // the finest pattern never changes: positions kept
-    else if (nnz_hint > 8LL * n) k_tpos_warp<<<grid_for((size_t)n * 32, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.tpos.p, F + AF_SYM);
-    else k_tpos<<<grid_for(n, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.tpos.p, F + AF_SYM);
-    k_strength<<<grid_for(n, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.A.v.p, o.theta, L.strong.p, L.dinv.p,
-                                              mixed ? L.dinv32.p : nullptr);
+    {
+      // (the finest pattern never changes: its positions are kept)
+      const unsigned nstr = grid_for(n, 128);
+      const bool wide = nnz_hint > 8LL * n, have = l == 0 && h.tpos0;
+      const unsigned nt = have ? 0 : wide ? grid_for((size_t)n * 32, 128) : nstr;
+      auto go = [&](auto kern) {
+        kern<<<nstr + nt, 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.A.v.p, o.theta, L.strong.p, L.dinv.p,
+                                       mixed ? L.dinv32.p : nullptr, nstr, L.tpos.p, F + AF_SYM);
+      };
+      if (wide) go(k_strength<32>); else go(k_strength<1>);
+    }
     h.hashw.ensure(n); h.newc.ensure(n); h.plist.ensure(2 * (size_t)n);
     k_pmis_init<<<grid_for(n, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.strong.p, L.tpos.p, o.seed, l,
                                                  h.hashw.p, L.cf.p, h.newc.p, F + AF_CNT, h.plist.p);
-    RS_LAUNCHED(3);
+    RS_LAUNCHED(2);
     RS_CHECK_LAUNCH();
     // full-grid rounds while the lists are long (the previous setup's
     // counts say how many), then the rest in one block until a list is empty
@@ -1274,7 +1309,6 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
     L.nc = nc;
     if (nc == 0) { h.coarse_dense = 0; break; }
     L.P.m = nc;
-    static thread_local csr_dev<double> AP;
     // R = P^T, from the moment P is complete, beside A P
     L.R.n = nc; L.R.m = n; L.R.nnz = L.P.nnz;
     L.R.rp.ensure(nc + 1); L.R.ci.ensure(L.P.nnz > 0 ? L.P.nnz : 1); L.R.v.ensure(L.P.nnz > 0 ? L.P.nnz : 1);
@@ -1305,14 +1339,23 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
       RS_CHECK_LAUNCH();
       RS_CUDA(cudaEventRecord(h.ev_r, sr));
     }
-    spgemm_fill(L.A, L.P, AP, ap_tot, ap_mx, F + AF_APNNZ, s);
+    spg_scratch &ap = spg(0), &rap = spg(1);
+    static thread_local csr_dev<double> apc;
+    row_ref AP;
+    if (ap_tot > SPG_PACK_MIN) {
+      spgemm_numeric(L.A, rows_of(L.P), ap, ap_tot, ap_mx, 0, s);
+      spgemm_pack(n, nc, ap, apc, nullptr, ap_tot, nullptr, s);
+      AP = rows_of(apc);
+    } else {
+      spgemm_numeric(L.A, rows_of(L.P), ap, ap_tot, ap_mx, 1, s);
+      AP = {ap.toff.p, ap.clen.p, ap.tci.p, ap.tv.p};
+    }
     RS_CUDA(cudaStreamWaitEvent(s, h.ev_r, 0));
     // A_{l+1} = R (A P)
-    spgemm_count(L.R, AP, F + AF_RAPTOT, F + AF_RAPMX, s);
+    spgemm_count(L.R, AP, rap, F + AF_RAPTOT, F + AF_RAPMX, false, s);
     hf = amg_read(h, AF_ZERO, AF_CNT - AF_ZERO, s);     // wait 2
-    AP.nnz = hf[AF_APNNZ];
-    spgemm_fill(L.R, AP, h.lev[l + 1].A, hf[AF_RAPTOT], hf[AF_RAPMX], F + AF_LNNZ + l + 1, s,
-                mixed ? &h.lev[l + 1].A32 : nullptr);
+    spgemm_numeric(L.R, AP, rap, hf[AF_RAPTOT], hf[AF_RAPMX], 0, s);
+    spgemm_pack(nc, nc, rap, h.lev[l + 1].A, mixed ? &h.lev[l + 1].A32 : nullptr, hf[AF_RAPTOT], F + AF_LNNZ + l + 1, s);
     if (mixed && o.interp == SIM_INTERP_EXTI) csr_cast(L.P, L.P32, s);
     l++;
   }

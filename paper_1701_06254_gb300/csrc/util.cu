@@ -90,18 +90,33 @@ __global__ void k_scan_empty(int *tail, int *tot2) {
   if (tail) *tail = 0;
   if (tot2) *tot2 = 0;
 }
-// one block over the whole array, chunk after chunk (short arrays: one
-// launch instead of two)
+// One block of 1024 threads over the whole array, 8192 values per pass (arrays
+// of up to SCAN_ONE_MAX: one launch of a few microseconds instead of two)
+#define SCAN_ONE_BS 1024
+#define SCAN_ONE_IT 8
 __device__ __forceinline__ void scan_one(const int *in, int *out, int n, int *tail, int *tot2) {
-  __shared__ int sh[SCAN_BS / 32]; __shared__ int tot;
+  __shared__ int sh[SCAN_ONE_BS / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int carry = 0;
-  for (int c0 = 0; c0 < n; c0 += SCAN_CHUNK) {
-    int base = c0 + threadIdx.x * SCAN_IT;
-    int v[SCAN_IT], s = 0;
-    for (int k = 0; k < SCAN_IT; k++) { v[k] = (base + k < n) ? in[base + k] : 0; s += v[k]; }
-    int e = block_excl_scan(s, sh, &tot) + carry;
-    for (int k = 0; k < SCAN_IT; k++) if (base + k < n) { out[base + k] = e; e += v[k]; }
-    carry += tot;
+  for (int c0 = 0; c0 < n; c0 += SCAN_ONE_BS * SCAN_ONE_IT) {
+    const int base = c0 + threadIdx.x * SCAN_ONE_IT;
+    int v[SCAN_ONE_IT], s = 0;
+#pragma unroll
+    for (int k = 0; k < SCAN_ONE_IT; k++) v[k] = base + k < n ? in[base + k] : 0;
+#pragma unroll
+    for (int k = 0; k < SCAN_ONE_IT; k++) s += v[k];
+    int x = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { int y = __shfl_up_sync(0xffffffffu, x, o); if (lane >= o) x += y; }
+    if (lane == 31) sh[wid] = x;
+    __syncthreads();
+    int w = sh[lane], z = w;                        // every warp scans the 32 warp totals for itself
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { int y = __shfl_up_sync(0xffffffffu, z, o); if (lane >= o) z += y; }
+    int e = carry + x - s + __shfl_sync(0xffffffffu, z - w, wid);
+    carry += __shfl_sync(0xffffffffu, z, 31);
+#pragma unroll
+    for (int k = 0; k < SCAN_ONE_IT; k++) if (base + k < n) { out[base + k] = e; e += v[k]; }
     __syncthreads();
   }
   if (threadIdx.x == 0) {
@@ -109,11 +124,14 @@ __device__ __forceinline__ void scan_one(const int *in, int *out, int n, int *ta
     if (tot2) *tot2 = carry;
   }
 }
-__global__ void k_scan_one(const int *in, int *out, int n, int *tail, int *tot2) { scan_one(in, out, n, tail, tot2); }
-__global__ void k_scan_one2(int *a, int *tail_a, int *tot_a, int *b, int *tail_b, int *tot_b, int n) {
+__global__ void __launch_bounds__(SCAN_ONE_BS) k_scan_one(const int *in, int *out, int n, int *tail, int *tot2) {
+  scan_one(in, out, n, tail, tot2);
+}
+__global__ void __launch_bounds__(SCAN_ONE_BS) k_scan_one2(int *a, int *tail_a, int *tot_a, int *b, int *tail_b,
+                                                           int *tot_b, int n) {
   if (blockIdx.x) scan_one(b, b, n, tail_b, tot_b); else scan_one(a, a, n, tail_a, tot_a);
 }
-static const int SCAN_ONE_MAX = 8 * SCAN_CHUNK;
+static const int SCAN_ONE_MAX = 3 * SCAN_ONE_BS * SCAN_ONE_IT;
 void rs_scan_dev(const int *in, int *out, int n, int *tail, int *tot2, cudaStream_t s, dbuf<int> *scratch) {
   if (n <= 0) {
     k_scan_empty<<<1, 1, 0, s>>>(tail, tot2);
@@ -121,7 +139,7 @@ void rs_scan_dev(const int *in, int *out, int n, int *tail, int *tot2, cudaStrea
     return;
   }
   if (n <= SCAN_ONE_MAX) {
-    k_scan_one<<<1, SCAN_BS, 0, s>>>(in, out, n, tail, tot2);
+    k_scan_one<<<1, SCAN_ONE_BS, 0, s>>>(in, out, n, tail, tot2);
     RS_LAUNCHED(1);
     RS_CHECK_LAUNCH();
     return;
@@ -141,7 +159,7 @@ void rs_scan_dev2(int *a, int *tail_a, int *tot_a, int *b, int *tail_b, int *tot
     rs_scan_dev(b, b, n, tail_b, tot_b, s);
     return;
   }
-  k_scan_one2<<<2, SCAN_BS, 0, s>>>(a, tail_a, tot_a, b, tail_b, tot_b, n);
+  k_scan_one2<<<2, SCAN_ONE_BS, 0, s>>>(a, tail_a, tot_a, b, tail_b, tot_b, n);
   RS_LAUNCHED(1);
   RS_CHECK_LAUNCH();
 }
