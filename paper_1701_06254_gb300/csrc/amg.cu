@@ -1406,47 +1406,73 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
 }
 
 // -------------------------------------------------------------- V-cycle ---
-template <class T>
-__global__ void k_vc_pre(int n, const int *rp, const int *ci, const T *v, const T *dinv, const T *f, T *x, T *r) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+// The cycle's four sweeps with L lanes per row (1 to 32).  MODE 0:
+// pre-smoothing (x = D^-1 f, r = f - A x; with u given, u already holds
+// D^-1 f); 1: y = A x (and, with o2 given, o2 = D_c^-1 y for the coarse
+// level's pre-smoothing); 2: t = x + P e; 3: post-smoothing (x = t + D^-1 (f
+// - A t)).  One lane per row sums its entries in order, starting from f (or
+// x); several lanes sum a strided part each (consecutive lanes read
+// consecutive entries) and shuffles combine the parts.
+//
+// The operators do not change within a solve, so a kernel fetches its row
+// pointers, its first B columns and values per lane (and the neighbours' D^-1
+// at level 0) before it waits for the kernel that makes its vectors: the
+// chain behind the wait is one gather, and on the coarse levels, a few
+// microseconds of latency per launch, most of it overlaps the kernel before.
+template <class T, int L, int MODE, int B>
+__global__ void __launch_bounds__(256) k_vc(int n, const int *__restrict__ rp, const int *__restrict__ ci,
+                                            const T *__restrict__ v, const T *__restrict__ dinv, const T *f,
+                                            const T *u, T *o1, T *o2) {
   pdl_trigger();
+  const int g = (blockIdx.x * blockDim.x + threadIdx.x) / L, k = threadIdx.x % L;
+  if (L == 1 && g >= n) return;
+  const int i = L == 1 || g < n ? g : n - 1;          // whole groups stay in the shuffles
+  const int q1 = rp[i + 1];
+  int q = rp[i] + k;
+  const bool fd = MODE == 0 && (L == 1 || !u);        // neighbours as f_j D_j^-1
+  const T di = MODE == 0 || MODE == 3 || (MODE == 1 && o2) ? dinv[i] : (T)0;
+  int c[B];
+  T a[B], dj[B];
+  auto fetch = [&]() {
+#pragma unroll
+    for (int b = 0; b < B; b++)
+      if (q + b * L < q1) { c[b] = __ldg(ci + q + b * L); a[b] = __ldg(v + q + b * L); }
+    if (fd) {
+#pragma unroll
+      for (int b = 0; b < B; b++) if (q + b * L < q1) dj[b] = __ldg(dinv + c[b]);
+    }
+  };
+  fetch();
   pdl_wait();
-  if (i >= n) return;
-  T s = f[i];
-  for (int q = rp[i]; q < rp[i + 1]; q++) { int j = ci[q]; s -= v[q] * (f[j] * dinv[j]); }
-  x[i] = f[i] * dinv[i];
-  r[i] = s;
-}
-template <class T>
-__global__ void k_prolong_add(int n, const int *rp, const int *ci, const T *v, const T *e, const T *x, T *t) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  pdl_trigger();
-  pdl_wait();
-  if (i >= n) return;
-  T s = x[i];
-  for (int q = rp[i]; q < rp[i + 1]; q++) s += v[q] * e[ci[q]];
-  t[i] = s;
-}
-template <class T>
-__global__ void k_vc_post(int n, const int *rp, const int *ci, const T *v, const T *dinv, const T *f, const T *t, T *x) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  pdl_trigger();
-  pdl_wait();
-  if (i >= n) return;
-  T s = f[i];
-  for (int q = rp[i]; q < rp[i + 1]; q++) s -= v[q] * t[ci[q]];
-  x[i] = t[i] + dinv[i] * s;
-}
-template <class T>
-__global__ void k_restrict_x(int n, const int *rp, const int *ci, const T *v, const T *u, const T *dinv, T *y, T *x) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  pdl_trigger();
-  pdl_wait();
-  if (i >= n) return;
-  T s = 0;
-  for (int q = rp[i]; q < rp[i + 1]; q++) s += v[q] * u[ci[q]];
-  y[i] = s;
-  x[i] = s * dinv[i];
+  const T *src = fd ? f : u;
+  T s = L == 1 && MODE != 1 ? f[i] : (T)0;
+  while (q < q1) {
+    T x[B];
+#pragma unroll
+    for (int b = 0; b < B; b++) if (q + b * L < q1) x[b] = src[c[b]];
+#pragma unroll
+    for (int b = 0; b < B; b++)
+      if (q + b * L < q1) {
+        const T xj = fd ? x[b] * dj[b] : x[b];
+        if (L == 1 && (MODE == 0 || MODE == 3)) s -= a[b] * xj; else s += a[b] * xj;
+      }
+    q += B * L;
+    if (q < q1) fetch();
+  }
+  if constexpr (L == 1) {
+    if (MODE == 0) { o1[i] = f[i] * di; o2[i] = s; }
+    else if (MODE == 1) { o1[i] = s; if (o2) o2[i] = s * di; }
+    else if (MODE == 2) o1[i] = s;                     // f = x (the smoothed iterate), u = e
+    else o1[i] = u[i] + di * s;                        // u = t
+  } else {
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, L);
+    if (k != 0 || g >= n) return;
+    if (MODE == 0) { if (!u) o1[i] = f[i] * di; o2[i] = f[i] - s; }   // with u, o1 = u holds it already
+    else if (MODE == 1) { o1[i] = s; if (o2) o2[i] = s * di; }
+    else if (MODE == 2) o1[i] = f[i] + s;
+    else o1[i] = u[i] + di * (f[i] - s);
+  }
 }
 template <class T>
 __global__ void k_jacobi(int n, const int *rp, const int *ci, const T *v, const T *dinv, const T *f, const T *x, T *y) {
@@ -1459,47 +1485,23 @@ __global__ void k_jacobi(int n, const int *rp, const int *ci, const T *v, const 
   y[i] = x[i] + dinv[i] * s;
 }
 template <class T>
-__global__ void k_dense_apply(int n, const double *invT, const T *f, T *x) {
-  // x_i = sum_c (A^{-1})_{ic} f_c, invT[c][i]; one warp per row
+__global__ void k_dense_apply(int n, const double *__restrict__ invT, const T *f, T *x) {
+  // x_i = sum_c (A^{-1})_{ic} f_c, invT[c][i]; one warp per row, the first
+  // 128 columns fetched before the wait
   pdl_trigger();
-  pdl_wait();
   int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= n) return;
+  double a[4];
+#pragma unroll
+  for (int b = 0; b < 4; b++) if (lane + 32 * b < n) a[b] = __ldg(invT + (size_t)(lane + 32 * b) * n + i);
+  pdl_wait();
   double s = 0.0;
-  for (int c = lane; c < n; c += 32) s += invT[(size_t)c * n + i] * (double)f[c];
+#pragma unroll
+  for (int b = 0; b < 4; b++) if (lane + 32 * b < n) s += a[b] * (double)f[lane + 32 * b];
+  for (int c = lane + 128; c < n; c += 32) s += invT[(size_t)c * n + i] * (double)f[c];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if (lane == 0) x[i] = (T)s;
-}
-
-// The same four sweeps with L lanes per row (L = 4..32): a row's entries are
-// read by consecutive lanes (coalesced), each lane sums a strided part of the
-// row and the parts are combined with shuffles.  MODE 0: pre-smoothing
-// (x = D^-1 f, r = f - A x; with u given, u already holds D^-1 f); 1: y = A x
-// (and, with o2 given, o2 = D_c^-1 y for the coarse level's pre-smoothing);
-// 2: t = x + P e; 3: post-smoothing (x = t + D^-1 (f - A t)).
-template <class T, int L, int MODE>
-__global__ void k_vc_lanes(int n, const int *__restrict__ rp, const int *__restrict__ ci, const T *__restrict__ v,
-                           const T *__restrict__ dinv, const T *__restrict__ f, const T *__restrict__ u, T *o1, T *o2) {
-  pdl_trigger();
-  pdl_wait();
-  int g = (blockIdx.x * blockDim.x + threadIdx.x) / L, k = threadIdx.x % L;
-  int i = g < n ? g : n - 1;                       // whole groups stay in the shuffles
-  int q0 = rp[i], q1 = rp[i + 1];
-  T s = 0;
-#pragma unroll 4
-  for (int q = q0 + k; q < q1; q += L) {
-    int j = ci[q];
-    T xj = MODE == 0 && !u ? f[j] * dinv[j] : u[j];
-    s += v[q] * xj;
-  }
-#pragma unroll
-  for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, L);
-  if (k != 0 || g >= n) return;
-  if (MODE == 0) { if (!u) o1[i] = f[i] * dinv[i]; o2[i] = f[i] - s; }   // with u, o1 = u holds it already
-  else if (MODE == 1) { o1[i] = s; if (o2) o2[i] = s * dinv[i]; }
-  else if (MODE == 2) o1[i] = f[i] + s;            // f = x (the smoothed iterate), u = e
-  else o1[i] = u[i] + dinv[i] * (f[i] - s);        // u = t
 }
 
 // lanes per row for a matrix's average row length: one thread per row for
@@ -1512,34 +1514,15 @@ static int lanes_for(long long nnz, int n) {
   return avg <= 8.0 ? 1 : avg <= 24.0 ? 4 : 16;
 }
 
-template <class T>
-__global__ void k_vc_pre(int n, const int *rp, const int *ci, const T *v, const T *dinv, const T *f, T *x, T *r);
-template <class T>
-__global__ void k_prolong_add(int n, const int *rp, const int *ci, const T *v, const T *e, const T *x, T *t);
-template <class T>
-__global__ void k_vc_post(int n, const int *rp, const int *ci, const T *v, const T *dinv, const T *f, const T *t, T *x);
-template <class T>
-__global__ void k_csr_spmv(int n, const int *rp, const int *ci, const T *v, const T *x, T *y);
-
 template <class T, int MODE>
 static void vc_sweep(int L, int n, const int *rp, const int *ci, const T *v, const T *dinv, const T *f, const T *u,
                      T *o1, T *o2, cudaStream_t s) {
   if (n <= 0) return;
-  if (L == 1) {
-    unsigned g = grid_for(n, 256);
-    if (MODE == 0) launch_pdl(k_vc_pre<T>, g, 256, 0, s, n, rp, ci, v, dinv, f, o1, o2);
-    else if (MODE == 1 && o2) launch_pdl(k_restrict_x<T>, g, 256, 0, s, n, rp, ci, v, u, dinv, o1, o2);
-    else if (MODE == 1) launch_pdl(k_csr_spmv<T>, g, 256, 0, s, n, rp, ci, v, u, o1);
-    else if (MODE == 2) launch_pdl(k_prolong_add<T>, g, 256, 0, s, n, rp, ci, v, u, f, o1);
-    else launch_pdl(k_vc_post<T>, g, 256, 0, s, n, rp, ci, v, dinv, f, u, o1);
-    RS_LAUNCHED(1);
-    return;
-  }
-  unsigned g = grid_for((size_t)n * L, 256);
-  if (L == 4) launch_pdl(k_vc_lanes<T, 4, MODE>, g, 256, 0, s, n, rp, ci, v, dinv, f, u, o1, o2);
-  else if (L == 8) launch_pdl(k_vc_lanes<T, 8, MODE>, g, 256, 0, s, n, rp, ci, v, dinv, f, u, o1, o2);
-  else if (L == 16) launch_pdl(k_vc_lanes<T, 16, MODE>, g, 256, 0, s, n, rp, ci, v, dinv, f, u, o1, o2);
-  else launch_pdl(k_vc_lanes<T, 32, MODE>, g, 256, 0, s, n, rp, ci, v, dinv, f, u, o1, o2);
+  const unsigned g = grid_for((size_t)n * L, 256);
+  auto go = [&](auto kern) { launch_pdl(kern, g, 256, 0, s, n, rp, ci, v, dinv, f, u, o1, o2); };
+  if (L == 1) go(k_vc<T, 1, MODE, 8>);
+  else if (L == 4) go(k_vc<T, 4, MODE, 6>);
+  else go(k_vc<T, 16, MODE, 4>);
   RS_LAUNCHED(1);
 }
 
@@ -1577,7 +1560,7 @@ int amg_vcycle(amg_hier &h, int l, cudaStream_t s) {
       return 1;
     }
     T *x = LP::x(L), *t = LP::t(L);
-    k_vc_pre<T><<<grid_for(n, 256), 256, 0, s>>>(n, A.rp, A.ci, A.v, LP::dinv(L), LP::f(L), x, LP::r(L));
+    k_vc<T, 1, 0, 8><<<grid_for(n, 256), 256, 0, s>>>(n, A.rp, A.ci, A.v, LP::dinv(L), LP::f(L), nullptr, x, LP::r(L));
     RS_LAUNCHED(1);
     for (int it = 1; it < 10; it++) {
       k_jacobi<T><<<grid_for(n, 256), 256, 0, s>>>(n, A.rp, A.ci, A.v, LP::dinv(L), LP::f(L), x, t);
@@ -1637,21 +1620,3 @@ void amg_vcycle_graph(amg_hier &h, cudaStream_t s) {
 }
 template void amg_vcycle_graph<double>(amg_hier &, cudaStream_t);
 template void amg_vcycle_graph<float>(amg_hier &, cudaStream_t);
-
-template <class T>
-__global__ void k_csr_spmv(int n, const int *rp, const int *ci, const T *v, const T *x, T *y) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  pdl_trigger();
-  pdl_wait();
-  if (i >= n) return;
-  T s = 0;
-  for (int q = rp[i]; q < rp[i + 1]; q++) s += v[q] * x[ci[q]];
-  y[i] = s;
-}
-template <class T>
-void csr_spmv(const int *rp, const int *ci, const T *v, const T *x, T *y, int n, cudaStream_t s) {
-  k_csr_spmv<T><<<grid_for(n, 256), 256, 0, s>>>(n, rp, ci, v, x, y);
-  RS_LAUNCHED(1);
-}
-template void csr_spmv<double>(const int *, const int *, const double *, const double *, double *, int, cudaStream_t);
-template void csr_spmv<float>(const int *, const int *, const float *, const float *, float *, int, cudaStream_t);

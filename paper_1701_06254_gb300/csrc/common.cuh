@@ -345,9 +345,6 @@ void ras_setup(sim_ls_s *ls);
 // SpMV kernels (block 2x2, values Tv, vectors Tx in / Ty out)
 template <class Tv, class Tx, class Ty>
 void bsr_spmv(const int *rp, const int *ci, const Tv *val, const Tx *x, Ty *y, const Ty *f, int nb, cudaStream_t s);
-template <class T>
-void csr_spmv(const int *rp, const int *ci, const T *v, const T *x, T *y, int n, cudaStream_t s);
-
 // simulator internals used by the ensemble driver (batch.cu)
 void sim_dims(sim_t h, int *n, int *n_wells);
 void sim_put_stats(sim_t h, const sim_stats *st);
