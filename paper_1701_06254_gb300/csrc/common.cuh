@@ -269,7 +269,7 @@ struct sim_ls_s {
   dbuf<float> Z32;
   dbuf<double> x64a, x64b;      // CPR work (FP64)
   dbuf<float> x32a, x32b, x32c; // CPR work (FP32)
-  double *hpin = nullptr;       // pinned host scalars: 4 per Arnoldi step (estimate, h_{j+1,j}, second pass)
+  double *hpin = nullptr;       // pinned host scalars: 4 per Arnoldi step (estimate, h_{j+1,j}, second pass, slot complete)
   // one Arnoldi step as a CUDA graph (recorded after each setup)
   int graph_mode = 1;           // 0 separate launches, 1 a graph per Arnoldi step, 2 a device-side loop
   cudaGraphExec_t it_exec = nullptr;

@@ -9,8 +9,10 @@
 #include "common.cuh"
 #define ORTHO_MAXV 64            // FGMRES restart length limit (m + 1 basis vectors)
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
+#include <thread>
 
 // ------------------------------------------------------------ timers -----
 rs_timed::rs_timed(sim_ls_s *l, int which) : ls(l), on(which > 0 && (l->timer_mask >> which) & 1u), fam(which) {
@@ -253,23 +255,24 @@ template <> struct vec2_t<float> { typedef float2 type; };
 // ascending block order.
 #define SPMV_WARPS 8
 #define SPMV_CHUNK 256
-template <class Tv, class Tx, class Tf, class Ty>
+// (The FP32 kernel of large systems stays at 32 registers, 8 blocks per SM,
+// only without the wait and without jd: 40 registers cost it 8%.)
+template <class Tv, class Tx, class Tf, class Ty, bool PDL>
 __global__ void __launch_bounds__(SPMV_WARPS * 32)
 k_bsr_spmv(int nb, const int *__restrict__ rp, const int *__restrict__ ci, const Tv *__restrict__ val,
-           const Tx *x, const Tf *f, Ty *y, int np, const Tx *e, Tx *xout, Ty *pout, const int *jd,
-           int pdl) {
+           const Tx *x, const Tf *f, Ty *y, int np, const Tx *e, Tx *xout, Ty *pout, const int *jd) {
   // (x, f and e come from the kernel before: no __restrict__, so that no load
   // of them can move above pdl_wait)
   __shared__ Ty prod[SPMV_WARPS][SPMV_CHUNK][2];
   int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int r0 = (blockIdx.x * SPMV_WARPS + wid) * 32;
-  if (pdl) pdl_trigger();
+  if (PDL) pdl_trigger();
   if (r0 >= nb) return;
   int r = r0 + lane, rend = min(r0 + 32, nb);
   int q0 = rp[r0], q1 = rp[rend];
   int myq0 = r < nb ? rp[r] : q1, myq1 = r < nb ? rp[r + 1] : q1;
-  if (pdl) pdl_wait();                         // the pattern is fixed; everything else is the previous kernels'
-  if (jd) xout += (size_t)*jd * 2 * nb;
+  if (PDL) pdl_wait();                         // the pattern is fixed; everything else is the previous kernels'
+  if (sizeof(Tv) == 8 && jd) xout += (size_t)*jd * 2 * nb;
   Ty a0 = 0, a1 = 0;
   typedef typename vec2_t<Tx>::type X2;
   for (int c0 = q0; c0 < q1; c0 += SPMV_CHUNK) {
@@ -321,9 +324,12 @@ static int arnoldi_pdl(int nb) { return nb <= 152 * 8 * SPMV_WARPS * 32; }
 template <class Tv, class Tx, class Tf, class Ty>
 static void spmv(const sim_ls_s *ls, const Tv *val, const Tx *x, const Tf *f, Ty *y, cudaStream_t s,
                  const Tx *e = nullptr, Tx *xout = nullptr, Ty *pout = nullptr, const int *jd = nullptr) {
-  const int pdl = arnoldi_pdl(ls->nb);
-  launch_pdl_if(pdl, k_bsr_spmv<Tv, Tx, Tf, Ty>, grid_for(ls->nb, SPMV_WARPS * 32), SPMV_WARPS * 32, 0, s, ls->nb,
-                ls->rp.p, ls->ci.p, val, x, f, y, ls->n, e, xout, pout, jd, pdl);
+  auto go = [&](bool pdl, auto kern) {
+    launch_pdl_if(pdl, kern, grid_for(ls->nb, SPMV_WARPS * 32), SPMV_WARPS * 32, 0, s, ls->nb, ls->rp.p, ls->ci.p, val, x,
+                  f, y, ls->n, e, xout, pout, jd);
+  };
+  if (arnoldi_pdl(ls->nb)) go(true, k_bsr_spmv<Tv, Tx, Tf, Ty, true>);
+  else go(false, k_bsr_spmv<Tv, Tx, Tf, Ty, false>);
   RS_LAUNCHED(1);
 }
 
@@ -673,10 +679,9 @@ __device__ __forceinline__ double warp_sum_df(float h, float l) {        // resu
   return (double)h + (double)l;
 }
 
-// The block that finishes last (atomic ticket) sums the per-block partials
-// part[k][b] into out[k] for k < nout, exactly as k_reduce_parts does (warp
-// per k, lanes over a fixed stride of blocks, shuffle tree), and resets the
-// ticket: the separate reduction launch between the sweeps disappears.
+// The per-block partials of one sum are added by one warp: lanes over a fixed
+// stride of blocks, then a fixed shuffle tree.  After an update (one sum) the
+// block that finishes last (atomic ticket) does it.
 __device__ __forceinline__ bool last_block(int *ticket) {
   __shared__ bool last;
   __threadfence();
@@ -685,34 +690,65 @@ __device__ __forceinline__ bool last_block(int *ticket) {
   __syncthreads();
   return last;
 }
-__device__ __forceinline__ void reduce_tail(int nout, int nblk, const double *part, double *out, int *ticket) {
+__device__ __forceinline__ double reduce_part(int nblk, const double *part) {   // one warp, total in lane 0
+  const int lane = threadIdx.x & 31;
+  double t = 0;
+  for (int b0 = lane; b0 < nblk; b0 += 32 * 8) {        // eight loads in flight, added in order
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; u++) if (b0 + 32 * u < nblk) v[u] = __ldcg(part + b0 + 32 * u);
+#pragma unroll
+    for (int u = 0; u < 8; u++) if (b0 + 32 * u < nblk) t += v[u];
+  }
+  return warp_sum_d(t);
+}
+// The block that finishes last adds the partials of every sum, a warp per sum,
+// and resets the ticket.
+__device__ __forceinline__ void reduce_tail(int nt, int nblk, const double *part, double *out, int *ticket) {
   __threadfence();
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int k = warp; k < nout; k += nw) {
-    double t = 0;
-    for (int b = lane; b < nblk; b += 32) t += __ldcg(part + (size_t)k * nblk + b);
-    t = warp_sum_d(t);
-    if (lane == 0) out[k] = t;
+  for (int k = threadIdx.x >> 5; k < nt; k += ORTHO_BS / 32) {
+    const double t = reduce_part(nblk, part + (size_t)k * nblk);
+    if ((threadIdx.x & 31) == 0) out[k] = t;
   }
   if (threadIdx.x == 0) *ticket = 0;
 }
+// out[k] = V_k . w (and ||w||^2): one block of one warp per k, a launch of its
+// own where launches overlap (arnoldi_pdl).  In the dots kernel's last block
+// one SM's FP64 pipe holds the chain for nt / 8 rounds of 24 additions (5 us
+// at 18 vectors, 11 us at 45: 155k cells, 45 iterations, 95 against 89 us of
+// Gram-Schmidt per step); on the 1M-cell case a launch costs as much (97
+// against 101 us).
+__global__ void __launch_bounds__(32) k_reduce_parts(int nt, int nblk, const double *part, double *out, const int *cond,
+                                                     const int *jd, int extra) {
+  pdl_trigger();
+  pdl_wait();
+  if (cond && *cond == 0) return;
+  if (jd) nt = *jd + 1 + extra;
+  const int k = blockIdx.x;
+  if (k >= nt) return;
+  const double t = reduce_part(nblk, part + (size_t)k * nblk);
+  if (threadIdx.x == 0) out[k] = t;
+}
 
-// After an update pass (thread 0 of its last block): h_{j+1,j} = ||w|| and its
+// After an update pass (its last block): ||w||^2, h_{j+1,j} = ||w|| and its
 // reciprocal (isp: split into hi + lo), the flag for a second pass when the
 // first kept less than 1% of w (||w_1||^2 < 1e-4 ||w||^2, the latter behind
 // the dot products), and in graph replay the step index for k_scale's blocks
-// (jd[0] moves on while they run).
-__device__ __forceinline__ void norm_tail(int nv, const double *nrm, int *flag, const double *h1, double *hnorm,
-                                          float *isp, int *jd) {
-  if (threadIdx.x != 0) return;
+// (jd[0] moves on while they run).  Resets the ticket.
+__device__ __forceinline__ void norm_tail(int nv, const double *part, double *nrm, int *flag, const double *h1,
+                                          double *hnorm, float *isp, int *jd, int *ticket) {
+  if (threadIdx.x >= 32) return;
   __threadfence();
-  const double n2 = *(volatile const double *)nrm;
+  const double n2 = reduce_part(gridDim.x, part);
+  if (threadIdx.x != 0) return;
+  *nrm = n2;
   if (flag) *flag = n2 < 1e-4 * h1[nv] ? 1 : 0;
   const double hn = sqrt(n2), inv = hn > 0.0 ? 1.0 / hn : 0.0;
   hnorm[0] = hn;
   hnorm[1] = inv;
   if (isp) { float a, b; df_split(inv, a, b); isp[0] = a; isp[1] = b; }
   if (jd) jd[1] = jd[0];
+  *ticket = 0;
 }
 
 // part[k][b] = V_k . w over the block's rows (k < nv); with_norm: part[nv][b] = w . w
@@ -754,7 +790,7 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots(int nu, int ch, int 
       part[(size_t)(k0 + threadIdx.x) * nblk + blockIdx.x] = s;
     }
   }
-  if (last_block(ticket)) reduce_tail(nt, nblk, part, out, ticket);   // out[k] = V_k . w (and ||w||^2)
+  if (!pdl && last_block(ticket)) reduce_tail(nt, nblk, part, out, ticket);
 }
 
 // w -= sum_k h_k V_k over the block's rows, then part[0][b] = ||w||^2
@@ -799,10 +835,7 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update(int nu, int ch, in
   for (int t = threadIdx.x; t < len; t += ORTHO_BS) { double v = ws[t]; w[i0 + t] = v; n2 += v * v; }
   double tot = block_sum_d(n2, sred);
   if (threadIdx.x == 0) part[blockIdx.x] = tot;
-  if (last_block(ticket)) {
-    reduce_tail(1, gridDim.x, part, nrm, ticket);
-    norm_tail(nv, nrm, flag, h1, hnorm, nullptr, jd);
-  }
+  if (last_block(ticket)) norm_tail(nv, part, nrm, flag, h1, hnorm, nullptr, jd, ticket);
 }
 
 // k_ortho_dots on pair planes: V vector k at V + 2k nu (hi) and + (2k+1) nu
@@ -867,7 +900,7 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots_df(int nu, int ch, i
       part[(size_t)(k0 + threadIdx.x) * nblk + blockIdx.x] = sum;
     }
   }
-  if (last_block(ticket)) reduce_tail(nt, nblk, part, out, ticket);   // out[k] = V_k . w (and ||w||^2)
+  if (!pdl && last_block(ticket)) reduce_tail(nt, nblk, part, out, ticket);
 }
 
 // k_ortho_update on pair planes: w -= sum_k h_k V_k (h FP64, split once per
@@ -942,10 +975,7 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update_df(int nu, int ch,
     for (int q = 0; q < ORTHO_BS / 32; q++) tot += sred[q];
     part[blockIdx.x] = tot;
   }
-  if (last_block(ticket)) {
-    reduce_tail(1, gridDim.x, part, nrm, ticket);        // nrm = ||w||^2 after the pass
-    norm_tail(nv, nrm, flag, h1, hnorm, isp, jd);
-  }
+  if (last_block(ticket)) norm_tail(nv, part, nrm, flag, h1, hnorm, isp, jd, ticket);
 }
 
 // Hessenberg column j: h = h1 + h2 (h1 without a second pass), h_{j+1,j} =
@@ -983,6 +1013,8 @@ __device__ __forceinline__ void arnoldi_col(int j, int m, const double *h1, cons
   host[0] = fabs(g[j + 1]);
   host[1] = hn;
   host[2] = re ? 1.0 : 0.0;
+  __threadfence_system();
+  host[3] = 1.0;                                 // the slot is complete (ls_solve polls it)
 }
 // The end of an Arnoldi step.  Block 0: the Hessenberg column, beside the
 // others' work instead of in front of it, and in graph replay the step
@@ -1244,6 +1276,23 @@ __global__ void k_loop_cond(cudaGraphConditionalHandle h, const int *jd, const d
 }
 __global__ void k_loop_params(double *lp, double thr, double cap) { lp[0] = thr; lp[1] = cap; lp[2] = 0.0; lp[3] = 0.0; }
 
+// Wait until the device has completed a step's pinned slot.  The Givens column
+// is written while the step's last kernel is still scaling the next basis
+// vector, so the decision is taken and the next step queued before the GPU
+// runs dry (a stream synchronisation left it idle for some 8 us per step).
+// The stream is asked now and then, so that a failed launch ends the wait.
+static void wait_slot(const volatile double *done, cudaStream_t s) {
+  for (unsigned it = 1; *done == 0.0; it++) {
+    if (it % 64 == 0) std::this_thread::yield();
+    if (it % 4096 == 0) {
+      const cudaError_t e = cudaStreamQuery(s);
+      if (e == cudaSuccess) break;
+      if (e != cudaErrorNotReady) RS_CUDA(e);
+    }
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
+}
+
 int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
   if (ls->o.krylov == SIM_KRYLOV_BICGSTAB) return ls_solve_bicgstab(ls, tol, its_out, relres, x0);
   cudaStream_t s = ls->st;
@@ -1297,22 +1346,29 @@ int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
     const int pdl = arnoldi_pdl(ls->nb);
     const col_args ca = {m, h1, h2, flag, hn, G, jdp ? hp_dev : hp_dev + 4 * j};
     auto ortho = [&](auto kern, auto... a) { launch_pdl_if(pdl, kern, nblk, ORTHO_BS, sm, c, nu, ch, nv, a..., pdl); };
+    auto reduce = [&](int nt, double *out, const int *cond, int extra) {   // (in graph replay enough blocks for any step)
+      if (pdl) launch_pdl(k_reduce_parts, jdp ? m + 1 : nt, 32, 0, c, nt, nblk, part, out, cond, jdp, extra);
+    };
     if (df) {
       float *w2 = ls->w2.p, *isp = ls->isp.p;  // w2 written by the double-float SpMV
       ortho(k_ortho_dots_df, V32, w2, part, 1, nullptr, jdp, tk, h1);
+      reduce(nv + 1, h1, nullptr, 1);
       ortho(k_ortho_update_df, V32, w2, h1, part, nullptr, jdp, tk, nrm, flag, h1, hn, isp);
       ortho(k_ortho_dots_df, V32, w2, part, 0, flag, jdp, tk, h2);
+      reduce(nv, h2, flag, 0);
       ortho(k_ortho_update_df, V32, w2, h2, part, flag, jdp, tk, nrm_b, nullptr, nullptr, hn, isp);
       launch_pdl_if(pdl, k_scale<true>, gs, 256, 0, c, nu, w2, isp, V32, j, jdp, jdp ? ls->vcur32.p : nullptr, ca, pdl);
     } else {
       double *w = ls->w.p, *V = ls->V.p;
       ortho(k_ortho_dots, V, w, part, 1, nullptr, jdp, tk, h1);
+      reduce(nv + 1, h1, nullptr, 1);
       ortho(k_ortho_update, V, w, h1, part, nullptr, jdp, tk, nrm, flag, h1, hn);
       ortho(k_ortho_dots, V, w, part, 0, flag, jdp, tk, h2);
+      reduce(nv, h2, flag, 0);
       ortho(k_ortho_update, V, w, h2, part, flag, jdp, tk, nrm_b, nullptr, nullptr, hn);
       launch_pdl_if(pdl, k_scale<false>, gs, 256, 0, c, nu, w, nullptr, V, j, jdp, jdp ? ls->vcur.p : nullptr, ca, pdl);
     }
-    RS_LAUNCHED(5);
+    RS_LAUNCHED(pdl ? 7 : 5);
   };
   // One Arnoldi step j (CPR, SpMV, orthogonalisation, Givens); its residual
   // estimate and h_{j+1,j} land in pinned slot j
@@ -1495,14 +1551,19 @@ int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
       if (lo[1] != 0.0) { *its_out = its; *relres = NAN; return 2; }
     }
     for (int j = 0; j < m && !use_loop; j++) {
+      hp[4 * j + 3] = 0.0;
       if (use_graph) {
         RS_CUDA(cudaGraphLaunch(ls->it_exec, s));
         RS_LAUNCHED(ls->it_launches);
       } else {
         enqueue(j);
       }
-      RS_CUDA(cudaStreamSynchronize(s));
-      if (use_graph) ls->graph_timers();
+      if (ls->timer_mask) {
+        RS_CUDA(cudaStreamSynchronize(s));
+        if (use_graph) ls->graph_timers();
+      } else {
+        wait_slot(hp + 4 * j + 3, s);
+      }
       if (ls->errw[0]) RS_FAIL(SIM_ERR_TIMEOUT, "RAS setup gave up (code %d)", ls->errw[0]);
       double est = hp[4 * j], hnv = hp[4 * j + 1];
       its++;
