@@ -978,31 +978,37 @@ template <> struct v2_t<double> { typedef double2 type; };
 // a block has two warps: half the FP64 instructions in each warp's chain,
 // and the four sub-partitions' pipes evenly used; slots that none of a warp's
 // rows has are skipped.
+// FP32 and BF16 use two lanes per row as well while all blocks are resident
+// (RAS_W2_MAX): each lane issues half the products and shuffles of a group.
+// Per launch, one against two lanes: 200k, FP32, 43 -> 37 us; 65k, BF16, 36 ->
+// 28 us; 150k with overlap 2, 44 -> 39 us; 155k, 33 -> 29 us.  Beyond one wave
+// the second warp's instructions compete with the other blocks' (1M cells:
+// one lane, 84 us).
 #define RAS_PF_BYTES 8192
 #define RAS_PF_STEP 2048
-template <class T> __host__ __device__ constexpr int ras_threads() { return sizeof(T) == 8 ? 64 : 32; }
+#define RAS_W2_MAX (152 * 8)
 template <int NP> struct ras_group { uint2 d; uint4 h; uint4 p[NP]; };
-template <class T, class Tin, bool ACC, class TB>
-__global__ void __launch_bounds__(ras_threads<T>(), sizeof(TB) == 2 ? 20 : sizeof(T) == 4 ? 16 : 8)
+template <class T, class Tin, bool ACC, class TB, int LPR>
+__global__ void __launch_bounds__(32 * LPR, LPR == 2 ? 8 : sizeof(TB) == 2 ? 20 : 16)
 k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const int *gidx_all, const uint16_t *gpos_all,
                    const int *nown, const uint2 *gdesc, const int *ngrp, const int *lrp_ptr, const int *sub_ptr,
                    const int *order, const Tin *f, T *x) {
-  constexpr bool D = sizeof(T) == 8;                   // FP64: two lanes per row
-  constexpr int BS = ras_threads<T>(), BPP = sizeof(TB) == 2 ? 2 : 1, NP = RAS_K / BPP + 1, AHEAD = ras_ahead<TB>();
+  constexpr bool D = sizeof(T) == 8, W2 = LPR == 2;    // W2: two lanes per row, one component each
+  constexpr int BS = 32 * LPR, BPP = sizeof(TB) == 2 ? 2 : 1, NP = RAS_K / BPP + 1, AHEAD = ras_ahead<TB>();
   typedef typename v2_t<T>::type T2;
   typedef typename v2_t<Tin>::type Tin2;
   extern __shared__ uint4 sm4[];
   T2 *y = reinterpret_cast<T2 *>(sm4);
-  const int tid = threadIdx.x, row_of = D ? tid >> 1 : tid, comp = tid & 1;
+  const int tid = threadIdx.x, row_of = tid / LPR, comp = tid & 1;
   const int s = order[blockIdx.x], base = sub_ptr[s], m = sub_ptr[s + 1] - base, no = nown[s];
   const int ngl = ngrp[2 * s], ng = ngrp[2 * s + 1];
   const int *gidx = gidx_all + base;
   const uint16_t *gpos = gpos_all + base;
   const unsigned char *st = blobs + blob_off[s];
-  const uint4 *st_h = reinterpret_cast<const uint4 *>(st) + row_of, *st_b = reinterpret_cast<const uint4 *>(st) + tid;
+  const uint4 *st_h = reinterpret_cast<const uint4 *>(st) + row_of, *st_b = reinterpret_cast<const uint4 *>(st) + (D ? tid : row_of);
   const uint2 *gd = gdesc + ras_group0(s, base, lrp_ptr[s]);
   const int bound = (int)(blob_off[s + 1] - blob_off[s]), glast = max(ng - 1, 0);
-  auto sync = [&]() { if (D) __syncthreads(); else __syncwarp(); };
+  auto sync = [&]() { if (W2) __syncthreads(); else __syncwarp(); };
   pdl_trigger();
   int pf = min(bound, RAS_PF_BYTES);                   // the stream is prefetched into L2 up to here
   if (tid == 0)
@@ -1047,7 +1053,7 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
   // gather the extended right-hand side, the first indices ahead of the wait
   // for the kernel that makes f (all other inputs are fixed between setups)
   const Tin2 *f2 = reinterpret_cast<const Tin2 *>(f);
-  constexpr int GU = D ? 8 : 16;
+  constexpr int GU = W2 ? 8 : 16;
   int gi[GU], pos[GU];
   auto indices = [&](int p0) {
 #pragma unroll
@@ -1085,7 +1091,7 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
     T2 yc[RAS_K];
     T a0;
     [[maybe_unused]] T a1 = 0;
-    if constexpr (D) a0 = reinterpret_cast<const double *>(y + row)[comp];
+    if constexpr (W2) a0 = reinterpret_cast<const T *>(y + row)[comp];
     else { const T2 t = y[row]; a0 = t.x; a1 = t.y; }
 #pragma unroll
     for (int e = 0; e < RAS_K; e++) yc[e] = y[col(e)];
@@ -1100,6 +1106,15 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
           const double bx = __hiloint2double(G.p[k].y, G.p[k].x), by = __hiloint2double(G.p[k].w, G.p[k].z);
           a0 = __fma_rn(-bx, yc[e].x, a0);
           a0 = __fma_rn(-by, yc[e].y, a0);
+        } else if constexpr (W2) {
+          float bx, by;
+          if constexpr (BPP == 2) {
+            const unsigned w = u ? (comp ? G.p[k].w : G.p[k].z) : (comp ? G.p[k].y : G.p[k].x);
+            bx = __uint_as_float(w << 16); by = __uint_as_float(w & 0xffff0000u);
+          } else {
+            bx = __uint_as_float(comp ? G.p[k].z : G.p[k].x); by = __uint_as_float(comp ? G.p[k].w : G.p[k].y);
+          }
+          a0 = __fsub_rn(a0, __fmaf_rn(bx, yc[e].x, __fmul_rn(by, yc[e].y)));
         } else {
           float b0, b1, b2, b3;
           if constexpr (BPP == 2) blk4(u ? G.p[k].z : G.p[k].x, u ? G.p[k].w : G.p[k].y, b0, b1, b2, b3);
@@ -1118,6 +1133,16 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
           const double o = __shfl_xor_sync(0xffffffffu, a0, 1);
           a0 = __fma_rn(comp ? dy : dx, a0, (comp ? dx : dy) * o);
         }
+      } else if constexpr (W2) {
+        float dx, dy;
+        if constexpr (BPP == 2) {
+          const unsigned w = comp ? G.p[0].y : G.p[0].x;
+          dx = __uint_as_float(w << 16); dy = __uint_as_float(w & 0xffff0000u);
+        } else {
+          dx = __uint_as_float(comp ? G.p[0].z : G.p[0].x); dy = __uint_as_float(comp ? G.p[0].w : G.p[0].y);
+        }
+        const float o = __shfl_xor_sync(0xffffffffu, a0, 1), ax = comp ? o : a0, ay = comp ? a0 : o;
+        a0 = dx * ax + dy * ay;
       } else {
         float d0, d1, d2, d3;
         if constexpr (BPP == 2) blk4(G.p[0].x, G.p[0].y, d0, d1, d2, d3);
@@ -1128,7 +1153,7 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
       }
     }
     if (row_of < rows) {
-      if constexpr (D) reinterpret_cast<double *>(y + row)[comp] = a0;
+      if constexpr (W2) reinterpret_cast<T *>(y + row)[comp] = a0;
       else { T2 t; t.x = a0; t.y = a1; y[row] = t; }
     }
   };
@@ -1190,9 +1215,12 @@ template <class T, class Tin, class TB>
 static void ras_apply_go(sim_ls_s *ls, const Tin *f, T *x, bool acc) {
   ras_data &R = ls->ras;
 #define RAS_APPLY_ARGS R.blob_off.p, R.blob.p, R.gidx.p, R.gpos.p, R.nown.p, R.gdesc.p, R.ngrp.p, R.lrp_ptr.p, R.sub_ptr.p, R.order.p, f, x
-  const int bs = ras_threads<T>();
-  if (acc) launch_pdl(k_ras_apply_stream<T, Tin, true, TB>, R.nsub, bs, R.smem_bytes, ls->st, RAS_APPLY_ARGS);
-  else launch_pdl(k_ras_apply_stream<T, Tin, false, TB>, R.nsub, bs, R.smem_bytes, ls->st, RAS_APPLY_ARGS);
+  auto go = [&](auto kern, int lpr) { launch_pdl(kern, R.nsub, 32 * lpr, R.smem_bytes, ls->st, RAS_APPLY_ARGS); };
+  if (sizeof(T) == 8 || R.nsub <= RAS_W2_MAX) {
+    if (acc) go(k_ras_apply_stream<T, Tin, true, TB, 2>, 2); else go(k_ras_apply_stream<T, Tin, false, TB, 2>, 2);
+  } else if constexpr (sizeof(T) == 4) {
+    if (acc) go(k_ras_apply_stream<T, Tin, true, TB, 1>, 1); else go(k_ras_apply_stream<T, Tin, false, TB, 1>, 1);
+  }
 #undef RAS_APPLY_ARGS
 }
 template <class T, class Tin> static void ras_apply_launch(sim_ls_s *ls, const Tin *f, T *x, bool acc);
@@ -1214,12 +1242,14 @@ template <class T, class Tin> void ls_ras_apply(sim_ls_s *ls, const Tin *f, T *x
   if (R.smem_path) {
     static bool attr = false;
     if (!attr) {
-#define RAS_ATTR(...) RS_CUDA(cudaFuncSetAttribute(k_ras_apply_stream<__VA_ARGS__>, cudaFuncAttributeMaxDynamicSharedMemorySize, RAS_SMEM_BUDGET))
-      RAS_ATTR(float, float, false, float); RAS_ATTR(float, float, true, float);
-      RAS_ATTR(float, double, false, float); RAS_ATTR(float, double, true, float);
-      RAS_ATTR(float, float, false, __nv_bfloat16); RAS_ATTR(float, float, true, __nv_bfloat16);
-      RAS_ATTR(float, double, false, __nv_bfloat16); RAS_ATTR(float, double, true, __nv_bfloat16);
-      RAS_ATTR(double, double, false, double); RAS_ATTR(double, double, true, double);
+#define RAS_ATTR(...)                                                                                              \
+  RS_CUDA(cudaFuncSetAttribute(k_ras_apply_stream<__VA_ARGS__>, cudaFuncAttributeMaxDynamicSharedMemorySize, RAS_SMEM_BUDGET))
+#define RAS_ATTR4(T, Tin, TB)                                                                                      \
+  RAS_ATTR(T, Tin, false, TB, 2); RAS_ATTR(T, Tin, true, TB, 2); RAS_ATTR(T, Tin, false, TB, 1); RAS_ATTR(T, Tin, true, TB, 1)
+      RAS_ATTR4(float, float, float); RAS_ATTR4(float, double, float);
+      RAS_ATTR4(float, float, __nv_bfloat16); RAS_ATTR4(float, double, __nv_bfloat16);
+      RAS_ATTR(double, double, false, double, 2); RAS_ATTR(double, double, true, double, 2);
+#undef RAS_ATTR4
 #undef RAS_ATTR
       attr = true;
     }
