@@ -82,6 +82,16 @@ __device__ __forceinline__ void mma16816(float c[4], const unsigned a[4], const 
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
+// Weight copies: per tap [CO rows][CI], stored as the 8 x 8 core matrices the
+// tcgen05 descriptors address (16-byte chunks of 8 inputs; the two chunks of
+// a 16-wide K block 128 bytes apart, 8-row groups 256 apart, K blocks CO / 8
+// groups apart), so that one bulk copy brings a layer's weights.  Element
+// offset of chunk ch of row o (rows padded to 16):
+__host__ __device__ constexpr int wrows(int co) { return co < 16 ? 16 : co; }
+__host__ __device__ inline int woffs(int rows, int o, int ch) {
+  return ((ch >> 1) * (rows / 8) + (o >> 3)) * 128 + (ch & 1) * 64 + (o & 7) * 8;
+}
+
 // --------------------------------------------------- implicit-GEMM conv ---
 // out[v, o] for v in this CTA's 128 voxels, o < NT*8.
 // MODE 0: BF16 out = act(acc + bias)           (forward)
@@ -131,13 +141,13 @@ __global__ void __launch_bounds__(128) k_conv(int nx, int ny, int nz, const bf16
       cp_async16(a + vrow[j] * S::AST + vch[j] * 8, src, ok ? 16 : 0);
     }
     bf16 *b = sB + stage * S::B_EL;
-    const bf16 *w = Wt + (size_t)tap * CO * CI;
+    const bf16 *w = Wt + (size_t)tap * wrows(CO) * CI;
 #pragma unroll
     for (int j = 0; j < BJ; j++) {
       int q = j * 128 + t;
       if (q < CO * CH) {
         int o = q / CH, ch = q % CH;
-        cp_async16(b + o * S::BST + ch * 8, w + o * CI + ch * 8, 16);
+        cp_async16(b + o * S::BST + ch * 8, w + woffs(wrows(CO), o, ch), 16);
       }
     }
   };
@@ -255,13 +265,13 @@ __global__ void __launch_bounds__(128) k_conv_halo(int nx, int ny, int nz, const
   }
   auto loadw = [&](int stage, int tap) {
     bf16 *b = sB + stage * S::B_EL;
-    const bf16 *w = Wt + (size_t)tap * CO * CI;
+    const bf16 *w = Wt + (size_t)tap * wrows(CO) * CI;
 #pragma unroll
     for (int j = 0; j < BJ; j++) {
       int q = j * 128 + t;
       if (q < CO * CH) {
         int o = q / CH, ch = q % CH;
-        cp_async16(b + o * S::BST + ch * 8, w + o * CI + ch * 8, 16);
+        cp_async16(b + o * S::BST + ch * 8, w + woffs(wrows(CO), o, ch), 16);
       }
     }
   };
@@ -339,30 +349,56 @@ __global__ void __launch_bounds__(128) k_conv_halo(int nx, int ny, int nz, const
 }
 
 // ------------------------------------------ implicit-GEMM conv, tcgen05 ---
-// The same contraction on the 5th-generation tensor cores: per CTA a tile of
-// 128 voxels (M) against CO output channels (N = 32 or 64), K = 27 taps x CI.
-// For every tap the CTA gathers the 128 shifted input rows (cp.async,
-// zero-filled outside the grid) and the tap's CO x CI weights into shared
-// memory in the K-major, no-swizzle core-matrix layout (8 rows x 16 bytes per
-// 128-byte core matrix; the two 8-element halves of a 16-wide K block 128 B
-// apart, 8-row groups 256 B apart), then one thread issues CI/16
-// tcgen05.mma.kind::f16 (BF16 x BF16 -> FP32) into a TMEM accumulator of
-// 128 lanes x CO columns.  Two stages: a stage is refilled once the MMAs that
-// read it have committed to that stage's mbarrier.  The epilogue reads the
-// accumulator with tcgen05.ld (thread = voxel row) and applies bias / ReLU or
-// the data-gradient mask.  Every wait is bounded; on a timeout the kernel
-// records an error and writes nothing.
-__device__ __forceinline__ uint64_t tc_desc(unsigned saddr) {
+// The same contraction on the 5th-generation tensor cores, the operands of
+// all 27 taps taken from one copy of the input halo in shared memory.
+//
+// A CTA owns an 8 x 16 x NZ box of output voxels; each z slice is one M = 128
+// accumulator of CO columns in TMEM (row r = x + 8 y).  The halo lies in
+// planes of 8 channels, [chunk][z][y][x] with 16 bytes per voxel: 8 voxels
+// consecutive in x are one core matrix (8 rows x 16 bytes, contiguous) from
+// any start, the next 8 rows (y + 1) lie 160 bytes on, the other half of a K
+// block one plane on.  So the A operand of a tap is the same memory from a
+// shifted start address, and nothing is gathered per tap; a plane's pad
+// keeps the copies' writes free of bank conflicts.  The weights of all taps
+// come by one bulk copy (they are stored as core matrices), issued before
+// the wait for the kernel that makes X.  One thread issues the 27 x CI / 16
+// x NZ MMAs, K ascending within each tap as in k_conv, slices innermost; the
+// results are the same bits as with mma.sync.  Epilogue: tcgen05.ld, thread
+// = voxel row, bias / ReLU or the data-gradient mask.  Every wait is
+// bounded; on a timeout the kernel records an error and writes nothing.
+__device__ __forceinline__ uint64_t tc_desc(unsigned saddr, unsigned lbo, unsigned sbo) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-  d |= (uint64_t)(128 >> 4) << 16;             // leading byte offset: the K halves of a block
-  d |= (uint64_t)(256 >> 4) << 32;             // stride byte offset: consecutive 8-row groups
+  d |= (uint64_t)(lbo >> 4) << 16;             // K-major: K halves of a block; MN-major: next 8 of K
+  d |= (uint64_t)(sbo >> 4) << 32;             // next 8 rows (K-major) or 8 of M / N (MN-major)
   d |= (uint64_t)1 << 46;                      // descriptor version; no swizzle, base offset 0
   return d;
 }
-__device__ __forceinline__ uint32_t tc_idesc(int n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+// BF16 x BF16 -> FP32, M = 128, N = n; MN-major operands when mn
+__device__ __forceinline__ uint32_t tc_idesc(int n, bool mn) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? 3u << 15 : 0u) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
+__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+               " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+               ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void tc_commit(uint64_t *bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void bar_init(uint64_t *bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+}
+// whole warp: allocate ncol TMEM columns (a power of two, at least 32)
+__device__ __forceinline__ void tc_alloc(uint32_t *slot, int ncol) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(ncol) : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tc_free(uint32_t taddr, int ncol) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncol) : "memory");
+}
+__device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ bool tc_wait(uint64_t *bar, unsigned parity) {
   for (int it = 0; it < (1 << 24); it++) {
     unsigned ok;
@@ -386,274 +422,343 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float *v) {
   for (int c = 0; c < 32; c++) v[c] = __uint_as_float(r[c]);
 }
 
-template <int CI, int CO>
-struct tc_smem {
-  static constexpr int KB = CI / 16;
-  static constexpr int A_BYTES = KB * (CBM / 8) * 256, B_BYTES = KB * (CO / 8) * 256;
-  static constexpr int STAGE = A_BYTES + B_BYTES;
-  static constexpr int NS = 4;                   // stages: 2 taps of copies ahead + 2 of MMA slack
-  static constexpr int BYTES = NS * STAGE;
-};
+__device__ __forceinline__ void tc_ld8(uint32_t taddr, float *v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int c = 0; c < 8; c++) v[c] = __uint_as_float(r[c]);
+}
 
-// MODE as for k_conv: 0 forward (bias, ReLU flag), 2 data gradient with mask,
-// 3 data gradient.  Persistent: each CTA walks tiles blockIdx.x, +gridDim.x, ...
-// with one TMEM allocation; taps flow through NS shared-memory stages, a
-// stage being refilled once the MMAs that read it have committed.
+constexpr int TBX = 8, TBY = 16, THX = TBX + 2, THY = TBY + 2, TSL = THX * THY;   // box, halo, halo voxels per slice
+__host__ __device__ constexpr int tc_plane(int ci, int nz) {                      // bytes of an 8-channel plane
+  return (TSL * (nz + 2) * 16 + 127) / 128 * 128 + 1024 / ci;
+}
+__host__ __device__ constexpr int tc_bytes(int ci, int co, int nz) { return 27 * ci * co * 2 + ci / 8 * tc_plane(ci, nz); }
+__host__ __device__ constexpr int tc_cols(int co, int nz) {                       // TMEM columns to allocate
+  int n = 32;
+  while (n < co * nz) n *= 2;
+  return n;
+}
+
+// MODE as for k_conv: 0 forward (bias, ReLU flag), 1 head forward (FP32, 8 of
+// the 16 columns), 2 data gradient with mask, 3 data gradient.
 template <int CI, int CO, int MODE>
-__global__ void __launch_bounds__(128) k_conv_tc(int nx, int ny, int nz, const bf16 *__restrict__ X, int ldx, int offx,
-                                                 const bf16 *__restrict__ Wt, const float *__restrict__ bias, int relu,
-                                                 bf16 *out, int ldo, int offo, const bf16 *__restrict__ mask, int ldm,
-                                                 int offm, int *err) {
-  typedef tc_smem<CI, CO> S;
-  constexpr int CH = CI / 8, AJ = CBM * CH / 128, BJ = (CO * CH + 127) / 128, NS = S::NS;
-  extern __shared__ __align__(1024) unsigned char smraw[];
-  __shared__ uint64_t bar[NS];
+__global__ void __launch_bounds__(256) k_conv_tc(int nx, int ny, int nz, int NZ, const bf16 *X, int ldx, int offx,
+                                                 const bf16 *Wt, const float *bias, int relu, void *out, int ldo,
+                                                 int offo, const bf16 *mask, int ldm, int offm, int *err) {
+  constexpr int CH = CI / 8, KB = CI / 16, W_BYTES = 27 * CI * CO * 2;
+  extern __shared__ __align__(128) unsigned char smtc[];
+  __shared__ uint64_t wbar, mbar;
   __shared__ uint32_t tslot;
-  const int V = nx * ny * nz, nxy = nx * ny, ntile = (V + CBM - 1) / CBM;
+  unsigned char *sA = smtc + W_BYTES;
+  const int plane = tc_plane(CI, NZ), ncol = tc_cols(CO, NZ);
+  const int tx = (nx + TBX - 1) / TBX, ty = (ny + TBY - 1) / TBY;
+  const int X0 = (int)(blockIdx.x % tx) * TBX, Y0 = (int)(blockIdx.x / tx % ty) * TBY, Z0 = (int)(blockIdx.x / (tx * ty)) * NZ;
   const int t = threadIdx.x, warp = t >> 5;
-  auto coff = [](int r, int ch) { return (r >> 3) * 256 + (ch & 1) * 128 + (r & 7) * 16; };
   if (t == 0) {
-    for (int k = 0; k < NS; k++) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar[k])) : "memory");
+    bar_init(&wbar);
+    bar_init(&mbar);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tslot)), "n"(CO) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (warp == 0) tc_alloc(&tslot, ncol);
+  tc_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t taddr = tslot, idesc = tc_idesc(CO);
-  bool ok = true;
-  long long g0 = 0;                               // taps issued by this CTA before the current tile
-  for (int tile = blockIdx.x; tile < ntile && ok; tile += gridDim.x, g0 += 27) {
-    const int v0 = tile * CBM;
-    int vx[AJ], vy[AJ], vz[AJ], vrow[AJ], vch[AJ];
-#pragma unroll
-    for (int j = 0; j < AJ; j++) {
-      int q = j * 128 + t;
-      vrow[j] = q / CH; vch[j] = q % CH;
-      int v = v0 + vrow[j];
-      if (v < V) { vz[j] = v / nxy; int r = v - vz[j] * nxy; vy[j] = r / nx; vx[j] = r - vy[j] * nx; }
-      else { vx[j] = -1000000; vy[j] = 0; vz[j] = 0; }
-    }
-    // tap u of this tile is global tap g0 + u: stage (g0 + u) % NS, and its
-    // commit is completion number (g0 + u) / NS of that stage's barrier
-    auto load = [&](int u) {
-      long long g = g0 + u;
-      int stage = (int)(g % NS);
-      if (g >= NS) ok = ok && tc_wait(&bar[stage], (unsigned)(((g - NS) / NS) & 1));   // MMAs of g - NS done
-      int dx = u % 3 - 1, dy = (u / 3) % 3 - 1, dz = u / 9 - 1;
-      unsigned char *a = smraw + stage * S::STAGE, *b = a + S::A_BYTES;
-#pragma unroll
-      for (int j = 0; j < AJ; j++) {
-        int x = vx[j] + dx, y = vy[j] + dy, z = vz[j] + dz;
-        bool in = x >= 0 && x < nx && y >= 0 && y < ny && z >= 0 && z < nz;
-        const bf16 *src = in ? X + ((size_t)(x + nx * (y + ny * z)) * ldx + offx + vch[j] * 8) : X;
-        cp_async16(a + (vch[j] >> 1) * (CBM / 8) * 256 + coff(vrow[j], vch[j]), src, in ? 16 : 0);
-      }
-      const bf16 *w = Wt + (size_t)u * CO * CI;
-#pragma unroll
-      for (int j = 0; j < BJ; j++) {
-        int q = j * 128 + t;
-        if (q < CO * CH) {
-          int o = q / CH, ch = q % CH;
-          cp_async16(b + (ch >> 1) * (CO / 8) * 256 + coff(o, ch), w + o * CI + ch * 8, 16);
-        }
-      }
-    };
-    // copies run LA = NS - 2 taps ahead, so the stage refilled at tap t was
-    // last read by the MMAs of tap t - 2, which have had a whole tap to finish
-    constexpr int LA = NS - 2;
-#pragma unroll 1
-    for (int u = 0; u < LA; u++) { load(u); cp_commit(); }
+  tc_after();
+  const uint32_t taddr = tslot;
+  // the next kernel may start only now: every CTA of this one has its TMEM,
+  // so CTAs of the next that hold theirs cannot keep this one from finishing
+  pdl_trigger();
+  if (t == 0) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&wbar)), "n"(W_BYTES) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_u32(smtc)), "l"(Wt), "n"(W_BYTES), "r"(smem_u32(&wbar)) : "memory");
+  }
+  pdl_wait();
+  const int nh = TSL * (NZ + 2) * CH;
+  for (int q = t; q < nh; q += 256) {
+    const int ch = q % CH, h = q / CH, hx = h % THX, r = h / THX, hy = r % THY, hz = r / THY;
+    const int x = X0 + hx - 1, y = Y0 + hy - 1, z = Z0 + hz - 1;
+    const bool in = x >= 0 && x < nx && y >= 0 && y < ny && z >= 0 && z < nz;
+    const bf16 *src = in ? X + ((size_t)x + (size_t)nx * (y + (size_t)ny * z)) * ldx + offx + ch * 8 : X;
+    cp_async16(sA + ch * plane + h * 16, src, in ? 16 : 0);
+  }
+  cp_commit();
+  cp_wait<0>();
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  bool ok = __syncthreads_and(tc_wait(&wbar, 0));
+  if (t == 0 && ok) {
+    tc_after();
+    const uint32_t idesc = tc_idesc(CO, false);
+    const uint64_t da0 = tc_desc(smem_u32(sA), plane, THX * 16);
+    uint64_t db = tc_desc(smem_u32(smtc), 128, 256);
+    uint32_t acc = 0;
     for (int tap = 0; tap < 27; tap++) {
-      int u = tap + LA;
-      if (u < 27) load(u);
-      cp_commit();                                // (possibly empty) group: one per tap
-      cp_wait<LA>();                              // this tap's copies have landed
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      ok = __syncthreads_and(ok);
-      if (t == 0 && ok) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        long long g = g0 + tap;
-        int stage = (int)(g % NS);
-        unsigned char *a = smraw + stage * S::STAGE, *b = a + S::A_BYTES;
+      const uint64_t da = da0 + tap % 3 + THX * (tap / 3 % 3) + TSL * (tap / 9);
 #pragma unroll
-        for (int kb = 0; kb < S::KB; kb++) {
-          uint64_t da = tc_desc(smem_u32(a + kb * (CBM / 8) * 256)), db = tc_desc(smem_u32(b + kb * (CO / 8) * 256));
-          uint32_t acc = (tap > 0 || kb > 0) ? 1u : 0u;
-          asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                       ::"r"(taddr), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                     ::"r"(smem_u32(&bar[stage])) : "memory");
+      for (int kb = 0; kb < KB; kb++) {
+        for (int z = 0; z < NZ; z++) tc_mma(taddr + z * CO, da + z * TSL + kb * (plane >> 3), db, idesc, acc);
+        acc = 1;
+        db += CO * 2;                                  // CO / 8 groups of 256 bytes
       }
     }
-    // the tile's last MMAs have committed
-    {
-      long long g = g0 + 26;
-      ok = ok && tc_wait(&bar[(int)(g % NS)], (unsigned)((g / NS) & 1));
-    }
-    ok = __syncthreads_and(ok);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (ok) {
-      int v = v0 + t;                             // TMEM lane = row = thread
-#pragma unroll
-      for (int c0 = 0; c0 < CO; c0 += 32) {
-        float acc[32];
-        tc_ld32(taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, acc);
-        if (v < V) {
-          if (MODE == 0) {
-#pragma unroll
-            for (int c = 0; c < 32; c++) { acc[c] += bias[c0 + c]; if (relu) acc[c] = fmaxf(acc[c], 0.f); }
-          } else if (MODE == 2) {
-            const bf16 *mk = mask + (size_t)v * ldm + offm + c0;
-#pragma unroll
-            for (int c = 0; c < 32; c++) if (!(__bfloat162float(mk[c]) > 0.f)) acc[c] = 0.f;
-          }
-          uint4 pk[4];
-          __nv_bfloat162 *h2 = reinterpret_cast<__nv_bfloat162 *>(pk);
-#pragma unroll
-          for (int c = 0; c < 16; c++) h2[c] = __floats2bfloat162_rn(acc[2 * c], acc[2 * c + 1]);
-          uint4 *dst = reinterpret_cast<uint4 *>(out + (size_t)v * ldo + offo + c0);
-#pragma unroll
-          for (int u = 0; u < 4; u++) dst[u] = pk[u];
-        }
-      }
-    }
-    // the accumulator is read before the next tile's first MMA overwrites it
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tc_commit(&mbar);
   }
-  if (!ok && t == 0) atomicExch(err, 1);
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (ok) ok = tc_wait(&mbar, 0);
+  ok = __syncthreads_and(ok);
+  tc_after();
+  if (ok) {
+    const int r = (warp & 3) * 32 + (t & 31), x = X0 + r % TBX, y = Y0 + r / TBX, nzv = min(NZ, nz - Z0);
+    const bool live = x < nx && y < ny;
+    for (int z = warp >> 2; z < nzv; z += 2) {
+      const size_t v = (size_t)x + (size_t)nx * (y + (size_t)ny * (Z0 + z));
+      const uint32_t ta = taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(z * CO);
+      if constexpr (MODE == 1) {
+        float acc[8];
+        tc_ld8(ta, acc);
+        if (live) {
+          float *op = reinterpret_cast<float *>(out) + v * ldo + offo;
+#pragma unroll
+          for (int c = 0; c < 8; c++) acc[c] += bias[c];
+          reinterpret_cast<float4 *>(op)[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+          reinterpret_cast<float4 *>(op)[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+        }
+      } else {
+#pragma unroll
+        for (int c0 = 0; c0 < CO; c0 += 32) {
+          float acc[32];
+          tc_ld32(ta + (uint32_t)c0, acc);
+          if (live) {
+            if (MODE == 0) {
+#pragma unroll
+              for (int c = 0; c < 32; c++) { acc[c] += bias[c0 + c]; if (relu) acc[c] = fmaxf(acc[c], 0.f); }
+            } else if (MODE == 2) {
+              const uint4 *mk = reinterpret_cast<const uint4 *>(mask + v * ldm + offm + c0);
+#pragma unroll
+              for (int u = 0; u < 4; u++) {
+                const uint4 m4 = mk[u];
+                const bf16 *m = reinterpret_cast<const bf16 *>(&m4);
+#pragma unroll
+                for (int c = 0; c < 8; c++) if (!(__bfloat162float(m[c]) > 0.f)) acc[8 * u + c] = 0.f;
+              }
+            }
+            uint4 pk[4];
+            __nv_bfloat162 *h2 = reinterpret_cast<__nv_bfloat162 *>(pk);
+#pragma unroll
+            for (int c = 0; c < 16; c++) h2[c] = __floats2bfloat162_rn(acc[2 * c], acc[2 * c + 1]);
+            uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<bf16 *>(out) + v * ldo + offo + c0);
+#pragma unroll
+            for (int u = 0; u < 4; u++) dst[u] = pk[u];
+          }
+        }
+      }
+    }
+  }
+  if (!ok && t == 0) *(volatile int *)err = 1;
+  tc_before();
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "n"(CO) : "memory");
+  if (warp == 0) tc_free(taddr, ncol);
 }
 
 // ------------------------------------------------------ weight gradient ---
-// part[tap][chunk][o][c] = sum over the chunk's voxels v of dZ[v, o] X[v + d(tap), c]
-// (o < CO, c < CI), and for the centre tap bpart[chunk][o] = sum_v dZ[v, o].
-constexpr int WCH = 256;      // voxels per sub-chunk (8 warps x 32)
-constexpr int WIT = 4;        // sub-chunks per CTA
-template <int CI, int MT>
-struct wg_smem {
-  static constexpr int ZST = MT * 16 + 8, XST = CI + 8;
-  static constexpr int Z_EL = WCH * ZST, X_EL = WCH * XST;
-  static constexpr int RED = 8 * MT * 16 * CI;           // floats
-  static constexpr int BYTES = (Z_EL + X_EL) * 2 + RED * 4;
+// part[tap][chunk][o][c] = sum over the chunk's voxels v of dZ[v, o] X[v + d(tap), c],
+// and for dz = 0 bpart[chunk][o] = sum_v dZ[v, o], of all layers in one launch.
+//
+// On tcgen05 with the voxels as K: M = 128 rows are four x shifts of 32 input
+// channels (three used), N the output channels, one accumulator per dy.  A
+// CTA owns a range of slices (8 x 16 voxels of one z), one dz and 32 of the
+// input channels.  Both operands are MN-major core matrices (8 channels of
+// 16 bytes, 8 voxels consecutive in y): X lies as [x][chunk][y], so that the
+// channel groups of x - 1, x, x + 1 follow each other at one stride, and dy is
+// a shift of the start by 16 bytes; dZ as [x][chunk][y].  One MMA contracts
+// the 16 voxels of an x column.  Four stages of a slice each; after WFL
+// slices (64 MMAs on an accumulator) the sums move to FP32 registers, so that
+// the tensor cores' accumulation chains stay short.
+constexpr int WYP = THY + 1, WYB = TBY + 1;                      // y pitches, odd: copies free of bank conflicts
+constexpr int WA_BYTES = 11 * 4 * WYP * 16 + 64, WB_BYTES = TBX * 4 * WYB * 16;
+constexpr int WSTAGE = WA_BYTES + WB_BYTES, WNS = 4, WLA = 2, WFL = 8;
+struct wg_layer {
+  const bf16 *X, *dZ;
+  float *part, *bpart;
+  int ldx, offx, ldz, nx, ny, nz, co, ci, nchunk, block0;
 };
+struct wg_table { wg_layer l[NLAYER]; };
 
-template <int CI, int MT>
-__global__ void __launch_bounds__(256) k_conv_wgrad(int nx, int ny, int nz, const bf16 *__restrict__ X, int ldx,
-                                                    int offx, const bf16 *__restrict__ dZ, int ldz, int offz, int co,
-                                                    float *part, float *bpart) {
-  typedef wg_smem<CI, MT> S;
-  constexpr int M16 = MT * 16, CH = CI / 8, NTL = CI / 8;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  bf16 *sZ = reinterpret_cast<bf16 *>(smraw);
-  bf16 *sX = sZ + S::Z_EL;
-  float *red = reinterpret_cast<float *>(sX + S::X_EL);
-  const int V = nx * ny * nz, nxy = nx * ny;
-  const int chunk = blockIdx.x, tap = blockIdx.y, nchunk = gridDim.x;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int dx = tap % 3 - 1, dy = (tap / 3) % 3 - 1, dz = tap / 9 - 1;
-  float acc[MT][NTL][4];
-#pragma unroll
-  for (int mt = 0; mt < MT; mt++)
-#pragma unroll
-    for (int nt = 0; nt < NTL; nt++)
-#pragma unroll
-      for (int e = 0; e < 4; e++) acc[mt][nt][e] = 0.f;
-  float bsum = 0.f;
-  for (int it = 0; it < WIT; it++) {
-    int vb = (chunk * WIT + it) * WCH;
-    if (vb >= V) break;
-    // dZ rows (zero past the end and in the padding channels)
-    for (int q = t; q < WCH * (M16 / 8); q += 256) {
-      int r = q / (M16 / 8), ch = q % (M16 / 8), v = vb + r;
-      bool ok = v < V && ch * 8 < co;
-      cp_async16(sZ + r * S::ZST + ch * 8, ok ? dZ + (size_t)v * ldz + offz + ch * 8 : dZ, ok ? 16 : 0);
+__global__ void __launch_bounds__(256) k_conv_wgrad(const __grid_constant__ wg_table tab, int *err) {
+  extern __shared__ __align__(128) unsigned char smtc[];
+  __shared__ uint64_t bar[WNS];
+  __shared__ uint32_t tslot;
+  __shared__ float bred[256];
+  const int t = threadIdx.x, warp = t >> 5;
+  int li = 0;
+  while (li + 1 < NLAYER && (int)blockIdx.x >= tab.l[li + 1].block0) li++;
+  const wg_layer &L = tab.l[li];
+  const int nx = L.nx, ny = L.ny, nz = L.nz, co = L.co, ci = L.ci, nchunk = L.nchunk, lb = (int)blockIdx.x - L.block0;
+  const int chunk = lb % nchunk, dz = lb / nchunk % 3, half = lb / (3 * nchunk);
+  const int lch = ci == 16 ? 1 : 2, chn = 1 << lch;              // 16-byte chunks of input channels
+  const int lno = co <= 16 ? 1 : 2, no = 8 << lno;               // N and its chunks
+  if (t == 0) {
+    for (int k = 0; k < WNS; k++) bar_init(&bar[k]);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tc_alloc(&tslot, 128);
+  tc_before();
+  __syncthreads();
+  tc_after();
+  pdl_trigger();
+  pdl_wait();
+  const uint32_t taddr = tslot, idesc = tc_idesc(no, true);
+  const int tx = (nx + TBX - 1) / TBX, ty = (ny + TBY - 1) / TBY;
+  const int zlo = dz == 0 ? 1 : 0, nzv = max(0, (dz == 2 ? nz - 1 : nz) - zlo);   // slices whose z + dz - 1 exists
+  const long long S = (long long)tx * ty * nzv;
+  const long long s0 = S * chunk / nchunk;
+  const int n = (int)(S * (chunk + 1) / nchunk - s0);
+  const bf16 *X = L.X + L.offx + half * 32, *dZ = L.dZ;
+  const int ldx = L.ldx, ldz = L.ldz;
+  bool ok = true;
+  auto load = [&](int u) {
+    const int stage = u % WNS;
+    if (u >= WNS) ok = ok && tc_wait(&bar[stage], (unsigned)((u / WNS - 1) & 1));
+    const long long s = s0 + u;
+    const int z = zlo + (int)(s / (tx * ty)), rr = (int)(s % (tx * ty)), X0 = rr % tx * TBX, Y0 = rr / tx * TBY;
+    unsigned char *a = smtc + stage * WSTAGE, *b = a + WA_BYTES;
+    const size_t zx = (size_t)ny * (z + dz - 1), zz = (size_t)ny * z;
+    for (int q = t; q < TSL << lch; q += 256) {
+      const int ch = q & (chn - 1), h = q >> lch, hx = h % THX, hy = h / THX, x = X0 + hx - 1, y = Y0 + hy - 1;
+      const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
+      cp_async16(a + (((hx << lch) + ch) * WYP + hy) * 16, in ? X + (x + nx * (y + zx)) * ldx + ch * 8 : X, in ? 16 : 0);
     }
-    // shifted X rows
-    for (int q = t; q < WCH * CH; q += 256) {
-      int r = q / CH, ch = q % CH, v = vb + r;
-      bool ok = false;
-      const bf16 *src = X;
-      if (v < V) {
-        int z = v / nxy, rr = v - z * nxy, y = rr / nx, x = rr - y * nx;
-        x += dx; y += dy; z += dz;
-        ok = x >= 0 && x < nx && y >= 0 && y < ny && z >= 0 && z < nz;
-        if (ok) src = X + (size_t)(x + nx * (y + ny * z)) * ldx + offx + ch * 8;
-      }
-      cp_async16(sX + r * S::XST + ch * 8, src, ok ? 16 : 0);
+    for (int q = t; q < (TBX * TBY) << lno; q += 256) {
+      const int ch = q & ((1 << lno) - 1), h = q >> lno, hx = h % TBX, hy = h / TBX, x = X0 + hx, y = Y0 + hy;
+      const bool in = x < nx && y < ny;
+      cp_async16(b + (((hx << lno) + ch) * WYB + hy) * 16, in ? dZ + (x + nx * (y + zz)) * ldz + ch * 8 : dZ, in ? 16 : 0);
     }
+  };
+  float sum[3][16], bsum = 0.f;
+#pragma unroll
+  for (int d = 0; d < 3; d++)
+#pragma unroll
+    for (int j = 0; j < 16; j++) sum[d][j] = 0.f;
+  // bias: thread = output channel and part of the slice's voxels
+  const bool bias = dz == 1 && half == 0;
+  const int bo = t & (no - 1), bx = (t >> (lno + 3)) % TBX, by0 = lno == 1 ? (t >> 7) * 8 : 0, by1 = lno == 1 ? by0 + 8 : TBY;
+#pragma unroll 1
+  for (int u = 0; u < WLA; u++) { if (u < n) load(u); cp_commit(); }
+  for (int i = 0; i < n; i++) {
+    if (i + WLA < n) load(i + WLA);
     cp_commit();
-    cp_wait<0>();
-    __syncthreads();
-    if (tap == 13 && t < co)
-      for (int r = 0; r < WCH; r++) bsum += __bfloat162float(sZ[r * S::ZST + t]);
+    cp_wait<WLA>();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    ok = __syncthreads_and(ok);
+    if (!ok) break;
+    const unsigned char *a = smtc + i % WNS * WSTAGE, *b = a + WA_BYTES;
+    if (t == 0) {
+      tc_after();
+      const uint64_t da = tc_desc(smem_u32(a), 128, WYP * 16), db = tc_desc(smem_u32(b), 128, WYB * 16);
 #pragma unroll
-    for (int ks = 0; ks < 2; ks++) {
-      int kb = warp * 32 + ks * 16;
-      unsigned af[MT][4];
+      for (int x = 0; x < TBX; x++)
 #pragma unroll
-      for (int mt = 0; mt < MT; mt++)
-        ldsm_x4_t(af[mt], sZ + (kb + (lane & 7) + ((lane >> 4) << 3)) * S::ZST + mt * 16 + ((lane >> 3) & 1) * 8);
+        for (int dy = 0; dy < 3; dy++)
+          tc_mma(taddr + dy * 32, da + (x << lch) * WYP + dy, db + (x << lno) * WYB, idesc, i % WFL > 0 || x > 0);
+      tc_commit(&bar[i % WNS]);
+    }
+    if (bias) {
+      const bf16 *zr = reinterpret_cast<const bf16 *>(b) + ((bx << lno) + (bo >> 3)) * WYB * 8 + (bo & 7);
+      for (int y = by0; y < by1; y++) bsum += __bfloat162float(zr[y * 8]);
+    }
+    if (i % WFL == WFL - 1 || i == n - 1) {
+      ok = __syncthreads_and(tc_wait(&bar[i % WNS], (unsigned)((i / WNS) & 1)));
+      if (!ok) break;
+      tc_after();
 #pragma unroll
-      for (int np = 0; np < NTL / 2; np++) {
-        unsigned r[4];
-        ldsm_x4_t(r, sX + (kb + (lane & 7) + (((lane >> 3) & 1) << 3)) * S::XST + np * 16 + (lane >> 4) * 8);
-        unsigned b0[2] = {r[0], r[1]}, b1[2] = {r[2], r[3]};
+      for (int d = 0; d < 3; d++) {
+        const uint32_t ta = taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(d * 32 + (warp >> 2) * (no / 2));
+        float v[8];
+        tc_ld8(ta, v);
 #pragma unroll
-        for (int mt = 0; mt < MT; mt++) {
-          mma16816(acc[mt][2 * np], af[mt], b0);
-          mma16816(acc[mt][2 * np + 1], af[mt], b1);
+        for (int j = 0; j < 8; j++) sum[d][j] += v[j];
+        if (lno == 2) {
+          tc_ld8(ta + 8, v);
+#pragma unroll
+          for (int j = 0; j < 8; j++) sum[d][8 + j] += v[j];
         }
       }
+      tc_before();
+      __syncthreads();
     }
-    __syncthreads();
   }
-  // cross-warp sum in a fixed order
+  if (ok) {
+    const int m = (warp & 3) * 32 + (t & 31), dx = m >> (lch + 3), c = half * 32 + (m & (8 * chn - 1));
+    if (dx < 3)
 #pragma unroll
-  for (int mt = 0; mt < MT; mt++)
+      for (int d = 0; d < 3; d++) {
+        float *dst = L.part + ((size_t)(dx + 3 * d + 9 * dz) * nchunk + chunk) * co * ci + c;
 #pragma unroll
-    for (int nt = 0; nt < NTL; nt++)
-#pragma unroll
-      for (int e = 0; e < 4; e++) {
-        int m = mt * 16 + (lane >> 2) + (e >> 1) * 8, n = nt * 8 + (lane & 3) * 2 + (e & 1);
-        red[(warp * M16 + m) * CI + n] = acc[mt][nt][e];
+        for (int j = 0; j < 16; j++) {
+          const int o = (warp >> 2) * (no / 2) + j;
+          if (j < no / 2 && o < co) dst[(size_t)o * ci] = sum[d][j];
+        }
       }
-  __syncthreads();
-  float *dst = part + ((size_t)tap * nchunk + chunk) * co * CI;
-  for (int q = t; q < co * CI; q += 256) {
-    float s = 0.f;
-#pragma unroll
-    for (int w = 0; w < 8; w++) s += red[w * M16 * CI + q];
-    dst[q] = s;
+    if (bias) {
+      bred[t] = bsum;
+      __syncthreads();
+      if (t < co) {
+        float s = 0.f;
+        for (int k = t; k < 256; k += no) s += bred[k];
+        L.bpart[(size_t)chunk * co + t] = s;
+      }
+    }
+  } else if (t == 0) {
+    *(volatile int *)err = 1;
   }
-  if (tap == 13 && t < co) bpart[(size_t)chunk * co + t] = bsum;
+  tc_before();
+  __syncthreads();
+  if (warp == 0) tc_free(taddr, 128);
 }
 
-// grad[tap][o][c] += sum over chunks (in order) of part[tap][chunk][o][c]; bias likewise
-__global__ void k_wgrad_reduce(int nchunk, int per_tap, const float *part, const float *bpart, int co, float *gW,
-                               float *gb) {
-  int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < 27 * per_tap) {
-    int tap = q / per_tap, e = q - tap * per_tap;
-    const float *p = part + (size_t)tap * nchunk * per_tap + e;
-    float s = 0.f;
-    for (int c = 0; c < nchunk; c++) s += p[(size_t)c * per_tap];
-    gW[q] += s;
-  } else if (q < 27 * per_tap + co) {
-    int o = q - 27 * per_tap;
-    float s = 0.f;
-    for (int c = 0; c < nchunk; c++) s += bpart[(size_t)c * co + o];
-    gb[o] += s;
+// G += sums over the chunks (in order) of all layers' partials, G in the flat
+// parameter order (a layer's weights, then its biases); the last block adds
+// the loss (see k_sum_parts)
+__device__ __forceinline__ void sum_parts(int n, const float *part, double scale, double *out, int accumulate) {
+  double t = 0.0;
+  for (int k = threadIdx.x; k < n; k += 32) t += (double)part[k];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if (threadIdx.x == 0) out[0] = (accumulate ? out[0] : 0.0) + scale * t;
+}
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const __grid_constant__ wg_table tab, int np, float *G, int nl,
+                                                      const float *lpart, double lscale, double *lsum) {
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == gridDim.x - 1) {
+    if (threadIdx.x < 32) sum_parts(nl, lpart, lscale, lsum, 1);
+    return;
   }
+  const int q = blockIdx.x * 256 + threadIdx.x;
+  if (q >= np) return;
+  int r = q, l = 0;
+  for (; l < NLAYER - 1; l++) {
+    const int sz = 27 * tab.l[l].co * tab.l[l].ci + tab.l[l].co;
+    if (r < sz) break;
+    r -= sz;
+  }
+  const wg_layer &L = tab.l[l];
+  const int per = L.co * L.ci, nc = L.nchunk;
+  const float *p;
+  size_t st;
+  if (r < 27 * per) { p = L.part + (size_t)(r / per) * nc * per + r % per; st = per; }
+  else { p = L.bpart + (r - 27 * per); st = L.co; }
+  float s = 0.f;
+  for (int c0 = 0; c0 < nc; c0 += 8) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; u++) v[u] = c0 + u < nc ? p[(c0 + u) * st] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; u++) if (c0 + u < nc) s += v[u];
+  }
+  G[q] += s;
 }
 
 // ------------------------------------------------------- pool and up ------
@@ -662,6 +767,8 @@ __host__ __device__ inline dims coarse(dims d) { return {(d.nx + 1) / 2, (d.ny +
 
 // P[V, c] = mean of the existing children, 32 channels, 8 per thread
 __global__ void k_pool(dims f, dims c, const bf16 *X, int ldx, int offx, bf16 *P) {
+  pdl_trigger();
+  pdl_wait();
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= c.V() * 4) return;
   int V = q >> 2, g = (q & 3) * 8;
@@ -689,6 +796,8 @@ __global__ void k_pool(dims f, dims c, const bf16 *X, int ldx, int offx, bf16 *P
 
 // out[v, off + c] = C[parent(v), c], 32 channels
 __global__ void k_up(dims f, dims c, const bf16 *C, bf16 *out, int ldo, int offo) {
+  pdl_trigger();
+  pdl_wait();
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= f.V() * 4) return;
   int v = q >> 2, g = (q & 3) * 8;
@@ -699,6 +808,8 @@ __global__ void k_up(dims f, dims c, const bf16 *C, bf16 *out, int ldo, int offo
 
 // dC[V, c] = sum over children of G[v, offg + c]  (32 channels)
 __global__ void k_up_back(dims f, dims c, const bf16 *G, int ldg, int offg, bf16 *dC) {
+  pdl_trigger();
+  pdl_wait();
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= c.V() * 4) return;
   int V = q >> 2, g = (q & 3) * 8;
@@ -725,6 +836,8 @@ __global__ void k_up_back(dims f, dims c, const bf16 *G, int ldg, int offg, bf16
 // (the skip gradient, already masked, plus the pooled path's gradient)
 __global__ void k_pool_back(dims f, dims c, const bf16 *dP, const bf16 *S, int lds, int offs, const bf16 *E, int lde,
                             int offe, bf16 *dE) {
+  pdl_trigger();
+  pdl_wait();
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= f.V() * 4) return;
   int v = q >> 2, g = (q & 3) * 8;
@@ -750,6 +863,8 @@ __global__ void k_pool_back(dims f, dims c, const bf16 *dP, const bf16 *S, int l
 // dY[v, c] = (Y[v, c] - T[v, c]) / V for c < 2, 0 for the other 14 channels;
 // part[block] = sum of the block's squared errors
 __global__ void k_loss(int V, const float *Y, const float *T, bf16 *dY, float *part) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ float sh[256];
   int v = blockIdx.x * blockDim.x + threadIdx.x;
   float s = 0.f;
@@ -776,34 +891,48 @@ __global__ void k_loss(int V, const float *Y, const float *T, bf16 *dY, float *p
 
 // out[0] (+)= scale * sum of the n partials (one warp, fixed order)
 __global__ void k_sum_parts(int n, const float *part, double scale, double *out, int accumulate) {
-  double t = 0.0;
-  for (int k = threadIdx.x; k < n; k += 32) t += (double)part[k];
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-  if (threadIdx.x == 0) out[0] = (accumulate ? out[0] : 0.0) + scale * t;
+  sum_parts(n, part, scale, out, accumulate);
 }
 
-// Adam (Kingma and Ba, Algorithm 1) on the flat parameter array; the
-// gradient is divided by `gdiv` (the number of samples accumulated)
-__global__ void k_adam(int n, float *p, float *m, float *v, const float *g, float lr, float b1, float b2, float c1,
-                       float c2, float eps, float gdiv) {
+// Adam (Kingma and Ba, Algorithm 1) on the flat parameter array (the gradient
+// is divided by `gdiv`, the number of samples accumulated, and cleared), and
+// the BF16 copies of all layers, core matrices as woffs describes:
+// Wf[t][o][c] = W[t][o][c] and Wb[26-t][c][o] = W[t][o][c].  Rows and columns
+// beyond co (the head's 8 outputs) stay zero.  One launch for both: one per
+// layer took 45 us of 1.2 ms per training step.
+struct pack_table { int w0[NLAYER], wf[NLAYER], wb[NLAYER], co[NLAYER], ci[NLAYER]; };
+template <bool ADAM>
+__global__ void k_adam_pack(int n, const __grid_constant__ pack_table T, float *p, float *m, float *v, float *g, float lr,
+                            float b1, float b2, float c1, float c2, float eps, float gdiv, bf16 *Wf, bf16 *Wb) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  float gi = g[i] / gdiv;
-  float mi = b1 * m[i] + (1.f - b1) * gi;
-  float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi; v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  float pi = p[i];
+  if (ADAM) {
+    float gi = g[i] / gdiv;
+    float mi = b1 * m[i] + (1.f - b1) * gi;
+    float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+    m[i] = mi; v[i] = vi;
+    pi -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = pi;
+    g[i] = 0.f;
+  }
+  int l = 0;
+  while (l + 1 < NLAYER && i >= T.w0[l + 1]) l++;
+  const int co = T.co[l], ci = T.ci[l], q = i - T.w0[l];
+  if (q >= 27 * co * ci) return;                       // a bias
+  const int t = q / (co * ci), r = q - t * co * ci, o = r / ci, c = r - o * ci, cr = wrows(co);
+  const bf16 w = __float2bfloat16_rn(pi);
+  Wf[(size_t)T.wf[l] + (size_t)t * cr * ci + woffs(cr, o, c >> 3) + (c & 7)] = w;
+  Wb[(size_t)T.wb[l] + (size_t)(26 - t) * ci * cr + woffs(ci, c, o >> 3) + (o & 7)] = w;
 }
 
-// BF16 copies of one layer: Wf[t][o][c] = W[t][o][c]; Wb[26-t][c][o] = W[t][o][c]
-// (Wb's o dimension padded to cob with zeros)
-__global__ void k_pack(int co, int ci, int cb, const float *W, bf16 *Wf, bf16 *Wb) {
-  int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= 27 * co * ci) return;
-  int t = q / (co * ci), r = q - t * co * ci, o = r / ci, c = r - o * ci;
-  bf16 w = __float2bfloat16_rn(W[q]);
-  Wf[q] = w;
-  Wb[((size_t)(26 - t) * ci + c) * cb + o] = w;
+// the exported layout (input layer's 8 used channels only) of the parameters,
+// or of the mean gradients
+__global__ void k_export(int n, const float *p, float div, float *out) {
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  constexpr int n0 = 27 * 32 * CIN_USED, d0 = 27 * 32 * (CIN_GPU - CIN_USED);
+  out[i] = p[i < n0 ? i / CIN_USED * CIN_GPU + i % CIN_USED : i + d0] / div;
 }
 
 // network input from FP32 features [V][8] -> BF16 [V][16]
@@ -839,7 +968,7 @@ struct sim_ws_s {
   dims cur = {0, 0, 0};
   level_bufs L[4];
   dbuf<bf16> X0, dY;
-  dbuf<float> Y, part, lpart, T32, F32;
+  dbuf<float> Y, part, lpart, T32, F32, E;
   dbuf<double> lsum;
   // dataset of (features, target) pairs taken from simulator solves
   struct sample { dims d; dbuf<bf16> X; dbuf<float> T; };
@@ -847,9 +976,13 @@ struct sim_ws_s {
   size_t max_samples = 1u << 30;
   unsigned long long seed = 0;
   std::mutex use;                         // one caller at a time (activations are shared)
-  bool tc = false;                        // tcgen05 convolutions (else mma.sync, the faster here)
-  dbuf<int> err;                          // set by a kernel whose bounded wait gave up
-  ~sim_ws_s() { if (st) cudaStreamDestroy(st); }
+  bool tc = true;                         // tcgen05 convolutions (else mma.sync)
+  int *err = nullptr, *err_dev = nullptr; // host-mapped: set by a kernel whose bounded wait gave up
+  pack_table tab;
+  ~sim_ws_s() {
+    if (st) cudaStreamDestroy(st);
+    if (err) cudaFreeHost(err);
+  }
 };
 
 namespace nn {
@@ -859,22 +992,22 @@ static void ws_layout(sim_ws_s *w) {
   for (int l = 0; l < NLAYER; l++) {
     w->woff[l] = o; o += (size_t)27 * LAYERS[l].co * LAYERS[l].ci;
     w->boff[l] = o; o += LAYERS[l].co;
-    w->wfoff[l] = fo; fo += (size_t)27 * LAYERS[l].co * LAYERS[l].ci;
+    w->wfoff[l] = fo; fo += (size_t)27 * cob(l) * LAYERS[l].ci;
     w->wboff[l] = bo; bo += (size_t)27 * LAYERS[l].ci * cob(l);
+    w->tab.w0[l] = (int)w->woff[l]; w->tab.wf[l] = (int)w->wfoff[l]; w->tab.wb[l] = (int)w->wboff[l];
+    w->tab.co[l] = LAYERS[l].co; w->tab.ci[l] = LAYERS[l].ci;
   }
   w->np = o;
   w->P.alloc(o); w->M.alloc(o); w->Vm.alloc(o); w->G.alloc(o);
   w->Wf.alloc(fo); w->Wb.alloc(bo);
+  RS_CUDA(cudaMemsetAsync(w->Wf.p, 0, fo * sizeof(bf16), w->st));
+  RS_CUDA(cudaMemsetAsync(w->Wb.p, 0, bo * sizeof(bf16), w->st));
 }
 
 static void ws_pack(sim_ws_s *w) {
-  RS_CUDA(cudaMemsetAsync(w->Wb.p, 0, w->Wb.n * sizeof(bf16), w->st));
-  for (int l = 0; l < NLAYER; l++) {
-    int n = 27 * LAYERS[l].co * LAYERS[l].ci;
-    k_pack<<<grid_for(n, 256), 256, 0, w->st>>>(LAYERS[l].co, LAYERS[l].ci, cob(l), w->P.p + w->woff[l],
-                                                 w->Wf.p + w->wfoff[l], w->Wb.p + w->wboff[l]);
-  }
-  RS_LAUNCHED(NLAYER);
+  k_adam_pack<false><<<grid_for(w->np, 256), 256, 0, w->st>>>((int)w->np, w->tab, w->P.p, nullptr, nullptr, nullptr, 0.f,
+                                                             0.f, 0.f, 0.f, 0.f, 0.f, 0.f, w->Wf.p, w->Wb.p);
+  RS_LAUNCHED(1);
   RS_CHECK_LAUNCH();
 }
 
@@ -907,24 +1040,41 @@ static void conv_halo_launch(sim_ws_s *w, dims d, const bf16 *X, int ldx, int of
   RS_LAUNCHED(1);
 }
 
+// Slices per CTA: more of them share a halo and the weights' copy, fewer fill
+// the chip on small grids.  Taken by a model of the time in units of one
+// slice's MMAs at 32 input channels (1 us): rounds of resident CTAs, each a
+// start (TMEM, copies, epilogue: 2) and its resident slices one after the other.
 template <int CI, int CO, int MODE>
 static void conv_tc_launch(sim_ws_s *w, dims d, const bf16 *X, int ldx, int offx, const bf16 *Wt, const float *bias,
                            int relu, void *out, int ldo, int offo, const bf16 *mask, int ldm, int offm) {
-  static int per_sm = 0;                      // resident CTAs per SM for this instantiation
+  static int per_sm[5] = {0, 0, 0, 0, 0};     // resident CTAs per SM by slices (0: does not fit)
   static int sms = 0;
-  int bytes = tc_smem<CI, CO>::BYTES;
-  if (!per_sm) {
-    RS_CUDA(cudaFuncSetAttribute(k_conv_tc<CI, CO, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    int dev = 0;
+  static std::once_flag once;
+  std::call_once(once, [&] {
+    int dev = 0, cap = 0;
     RS_CUDA(cudaGetDevice(&dev));
     RS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    RS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_conv_tc<CI, CO, MODE>, 128, bytes));
-    if (per_sm < 1) per_sm = 1;
+    RS_CUDA(cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    int top = 0;
+    for (int z = 1; z <= 4; z++) if (tc_bytes(CI, CO, z) + 128 <= cap) top = z;
+    RS_CUDA(cudaFuncSetAttribute(k_conv_tc<CI, CO, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_bytes(CI, CO, top)));
+    for (int z = 1; z <= top; z++) {
+      RS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[z], k_conv_tc<CI, CO, MODE>, 256, tc_bytes(CI, CO, z)));
+      per_sm[z] = std::max(1, std::min(per_sm[z], 512 / tc_cols(CO, z)));
+    }
+  });
+  const long long txy = (long long)((d.nx + TBX - 1) / TBX) * ((d.ny + TBY - 1) / TBY);
+  int NZ = 1;
+  double best = 1e300;
+  for (int z = 1; z <= 4 && per_sm[z]; z++) {
+    const long long tiles = txy * ((d.nz + z - 1) / z), r = std::min<long long>(per_sm[z], (tiles + sms - 1) / sms),
+                    rounds = (tiles + sms * r - 1) / (sms * r);
+    const double c = rounds * (2.0 + r * z * (CI / 32.0));
+    if (c < best) { best = c; NZ = z; }
   }
-  unsigned tiles = grid_for(d.V(), CBM), cap = (unsigned)(sms * per_sm), grid = tiles < cap ? tiles : cap;
-  k_conv_tc<CI, CO, MODE><<<grid, 128, bytes, w->st>>>(d.nx, d.ny, d.nz, X, ldx, offx, Wt, bias, relu,
-                                                                        reinterpret_cast<bf16 *>(out), ldo, offo, mask,
-                                                                        ldm, offm, w->err.p);
+  const unsigned tiles = (unsigned)(txy * ((d.nz + NZ - 1) / NZ));
+  launch_pdl(k_conv_tc<CI, CO, MODE>, tiles, 256, (size_t)tc_bytes(CI, CO, NZ), w->st, d.nx, d.ny, d.nz, NZ, X, ldx, offx,
+             Wt, bias, relu, out, ldo, offo, mask, ldm, offm, w->err_dev);
   RS_LAUNCHED(1);
 }
 
@@ -933,12 +1083,13 @@ static void fwd(sim_ws_s *w, int l, dims d, const bf16 *X, int ldx, int offx, vo
   const bf16 *Wt = w->Wf.p + w->wfoff[l];
   const float *b = w->P.p + w->boff[l];
   int ci = LAYERS[l].ci;
-  if (l == HEAD) conv_halo_launch<32, 1, 1>(w, d, X, ldx, offx, Wt, b, 0, out, ldo, offo);
-  else if (w->tc) {
-    if (ci == 16) conv_tc_launch<16, 32, 0>(w, d, X, ldx, offx, Wt, b, 1, out, ldo, offo, nullptr, 0, 0);
+  if (w->tc) {
+    if (l == HEAD) conv_tc_launch<32, 16, 1>(w, d, X, ldx, offx, Wt, b, 0, out, ldo, offo, nullptr, 0, 0);
+    else if (ci == 16) conv_tc_launch<16, 32, 0>(w, d, X, ldx, offx, Wt, b, 1, out, ldo, offo, nullptr, 0, 0);
     else if (ci == 32) conv_tc_launch<32, 32, 0>(w, d, X, ldx, offx, Wt, b, 1, out, ldo, offo, nullptr, 0, 0);
     else conv_tc_launch<64, 32, 0>(w, d, X, ldx, offx, Wt, b, 1, out, ldo, offo, nullptr, 0, 0);
   }
+  else if (l == HEAD) conv_halo_launch<32, 1, 1>(w, d, X, ldx, offx, Wt, b, 0, out, ldo, offo);
   else if (ci == 16) conv_halo_launch<16, 4, 0>(w, d, X, ldx, offx, Wt, b, 1, out, ldo, offo);
   else if (ci == 32) conv_halo_launch<32, 4, 0>(w, d, X, ldx, offx, Wt, b, 1, out, ldo, offo);
   else conv_halo_launch<64, 4, 0>(w, d, X, ldx, offx, Wt, b, 1, out, ldo, offo);
@@ -977,33 +1128,49 @@ static void bwd_data(sim_ws_s *w, int l, dims d, const bf16 *dZ, int ldz, int of
   }
 }
 
-template <int CI, int MT>
-static void wgrad_launch(sim_ws_s *w, int l, dims d, const bf16 *X, int ldx, int offx, const bf16 *dZ, int ldz, int offz) {
-  static bool attr = false;
-  int bytes = wg_smem<CI, MT>::BYTES;
-  if (!attr) {
-    RS_CUDA(cudaFuncSetAttribute(k_conv_wgrad<CI, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    attr = true;
+// Weight gradients of all layers, from the activations and the gradients that
+// the data-gradient passes left (each in a buffer of its own): one launch of
+// about two CTAs per SM, shared out by the layers' slices, and one that adds
+// the chunks and the loss.
+struct wg_in { const bf16 *X; int ldx, offx; const bf16 *dZ; int ldz; dims d; };
+static void wgrad(sim_ws_s *w, const wg_in in[NLAYER], int nl, double lscale) {
+  wg_table tab;
+  double units = 0.0;
+  auto slices = [](dims d) { return (long long)((d.nx + TBX - 1) / TBX) * ((d.ny + TBY - 1) / TBY) * d.nz; };
+  for (int l = 0; l < NLAYER; l++) units += 3.0 * slices(in[l].d) * ((LAYERS[l].ci + 31) / 32);
+  static int cap = 0;                             // CTAs to aim at
+  static std::once_flag once;
+  std::call_once(once, [&] {
+    int dev = 0, sms = 0;
+    RS_CUDA(cudaGetDevice(&dev));
+    RS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    RS_CUDA(cudaFuncSetAttribute(k_conv_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, WNS * WSTAGE));
+    cap = 2 * sms;
+  });
+  int block = 0;
+  size_t need = 0;
+  for (int l = 0; l < NLAYER; l++) {
+    wg_layer &L = tab.l[l];
+    const int co = LAYERS[l].co, ci = LAYERS[l].ci;
+    const long long S = slices(in[l].d);
+    L.X = in[l].X; L.ldx = in[l].ldx; L.offx = in[l].offx; L.dZ = in[l].dZ; L.ldz = in[l].ldz;
+    L.nx = in[l].d.nx; L.ny = in[l].d.ny; L.nz = in[l].d.nz; L.co = co; L.ci = ci;
+    L.nchunk = (int)std::max(1.0, std::min((double)S, std::floor(cap * (double)S / units)));
+    L.block0 = block;
+    block += L.nchunk * 3 * ((ci + 31) / 32);
+    need += (size_t)L.nchunk * (27 * co * ci + co);
   }
-  int co = LAYERS[l].co;
-  int nchunk = (d.V() + WCH * WIT - 1) / (WCH * WIT);
-  size_t need = (size_t)27 * nchunk * co * CI;
-  w->part.ensure(need + (size_t)nchunk * co);
-  float *bpart = w->part.p + need;
-  k_conv_wgrad<CI, MT><<<dim3(nchunk, 27), 256, bytes, w->st>>>(d.nx, d.ny, d.nz, X, ldx, offx, dZ, ldz, offz, co,
-                                                                 w->part.p, bpart);
-  int per_tap = co * CI;
-  k_wgrad_reduce<<<grid_for(27 * per_tap + co, 256), 256, 0, w->st>>>(nchunk, per_tap, w->part.p, bpart, co,
-                                                                       w->G.p + w->woff[l], w->G.p + w->boff[l]);
+  w->part.ensure(need);
+  float *p = w->part.p;
+  for (int l = 0; l < NLAYER; l++) {
+    wg_layer &L = tab.l[l];
+    L.part = p; p += (size_t)L.nchunk * 27 * L.co * L.ci;
+    L.bpart = p; p += (size_t)L.nchunk * L.co;
+  }
+  launch_pdl(k_conv_wgrad, (unsigned)block, 256, (size_t)WNS * WSTAGE, w->st, tab, w->err_dev);
+  launch_pdl(k_wgrad_reduce, grid_for(w->np, 256) + 1, 256, 0, w->st, tab, (int)w->np, w->G.p, nl, w->lpart.p, lscale,
+             w->lsum.p);
   RS_LAUNCHED(2);
-}
-
-static void wgrad(sim_ws_s *w, int l, dims d, const bf16 *X, int ldx, int offx, const bf16 *dZ, int ldz, int offz) {
-  int ci = LAYERS[l].ci;
-  if (l == HEAD) wgrad_launch<32, 1>(w, l, d, X, ldx, offx, dZ, ldz, offz);
-  else if (ci == 16) wgrad_launch<16, 2>(w, l, d, X, ldx, offx, dZ, ldz, offz);
-  else if (ci == 32) wgrad_launch<32, 2>(w, l, d, X, ldx, offx, dZ, ldz, offz);
-  else wgrad_launch<64, 2>(w, l, d, X, ldx, offx, dZ, ldz, offz);
 }
 
 static void ensure_dims(sim_ws_s *w, dims d) {
@@ -1033,7 +1200,7 @@ static void forward(sim_ws_s *w) {
   fwd(w, C00, L[0].d, w->X0.p, CIN_GPU, 0, L[0].a.p, 32, 0);
   fwd(w, C01, L[0].d, L[0].a.p, 32, 0, L[0].cat.p, 64, 32);
   for (int k = 1; k <= 3; k++) {
-    k_pool<<<grid_for((size_t)L[k].d.V() * 4, 256), 256, 0, w->st>>>(L[k - 1].d, L[k].d, L[k - 1].cat.p, 64, 32, L[k].p.p);
+    launch_pdl(k_pool, grid_for((size_t)L[k].d.V() * 4, 256), 256, 0, w->st, L[k - 1].d, L[k].d, L[k - 1].cat.p, 64, 32, L[k].p.p);
     RS_LAUNCHED(1);
     int c0 = k == 1 ? C10 : k == 2 ? C20 : C30;
     fwd(w, c0, L[k].d, L[k].p.p, 32, 0, L[k].a.p, 32, 0);
@@ -1041,7 +1208,7 @@ static void forward(sim_ws_s *w) {
     else fwd(w, c0 + 1, L[k].d, L[k].a.p, 32, 0, L[k].b.p, 32, 0);
   }
   for (int k = 2; k >= 0; k--) {
-    k_up<<<grid_for((size_t)L[k].d.V() * 4, 256), 256, 0, w->st>>>(L[k].d, L[k + 1].d, L[k + 1].b.p, L[k].cat.p, 64, 0);
+    launch_pdl(k_up, grid_for((size_t)L[k].d.V() * 4, 256), 256, 0, w->st, L[k].d, L[k + 1].d, L[k + 1].b.p, L[k].cat.p, 64, 0);
     RS_LAUNCHED(1);
     int d0 = k == 2 ? D20 : k == 1 ? D10 : D00;
     fwd(w, d0, L[k].d, L[k].cat.p, 64, 0, L[k].da.p, 32, 0);
@@ -1056,47 +1223,46 @@ static void forward(sim_ws_s *w) {
 static void backward(sim_ws_s *w, const float *T) {
   level_bufs *L = w->L;
   int V = L[0].d.V();
-  k_loss<<<grid_for(V, 256), 256, 0, w->st>>>(V, w->Y.p, T, w->dY.p, w->lpart.p);
-  k_sum_parts<<<1, 32, 0, w->st>>>((int)grid_for(V, 256), w->lpart.p, 0.5 / V, w->lsum.p, 1);
-  RS_LAUNCHED(2);
+  wg_in in[NLAYER];
+  auto wgrad = [&](int l, dims d, const bf16 *X, int ldx, int offx, const bf16 *dZ, int ldz) { in[l] = {X, ldx, offx, dZ, ldz, d}; };
+  launch_pdl(k_loss, grid_for(V, 256), 256, 0, w->st, V, w->Y.p, T, w->dY.p, w->lpart.p);
+  RS_LAUNCHED(1);
   // head: input b0, output dY
-  wgrad(w, HEAD, L[0].d, L[0].b.p, 32, 0, w->dY.p, 16, 0);
+  wgrad(HEAD, L[0].d, L[0].b.p, 32, 0, w->dY.p, 16);
   bwd_data(w, HEAD, L[0].d, w->dY.p, 16, 0, L[0].gb.p, 32, 0, L[0].b.p, 32, 0);
   // decoder, finest level first
   for (int k = 0; k <= 2; k++) {
     int d0 = k == 2 ? D20 : k == 1 ? D10 : D00;
     // second decoder conv: input da, output gradient gb
-    wgrad(w, d0 + 1, L[k].d, L[k].da.p, 32, 0, L[k].gb.p, 32, 0);
+    wgrad(d0 + 1, L[k].d, L[k].da.p, 32, 0, L[k].gb.p, 32);
     bwd_data(w, d0 + 1, L[k].d, L[k].gb.p, 32, 0, L[k].gda.p, 32, 0, L[k].da.p, 32, 0);
     // first decoder conv: input cat, output gradient gda
-    wgrad(w, d0, L[k].d, L[k].cat.p, 64, 0, L[k].gda.p, 32, 0);
+    wgrad(d0, L[k].d, L[k].cat.p, 64, 0, L[k].gda.p, 32);
     bwd_data(w, d0, L[k].d, L[k].gda.p, 32, 0, L[k].gcat.p, 64, 0, L[k].cat.p, 64, 0);
     // up-sampled half -> gradient of the coarser level's output (gb there)
-    k_up_back<<<grid_for((size_t)L[k + 1].d.V() * 4, 256), 256, 0, w->st>>>(L[k].d, L[k + 1].d, L[k].gcat.p, 64, 0,
-                                                                           L[k + 1].gb.p);
+    launch_pdl(k_up_back, grid_for((size_t)L[k + 1].d.V() * 4, 256), 256, 0, w->st, L[k].d, L[k + 1].d, L[k].gcat.p, 64, 0, L[k + 1].gb.p);
     RS_LAUNCHED(1);
   }
   // bottom: c31 (input a3, output b3), c30 (input p3)
-  wgrad(w, C31, L[3].d, L[3].a.p, 32, 0, L[3].gb.p, 32, 0);
+  wgrad(C31, L[3].d, L[3].a.p, 32, 0, L[3].gb.p, 32);
   bwd_data(w, C31, L[3].d, L[3].gb.p, 32, 0, L[3].ga.p, 32, 0, L[3].a.p, 32, 0);
-  wgrad(w, C30, L[3].d, L[3].p.p, 32, 0, L[3].ga.p, 32, 0);
+  wgrad(C30, L[3].d, L[3].p.p, 32, 0, L[3].ga.p, 32);
   bwd_data(w, C30, L[3].d, L[3].ga.p, 32, 0, L[3].gp.p, 32, 0, nullptr, 0, 0);
   // encoder, coarse to fine: ge(k) = mask * (skip part of gcat(k) + pool-back of gp(k+1))
   for (int k = 2; k >= 0; k--) {
-    k_pool_back<<<grid_for((size_t)L[k].d.V() * 4, 256), 256, 0, w->st>>>(L[k].d, L[k + 1].d, L[k + 1].gp.p,
-                                                                         L[k].gcat.p, 64, 32, L[k].cat.p, 64, 32,
-                                                                         L[k].ge.p);
+    launch_pdl(k_pool_back, grid_for((size_t)L[k].d.V() * 4, 256), 256, 0, w->st, L[k].d, L[k + 1].d, L[k + 1].gp.p, L[k].gcat.p, 64, 32, L[k].cat.p, 64, 32, L[k].ge.p);
     RS_LAUNCHED(1);
     int c0 = k == 2 ? C20 : k == 1 ? C10 : C00;
-    wgrad(w, c0 + 1, L[k].d, L[k].a.p, 32, 0, L[k].ge.p, 32, 0);
+    wgrad(c0 + 1, L[k].d, L[k].a.p, 32, 0, L[k].ge.p, 32);
     bwd_data(w, c0 + 1, L[k].d, L[k].ge.p, 32, 0, L[k].ga.p, 32, 0, L[k].a.p, 32, 0);
     if (k > 0) {
-      wgrad(w, c0, L[k].d, L[k].p.p, 32, 0, L[k].ga.p, 32, 0);
+      wgrad(c0, L[k].d, L[k].p.p, 32, 0, L[k].ga.p, 32);
       bwd_data(w, c0, L[k].d, L[k].ga.p, 32, 0, L[k].gp.p, 32, 0, nullptr, 0, 0);
     } else {
-      wgrad(w, C00, L[0].d, w->X0.p, CIN_GPU, 0, L[0].ga.p, 32, 0);
+      wgrad(C00, L[0].d, w->X0.p, CIN_GPU, 0, L[0].ga.p, 32);
     }
   }
+  nn::wgrad(w, in, (int)grid_for(V, 256), 0.5 / V);
   RS_CHECK_LAUNCH();
   w->accum++;
 }
@@ -1111,11 +1277,12 @@ static void adam(sim_ws_s *w, double lr) {
   w->tstep++;
   const double b1 = 0.9, b2 = 0.999;
   float c1 = (float)(1.0 - std::pow(b1, (double)w->tstep)), c2 = (float)(1.0 - std::pow(b2, (double)w->tstep));
-  k_adam<<<grid_for(w->np, 256), 256, 0, w->st>>>((int)w->np, w->P.p, w->M.p, w->Vm.p, w->G.p, (float)lr, (float)b1,
-                                                 (float)b2, c1, c2, 1e-8f, (float)w->accum);
+  k_adam_pack<true><<<grid_for(w->np, 256), 256, 0, w->st>>>((int)w->np, w->tab, w->P.p, w->M.p, w->Vm.p, w->G.p, (float)lr,
+                                                            (float)b1, (float)b2, c1, c2, 1e-8f, (float)w->accum, w->Wf.p,
+                                                            w->Wb.p);
   RS_LAUNCHED(1);
-  ws_pack(w);
-  zero_grad(w);
+  RS_CHECK_LAUNCH();
+  w->accum = 0;
 }
 
 // splitmix64 (Steele, Lea and Flood 2014) and a Box-Muller normal draw for
@@ -1148,15 +1315,15 @@ static size_t export_count() {
 }
 
 // a tensor-core kernel whose bounded wait gave up leaves a flag; report it
+// (the caller has synchronised with the kernels)
 static void check_err(sim_ws_s *w) {
-  int e = 0;
-  RS_CUDA(cudaMemcpyAsync(&e, w->err.p, sizeof(int), cudaMemcpyDeviceToHost, w->st));
-  RS_CUDA(cudaStreamSynchronize(w->st));
-  if (e) {
-    RS_CUDA(cudaMemsetAsync(w->err.p, 0, sizeof(int), w->st));
+  volatile int *e = w->err;
+  if (*e) {
+    *e = 0;
     RS_FAIL(SIM_ERR_TIMEOUT, "warm-start network: a tensor-core pipeline wait gave up");
   }
 }
+void ws_check(sim_ws_s *w) { check_err(w); }
 
 extern "C" sim_status sim_ws_create(sim_ws_t *out, unsigned long long seed) {
   ABI_BEGIN
@@ -1185,8 +1352,9 @@ extern "C" sim_status sim_ws_create(sim_ws_t *out, unsigned long long seed) {
   RS_CUDA(cudaMemsetAsync(w->M.p, 0, w->np * sizeof(float), w->st));
   RS_CUDA(cudaMemsetAsync(w->Vm.p, 0, w->np * sizeof(float), w->st));
   w->lsum.alloc(2);
-  w->err.alloc(1);
-  RS_CUDA(cudaMemsetAsync(w->err.p, 0, sizeof(int), w->st));
+  RS_CUDA(cudaHostAlloc((void **)&w->err, sizeof(int), cudaHostAllocMapped));
+  *w->err = 0;
+  RS_CUDA(cudaHostGetDevicePointer((void **)&w->err_dev, w->err, 0));
   zero_grad(w.get());
   ws_pack(w.get());
   RS_CUDA(cudaStreamSynchronize(w->st));
@@ -1213,16 +1381,12 @@ extern "C" sim_status sim_ws_params(sim_ws_t w, int which, float *dst, size_t n,
   if (needed) *needed = ne;
   if (!dst) return SIM_OK;
   if (n < ne) RS_FAIL(SIM_ERR_ARG, "sim_ws_params: buffer holds %zu of %zu values", n, ne);
-  std::vector<float> h = d2h(which == 0 ? w->P.p : w->G.p, w->np, w->st);
-  float div = which == 1 && w->accum > 0 ? (float)w->accum : 1.f;
-  size_t q = 0;
-  for (int l = 0; l < NLAYER; l++) {
-    int co = LAYERS[l].co, ci = LAYERS[l].ci, ct = ci_true(l);
-    for (int t = 0; t < 27; t++)
-      for (int o = 0; o < co; o++)
-        for (int c = 0; c < ct; c++) dst[q++] = h[w->woff[l] + ((size_t)t * co + o) * ci + c] / div;
-    for (int o = 0; o < co; o++) dst[q++] = h[w->boff[l] + o] / div;
-  }
+  w->E.ensure(ne);
+  k_export<<<grid_for(ne, 256), 256, 0, w->st>>>((int)ne, which == 0 ? w->P.p : w->G.p,
+                                                which == 1 && w->accum > 0 ? (float)w->accum : 1.f, w->E.p);
+  RS_LAUNCHED(1);
+  RS_CUDA(cudaMemcpyAsync(dst, w->E.p, ne * sizeof(float), cudaMemcpyDefault, w->st));
+  RS_CUDA(cudaStreamSynchronize(w->st));
   ABI_END
 }
 

@@ -591,6 +591,7 @@ static int s_solve(sim_s *h, double eta, double bn, int *its, double *rel) {
     for (int i = 0; i < m; i++) { xs[q] = u[i]; ys[q] = ls->b.p; q++; }
     double dv[9];
     rs_dots(xs, ys, q, nu, dv, st);
+    ws_check(h->ws);                                   // (rs_dots has synchronised)
     double G[3][3] = {{0}}, r[3] = {0};
     q = 0;
     for (int i = 0; i < m; i++) for (int j = 0; j <= i; j++) { G[i][j] = G[j][i] = dv[q]; q++; }
