@@ -378,13 +378,23 @@ __device__ __forceinline__ uint64_t tc_desc(unsigned saddr, unsigned lbo, unsign
 __device__ __forceinline__ uint32_t tc_idesc(int n, bool mn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? 3u << 15 : 0u) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
-__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-               " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-               ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+// MMAs are issued by a whole warp with one elected lane's predicate on the
+// instruction only: the descriptors then stay in uniform registers, while in
+// a branch of one thread each MMA cost 80 to 170 cycles to issue.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e;
 }
-__device__ __forceinline__ void tc_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+__device__ __forceinline__ void tc_mma(uint32_t e, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+               " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+               ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(e) : "memory");
+}
+__device__ __forceinline__ void tc_commit(uint32_t e, uint64_t *bar) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+               " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n"
+               ::"r"(smem_u32(bar)), "r"(e) : "memory");
 }
 __device__ __forceinline__ void bar_init(uint64_t *bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
@@ -445,19 +455,43 @@ __host__ __device__ constexpr int tc_cols(int co, int nz) {                     
 
 // MODE as for k_conv: 0 forward (bias, ReLU flag), 1 head forward (FP32, 8 of
 // the 16 columns), 2 data gradient with mask, 3 data gradient.
+template <int CI, int CO, int NZ>
+__device__ __forceinline__ void tc_conv_issue(uint32_t taddr, unsigned sA, unsigned sW, uint64_t *bar) {
+  constexpr int KB = CI / 16, PL = tc_plane(CI, NZ);
+  const uint32_t idesc = tc_idesc(CO, false), e = elect_one();
+  uint64_t da = tc_desc(sA, PL, THX * 16), db = tc_desc(sW, 128, 256);
+  uint32_t acc = 0;
+#pragma unroll 1
+  for (int ryz = 0; ryz < 9; ryz++) {                  // (dy, dz)
+#pragma unroll
+    for (int dx = 0; dx < 3; dx++)
+#pragma unroll
+      for (int kb = 0; kb < KB; kb++) {
+#pragma unroll
+        for (int z = 0; z < NZ; z++) tc_mma(e, taddr + z * CO, da + dx + z * TSL + kb * (PL >> 3), db, idesc, acc);
+        acc = 1;
+        db += CO * 2;                                  // CO / 8 groups of 256 bytes
+      }
+    da += ryz % 3 == 2 ? TSL - 2 * THX : THX;
+  }
+  tc_commit(e, bar);
+}
+
 template <int CI, int CO, int MODE>
 __global__ void __launch_bounds__(256) k_conv_tc(int nx, int ny, int nz, int NZ, const bf16 *X, int ldx, int offx,
                                                  const bf16 *Wt, const float *bias, int relu, void *out, int ldo,
                                                  int offo, const bf16 *mask, int ldm, int offm, int *err) {
-  constexpr int CH = CI / 8, KB = CI / 16, W_BYTES = 27 * CI * CO * 2;
+  constexpr int CH = CI / 8, W_BYTES = 27 * CI * CO * 2;
   extern __shared__ __align__(128) unsigned char smtc[];
   __shared__ uint64_t wbar, mbar;
   __shared__ uint32_t tslot;
+  __shared__ float sbias[32];
   unsigned char *sA = smtc + W_BYTES;
   const int plane = tc_plane(CI, NZ), ncol = tc_cols(CO, NZ);
   const int tx = (nx + TBX - 1) / TBX, ty = (ny + TBY - 1) / TBY;
   const int X0 = (int)(blockIdx.x % tx) * TBX, Y0 = (int)(blockIdx.x / tx % ty) * TBY, Z0 = (int)(blockIdx.x / (tx * ty)) * NZ;
-  const int t = threadIdx.x, warp = t >> 5;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0);
+  if (MODE <= 1 && t < (MODE == 1 ? 8 : 32)) sbias[t] = bias[t];
   if (t == 0) {
     bar_init(&wbar);
     bar_init(&mbar);
@@ -478,41 +512,50 @@ __global__ void __launch_bounds__(256) k_conv_tc(int nx, int ny, int nz, int NZ,
                  ::"r"(smem_u32(smtc)), "l"(Wt), "n"(W_BYTES), "r"(smem_u32(&wbar)) : "memory");
   }
   pdl_wait();
-  const int nh = TSL * (NZ + 2) * CH;
-  for (int q = t; q < nh; q += 256) {
-    const int ch = q % CH, h = q / CH, hx = h % THX, r = h / THX, hy = r % THY, hz = r / THY;
-    const int x = X0 + hx - 1, y = Y0 + hy - 1, z = Z0 + hz - 1;
-    const bool in = x >= 0 && x < nx && y >= 0 && y < ny && z >= 0 && z < nz;
-    const bf16 *src = in ? X + ((size_t)x + (size_t)nx * (y + (size_t)ny * z)) * ldx + offx + ch * 8 : X;
-    cp_async16(sA + ch * plane + h * 16, src, in ? 16 : 0);
+  {
+    // thread: chunk ch of voxels h, h + DH, ... of the halo, coordinates carried along
+    constexpr int DH = 256 / CH, DX = DH % THX, DY = DH / THX;
+    const int ch = t % CH;
+    int h = t / CH, hx = h % THX, hy = h / THX, hz = 0;
+    if (hy >= THY) { hy -= THY; hz++; }
+    const bf16 *Xc = X + offx + ch * 8;
+    unsigned char *dst = sA + ch * plane;
+    for (; h < TSL * (NZ + 2); h += DH) {
+      const int x = X0 + hx - 1, y = Y0 + hy - 1, z = Z0 + hz - 1;
+      const bool in = x >= 0 && x < nx && y >= 0 && y < ny && z >= 0 && z < nz;
+      cp_async16(dst + h * 16, in ? Xc + ((size_t)x + (size_t)nx * (y + (size_t)ny * z)) * ldx : X, in ? 16 : 0);
+      hx += DX; hy += DY;
+      if (hx >= THX) { hx -= THX; hy++; }
+      if (hy >= THY) { hy -= THY; hz++; }
+    }
   }
   cp_commit();
   cp_wait<0>();
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   bool ok = __syncthreads_and(tc_wait(&wbar, 0));
-  if (t == 0 && ok) {
+  if (warp == 0 && ok) {
     tc_after();
-    const uint32_t idesc = tc_idesc(CO, false);
-    const uint64_t da0 = tc_desc(smem_u32(sA), plane, THX * 16);
-    uint64_t db = tc_desc(smem_u32(smtc), 128, 256);
-    uint32_t acc = 0;
-    for (int tap = 0; tap < 27; tap++) {
-      const uint64_t da = da0 + tap % 3 + THX * (tap / 3 % 3) + TSL * (tap / 9);
-#pragma unroll
-      for (int kb = 0; kb < KB; kb++) {
-        for (int z = 0; z < NZ; z++) tc_mma(taddr + z * CO, da + z * TSL + kb * (plane >> 3), db, idesc, acc);
-        acc = 1;
-        db += CO * 2;                                  // CO / 8 groups of 256 bytes
-      }
-    }
-    tc_commit(&mbar);
+    const unsigned a = smem_u32(sA), b = smem_u32(smtc);
+    if (NZ == 4) tc_conv_issue<CI, CO, 4>(taddr, a, b, &mbar);
+    else if (NZ == 3) tc_conv_issue<CI, CO, 3>(taddr, a, b, &mbar);
+    else if (NZ == 2) tc_conv_issue<CI, CO, 2>(taddr, a, b, &mbar);
+    else tc_conv_issue<CI, CO, 1>(taddr, a, b, &mbar);
   }
+  const int r = (warp & 3) * 32 + (t & 31), x = X0 + r % TBX, y = Y0 + r / TBX, nzv = min(NZ, nz - Z0);
+  const bool live = x < nx && y < ny;
+  [[maybe_unused]] uint4 mk[CO / 8];                   // the mask of this thread's next voxel, ahead of the MMAs
+  auto load_mask = [&](int z) {
+    if (MODE == 2 && live && z < nzv) {
+      const uint4 *p = reinterpret_cast<const uint4 *>(mask + ((size_t)x + (size_t)nx * (y + (size_t)ny * (Z0 + z))) * ldm + offm);
+#pragma unroll
+      for (int u = 0; u < CO / 8; u++) mk[u] = p[u];
+    }
+  };
+  load_mask(warp >> 2);
   if (ok) ok = tc_wait(&mbar, 0);
   ok = __syncthreads_and(ok);
   tc_after();
   if (ok) {
-    const int r = (warp & 3) * 32 + (t & 31), x = X0 + r % TBX, y = Y0 + r / TBX, nzv = min(NZ, nz - Z0);
-    const bool live = x < nx && y < ny;
     for (int z = warp >> 2; z < nzv; z += 2) {
       const size_t v = (size_t)x + (size_t)nx * (y + (size_t)ny * (Z0 + z));
       const uint32_t ta = taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(z * CO);
@@ -522,7 +565,7 @@ __global__ void __launch_bounds__(256) k_conv_tc(int nx, int ny, int nz, int NZ,
         if (live) {
           float *op = reinterpret_cast<float *>(out) + v * ldo + offo;
 #pragma unroll
-          for (int c = 0; c < 8; c++) acc[c] += bias[c];
+          for (int c = 0; c < 8; c++) acc[c] += sbias[c];
           reinterpret_cast<float4 *>(op)[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
           reinterpret_cast<float4 *>(op)[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
         }
@@ -534,13 +577,11 @@ __global__ void __launch_bounds__(256) k_conv_tc(int nx, int ny, int nz, int NZ,
           if (live) {
             if (MODE == 0) {
 #pragma unroll
-              for (int c = 0; c < 32; c++) { acc[c] += bias[c0 + c]; if (relu) acc[c] = fmaxf(acc[c], 0.f); }
+              for (int c = 0; c < 32; c++) { acc[c] += sbias[c0 + c]; if (relu) acc[c] = fmaxf(acc[c], 0.f); }
             } else if (MODE == 2) {
-              const uint4 *mk = reinterpret_cast<const uint4 *>(mask + v * ldm + offm + c0);
 #pragma unroll
               for (int u = 0; u < 4; u++) {
-                const uint4 m4 = mk[u];
-                const bf16 *m = reinterpret_cast<const bf16 *>(&m4);
+                const bf16 *m = reinterpret_cast<const bf16 *>(&mk[c0 / 8 + u]);
 #pragma unroll
                 for (int c = 0; c < 8; c++) if (!(__bfloat162float(m[c]) > 0.f)) acc[8 * u + c] = 0.f;
               }
@@ -554,6 +595,7 @@ __global__ void __launch_bounds__(256) k_conv_tc(int nx, int ny, int nz, int NZ,
             for (int u = 0; u < 4; u++) dst[u] = pk[u];
           }
         }
+        load_mask(z + 2);
       }
     }
   }
@@ -587,12 +629,12 @@ struct wg_layer {
 };
 struct wg_table { wg_layer l[NLAYER]; };
 
-__global__ void __launch_bounds__(256) k_conv_wgrad(const __grid_constant__ wg_table tab, int *err) {
+constexpr int WG_T = 288;                                        // 8 warps copy and sum, the ninth issues the MMAs
+__global__ void __launch_bounds__(WG_T, 2) k_conv_wgrad(const __grid_constant__ wg_table tab, int *err) {
   extern __shared__ __align__(128) unsigned char smtc[];
   __shared__ uint64_t bar[WNS];
   __shared__ uint32_t tslot;
-  __shared__ float bred[256];
-  const int t = threadIdx.x, warp = t >> 5;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0);
   int li = 0;
   while (li + 1 < NLAYER && (int)blockIdx.x >= tab.l[li + 1].block0) li++;
   const wg_layer &L = tab.l[li];
@@ -619,71 +661,104 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(const __grid_constant__ wg_t
   const bf16 *X = L.X + L.offx + half * 32, *dZ = L.dZ;
   const int ldx = L.ldx, ldz = L.ldz;
   bool ok = true;
+  // the chunks this thread copies of every slice: halo column and offset in
+  // shared memory (X: up to three, dZ: up to two)
+  int xh[3], yh[3], xo[3], xz[2], yz[2], zo[2];
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const int q = t + 256 * k, ch = q & (chn - 1), h = q >> lch;
+    xh[k] = h % THX - 1; yh[k] = h / THX - 1;
+    xo[k] = t < 256 && h < TSL ? ((((xh[k] + 1) << lch) + ch) * WYP + yh[k] + 1) * 16 : -1;
+  }
+  const int xch = (t & (chn - 1)) * 8, zch = (t & ((1 << lno) - 1)) * 8;
+#pragma unroll
+  for (int k = 0; k < 2; k++) {
+    const int q = t + 256 * k, ch = q & ((1 << lno) - 1), h = q >> lno;
+    xz[k] = h % TBX; yz[k] = h / TBX;
+    zo[k] = t < 256 && h < TBX * TBY ? WA_BYTES + (((xz[k] << lno) + ch) * WYB + yz[k]) * 16 : -1;
+  }
+  int lz = zlo + (int)(s0 / (tx * ty)), lr = (int)(s0 % (tx * ty)), lx = lr % tx * TBX, ly = lr / tx * TBY;   // next slice to copy
   auto load = [&](int u) {
     const int stage = u % WNS;
     if (u >= WNS) ok = ok && tc_wait(&bar[stage], (unsigned)((u / WNS - 1) & 1));
-    const long long s = s0 + u;
-    const int z = zlo + (int)(s / (tx * ty)), rr = (int)(s % (tx * ty)), X0 = rr % tx * TBX, Y0 = rr / tx * TBY;
-    unsigned char *a = smtc + stage * WSTAGE, *b = a + WA_BYTES;
-    const size_t zx = (size_t)ny * (z + dz - 1), zz = (size_t)ny * z;
-    for (int q = t; q < TSL << lch; q += 256) {
-      const int ch = q & (chn - 1), h = q >> lch, hx = h % THX, hy = h / THX, x = X0 + hx - 1, y = Y0 + hy - 1;
-      const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
-      cp_async16(a + (((hx << lch) + ch) * WYP + hy) * 16, in ? X + (x + nx * (y + zx)) * ldx + ch * 8 : X, in ? 16 : 0);
-    }
-    for (int q = t; q < (TBX * TBY) << lno; q += 256) {
-      const int ch = q & ((1 << lno) - 1), h = q >> lno, hx = h % TBX, hy = h / TBX, x = X0 + hx, y = Y0 + hy;
-      const bool in = x < nx && y < ny;
-      cp_async16(b + (((hx << lno) + ch) * WYB + hy) * 16, in ? dZ + (x + nx * (y + zz)) * ldz + ch * 8 : dZ, in ? 16 : 0);
-    }
+    unsigned char *a = smtc + stage * WSTAGE;
+    const size_t zx = (size_t)ny * (lz + dz - 1), zz = (size_t)ny * lz;
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+      if (xo[k] >= 0) {
+        const int x = lx + xh[k], y = ly + yh[k];
+        const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
+        cp_async16(a + xo[k], in ? X + (x + nx * (y + zx)) * ldx + xch : X, in ? 16 : 0);
+      }
+#pragma unroll
+    for (int k = 0; k < 2; k++)
+      if (zo[k] >= 0) {
+        const int x = lx + xz[k], y = ly + yz[k];
+        const bool in = x < nx && y < ny;
+        cp_async16(a + zo[k], in ? dZ + (x + nx * (y + zz)) * ldz + zch : dZ, in ? 16 : 0);
+      }
+    lx += TBX;
+    if (lx >= nx) { lx = 0; ly += TBY; if (ly >= ny) { ly = 0; lz++; } }
   };
-  float sum[3][16], bsum = 0.f;
+  float sum[3][16], bsum[8];
 #pragma unroll
   for (int d = 0; d < 3; d++)
 #pragma unroll
     for (int j = 0; j < 16; j++) sum[d][j] = 0.f;
-  // bias: thread = output channel and part of the slice's voxels
-  const bool bias = dz == 1 && half == 0;
-  const int bo = t & (no - 1), bx = (t >> (lno + 3)) % TBX, by0 = lno == 1 ? (t >> 7) * 8 : 0, by1 = lno == 1 ? by0 + 8 : TBY;
+#pragma unroll
+  for (int j = 0; j < 8; j++) bsum[j] = 0.f;
+  const bool bias = dz == 1 && half == 0;              // bias: thread = chunk (t >> 4) % (no / 8) of dZ, voxels by y
+  const uint32_t e = elect_one();
 #pragma unroll 1
-  for (int u = 0; u < WLA; u++) { if (u < n) load(u); cp_commit(); }
+  for (int u = 0; u < WLA; u++) { if (warp < 8 && u < n) load(u); cp_commit(); }
+#pragma unroll 1
   for (int i = 0; i < n; i++) {
-    if (i + WLA < n) load(i + WLA);
+    if (warp < 8 && i + WLA < n) load(i + WLA);
     cp_commit();
     cp_wait<WLA>();
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     ok = __syncthreads_and(ok);
     if (!ok) break;
     const unsigned char *a = smtc + i % WNS * WSTAGE, *b = a + WA_BYTES;
-    if (t == 0) {
+    if (warp == 8) {
       tc_after();
       const uint64_t da = tc_desc(smem_u32(a), 128, WYP * 16), db = tc_desc(smem_u32(b), 128, WYB * 16);
+      const int ax = WYP << lch, bx = WYB << lno;
 #pragma unroll
       for (int x = 0; x < TBX; x++)
 #pragma unroll
         for (int dy = 0; dy < 3; dy++)
-          tc_mma(taddr + dy * 32, da + (x << lch) * WYP + dy, db + (x << lno) * WYB, idesc, i % WFL > 0 || x > 0);
-      tc_commit(&bar[i % WNS]);
-    }
-    if (bias) {
-      const bf16 *zr = reinterpret_cast<const bf16 *>(b) + ((bx << lno) + (bo >> 3)) * WYB * 8 + (bo & 7);
-      for (int y = by0; y < by1; y++) bsum += __bfloat162float(zr[y * 8]);
+          tc_mma(e, taddr + dy * 32, da + x * ax + dy, db + x * bx, idesc, x > 0 || i % WFL > 0);
+      tc_commit(e, &bar[i % WNS]);
+    } else if (bias) {
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        const int u = t + 256 * k;
+        if (u >> 4 < TBX << lno) {
+          const uint4 v = *reinterpret_cast<const uint4 *>(b + ((u >> 4) * WYB + (u & 15)) * 16);
+          const bf16 *p = reinterpret_cast<const bf16 *>(&v);
+#pragma unroll
+          for (int j = 0; j < 8; j++) bsum[j] += __bfloat162float(p[j]);
+        }
+      }
     }
     if (i % WFL == WFL - 1 || i == n - 1) {
       ok = __syncthreads_and(tc_wait(&bar[i % WNS], (unsigned)((i / WNS) & 1)));
       if (!ok) break;
       tc_after();
+      if (warp < 8) {
 #pragma unroll
-      for (int d = 0; d < 3; d++) {
-        const uint32_t ta = taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(d * 32 + (warp >> 2) * (no / 2));
-        float v[8];
-        tc_ld8(ta, v);
+        for (int d = 0; d < 3; d++) {
+          const uint32_t ta = taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(d * 32 + (warp >> 2) * (no / 2));
+          float v[8];
+          tc_ld8(ta, v);
 #pragma unroll
-        for (int j = 0; j < 8; j++) sum[d][j] += v[j];
-        if (lno == 2) {
-          tc_ld8(ta + 8, v);
+          for (int j = 0; j < 8; j++) sum[d][j] += v[j];
+          if (lno == 2) {
+            tc_ld8(ta + 8, v);
 #pragma unroll
-          for (int j = 0; j < 8; j++) sum[d][8 + j] += v[j];
+            for (int j = 0; j < 8; j++) sum[d][8 + j] += v[j];
+          }
         }
       }
       tc_before();
@@ -692,7 +767,7 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(const __grid_constant__ wg_t
   }
   if (ok) {
     const int m = (warp & 3) * 32 + (t & 31), dx = m >> (lch + 3), c = half * 32 + (m & (8 * chn - 1));
-    if (dx < 3)
+    if (warp < 8 && dx < 3)
 #pragma unroll
       for (int d = 0; d < 3; d++) {
         float *dst = L.part + ((size_t)(dx + 3 * d + 9 * dz) * nchunk + chunk) * co * ci + c;
@@ -702,12 +777,17 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(const __grid_constant__ wg_t
           if (j < no / 2 && o < co) dst[(size_t)o * ci] = sum[d][j];
         }
       }
-    if (bias) {
-      bred[t] = bsum;
+    if (bias) {                                        // (the last slice's MMAs are done: the stages are free)
+      float *bred = reinterpret_cast<float *>(smtc);
+      __syncthreads();
+      if (warp < 8)
+#pragma unroll
+        for (int j = 0; j < 8; j++) bred[t * 8 + j] = bsum[j];
       __syncthreads();
       if (t < co) {
         float s = 0.f;
-        for (int k = t; k < 256; k += no) s += bred[k];
+        for (int k = 0; k < 256; k++)
+          if (((k >> 4) & ((1 << lno) - 1)) == t >> 3) s += bred[k * 8 + (t & 7)];
         L.bpart[(size_t)chunk * co + t] = s;
       }
     }
@@ -1167,7 +1247,7 @@ static void wgrad(sim_ws_s *w, const wg_in in[NLAYER], int nl, double lscale) {
     L.part = p; p += (size_t)L.nchunk * 27 * L.co * L.ci;
     L.bpart = p; p += (size_t)L.nchunk * L.co;
   }
-  launch_pdl(k_conv_wgrad, (unsigned)block, 256, (size_t)WNS * WSTAGE, w->st, tab, w->err_dev);
+  launch_pdl(k_conv_wgrad, (unsigned)block, WG_T, (size_t)WNS * WSTAGE, w->st, tab, w->err_dev);
   launch_pdl(k_wgrad_reduce, grid_for(w->np, 256) + 1, 256, 0, w->st, tab, (int)w->np, w->G.p, nl, w->lpart.p, lscale,
              w->lsum.p);
   RS_LAUNCHED(2);
