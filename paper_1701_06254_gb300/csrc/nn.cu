@@ -396,8 +396,11 @@ __device__ __forceinline__ void tc_commit(uint32_t e, uint64_t *bar) {
                " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n"
                ::"r"(smem_u32(bar)), "r"(e) : "memory");
 }
-__device__ __forceinline__ void bar_init(uint64_t *bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+__device__ __forceinline__ void bar_init(uint64_t *bar, int count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 // whole warp: allocate ncol TMEM columns (a power of two, at least 32)
 __device__ __forceinline__ void tc_alloc(uint32_t *slot, int ncol) {
@@ -441,6 +444,16 @@ __device__ __forceinline__ void tc_ld8(uint32_t taddr, float *v) {
 #pragma unroll
   for (int c = 0; c < 8; c++) v[c] = __uint_as_float(r[c]);
 }
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, float *v) {
+  uint32_t r[16];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int c = 0; c < 16; c++) v[c] = __uint_as_float(r[c]);
+}
 
 constexpr int TBX = 8, TBY = 16, THX = TBX + 2, THY = TBY + 2, TSL = THX * THY;   // box, halo, halo voxels per slice
 __host__ __device__ constexpr int tc_plane(int ci, int nz) {                      // bytes of an 8-channel plane
@@ -455,35 +468,14 @@ __host__ __device__ constexpr int tc_cols(int co, int nz) {                     
 
 // MODE as for k_conv: 0 forward (bias, ReLU flag), 1 head forward (FP32, 8 of
 // the 16 columns), 2 data gradient with mask, 3 data gradient.
-template <int CI, int CO, int NZ>
-__device__ __forceinline__ void tc_conv_issue(uint32_t taddr, unsigned sA, unsigned sW, uint64_t *bar) {
-  constexpr int KB = CI / 16, PL = tc_plane(CI, NZ);
-  const uint32_t idesc = tc_idesc(CO, false), e = elect_one();
-  uint64_t da = tc_desc(sA, PL, THX * 16), db = tc_desc(sW, 128, 256);
-  uint32_t acc = 0;
-#pragma unroll 1
-  for (int ryz = 0; ryz < 9; ryz++) {                  // (dy, dz)
-#pragma unroll
-    for (int dx = 0; dx < 3; dx++)
-#pragma unroll
-      for (int kb = 0; kb < KB; kb++) {
-#pragma unroll
-        for (int z = 0; z < NZ; z++) tc_mma(e, taddr + z * CO, da + dx + z * TSL + kb * (PL >> 3), db, idesc, acc);
-        acc = 1;
-        db += CO * 2;                                  // CO / 8 groups of 256 bytes
-      }
-    da += ryz % 3 == 2 ? TSL - 2 * THX : THX;
-  }
-  tc_commit(e, bar);
-}
-
+constexpr int TC_T = 288;                              // 8 warps copy and store, the ninth issues the MMAs
 template <int CI, int CO, int MODE>
-__global__ void __launch_bounds__(256) k_conv_tc(int nx, int ny, int nz, int NZ, const bf16 *X, int ldx, int offx,
+__global__ void __launch_bounds__(TC_T) k_conv_tc(int nx, int ny, int nz, int NZ, const bf16 *X, int ldx, int offx,
                                                  const bf16 *Wt, const float *bias, int relu, void *out, int ldo,
                                                  int offo, const bf16 *mask, int ldm, int offm, int *err) {
   constexpr int CH = CI / 8, W_BYTES = 27 * CI * CO * 2;
   extern __shared__ __align__(128) unsigned char smtc[];
-  __shared__ uint64_t wbar, mbar;
+  __shared__ uint64_t wbar, full[4], done[4];           // weights; halo of slice z complete; its MMAs complete
   __shared__ uint32_t tslot;
   __shared__ float sbias[32];
   unsigned char *sA = smtc + W_BYTES;
@@ -493,8 +485,8 @@ __global__ void __launch_bounds__(256) k_conv_tc(int nx, int ny, int nz, int NZ,
   const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0);
   if (MODE <= 1 && t < (MODE == 1 ? 8 : 32)) sbias[t] = bias[t];
   if (t == 0) {
-    bar_init(&wbar);
-    bar_init(&mbar);
+    bar_init(&wbar, 1);
+    for (int z = 0; z < 4; z++) { bar_init(&full[z], 256); bar_init(&done[z], 1); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -511,52 +503,77 @@ __global__ void __launch_bounds__(256) k_conv_tc(int nx, int ny, int nz, int NZ,
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_u32(smtc)), "l"(Wt), "n"(W_BYTES), "r"(smem_u32(&wbar)) : "memory");
   }
-  pdl_wait();
-  {
-    // thread: chunk ch of voxels h, h + DH, ... of the halo, coordinates carried along
+  const int nzv = min(NZ, nz - Z0);
+  bool ok = true;
+  if (warp == 8) {
+    ok = tc_wait(&wbar, 0);
+    const uint32_t idesc = tc_idesc(CO, false), e = elect_one();
+    const uint64_t da0 = tc_desc(smem_u32(sA), plane, THX * 16), db0 = tc_desc(smem_u32(smtc), 128, 256);
+    const int kstep = plane >> 3;                      // two planes, in 16-byte units
+    for (int z = 0; z < nzv && ok; z++) {
+      ok = tc_wait(&full[z], 0);
+      if (!ok) break;
+      tc_after();
+      uint64_t da = da0 + z * TSL, db = db0;
+      uint32_t acc = 0;
+#pragma unroll 1
+      for (int ryz = 0; ryz < 9; ryz++) {              // (dy, dz)
+#pragma unroll
+        for (int dx = 0; dx < 3; dx++)
+#pragma unroll
+          for (int kb = 0; kb < CI / 16; kb++) {
+            tc_mma(e, taddr + z * CO, da + dx + kb * kstep, db, idesc, acc);
+            acc = 1;
+            db += CO * 2;                              // CO / 8 groups of 256 bytes
+          }
+        da += ryz % 3 == 2 ? TSL - 2 * THX : THX;
+      }
+      tc_commit(e, &done[z]);
+    }
+  } else {
+    pdl_wait();
+    // thread: chunk ch of voxels h, h + DH, ... of the halo, coordinates
+    // carried along; slice z's MMAs can start when z + 3 halo slices are there
     constexpr int DH = 256 / CH, DX = DH % THX, DY = DH / THX;
     const int ch = t % CH;
     int h = t / CH, hx = h % THX, hy = h / THX, hz = 0;
-    if (hy >= THY) { hy -= THY; hz++; }
     const bf16 *Xc = X + offx + ch * 8;
     unsigned char *dst = sA + ch * plane;
-    for (; h < TSL * (NZ + 2); h += DH) {
-      const int x = X0 + hx - 1, y = Y0 + hy - 1, z = Z0 + hz - 1;
-      const bool in = x >= 0 && x < nx && y >= 0 && y < ny && z >= 0 && z < nz;
-      cp_async16(dst + h * 16, in ? Xc + ((size_t)x + (size_t)nx * (y + (size_t)ny * z)) * ldx : X, in ? 16 : 0);
-      hx += DX; hy += DY;
-      if (hx >= THX) { hx -= THX; hy++; }
-      if (hy >= THY) { hy -= THY; hz++; }
+    for (int g = 0; g < nzv; g++) {
+      for (; h < TSL * (3 + g); h += DH) {
+        const int x = X0 + hx - 1, y = Y0 + hy - 1, z = Z0 + hz - 1;
+        const bool in = x >= 0 && x < nx && y >= 0 && y < ny && z >= 0 && z < nz;
+        cp_async16(dst + h * 16, in ? Xc + ((size_t)x + (size_t)nx * (y + (size_t)ny * z)) * ldx : X, in ? 16 : 0);
+        hx += DX; hy += DY;
+        if (hx >= THX) { hx -= THX; hy++; }
+        if (hy >= THY) { hy -= THY; hz++; }
+      }
+      cp_commit();
     }
-  }
-  cp_commit();
-  cp_wait<0>();
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  bool ok = __syncthreads_and(tc_wait(&wbar, 0));
-  if (warp == 0 && ok) {
-    tc_after();
-    const unsigned a = smem_u32(sA), b = smem_u32(smtc);
-    if (NZ == 4) tc_conv_issue<CI, CO, 4>(taddr, a, b, &mbar);
-    else if (NZ == 3) tc_conv_issue<CI, CO, 3>(taddr, a, b, &mbar);
-    else if (NZ == 2) tc_conv_issue<CI, CO, 2>(taddr, a, b, &mbar);
-    else tc_conv_issue<CI, CO, 1>(taddr, a, b, &mbar);
-  }
-  const int r = (warp & 3) * 32 + (t & 31), x = X0 + r % TBX, y = Y0 + r / TBX, nzv = min(NZ, nz - Z0);
-  const bool live = x < nx && y < ny;
-  [[maybe_unused]] uint4 mk[CO / 8];                   // the mask of this thread's next voxel, ahead of the MMAs
-  auto load_mask = [&](int z) {
-    if (MODE == 2 && live && z < nzv) {
-      const uint4 *p = reinterpret_cast<const uint4 *>(mask + ((size_t)x + (size_t)nx * (y + (size_t)ny * (Z0 + z))) * ldm + offm);
+    const int r = (warp & 3) * 32 + (t & 31), x = X0 + r % TBX, y = Y0 + r / TBX;
+    const bool live = x < nx && y < ny;
+    [[maybe_unused]] uint4 mk[CO / 8];                 // the mask of this thread's next voxel, ahead of the MMAs
+    auto load_mask = [&](int z) {
+      if (MODE == 2 && live && z < nzv) {
+        const uint4 *p = reinterpret_cast<const uint4 *>(mask + ((size_t)x + (size_t)nx * (y + (size_t)ny * (Z0 + z))) * ldm + offm);
 #pragma unroll
-      for (int u = 0; u < CO / 8; u++) mk[u] = p[u];
+        for (int u = 0; u < CO / 8; u++) mk[u] = p[u];
+      }
+    };
+    load_mask(warp >> 2);
+    for (int g = 0; g < nzv; g++) {
+      const int pending = nzv - 1 - g;
+      if (pending == 3) cp_wait<3>();
+      else if (pending == 2) cp_wait<2>();
+      else if (pending == 1) cp_wait<1>();
+      else cp_wait<0>();
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      bar_arrive(&full[g]);
     }
-  };
-  load_mask(warp >> 2);
-  if (ok) ok = tc_wait(&mbar, 0);
-  ok = __syncthreads_and(ok);
-  tc_after();
-  if (ok) {
     for (int z = warp >> 2; z < nzv; z += 2) {
+      ok = tc_wait(&done[z], 0);
+      if (!ok) break;
+      tc_after();
       const size_t v = (size_t)x + (size_t)nx * (y + (size_t)ny * (Z0 + z));
       const uint32_t ta = taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(z * CO);
       if constexpr (MODE == 1) {
@@ -599,38 +616,58 @@ __global__ void __launch_bounds__(256) k_conv_tc(int nx, int ny, int nz, int NZ,
       }
     }
   }
-  if (!ok && t == 0) *(volatile int *)err = 1;
+  if (!ok) *(volatile int *)err = 1;
   tc_before();
   __syncthreads();
   if (warp == 0) tc_free(taddr, ncol);
 }
 
 // ------------------------------------------------------ weight gradient ---
-// part[tap][chunk][o][c] = sum over the chunk's voxels v of dZ[v, o] X[v + d(tap), c],
-// and for dz = 0 bpart[chunk][o] = sum_v dZ[v, o], of all layers in one launch.
+// part[tap][chunk][o][c] = sum over the chunk's voxels u of dZ[u - d(tap), o] X[u, c],
+// and bpart[chunk][o] = sum_u dZ[u, o], of all layers in one launch.
 //
 // On tcgen05 with the voxels as K: M = 128 rows are four x shifts of 32 input
-// channels (three used), N the output channels, one accumulator per dy.  A
-// CTA owns a range of slices (8 x 16 voxels of one z), one dz and 32 of the
-// input channels.  Both operands are MN-major core matrices (8 channels of
-// 16 bytes, 8 voxels consecutive in y): X lies as [x][chunk][y], so that the
-// channel groups of x - 1, x, x + 1 follow each other at one stride, and dy is
-// a shift of the start by 16 bytes; dZ as [x][chunk][y].  One MMA contracts
-// the 16 voxels of an x column.  Four stages of a slice each; after WFL
-// slices (64 MMAs on an accumulator) the sums move to FP32 registers, so that
-// the tensor cores' accumulation chains stay short.
+// channels (three used), N three z shifts of the output channels, one
+// accumulator per dy; so an MMA reads 7 KB of shared memory (which bounds it:
+// 56 cycles) for three taps in z, where one per dz would read 15.  A CTA owns
+// a range of X slices (8 x 16 voxels of one z, z fastest) and 32 of the input
+// channels.  Both operands are MN-major core matrices (8 channels of 16
+// bytes, 8 voxels consecutive in y).  X lies as [x][chunk][y] with a halo of
+// one, so that the channel groups of x - 1, x, x + 1 follow each other at one
+// stride and dy is a shift of the start by 16 bytes.  dZ lies as
+// [x][slot][chunk][y] in a ring of six z slices, the first two slots held
+// twice, so that three consecutive slices are always adjacent.  One MMA
+// contracts the 16 voxels of an x column.
+//
+// Step i brings dZ slice z and X slice z - 1 and then contracts the latter
+// with dZ slices z - 2, z - 1, z (zero outside the grid); two steps at the
+// start of a column only load.  Eight warps copy two steps ahead, the ninth
+// issues the MMAs; after WFL slices (64 MMAs on an accumulator) all twelve
+// move the sums to FP32 registers, one z shift per four warps, so that the
+// tensor cores' accumulation chains stay short.
 constexpr int WYP = THY + 1, WYB = TBY + 1;                      // y pitches, odd: copies free of bank conflicts
-constexpr int WA_BYTES = 11 * 4 * WYP * 16 + 64, WB_BYTES = TBX * 4 * WYB * 16;
-constexpr int WSTAGE = WA_BYTES + WB_BYTES, WNS = 4, WLA = 2, WFL = 8;
+constexpr int WR = 6, WSLOT = WR + 2;                            // dZ ring: slots, with the two copies
+constexpr int WA_BYTES = 11 * 4 * WYP * 16 + 64, WNS = 4, WLA = 2, WFL = 8;
+constexpr int WB_OFF = WNS * WA_BYTES, WG_BYTES = WB_OFF + TBX * (WSLOT * 4 * WYB + 4) * 16;
 struct wg_layer {
   const bf16 *X, *dZ;
   float *part, *bpart;
   int ldx, offx, ldz, nx, ny, nz, co, ci, nchunk, block0;
 };
 struct wg_table { wg_layer l[NLAYER]; };
+// the steps of X slices s, s + 1, ... (col nz + z): zz runs from za - 1 to zb in each column
+struct wg_steps {
+  int col, za, zb, zz, left;
+  __device__ void start(long long s, int n, int nz) {
+    col = (int)(s / nz); za = (int)(s % nz); zb = min(nz, za + n); zz = za - 1; left = n - (zb - za);
+  }
+  __device__ void next(int nz) {
+    if (++zz > zb && left > 0) { col++; za = 0; zb = min(nz, left); left -= zb; zz = -1; }
+  }
+};
 
-constexpr int WG_T = 288;                                        // 8 warps copy and sum, the ninth issues the MMAs
-__global__ void __launch_bounds__(WG_T, 2) k_conv_wgrad(const __grid_constant__ wg_table tab, int *err) {
+constexpr int WG_T = 384;
+__global__ void __launch_bounds__(WG_T, 1) k_conv_wgrad(const __grid_constant__ wg_table tab, int *err) {
   extern __shared__ __align__(128) unsigned char smtc[];
   __shared__ uint64_t bar[WNS];
   __shared__ uint32_t tslot;
@@ -639,30 +676,30 @@ __global__ void __launch_bounds__(WG_T, 2) k_conv_wgrad(const __grid_constant__ 
   while (li + 1 < NLAYER && (int)blockIdx.x >= tab.l[li + 1].block0) li++;
   const wg_layer &L = tab.l[li];
   const int nx = L.nx, ny = L.ny, nz = L.nz, co = L.co, ci = L.ci, nchunk = L.nchunk, lb = (int)blockIdx.x - L.block0;
-  const int chunk = lb % nchunk, dz = lb / nchunk % 3, half = lb / (3 * nchunk);
+  const int chunk = lb % nchunk, half = lb / nchunk;
   const int lch = ci == 16 ? 1 : 2, chn = 1 << lch;              // 16-byte chunks of input channels
-  const int lno = co <= 16 ? 1 : 2, no = 8 << lno;               // N and its chunks
+  const int lno = co <= 16 ? 1 : 2, no = 8 << lno;               // output channels (padded) and their chunks
+  const int xsb = (WSLOT << lno) * WYB + 4;                      // x stride of dZ (16-byte units)
   if (t == 0) {
-    for (int k = 0; k < WNS; k++) bar_init(&bar[k]);
+    for (int k = 0; k < WNS; k++) bar_init(&bar[k], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) tc_alloc(&tslot, 128);
+  if (warp == 0) tc_alloc(&tslot, 512);
   tc_before();
   __syncthreads();
   tc_after();
   pdl_trigger();
   pdl_wait();
-  const uint32_t taddr = tslot, idesc = tc_idesc(no, true);
+  const uint32_t taddr = tslot, idesc = tc_idesc(3 * no, true);
   const int tx = (nx + TBX - 1) / TBX, ty = (ny + TBY - 1) / TBY;
-  const int zlo = dz == 0 ? 1 : 0, nzv = max(0, (dz == 2 ? nz - 1 : nz) - zlo);   // slices whose z + dz - 1 exists
-  const long long S = (long long)tx * ty * nzv;
-  const long long s0 = S * chunk / nchunk;
-  const int n = (int)(S * (chunk + 1) / nchunk - s0);
+  const long long S = (long long)tx * ty * nz, s0 = S * chunk / nchunk, s1 = S * (chunk + 1) / nchunk;
+  const int n = (int)(s1 - s0);                                  // at least 1: nchunk <= S
+  const int nstep = n + 2 * (int)((s1 - 1) / nz - s0 / nz + 1);
   const bf16 *X = L.X + L.offx + half * 32, *dZ = L.dZ;
   const int ldx = L.ldx, ldz = L.ldz;
   bool ok = true;
-  // the chunks this thread copies of every slice: halo column and offset in
-  // shared memory (X: up to three, dZ: up to two)
+  // the chunks this thread copies of every slice: voxel in the box and offset
+  // in shared memory (X: up to three, dZ: up to two)
   int xh[3], yh[3], xo[3], xz[2], yz[2], zo[2];
 #pragma unroll
   for (int k = 0; k < 3; k++) {
@@ -675,109 +712,121 @@ __global__ void __launch_bounds__(WG_T, 2) k_conv_wgrad(const __grid_constant__ 
   for (int k = 0; k < 2; k++) {
     const int q = t + 256 * k, ch = q & ((1 << lno) - 1), h = q >> lno;
     xz[k] = h % TBX; yz[k] = h / TBX;
-    zo[k] = t < 256 && h < TBX * TBY ? WA_BYTES + (((xz[k] << lno) + ch) * WYB + yz[k]) * 16 : -1;
+    zo[k] = t < 256 && h < TBX * TBY ? WB_OFF + (xz[k] * xsb + ch * WYB + yz[k]) * 16 : -1;
   }
-  int lz = zlo + (int)(s0 / (tx * ty)), lr = (int)(s0 % (tx * ty)), lx = lr % tx * TBX, ly = lr / tx * TBY;   // next slice to copy
+  wg_steps ls, ms;                                               // the copies' and the MMAs' steps
+  ls.start(s0, n, nz);
+  ms = ls;
+  int lx = ls.col % tx * TBX, ly = ls.col / tx * TBY;
   auto load = [&](int u) {
-    const int stage = u % WNS;
-    if (u >= WNS) ok = ok && tc_wait(&bar[stage], (unsigned)((u / WNS - 1) & 1));
-    unsigned char *a = smtc + stage * WSTAGE;
-    const size_t zx = (size_t)ny * (lz + dz - 1), zz = (size_t)ny * lz;
-#pragma unroll
-    for (int k = 0; k < 3; k++)
-      if (xo[k] >= 0) {
-        const int x = lx + xh[k], y = ly + yh[k];
-        const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
-        cp_async16(a + xo[k], in ? X + (x + nx * (y + zx)) * ldx + xch : X, in ? 16 : 0);
-      }
+    // the slot and the stage were last read by the MMAs of step u - 4
+    if (u >= WNS) ok = ok && tc_wait(&bar[u % WNS], (unsigned)((u / WNS - 1) & 1));
+    const int slot = u % WR;
+    const bool zin = ls.zz >= 0 && ls.zz < nz;
+    const size_t zz = (size_t)ny * ls.zz, zx = (size_t)ny * (ls.zz - 1);
 #pragma unroll
     for (int k = 0; k < 2; k++)
       if (zo[k] >= 0) {
         const int x = lx + xz[k], y = ly + yz[k];
-        const bool in = x < nx && y < ny;
-        cp_async16(a + zo[k], in ? dZ + (x + nx * (y + zz)) * ldz + zch : dZ, in ? 16 : 0);
+        const bool in = zin && x < nx && y < ny;
+        const bf16 *src = in ? dZ + (x + nx * (y + zz)) * ldz + zch : dZ;
+        unsigned char *d = smtc + zo[k] + (slot << lno) * WYB * 16;
+        cp_async16(d, src, in ? 16 : 0);
+        if (slot < 2) cp_async16(d + (WR << lno) * WYB * 16, src, in ? 16 : 0);
       }
-    lx += TBX;
-    if (lx >= nx) { lx = 0; ly += TBY; if (ly >= ny) { ly = 0; lz++; } }
+    if (ls.zz - 1 >= ls.za) {
+      unsigned char *a = smtc + u % WNS * WA_BYTES;
+#pragma unroll
+      for (int k = 0; k < 3; k++)
+        if (xo[k] >= 0) {
+          const int x = lx + xh[k], y = ly + yh[k];
+          const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
+          cp_async16(a + xo[k], in ? X + (x + nx * (y + zx)) * ldx + xch : X, in ? 16 : 0);
+        }
+    }
+    const int col = ls.col;
+    ls.next(nz);
+    if (ls.col != col) { lx += TBX; if (lx >= nx) { lx = 0; ly += TBY; } }
   };
-  float sum[3][16], bsum[8];
+  float sum[3][32], bsum[8];                                     // dy, output channel; z shift warp / 4
 #pragma unroll
   for (int d = 0; d < 3; d++)
 #pragma unroll
-    for (int j = 0; j < 16; j++) sum[d][j] = 0.f;
+    for (int j = 0; j < 32; j++) sum[d][j] = 0.f;
 #pragma unroll
   for (int j = 0; j < 8; j++) bsum[j] = 0.f;
-  const bool bias = dz == 1 && half == 0;              // bias: thread = chunk (t >> 4) % (no / 8) of dZ, voxels by y
   const uint32_t e = elect_one();
+  int done = 0;                                                  // X slices contracted
 #pragma unroll 1
-  for (int u = 0; u < WLA; u++) { if (warp < 8 && u < n) load(u); cp_commit(); }
+  for (int u = 0; u < WLA; u++) { if (warp < 8) load(u); cp_commit(); }   // (nstep >= 3)
 #pragma unroll 1
-  for (int i = 0; i < n; i++) {
-    if (warp < 8 && i + WLA < n) load(i + WLA);
+  for (int i = 0; i < nstep; i++) {
+    if (warp < 8 && i + WLA < nstep) load(i + WLA);
     cp_commit();
     cp_wait<WLA>();
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     ok = __syncthreads_and(ok);
     if (!ok) break;
-    const unsigned char *a = smtc + i % WNS * WSTAGE, *b = a + WA_BYTES;
+    const bool work = ms.zz - 1 >= ms.za;
+    ms.next(nz);
     if (warp == 8) {
-      tc_after();
-      const uint64_t da = tc_desc(smem_u32(a), 128, WYP * 16), db = tc_desc(smem_u32(b), 128, WYB * 16);
-      const int ax = WYP << lch, bx = WYB << lno;
+      if (work) {
+        tc_after();
+        const uint64_t da = tc_desc(smem_u32(smtc + i % WNS * WA_BYTES), 128, WYP * 16),
+                       db = tc_desc(smem_u32(smtc + WB_OFF + ((i - 2) % WR << lno) * WYB * 16), 128, WYB * 16);
+        const int ax = WYP << lch;
 #pragma unroll
-      for (int x = 0; x < TBX; x++)
+        for (int x = 0; x < TBX; x++)
 #pragma unroll
-        for (int dy = 0; dy < 3; dy++)
-          tc_mma(e, taddr + dy * 32, da + x * ax + dy, db + x * bx, idesc, x > 0 || i % WFL > 0);
+          for (int dy = 0; dy < 3; dy++)
+            tc_mma(e, taddr + dy * 96, da + x * ax + dy, db + x * xsb, idesc, x > 0 || done % WFL > 0);
+      }
       tc_commit(e, &bar[i % WNS]);
-    } else if (bias) {
+    } else if (warp < 8 && work && half == 0) {                  // bias: the middle one of the three slices
+      const unsigned char *b = smtc + WB_OFF + ((i - 1) % WR << lno) * WYB * 16;
 #pragma unroll
       for (int k = 0; k < 2; k++) {
-        const int u = t + 256 * k;
-        if (u >> 4 < TBX << lno) {
-          const uint4 v = *reinterpret_cast<const uint4 *>(b + ((u >> 4) * WYB + (u & 15)) * 16);
+        const int u = t + 256 * k, g = u >> 4;
+        if (g < TBX << lno) {
+          const uint4 v = *reinterpret_cast<const uint4 *>(b + ((g >> lno) * xsb + (g & ((1 << lno) - 1)) * WYB + (u & 15)) * 16);
           const bf16 *p = reinterpret_cast<const bf16 *>(&v);
 #pragma unroll
           for (int j = 0; j < 8; j++) bsum[j] += __bfloat162float(p[j]);
         }
       }
     }
-    if (i % WFL == WFL - 1 || i == n - 1) {
+    if (!work) continue;
+    done++;
+    if (done % WFL == 0 || done == n) {
       ok = __syncthreads_and(tc_wait(&bar[i % WNS], (unsigned)((i / WNS) & 1)));
       if (!ok) break;
       tc_after();
-      if (warp < 8) {
 #pragma unroll
-        for (int d = 0; d < 3; d++) {
-          const uint32_t ta = taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(d * 32 + (warp >> 2) * (no / 2));
-          float v[8];
-          tc_ld8(ta, v);
+      for (int d = 0; d < 3; d++)
 #pragma unroll
-          for (int j = 0; j < 8; j++) sum[d][j] += v[j];
-          if (lno == 2) {
-            tc_ld8(ta + 8, v);
+        for (int k = 0; k < 2; k++)
+          if (k < lno) {
+            float v[16];
+            tc_ld16(taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(d * 96 + (warp >> 2) * no + 16 * k), v);
 #pragma unroll
-            for (int j = 0; j < 8; j++) sum[d][8 + j] += v[j];
+            for (int j = 0; j < 16; j++) sum[d][16 * k + j] += v[j];
           }
-        }
-      }
       tc_before();
       __syncthreads();
     }
   }
   if (ok) {
     const int m = (warp & 3) * 32 + (t & 31), dx = m >> (lch + 3), c = half * 32 + (m & (8 * chn - 1));
-    if (warp < 8 && dx < 3)
+    if (dx < 3)
 #pragma unroll
       for (int d = 0; d < 3; d++) {
+        const int dz = 2 - (warp >> 2);                // of dZ slice z - 1 + warp / 4
         float *dst = L.part + ((size_t)(dx + 3 * d + 9 * dz) * nchunk + chunk) * co * ci + c;
 #pragma unroll
-        for (int j = 0; j < 16; j++) {
-          const int o = (warp >> 2) * (no / 2) + j;
-          if (j < no / 2 && o < co) dst[(size_t)o * ci] = sum[d][j];
-        }
+        for (int o = 0; o < 32; o++)
+          if (o < co) dst[(size_t)o * ci] = sum[d][o];
       }
-    if (bias) {                                        // (the last slice's MMAs are done: the stages are free)
+    if (half == 0) {                                   // (the last MMAs are done: the stages are free)
       float *bred = reinterpret_cast<float *>(smtc);
       __syncthreads();
       if (warp < 8)
@@ -796,7 +845,7 @@ __global__ void __launch_bounds__(WG_T, 2) k_conv_wgrad(const __grid_constant__ 
   }
   tc_before();
   __syncthreads();
-  if (warp == 0) tc_free(taddr, 128);
+  if (warp == 0) tc_free(taddr, 512);
 }
 
 // G += sums over the chunks (in order) of all layers' partials, G in the flat
@@ -855,18 +904,22 @@ __global__ void k_pool(dims f, dims c, const bf16 *X, int ldx, int offx, bf16 *P
   int Z = V / (c.nx * c.ny), r = V - Z * c.nx * c.ny, Y = r / c.nx, Xc = r - Y * c.nx;
   float s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   int cnt = 0;
-  for (int k = 0; k < 2; k++)
-    for (int j = 0; j < 2; j++)
-      for (int i = 0; i < 2; i++) {
-        int x = 2 * Xc + i, y = 2 * Y + j, z = 2 * Z + k;
-        if (x >= f.nx || y >= f.ny || z >= f.nz) continue;
-        const bf16 *p = X + (size_t)(x + f.nx * (y + f.ny * z)) * ldx + offx + g;
-        uint4 u = *reinterpret_cast<const uint4 *>(p);
-        const bf16 *e = reinterpret_cast<const bf16 *>(&u);
+  uint4 u[8];                                          // the children's loads together, then the sums in order
+  bool in[8];
 #pragma unroll
-        for (int a = 0; a < 8; a++) s[a] += __bfloat162float(e[a]);
-        cnt++;
-      }
+  for (int k = 0; k < 8; k++) {
+    int x = 2 * Xc + (k & 1), y = 2 * Y + (k >> 1 & 1), z = 2 * Z + (k >> 2);
+    in[k] = x < f.nx && y < f.ny && z < f.nz;
+    if (in[k]) u[k] = *reinterpret_cast<const uint4 *>(X + (size_t)(x + f.nx * (y + f.ny * z)) * ldx + offx + g);
+  }
+#pragma unroll
+  for (int k = 0; k < 8; k++)
+    if (in[k]) {
+      const bf16 *e = reinterpret_cast<const bf16 *>(&u[k]);
+#pragma unroll
+      for (int a = 0; a < 8; a++) s[a] += __bfloat162float(e[a]);
+      cnt++;
+    }
   uint4 o;
   bf16 *e = reinterpret_cast<bf16 *>(&o);
 #pragma unroll
@@ -895,16 +948,21 @@ __global__ void k_up_back(dims f, dims c, const bf16 *G, int ldg, int offg, bf16
   int V = q >> 2, g = (q & 3) * 8;
   int Z = V / (c.nx * c.ny), r = V - Z * c.nx * c.ny, Y = r / c.nx, Xc = r - Y * c.nx;
   float s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int k = 0; k < 2; k++)
-    for (int j = 0; j < 2; j++)
-      for (int i = 0; i < 2; i++) {
-        int x = 2 * Xc + i, y = 2 * Y + j, z = 2 * Z + k;
-        if (x >= f.nx || y >= f.ny || z >= f.nz) continue;
-        uint4 u = *reinterpret_cast<const uint4 *>(G + (size_t)(x + f.nx * (y + f.ny * z)) * ldg + offg + g);
-        const bf16 *e = reinterpret_cast<const bf16 *>(&u);
+  uint4 u[8];
+  bool in[8];
 #pragma unroll
-        for (int a = 0; a < 8; a++) s[a] += __bfloat162float(e[a]);
-      }
+  for (int k = 0; k < 8; k++) {
+    int x = 2 * Xc + (k & 1), y = 2 * Y + (k >> 1 & 1), z = 2 * Z + (k >> 2);
+    in[k] = x < f.nx && y < f.ny && z < f.nz;
+    if (in[k]) u[k] = *reinterpret_cast<const uint4 *>(G + (size_t)(x + f.nx * (y + f.ny * z)) * ldg + offg + g);
+  }
+#pragma unroll
+  for (int k = 0; k < 8; k++)
+    if (in[k]) {
+      const bf16 *e = reinterpret_cast<const bf16 *>(&u[k]);
+#pragma unroll
+      for (int a = 0; a < 8; a++) s[a] += __bfloat162float(e[a]);
+    }
   uint4 o;
   bf16 *e = reinterpret_cast<bf16 *>(&o);
 #pragma unroll
@@ -1019,9 +1077,15 @@ __global__ void k_export(int n, const float *p, float div, float *out) {
 __global__ void k_feat_in(int V, const float *F, bf16 *X) {
   int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= V) return;
-  bf16 *o = X + (size_t)v * CIN_GPU;
-  for (int c = 0; c < CIN_USED; c++) o[c] = __float2bfloat16_rn(F[(size_t)v * CIN_USED + c]);
-  for (int c = CIN_USED; c < CIN_GPU; c++) o[c] = __float2bfloat16_rn(0.f);
+  const float4 *f = reinterpret_cast<const float4 *>(F + (size_t)v * CIN_USED);
+  const float4 a = f[0], b = f[1];
+  uint4 o;
+  __nv_bfloat162 *h = reinterpret_cast<__nv_bfloat162 *>(&o);
+  h[0] = __floats2bfloat162_rn(a.x, a.y); h[1] = __floats2bfloat162_rn(a.z, a.w);
+  h[2] = __floats2bfloat162_rn(b.x, b.y); h[3] = __floats2bfloat162_rn(b.z, b.w);
+  uint4 *d = reinterpret_cast<uint4 *>(X + (size_t)v * CIN_GPU);
+  d[0] = o;
+  d[1] = make_uint4(0, 0, 0, 0);
 }
 
 // ------------------------------------------------------------ the net -----
@@ -1139,7 +1203,7 @@ static void conv_tc_launch(sim_ws_s *w, dims d, const bf16 *X, int ldx, int offx
     for (int z = 1; z <= 4; z++) if (tc_bytes(CI, CO, z) + 128 <= cap) top = z;
     RS_CUDA(cudaFuncSetAttribute(k_conv_tc<CI, CO, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_bytes(CI, CO, top)));
     for (int z = 1; z <= top; z++) {
-      RS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[z], k_conv_tc<CI, CO, MODE>, 256, tc_bytes(CI, CO, z)));
+      RS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[z], k_conv_tc<CI, CO, MODE>, TC_T, tc_bytes(CI, CO, z)));
       per_sm[z] = std::max(1, std::min(per_sm[z], 512 / tc_cols(CO, z)));
     }
   });
@@ -1153,7 +1217,7 @@ static void conv_tc_launch(sim_ws_s *w, dims d, const bf16 *X, int ldx, int offx
     if (c < best) { best = c; NZ = z; }
   }
   const unsigned tiles = (unsigned)(txy * ((d.nz + NZ - 1) / NZ));
-  launch_pdl(k_conv_tc<CI, CO, MODE>, tiles, 256, (size_t)tc_bytes(CI, CO, NZ), w->st, d.nx, d.ny, d.nz, NZ, X, ldx, offx,
+  launch_pdl(k_conv_tc<CI, CO, MODE>, tiles, TC_T, (size_t)tc_bytes(CI, CO, NZ), w->st, d.nx, d.ny, d.nz, NZ, X, ldx, offx,
              Wt, bias, relu, out, ldo, offo, mask, ldm, offm, w->err_dev);
   RS_LAUNCHED(1);
 }
@@ -1210,34 +1274,39 @@ static void bwd_data(sim_ws_s *w, int l, dims d, const bf16 *dZ, int ldz, int of
 
 // Weight gradients of all layers, from the activations and the gradients that
 // the data-gradient passes left (each in a buffer of its own): one launch of
-// about two CTAs per SM, shared out by the layers' slices, and one that adds
+// at most a CTA per SM, shared out by the layers' slices, and one that adds
 // the chunks and the loss.
 struct wg_in { const bf16 *X; int ldx, offx; const bf16 *dZ; int ldz; dims d; };
 static void wgrad(sim_ws_s *w, const wg_in in[NLAYER], int nl, double lscale) {
   wg_table tab;
-  double units = 0.0;
-  auto slices = [](dims d) { return (long long)((d.nx + TBX - 1) / TBX) * ((d.ny + TBY - 1) / TBY) * d.nz; };
-  for (int l = 0; l < NLAYER; l++) units += 3.0 * slices(in[l].d) * ((LAYERS[l].ci + 31) / 32);
-  static int cap = 0;                             // CTAs to aim at
+  static int sms = 0;
   static std::once_flag once;
   std::call_once(once, [&] {
-    int dev = 0, sms = 0;
+    int dev = 0;
     RS_CUDA(cudaGetDevice(&dev));
     RS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    RS_CUDA(cudaFuncSetAttribute(k_conv_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, WNS * WSTAGE));
-    cap = 2 * sms;
+    RS_CUDA(cudaFuncSetAttribute(k_conv_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_BYTES));
   });
+  auto slices = [&](int l) { return (long long)((in[l].d.nx + TBX - 1) / TBX) * ((in[l].d.ny + TBY - 1) / TBY) * in[l].d.nz; };
+  auto halves = [](int l) { return (LAYERS[l].ci + 31) / 32; };
+  // the fewest slices per CTA that need no second round
+  long long units = 0, per = 1;
+  for (int l = 0; l < NLAYER; l++) units += slices(l) * halves(l);
+  for (per = std::max(1LL, units / sms);; per += 1 + per / 64) {
+    long long ctas = 0;
+    for (int l = 0; l < NLAYER; l++) ctas += halves(l) * ((slices(l) + per - 1) / per);
+    if (ctas <= sms || per >= units) break;
+  }
   int block = 0;
   size_t need = 0;
   for (int l = 0; l < NLAYER; l++) {
     wg_layer &L = tab.l[l];
     const int co = LAYERS[l].co, ci = LAYERS[l].ci;
-    const long long S = slices(in[l].d);
     L.X = in[l].X; L.ldx = in[l].ldx; L.offx = in[l].offx; L.dZ = in[l].dZ; L.ldz = in[l].ldz;
     L.nx = in[l].d.nx; L.ny = in[l].d.ny; L.nz = in[l].d.nz; L.co = co; L.ci = ci;
-    L.nchunk = (int)std::max(1.0, std::min((double)S, std::floor(cap * (double)S / units)));
+    L.nchunk = (int)((slices(l) + per - 1) / per);
     L.block0 = block;
-    block += L.nchunk * 3 * ((ci + 31) / 32);
+    block += L.nchunk * halves(l);
     need += (size_t)L.nchunk * (27 * co * ci + co);
   }
   w->part.ensure(need);
@@ -1247,7 +1316,7 @@ static void wgrad(sim_ws_s *w, const wg_in in[NLAYER], int nl, double lscale) {
     L.part = p; p += (size_t)L.nchunk * 27 * L.co * L.ci;
     L.bpart = p; p += (size_t)L.nchunk * L.co;
   }
-  launch_pdl(k_conv_wgrad, (unsigned)block, WG_T, (size_t)WNS * WSTAGE, w->st, tab, w->err_dev);
+  launch_pdl(k_conv_wgrad, (unsigned)block, WG_T, (size_t)WG_BYTES, w->st, tab, w->err_dev);
   launch_pdl(k_wgrad_reduce, grid_for(w->np, 256) + 1, 256, 0, w->st, tab, (int)w->np, w->G.p, nl, w->lpart.p, lscale,
              w->lsum.p);
   RS_LAUNCHED(2);
