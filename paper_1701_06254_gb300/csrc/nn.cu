@@ -29,6 +29,7 @@
 // the voxel-major tiles, one CTA per (voxel chunk, tap), partials reduced in
 // a fixed order so results do not depend on scheduling.
 #include "common.cuh"
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <algorithm>
 #include <cmath>
@@ -1739,25 +1740,46 @@ __global__ void k_ws_target(int n, const double *y, const double *sc, float *T) 
   T[i] = s > 0.0 ? (float)(y[i] / s) : 0.f;
 }
 
-// rms over the n cells of the two interleaved components of v -> out[0], out[1]
-__global__ void k_rms2(int n, const double *v, double *out) {
-  __shared__ double sh[2][1024];
+// rms over the n cells of the two interleaved components of v -> out[0], out[1].
+// One cluster of eight CTAs, whose partial sums the first adds through
+// distributed shared memory: no workspace and a fixed order.  With a single
+// CTA its SM's FP64 pipe and latency bounded the sum.
+constexpr int RMS_C = 8, RMS_U = 4;
+__global__ void __cluster_dims__(RMS_C, 1, 1) __launch_bounds__(1024) k_rms2(int n, const double *v, double *out) {
+  __shared__ double sh[2][32];
+  __shared__ double all[2][RMS_C];
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int t = threadIdx.x, rank = (int)cl.block_rank(), step = RMS_C * 1024;
   double s0 = 0.0, s1 = 0.0;
-  for (int c = threadIdx.x; c < n; c += blockDim.x) {
-    double a = v[2 * (size_t)c], b = v[2 * (size_t)c + 1];
-    s0 += a * a; s1 += b * b;
+  for (int c0 = rank * 1024 + t; c0 < n; c0 += RMS_U * step) {
+    double2 a[RMS_U];
+#pragma unroll
+    for (int u = 0; u < RMS_U; u++)
+      a[u] = c0 + (long long)u * step < n ? reinterpret_cast<const double2 *>(v)[c0 + u * step] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int u = 0; u < RMS_U; u++) { s0 += a[u].x * a[u].x; s1 += a[u].y * a[u].y; }
   }
-  sh[0][threadIdx.x] = s0; sh[1][threadIdx.x] = s1;
+  auto warp_sum = [](double x) {
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    return x;
+  };
+  s0 = warp_sum(s0); s1 = warp_sum(s1);
+  if ((t & 31) == 0) { sh[0][t >> 5] = s0; sh[1][t >> 5] = s1; }
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) { sh[0][threadIdx.x] += sh[0][threadIdx.x + o]; sh[1][threadIdx.x] += sh[1][threadIdx.x + o]; }
-    __syncthreads();
+  if (t < 64) {
+    const double x = warp_sum(sh[t >> 5][t & 31]);
+    if ((t & 31) == 0) *cl.map_shared_rank(&all[t >> 5][rank], 0) = x;
   }
-  if (threadIdx.x == 0) { out[0] = sqrt(sh[0][0] / n); out[1] = sqrt(sh[1][0] / n); }
+  cl.sync();
+  if (rank == 0 && t < 2) {
+    double x = 0.0;
+    for (int k = 0; k < RMS_C; k++) x += all[t][k];
+    out[t] = sqrt(x / n);
+  }
 }
 
 void ws_rms2(int n, const double *v, double *out, cudaStream_t s) {
-  k_rms2<<<1, 1024, 0, s>>>(n, v, out);
+  k_rms2<<<RMS_C, 1024, 0, s>>>(n, v, out);
   RS_LAUNCHED(1);
 }
 
