@@ -117,6 +117,8 @@ __device__ __forceinline__ void warp_append(bool on, int i, int *count, int *lis
 __global__ void k_pmis_init(int n, const int *rp, const int *ci, const uint8_t *S, const int *tpos,
                             uint64_t seed, int level, double *w, int8_t *cf, int8_t *newc, int *undecided,
                             int *list) {
+  pdl_trigger();
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   int cnt = 0;
   if (i < n) {
@@ -229,6 +231,8 @@ __device__ __forceinline__ void pmis_update_pts(const int *rp, const int *ci, co
 template <int L>
 __global__ void k_pmis_select_w(const int *rp, const int *ci, const uint8_t *S, const int *tpos, const double *w,
                                 const int8_t *cf, int8_t *newc, const int *list, const int *cnt) {
+  pdl_trigger();
+  pdl_wait();
   int m = *cnt;
   if (m == 0) return;
   pmis_select_pts<L>(rp, ci, S, tpos, w, cf, newc, list, m, (blockIdx.x * blockDim.x + threadIdx.x) / L,
@@ -238,6 +242,8 @@ __global__ void k_pmis_select_w(const int *rp, const int *ci, const uint8_t *S, 
 template <int L>
 __global__ void k_pmis_update_w(const int *rp, const int *ci, const uint8_t *S, int8_t *cf, const int8_t *newc,
                                 const int *list, const int *cnt, int *next, int *cnt_next) {
+  pdl_trigger();
+  pdl_wait();
   int m = *cnt;
   if (m == 0) return;
   pmis_update_pts<L>(rp, ci, S, cf, newc, list, m, (blockIdx.x * blockDim.x + threadIdx.x) / L,
@@ -253,6 +259,8 @@ template <int L>
 __global__ void __launch_bounds__(1024) k_pmis_tail(const int *rp, const int *ci, const uint8_t *S, const int *tpos,
                                                     const double *w, int8_t *cf, int8_t *newc, int *plist, int n,
                                                     int *cnt, int r0, int rmax, int *z) {
+  pdl_trigger();
+  pdl_wait();
   const volatile int *vcnt = cnt;
   __shared__ int zs;
   if (threadIdx.x == 0) {
@@ -310,6 +318,8 @@ __device__ __forceinline__ void row_products(int i, int n, const int *arp, const
 }
 __global__ void k_row_products(int n, const int *arp, const int *aci, const int *bbeg, const int *bend, int *prod,
                                int *mx, int merge_p) {
+  pdl_trigger();
+  pdl_wait();
   row_products(blockIdx.x * blockDim.x + threadIdx.x, n, arp, aci, bbeg, bend, prod, mx, merge_p);
 }
 
@@ -523,11 +533,15 @@ __global__ void k_exti_fill(int n, const int *rp, const int *ci, const double *v
 
 // ------------------------------------------------------------ transpose ---
 __global__ void k_col_count(int nnz, const int *ci, int *cnt) {
+  pdl_trigger();
+  pdl_wait();
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < nnz) atomicAdd(&cnt[ci[q]], 1);
 }
 __global__ void k_transpose_fill(int n, const int *rp, const int *ci, const double *v, const int *trp, int *fill,
                                  int *tci, double *tv) {
+  pdl_trigger();
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   for (int q = rp[i]; q < rp[i + 1]; q++) {
@@ -565,6 +579,8 @@ __device__ __forceinline__ void warp_sort64(int M, int lane, int &k0, int &k1, d
 // row held up a whole level: 28 us on one of 1,600 rows).  v32: the FP32 copy
 // of v (mixed precision) or nullptr.
 __global__ void k_sort_rows_warp(int n, const int *rp, int *ci, double *v, float *v32) {
+  pdl_trigger();
+  pdl_wait();
   int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (i >= n) return;
   int a0 = rp[i], len = rp[i + 1] - a0;
@@ -593,6 +609,8 @@ __global__ void k_sort_rows_warp(int n, const int *rp, int *ci, double *v, float
 // entries), longer rows by an insertion sort in the group's first lane
 template <int G>
 __global__ void k_sort_rows_g(int n, const int *rp, int *ci, double *v, float *v32) {
+  pdl_trigger();
+  pdl_wait();
   if (n <= 0) return;
   int gi = (blockIdx.x * blockDim.x + threadIdx.x) / G, k = threadIdx.x % G;
   bool valid = gi < n;
@@ -637,6 +655,8 @@ __global__ void k_sort_rows_g(int n, const int *rp, int *ci, double *v, float *v
 // (cv32: the FP32 copy of cv or nullptr)
 __global__ void k_pack_rows(int n, const int *toff, const int *clen, const int *crp, const int *tci, const double *tv,
                             int *cci, double *cv, float *cv32) {
+  pdl_trigger();
+  pdl_wait();
   int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, lane = threadIdx.x & 7;
   if (row >= n) return;
   int a = toff[row], b = crp[row], len = clen[row];
@@ -661,6 +681,8 @@ __global__ void __launch_bounds__(128) k_spgemm_merge(int n, const int *arp, con
                                                       const int *bbeg, const int *bend, const int *bci,
                                                       const double *bv, const int *toff, int *clen, int *cci,
                                                       double *cv, int merge_p, int ends) {
+  pdl_trigger();
+  pdl_wait();
   int row = blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= n) return;
   int a0 = arp[row], k = arp[row + 1] - a0;
@@ -734,6 +756,8 @@ __global__ void __launch_bounds__(256) k_spgemm_hash(int n, const int *arp, cons
                                                      const double *bv, const int *toff, int *clen, int *cci,
                                                      double *cv, int tcap, int lo_p, double *gscratch, int merge_p,
                                                      int ends) {
+  pdl_trigger();
+  pdl_wait();
   extern __shared__ double sm_hash[];
   const int warps = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned FULL = 0xffffffffu;
@@ -873,7 +897,7 @@ static void spgemm_count(const csr_dev<double> &A, const row_ref &B, spg_scratch
   int n = A.n;
   if (!counted) {
     z.toff.ensure(n + 1); z.clen.ensure(n + 1);
-    k_row_products<<<grid_for(n, 128), 128, 0, s>>>(n, A.rp.p, A.ci.p, B.beg, B.end, z.toff.p, mx, spg_merge_p(n));
+    launch_small(k_row_products, grid_for(n, 128), 128, 0, s, n, A.rp.p, A.ci.p, B.beg, B.end, z.toff.p, mx, spg_merge_p(n));
     RS_LAUNCHED(1);
   }
   rs_scan_dev(z.toff.p, z.toff.p, n, z.toff.p + n, tot, s);      // row offsets into the scratch arrays
@@ -900,19 +924,19 @@ static void spgemm_numeric(const csr_dev<double> &A, const row_ref &B, spg_scrat
   z.tci.ensure(std::max(total, 1)); z.tv.ensure(std::max(total, 1));
   int mp = spg_merge_p(n);
   if (mp >= 0) {
-    k_spgemm_merge<SPG_KMAX><<<grid_for(n, 128), 128, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, B.beg, B.end, B.ci, B.v,
+    launch_small(k_spgemm_merge<SPG_KMAX>, grid_for(n, 128), 128, 0, s, n, A.rp.p, A.ci.p, A.v.p, B.beg, B.end, B.ci, B.v,
                                                               z.toff.p, z.clen.p, z.tci.p, z.tv.p, mp, ends);
     RS_LAUNCHED(1);
   }
   if (mx1 > 0) {                                       // rows for the hash kernel
     unsigned grid = (unsigned)std::min<size_t>((n + warps - 1) / warps, 152 * 32);
-    k_spgemm_hash<<<grid, warps * 32, smem, s>>>(n, A.rp.p, A.ci.p, A.v.p, B.beg, B.end, B.ci, B.v, z.toff.p,
+    launch_small(k_spgemm_hash, grid, warps * 32, (size_t)(smem), s, n, A.rp.p, A.ci.p, A.v.p, B.beg, B.end, B.ci, B.v, z.toff.p,
                                                  z.clen.p, z.tci.p, z.tv.p, tcap, -1, nullptr, mp, ends);
     RS_LAUNCHED(1);
     if (tall > tcap) {                                 // rows beyond the shared-memory capacity
       const int gw = 4, gblocks = 64;
       gs.ensure((size_t)gblocks * gw * spg_warp_doubles(tall));
-      k_spgemm_hash<<<gblocks, gw * 32, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, B.beg, B.end, B.ci, B.v, z.toff.p, z.clen.p,
+      launch_small(k_spgemm_hash, gblocks, gw * 32, 0, s, n, A.rp.p, A.ci.p, A.v.p, B.beg, B.end, B.ci, B.v, z.toff.p, z.clen.p,
                                                 z.tci.p, z.tv.p, tall, tcap, gs.p, mp, ends);
       RS_LAUNCHED(1);
     }
@@ -928,7 +952,7 @@ static void spgemm_pack(int n, int m, spg_scratch &z, csr_dev<double> &C, csr_de
   rs_scan_dev(z.clen.p, C.rp.p, n, C.rp.p + n, nnz, s);
   C.ci.ensure(std::max(total, 1)); C.v.ensure(std::max(total, 1));
   if (C32) C32->v.ensure(std::max(total, 1));
-  k_pack_rows<<<grid_for((size_t)n * 8, 256), 256, 0, s>>>(n, z.toff.p, z.clen.p, C.rp.p, z.tci.p, z.tv.p, C.ci.p,
+  launch_small(k_pack_rows, grid_for((size_t)n * 8, 256), 256, 0, s, n, z.toff.p, z.clen.p, C.rp.p, z.tci.p, z.tv.p, C.ci.p,
                                                           C.v.p, C32 ? C32->v.p : nullptr);
   RS_LAUNCHED(1);
   RS_CHECK_LAUNCH();
@@ -947,6 +971,8 @@ __global__ void k_l1(int n, const int *rp, const int *ci, const double *v, doubl
 
 // --------------------------------------------------------- dense coarsest -
 __global__ void k_dense_build(int n, const int *rp, const int *ci, const double *v, double *a) {
+  pdl_trigger();
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   for (int j = 0; j < n; j++) a[(size_t)i * n + j] = 0.0;
@@ -955,6 +981,8 @@ __global__ void k_dense_build(int n, const int *rp, const int *ci, const double 
 // LU with partial pivoting (first row of maximal |a_ik|), then the inverse
 // column by column; one block.
 __global__ void k_dense_lu_inv(int n, double *a, int *piv, double *inv) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ double smx[1024]; __shared__ int sid[1024];
   int t = threadIdx.x, nt = blockDim.x;
   for (int k = 0; k < n; k++) {
@@ -1004,6 +1032,8 @@ __global__ void k_dense_lu_inv(int n, double *a, int *piv, double *inv) {
 // and every lane columns j > k: a_ij -= l_ik a_kj.  Two block barriers per
 // step; n^3/3 multiply-adds in all.
 __global__ void __launch_bounds__(512) k_dense_lu_smem(int n, const double *ag, int *piv, double *lu, double *rdiag) {
+  pdl_trigger();
+  pdl_wait();
   extern __shared__ double sa[];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
   for (int e = t; e < n * n; e += blockDim.x) sa[e] = ag[e];
@@ -1050,6 +1080,8 @@ __global__ void __launch_bounds__(512) k_dense_lu_smem(int n, const double *ag, 
 template <int NR>
 __global__ void __launch_bounds__(64) k_dense_inv_cols(int n, const double *lu, const int *piv, const double *rdiag,
                                                       double *inv) {
+  pdl_trigger();
+  pdl_wait();
   extern __shared__ double sl[];
   double *sr = sl + (size_t)n * n;
   int *sp = reinterpret_cast<int *>(sr + n);
@@ -1151,9 +1183,9 @@ static void pmis_rounds(amg_level &L, amg_hier &h, int n, int lanes, int r0, int
     int *nxt = h.plist.p + (size_t)((r + 1) & 1) * n;
 #define PMIS_ROUND(LL)                                                                                        \
     if (lanes == LL) {                                                                                        \
-      k_pmis_select_w<LL><<<g, 128, 0, s>>>(L.A.rp.p, L.A.ci.p, L.strong.p, L.tpos.p, h.hashw.p, L.cf.p,      \
+      launch_small(k_pmis_select_w<LL>, g, 128, 0, s, L.A.rp.p, L.A.ci.p, L.strong.p, L.tpos.p, h.hashw.p, L.cf.p,      \
                                             h.newc.p, lst, cnt + r);                                          \
-      k_pmis_update_w<LL><<<g, 128, 0, s>>>(L.A.rp.p, L.A.ci.p, L.strong.p, L.cf.p, h.newc.p, lst, cnt + r,   \
+      launch_small(k_pmis_update_w<LL>, g, 128, 0, s, L.A.rp.p, L.A.ci.p, L.strong.p, L.cf.p, h.newc.p, lst, cnt + r,   \
                                             nxt, cnt + r + 1);                                                \
     }
     PMIS_ROUND(1) PMIS_ROUND(4) PMIS_ROUND(16)
@@ -1169,7 +1201,7 @@ static void pmis_tail(amg_level &L, amg_hier &h, int n, int lanes, int r0, cudaS
   int *F = h.flag.p;
 #define PMIS_TAIL(LL)                                                                                          \
   if (lanes == LL)                                                                                             \
-    k_pmis_tail<LL><<<1, 1024, 0, s>>>(L.A.rp.p, L.A.ci.p, L.strong.p, L.tpos.p, h.hashw.p, L.cf.p, h.newc.p,  \
+    launch_small(k_pmis_tail<LL>, 1, 1024, 0, s, L.A.rp.p, L.A.ci.p, L.strong.p, L.tpos.p, h.hashw.p, L.cf.p, h.newc.p,  \
                                        h.plist.p, n, F + AF_CNT, r0, AF_ROUNDS_MAX, F + AF_PRND);
   PMIS_TAIL(1) PMIS_TAIL(4) PMIS_TAIL(16)
 #undef PMIS_TAIL
@@ -1281,7 +1313,7 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
       if (wide) go(k_strength<32>); else go(k_strength<1>);
     }
     h.hashw.ensure(n); h.newc.ensure(n); h.plist.ensure(2 * (size_t)n);
-    k_pmis_init<<<grid_for(n, 128), 128, 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.strong.p, L.tpos.p, o.seed, l,
+    launch_small(k_pmis_init, grid_for(n, 128), 128, 0, s, n, L.A.rp.p, L.A.ci.p, L.strong.p, L.tpos.p, o.seed, l,
                                                  h.hashw.p, L.cf.p, h.newc.p, F + AF_CNT, h.plist.p);
     RS_LAUNCHED(2);
     RS_CHECK_LAUNCH();
@@ -1321,20 +1353,20 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
       RS_CUDA(cudaStreamWaitEvent(sr, h.ev_p, 0));
       rs_fill_i(L.R.rp.p, 0, nc + 1, sr);
       rs_fill_i(fill.p, 0, nc + 1, sr);
-      k_col_count<<<grid_for(L.P.nnz, 256), 256, 0, sr>>>(L.P.nnz, L.P.ci.p, L.R.rp.p);
+      launch_small(k_col_count, grid_for(L.P.nnz, 256), 256, 0, sr, L.P.nnz, L.P.ci.p, L.R.rp.p);
       RS_LAUNCHED(1);
       rs_scan_dev(L.R.rp.p, L.R.rp.p, nc, L.R.rp.p + nc, nullptr, sr, &h.scan_r);
-      k_transpose_fill<<<grid_for(n, 256), 256, 0, sr>>>(n, L.P.rp.p, L.P.ci.p, L.P.v.p, L.R.rp.p, fill.p, L.R.ci.p,
+      launch_small(k_transpose_fill, grid_for(n, 256), 256, 0, sr, n, L.P.rp.p, L.P.ci.p, L.P.v.p, L.R.rp.p, fill.p, L.R.ci.p,
                                                          L.R.v.p);
       // rows of R: lanes per row by their mean length (a row longer than its
       // group falls to one lane's insertion sort: groups of 16 only where
       // rows average at most 8 entries)
       double avg = nc ? (double)L.P.nnz / nc : 0.0;
       if (avg <= 4.0)
-        k_sort_rows_g<8><<<grid_for((size_t)nc * 8, 128), 128, 0, sr>>>(nc, L.R.rp.p, L.R.ci.p, L.R.v.p, r32);
+        launch_small(k_sort_rows_g<8>, grid_for((size_t)nc * 8, 128), 128, 0, sr, nc, L.R.rp.p, L.R.ci.p, L.R.v.p, r32);
       else if (avg <= 8.0)
-        k_sort_rows_g<16><<<grid_for((size_t)nc * 16, 128), 128, 0, sr>>>(nc, L.R.rp.p, L.R.ci.p, L.R.v.p, r32);
-      else k_sort_rows_warp<<<grid_for((size_t)nc * 32, 128), 128, 0, sr>>>(nc, L.R.rp.p, L.R.ci.p, L.R.v.p, r32);
+        launch_small(k_sort_rows_g<16>, grid_for((size_t)nc * 16, 128), 128, 0, sr, nc, L.R.rp.p, L.R.ci.p, L.R.v.p, r32);
+      else launch_small(k_sort_rows_warp, grid_for((size_t)nc * 32, 128), 128, 0, sr, nc, L.R.rp.p, L.R.ci.p, L.R.v.p, r32);
       RS_LAUNCHED(2);
       RS_CHECK_LAUNCH();
       RS_CUDA(cudaEventRecord(h.ev_r, sr));
@@ -1374,7 +1406,7 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
     if (n > 2048) RS_FAIL(SIM_ERR_ARG, "AMG: coarsest level of %d rows is too large for the dense solve", n);
     dbuf<double> &a = h.dense_a;
     a.ensure((size_t)n * n); h.lu.ensure((size_t)n * n); h.piv.ensure(n);
-    k_dense_build<<<grid_for(n, 128), 128, 0, s>>>(n, C.A.rp.p, C.A.ci.p, C.A.v.p, a.p);
+    launch_small(k_dense_build, grid_for(n, 128), 128, 0, s, n, C.A.rp.p, C.A.ci.p, C.A.v.p, a.p);
     if (n <= 128) {
       static bool attr = false;
       if (!attr) {
@@ -1387,18 +1419,18 @@ void amg_setup(amg_hier &h, const rs_opts &o, cudaStream_t s) {
       }
       h.dense_lu.ensure((size_t)n * n);
       h.dense_rd.ensure(n);
-      k_dense_lu_smem<<<1, 512, (size_t)n * n * 8, s>>>(n, a.p, h.piv.p, h.dense_lu.p, h.dense_rd.p);
+      launch_small(k_dense_lu_smem, 1, 512, (size_t)((size_t)n * n * 8), s, n, a.p, h.piv.p, h.dense_lu.p, h.dense_rd.p);
       const size_t csm = (size_t)n * n * 8 + (size_t)n * 12;
       const unsigned cg = (unsigned)((n + 1) / 2);
       switch ((n + 31) / 32) {
-        case 1: k_dense_inv_cols<1><<<cg, 64, csm, s>>>(n, h.dense_lu.p, h.piv.p, h.dense_rd.p, h.lu.p); break;
-        case 2: k_dense_inv_cols<2><<<cg, 64, csm, s>>>(n, h.dense_lu.p, h.piv.p, h.dense_rd.p, h.lu.p); break;
-        case 3: k_dense_inv_cols<3><<<cg, 64, csm, s>>>(n, h.dense_lu.p, h.piv.p, h.dense_rd.p, h.lu.p); break;
-        default: k_dense_inv_cols<4><<<cg, 64, csm, s>>>(n, h.dense_lu.p, h.piv.p, h.dense_rd.p, h.lu.p); break;
+        case 1: launch_small(k_dense_inv_cols<1>, cg, 64, (size_t)(csm), s, n, h.dense_lu.p, h.piv.p, h.dense_rd.p, h.lu.p); break;
+        case 2: launch_small(k_dense_inv_cols<2>, cg, 64, (size_t)(csm), s, n, h.dense_lu.p, h.piv.p, h.dense_rd.p, h.lu.p); break;
+        case 3: launch_small(k_dense_inv_cols<3>, cg, 64, (size_t)(csm), s, n, h.dense_lu.p, h.piv.p, h.dense_rd.p, h.lu.p); break;
+        default: launch_small(k_dense_inv_cols<4>, cg, 64, (size_t)(csm), s, n, h.dense_lu.p, h.piv.p, h.dense_rd.p, h.lu.p); break;
       }
       RS_LAUNCHED(1);
     } else {
-      k_dense_lu_inv<<<1, 512, 0, s>>>(n, a.p, h.piv.p, h.lu.p);
+      launch_small(k_dense_lu_inv, 1, 512, 0, s, n, a.p, h.piv.p, h.lu.p);
     }
     RS_LAUNCHED(2);
   }

@@ -91,6 +91,15 @@ inline void launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, si
                        Args... args) {
   launch_pdl_if(true, kern, grid, block, smem, s, args...);
 }
+// For chains of kernels of any size (the setups): programmatic while the grid
+// is small; the blocks of a large one would take the room of the kernel
+// before it while they wait.
+constexpr unsigned PDL_SMALL = 152 * 8;
+template <typename... KArgs, typename... Args>
+inline void launch_small(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                         Args... args) {
+  launch_pdl_if(grid <= PDL_SMALL, kern, grid, block, smem, s, args...);
+}
 
 // ------------------------------------------------------- device helpers --
 // Arithmetic used where a floating-point value decides an integer (the

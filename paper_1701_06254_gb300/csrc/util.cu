@@ -42,6 +42,8 @@ __device__ __forceinline__ int block_excl_scan(int v, int *sh, int *total) {
 }
 
 __global__ void k_scan_partials(const int *in, int n, int *part) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ int sh[SCAN_BS / 32]; __shared__ int tot;
   int base = blockIdx.x * SCAN_CHUNK + threadIdx.x * SCAN_IT, s = 0;
   for (int k = 0; k < SCAN_IT; k++) if (base + k < n) s += in[base + k];
@@ -54,6 +56,8 @@ __global__ void k_scan_partials(const int *in, int n, int *part) {
 // thousand integers, read from L2) instead of waiting for a separate scan of
 // the partials; the last block writes the total.
 __global__ void k_scan_final(const int *in, int *out, int n, int *part, int nblk, int *tail, int *tot2) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ int sh[SCAN_BS / 32]; __shared__ int tot, off;
   int o = 0;
   for (int k = threadIdx.x; k < (int)blockIdx.x; k += SCAN_BS) o += part[k];
@@ -76,8 +80,8 @@ int rs_scan(const int *in, int *out, int n, cudaStream_t s) {
   int nblk = (n + SCAN_CHUNK - 1) / SCAN_CHUNK;
   static thread_local dbuf<int> part;
   part.ensure(nblk + 1);
-  k_scan_partials<<<nblk, SCAN_BS, 0, s>>>(in, n, part.p);
-  k_scan_final<<<nblk, SCAN_BS, 0, s>>>(in, out, n, part.p, nblk, nullptr, nullptr);
+  launch_small(k_scan_partials, nblk, SCAN_BS, 0, s, in, n, part.p);
+  launch_small(k_scan_final, nblk, SCAN_BS, 0, s, in, out, n, part.p, nblk, nullptr, nullptr);
   RS_LAUNCHED(2);
   RS_CHECK_LAUNCH();
   int tot = 0;
@@ -125,10 +129,14 @@ __device__ __forceinline__ void scan_one(const int *in, int *out, int n, int *ta
   }
 }
 __global__ void __launch_bounds__(SCAN_ONE_BS) k_scan_one(const int *in, int *out, int n, int *tail, int *tot2) {
+  pdl_trigger();
+  pdl_wait();
   scan_one(in, out, n, tail, tot2);
 }
 __global__ void __launch_bounds__(SCAN_ONE_BS) k_scan_one2(int *a, int *tail_a, int *tot_a, int *b, int *tail_b,
                                                            int *tot_b, int n) {
+  pdl_trigger();
+  pdl_wait();
   if (blockIdx.x) scan_one(b, b, n, tail_b, tot_b); else scan_one(a, a, n, tail_a, tot_a);
 }
 static const int SCAN_ONE_MAX = 3 * SCAN_ONE_BS * SCAN_ONE_IT;
@@ -139,7 +147,7 @@ void rs_scan_dev(const int *in, int *out, int n, int *tail, int *tot2, cudaStrea
     return;
   }
   if (n <= SCAN_ONE_MAX) {
-    k_scan_one<<<1, SCAN_ONE_BS, 0, s>>>(in, out, n, tail, tot2);
+    launch_small(k_scan_one, 1, SCAN_ONE_BS, 0, s, in, out, n, tail, tot2);
     RS_LAUNCHED(1);
     RS_CHECK_LAUNCH();
     return;
@@ -148,8 +156,8 @@ void rs_scan_dev(const int *in, int *out, int n, int *tail, int *tot2, cudaStrea
   static thread_local dbuf<int> own;
   dbuf<int> &part = scratch ? *scratch : own;
   part.ensure(nblk + 1);
-  k_scan_partials<<<nblk, SCAN_BS, 0, s>>>(in, n, part.p);
-  k_scan_final<<<nblk, SCAN_BS, 0, s>>>(in, out, n, part.p, nblk, tail, tot2);
+  launch_small(k_scan_partials, nblk, SCAN_BS, 0, s, in, n, part.p);
+  launch_small(k_scan_final, nblk, SCAN_BS, 0, s, in, out, n, part.p, nblk, tail, tot2);
   RS_LAUNCHED(2);
   RS_CHECK_LAUNCH();
 }
@@ -159,7 +167,7 @@ void rs_scan_dev2(int *a, int *tail_a, int *tot_a, int *b, int *tail_b, int *tot
     rs_scan_dev(b, b, n, tail_b, tot_b, s);
     return;
   }
-  k_scan_one2<<<2, SCAN_ONE_BS, 0, s>>>(a, tail_a, tot_a, b, tail_b, tot_b, n);
+  launch_small(k_scan_one2, 2, SCAN_ONE_BS, 0, s, a, tail_a, tot_a, b, tail_b, tot_b, n);
   RS_LAUNCHED(1);
   RS_CHECK_LAUNCH();
 }
@@ -233,12 +241,14 @@ void rs_dots(const double *const *x, const double *const *y, int m, int n, doubl
 }
 
 template <class T> __global__ void k_fill(T *p, T v, size_t n) {
+  pdl_trigger();
+  pdl_wait();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) p[i] = v;
 }
 static unsigned gs(size_t n) { size_t g = (n + 255) / 256; return (unsigned)(g < 1 ? 1 : (g > 4096 ? 4096 : g)); }
-void rs_fill_i(int *p, int v, size_t n, cudaStream_t s) { if (n) { k_fill<<<gs(n), 256, 0, s>>>(p, v, n); RS_LAUNCHED(1); } }
-void rs_fill_d(double *p, double v, size_t n, cudaStream_t s) { if (n) { k_fill<<<gs(n), 256, 0, s>>>(p, v, n); RS_LAUNCHED(1); } }
-void rs_fill_f(float *p, float v, size_t n, cudaStream_t s) { if (n) { k_fill<<<gs(n), 256, 0, s>>>(p, v, n); RS_LAUNCHED(1); } }
+void rs_fill_i(int *p, int v, size_t n, cudaStream_t s) { if (n) { launch_small(k_fill<int>, gs(n), 256, 0, s, p, v, n); RS_LAUNCHED(1); } }
+void rs_fill_d(double *p, double v, size_t n, cudaStream_t s) { if (n) { launch_small(k_fill<double>, gs(n), 256, 0, s, p, v, n); RS_LAUNCHED(1); } }
+void rs_fill_f(float *p, float v, size_t n, cudaStream_t s) { if (n) { launch_small(k_fill<float>, gs(n), 256, 0, s, p, v, n); RS_LAUNCHED(1); } }
 __global__ void k_d2f(const double *a, float *b, size_t n) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) b[i] = (float)a[i];
 }
