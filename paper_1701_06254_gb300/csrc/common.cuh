@@ -300,8 +300,8 @@ struct sim_ls_s {
   dbuf<float> w2, isp;          // double-float w planes; split 1 / h_{j+1,j}
   dbuf<int> ticket;             // last-block ticket of the Gram-Schmidt sweeps (zero between launches)
   dbuf<float> vallo;            // lo plane of the decoupled matrix (hi: val32)
-  dbuf<double> bcg;             // BiCGSTAB vectors: rh, p, v, s, t, ph, sh, x (2 nb each)
-  dbuf<float> bcg32;            // mixed precision: the FP32 preconditioned vector
+  dbuf<double> bcg;             // BiCGSTAB: rh, p, v, s, t (2 nb each), scalars, partial sums, FP64: ph, sh
+  dbuf<float> bcg32;            // mixed precision: the FP32 preconditioned vectors ph, sh
   dbuf<float> cprt32;           // CPR: the first RAS stage's output (FP32)
   // timer brackets recorded inside the graph (event nodes): pairs of events
   // and the family of each pair, read back after every replay

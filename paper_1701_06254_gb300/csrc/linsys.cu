@@ -1135,39 +1135,175 @@ __global__ void k_xupdate(int nu, int jend, const double *yk, const Tz *Z, doubl
 // Right-preconditioned BiCGSTAB (van der Vorst), the paper's other Krylov
 // method (its Examples 3, 6 and 7): two CPR applications per iteration.
 // FP64 vectors throughout; in mixed precision the preconditioner returns an
-// FP32 vector, widened to FP64 before its product with A.
-__global__ void k_bcg_p(int nu, const double *r, const double *v, double beta, double omega, double *p) {
+// FP32 vector (Tz), which the product with A and the update of x widen.
+//
+// The scalars stay on the device (sc = {rho, alpha, omega, beta}); the host
+// learns of them through two pinned slots per iteration, after s (slot 0:
+// {(rh, v), (s, s)}) and after r (slot 1: {omega, (r, r), (rh, r)}), and polls
+// those.  Each vector update also adds up the dot products that follow it,
+// summed like rs_dots (the grid of k_dot_partials, the last block as
+// k_sum_partials), so the bits do not depend on where they are taken.  With a
+// synchronisation after each of six products, and kernels of their own for
+// each of them and for the widening, an iteration spent 170 us outside CPR
+// and A x (150k cells), now 115 (25.3 -> 23.1 ms per step).
+constexpr int BCG_BS = 256, BCG_U = 4;
+static int bcg_blocks(int nu) { return std::min(std::max((nu + 4095) / 4096, 1), 1024); }
+__device__ __forceinline__ double bcg_block_sum(double s) {           // BCG_BS threads; the sum in thread 0
+  __shared__ double sh[BCG_BS / 32];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    s = threadIdx.x < BCG_BS / 32 ? sh[threadIdx.x] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  }
+  return s;
+}
+// s[k] of all threads of the grid added up; true in one thread, which has the totals
+template <int ND> __device__ __forceinline__ bool bcg_total(double (&s)[ND], double *part, int *ticket) {
+#pragma unroll
+  for (int k = 0; k < ND; k++) {
+    const double b = bcg_block_sum(s[k]);
+    if (threadIdx.x == 0) part[k * gridDim.x + blockIdx.x] = b;
+  }
+  if (!last_block(ticket)) return false;
+#pragma unroll
+  for (int k = 0; k < ND; k++) {
+    double t = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += BCG_BS) t += __ldcg(part + k * gridDim.x + i);
+    s[k] = bcg_block_sum(t);
+  }
+  if (threadIdx.x != 0) return false;
+  *ticket = 0;
+  return true;
+}
+__device__ __forceinline__ void bcg_post(volatile double *host, double a, double b, double c) {
+  host[0] = a; host[1] = b; host[2] = c;
+  __threadfence_system();
+  host[3] = 1.0;
+}
+// elements i0 + u * step of the thread, BCG_U at a time: f loads, g uses them in order
+template <class T, class F, class G> __device__ __forceinline__ void bcg_each(int nu, F f, G g) {
+  const int step = gridDim.x * BCG_BS;
+  for (int i0 = blockIdx.x * BCG_BS + threadIdx.x; i0 < nu; i0 += BCG_U * step) {
+    T a[BCG_U];
+#pragma unroll
+    for (int u = 0; u < BCG_U; u++) if ((long long)i0 + (long long)u * step < nu) a[u] = f(i0 + u * step);
+#pragma unroll
+    for (int u = 0; u < BCG_U; u++) if ((long long)i0 + (long long)u * step < nu) g(i0 + u * step, a[u]);
+  }
+}
+// rh = r, p = v = 0, rho = (rh, r); alpha = omega = the previous rho = 1
+__global__ void __launch_bounds__(BCG_BS) k_bcg_start(int nu, const double *r, double *rh, double *p, double *v,
+                                                      double *part, int *ticket, double *sc, volatile double *host) {
+  double s[1] = {0.0};
+  bcg_each<double>(nu, [&](int i) { return r[i]; }, [&](int i, double a) {
+    rh[i] = a; p[i] = 0.0; v[i] = 0.0;
+    s[0] += a * a;
+  });
+  if (bcg_total(s, part, ticket)) {
+    sc[0] = s[0]; sc[1] = 1.0; sc[2] = 1.0; sc[3] = s[0];
+    bcg_post(host, 1.0, 0.0, s[0]);
+  }
+}
+__global__ void k_bcg_p(int nu, const double *r, const double *v, const double *sc, double *p) {
+  pdl_trigger();
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const double omega = sc[2], beta = sc[3];
   if (i < nu) p[i] = r[i] + beta * (p[i] - omega * v[i]);
 }
-__global__ void k_bcg_s(int nu, const double *r, const double *v, double alpha, double *s) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nu) s[i] = r[i] - alpha * v[i];
+// alpha = rho / (rh, v)
+__global__ void __launch_bounds__(BCG_BS) k_bcg_rv(int nu, const double *rh, const double *v, double *part, int *ticket,
+                                                   double *sc) {
+  pdl_trigger();
+  pdl_wait();
+  double s[1] = {0.0};
+  bcg_each<double2>(nu, [&](int i) { return make_double2(rh[i], v[i]); }, [&](int, double2 a) { s[0] += a.x * a.y; });
+  if (bcg_total(s, part, ticket)) { sc[1] = sc[0] / s[0]; sc[4] = s[0]; }
 }
-__global__ void k_bcg_xr(int nu, double alpha, const double *ph, double omega, const double *sh, const double *s,
-                         const double *t, double *x, double *r) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nu) { x[i] += alpha * ph[i] + omega * sh[i]; r[i] = s[i] - omega * t[i]; }
+// s = r - alpha v, (s, s)
+__global__ void __launch_bounds__(BCG_BS) k_bcg_s(int nu, const double *r, const double *v, double *sv, double *part,
+                                                  int *ticket, const double *sc, volatile double *host) {
+  pdl_trigger();
+  pdl_wait();
+  const double alpha = sc[1];
+  double s[1] = {0.0};
+  bcg_each<double2>(nu, [&](int i) { return make_double2(r[i], v[i]); }, [&](int i, double2 a) {
+    const double x = a.x - alpha * a.y;
+    sv[i] = x;
+    s[0] += x * x;
+  });
+  if (bcg_total(s, part, ticket)) bcg_post(host, sc[4], s[0], 0.0);
 }
-__global__ void k_bcg_xa(int nu, double alpha, const double *ph, double *x) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nu) x[i] += alpha * ph[i];
+// omega = (t, s) / (t, t), 0 without t
+__global__ void __launch_bounds__(BCG_BS) k_bcg_t(int nu, const double *t, const double *sv, double *part, int *ticket,
+                                                  double *sc) {
+  pdl_trigger();
+  pdl_wait();
+  double s[2] = {0.0, 0.0};
+  bcg_each<double2>(nu, [&](int i) { return make_double2(t[i], sv[i]); }, [&](int, double2 a) {
+    s[0] += a.x * a.x;
+    s[1] += a.x * a.y;
+  });
+  if (bcg_total(s, part, ticket)) sc[2] = s[0] > 0.0 ? s[1] / s[0] : 0.0;
 }
-__global__ void k_widen(int nu, const float *a, double *b) {
+// x += alpha ph + omega sh, r = s - omega t, (r, r), the next rho = (rh, r) and beta
+template <class Tz> struct bcg_row { double s, t, x, rh; Tz ph, sh; };
+template <class Tz>
+__global__ void __launch_bounds__(BCG_BS) k_bcg_xr(int nu, const Tz *ph, const Tz *sh, const double *sv, const double *t,
+                                                   const double *rh, double *x, double *r, double *part, int *ticket,
+                                                   double *sc, volatile double *host) {
+  pdl_trigger();
+  pdl_wait();
+  const double rho = sc[0], alpha = sc[1], omega = sc[2];
+  double s[2] = {0.0, 0.0};
+  bcg_each<bcg_row<Tz>>(nu, [&](int i) { return bcg_row<Tz>{sv[i], t[i], x[i], rh[i], ph[i], sh[i]}; },
+                        [&](int i, const bcg_row<Tz> &a) {
+    x[i] = a.x + (alpha * (double)a.ph + omega * (double)a.sh);
+    const double y = a.s - omega * a.t;
+    r[i] = y;
+    s[0] += y * y;
+    s[1] += a.rh * y;
+  });
+  if (bcg_total(s, part, ticket)) {
+    sc[0] = s[1];
+    sc[3] = (s[1] / rho) * (alpha / omega);
+    bcg_post(host, omega, s[0], s[1]);
+  }
+}
+template <class Tz> __global__ void k_bcg_xa(int nu, const double *sc, const Tz *ph, double *x) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nu) b[i] = (double)a[i];
+  if (i < nu) x[i] += sc[1] * (double)ph[i];
 }
 
-// z = M^-1 v (CPR-FPF) in FP64
-static void bcg_precond(sim_ls_s *ls, const double *v, double *z) {
-  int nu = 2 * ls->nb;
-  if (ls->o.precision != SIM_PREC_FP64) {
-    ls_cpr(ls, v, nullptr, ls->bcg32.p);
-    k_widen<<<grid_for(nu, 256), 256, 0, ls->st>>>(nu, ls->bcg32.p, z);
-    RS_LAUNCHED(1);
-  } else {
-    ls_cpr(ls, v, z, nullptr);
+// z = M^-1 v (CPR-FPF), y = A z
+static void bcg_product(sim_ls_s *ls, const double *v, double *z, double *y) {
+  ls_cpr(ls, v, z, nullptr);
+  ls_spmv64(ls, z, y);
+}
+static void bcg_product(sim_ls_s *ls, const double *v, float *z, double *y) {
+  ls_cpr(ls, v, nullptr, z);
+  rs_timed tm(ls, SIM_T_SPMV64);
+  spmv<double, float, double, double>(ls, ls->val.p, z, (const double *)nullptr, y, ls->st);
+}
+
+// Wait until the device has completed a step's pinned slot.  The Givens column
+// is written while the step's last kernel is still scaling the next basis
+// vector, so the decision is taken and the next step queued before the GPU
+// runs dry (a stream synchronisation left it idle for some 8 us per step).
+// The stream is asked now and then, so that a failed launch ends the wait.
+static void wait_slot(const volatile double *done, cudaStream_t s) {
+  for (unsigned it = 1; *done == 0.0; it++) {
+    if (it % 64 == 0) std::this_thread::yield();
+    if (it % 4096 == 0) {
+      const cudaError_t e = cudaStreamQuery(s);
+      if (e == cudaSuccess) break;
+      if (e != cudaErrorNotReady) RS_CUDA(e);
+    }
   }
+  std::atomic_thread_fence(std::memory_order_acquire);
 }
 
 // Solves A M^-1 u = b, x = M^-1 u, from x = 0 or from the initial guess in
@@ -1176,14 +1312,30 @@ static void bcg_precond(sim_ls_s *ls, const double *v, double *z) {
 // b - A x; when that misses the tolerance, or on a breakdown (rho, (rh, v)
 // or omega zero), it restarts from the true residual with rh = r.  At most
 // max_lin iterations.  0 = converged, 1 = iteration cap, 2 = non-finite.
+template <class Tz>
 static int ls_solve_bicgstab(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
   cudaStream_t st = ls->st;
   int nu = 2 * ls->nb, maxit = ls->o.max_lin, its = 0, rc = 1;
-  ls->bcg.ensure(8 * (size_t)nu);
-  if (ls->o.precision != SIM_PREC_FP64) ls->bcg32.ensure(nu);
-  double *rh = ls->bcg.p, *p = rh + nu, *v = p + nu, *sv = v + nu, *t = sv + nu, *ph = t + nu, *sh = ph + nu;
+  const int nblk = bcg_blocks(nu);
+  const bool pdl = arnoldi_pdl(ls->nb);
+  ls->bcg.ensure((sizeof(Tz) == 8 ? 7 : 5) * (size_t)nu + 8 + 2 * (size_t)nblk);
+  double *rh = ls->bcg.p, *p = rh + nu, *v = p + nu, *sv = v + nu, *t = sv + nu, *sc = t + nu, *part = sc + 8;
+  Tz *ph, *sh;
+  if constexpr (sizeof(Tz) == 8) { ph = part + 2 * (size_t)nblk; sh = ph + nu; }
+  else { ls->bcg32.ensure(2 * (size_t)nu); ph = ls->bcg32.p; sh = ph + nu; }
+  if (!ls->ticket.p) { ls->ticket.ensure(1); RS_CUDA(cudaMemsetAsync(ls->ticket.p, 0, sizeof(int), st)); }
+  int *tk = ls->ticket.p;
+  volatile double *hp = ls->hpin;
+  double *hp_dev = nullptr;
+  RS_CUDA(cudaHostGetDevicePointer((void **)&hp_dev, ls->hpin, 0));
   double *x = ls->y.p, *r = ls->r.p;
   unsigned g = grid_for(nu, 256);
+  auto go = [&](auto kern, auto... a) { launch_pdl_if(pdl, kern, nblk, BCG_BS, 0, st, nu, a...); RS_LAUNCHED(1); };
+  auto expect = [&](int slot) { hp[4 * slot + 3] = 0.0; return hp_dev + 4 * slot; };
+  auto wait = [&](int slot) {
+    if (ls->timer_mask) RS_CUDA(cudaStreamSynchronize(st));
+    else wait_slot(hp + 4 * slot + 3, st);
+  };
   double bn = rs_norm2(ls->b.p, nu, st), rn = bn;
   if (bn == 0.0) { rs_fill_d(x, 0.0, nu, st); *its_out = 0; *relres = 0.0; return 0; }
   if (!std::isfinite(bn)) { rs_fill_d(x, 0.0, nu, st); *its_out = 0; *relres = NAN; return 2; }
@@ -1201,50 +1353,46 @@ static int ls_solve_bicgstab(sim_ls_s *ls, double tol, int *its_out, double *rel
     if (ls->errw[0]) RS_FAIL(SIM_ERR_TIMEOUT, "RAS setup gave up (code %d)", ls->errw[0]);
   };
   for (;;) {
-    RS_CUDA(cudaMemcpyAsync(rh, r, nu * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    rs_fill_d(p, 0.0, nu, st); rs_fill_d(v, 0.0, nu, st);
-    double rho_prev = 1.0, alpha = 1.0, omega = 1.0;
+    launch_pdl_if(false, k_bcg_start, nblk, BCG_BS, 0, st, nu, r, rh, p, v, part, tk, sc, expect(1));
+    RS_LAUNCHED(1);
+    RS_CHECK_LAUNCH();
+    wait(1);
     bool broke = false, done = false;
     while (its < maxit) {
-      double rho;
-      { const double *xs[1] = {rh}, *ys[1] = {r}; rs_dots(xs, ys, 1, nu, &rho, st); }
+      const double rho = hp[4 + 2];
       if (!std::isfinite(rho)) { *its_out = its; *relres = NAN; return 2; }
       if (rho == 0.0) { broke = true; break; }
-      double beta = (rho / rho_prev) * (alpha / omega);
-      k_bcg_p<<<g, 256, 0, st>>>(nu, r, v, beta, omega, p);
+      launch_pdl_if(pdl, k_bcg_p, g, 256, 0, st, nu, r, v, sc, p);
       RS_LAUNCHED(1);
-      bcg_precond(ls, p, ph);
-      ls_spmv64(ls, ph, v);
-      double rv;
-      { const double *xs[1] = {rh}, *ys[1] = {v}; rs_dots(xs, ys, 1, nu, &rv, st); }
+      bcg_product(ls, p, ph, v);
+      go(k_bcg_rv, rh, v, part, tk, sc);
+      go(k_bcg_s, r, v, sv, part, tk, sc, expect(0));
+      RS_CHECK_LAUNCH();
+      wait(0);
       check();
+      const double rv = hp[0];
       if (!std::isfinite(rv)) { *its_out = its; *relres = NAN; return 2; }
       if (rv == 0.0) { broke = true; break; }
-      alpha = rho / rv;
-      k_bcg_s<<<g, 256, 0, st>>>(nu, r, v, alpha, sv);
-      RS_LAUNCHED(1);
       its++;
-      double sn = rs_norm2(sv, nu, st);
+      const double sn = std::sqrt((double)hp[1]);
       if (!std::isfinite(sn)) { *its_out = its; *relres = NAN; return 2; }
       if (sn <= tol * bn) {
-        k_bcg_xa<<<g, 256, 0, st>>>(nu, alpha, ph, x);
+        launch_pdl_if(false, k_bcg_xa<Tz>, g, 256, 0, st, nu, sc, ph, x);
         RS_LAUNCHED(1);
         done = true;
         break;
       }
-      bcg_precond(ls, sv, sh);
-      ls_spmv64(ls, sh, t);
-      double tt_ts[2];
-      { const double *xs[2] = {t, t}, *ys[2] = {t, sv}; rs_dots(xs, ys, 2, nu, tt_ts, st); }
+      bcg_product(ls, sv, sh, t);
+      go(k_bcg_t, t, sv, part, tk, sc);
+      go(k_bcg_xr<Tz>, ph, sh, sv, t, rh, x, r, part, tk, sc, expect(1));
+      RS_CHECK_LAUNCH();
+      wait(1);
       check();
-      omega = tt_ts[0] > 0.0 ? tt_ts[1] / tt_ts[0] : 0.0;
-      k_bcg_xr<<<g, 256, 0, st>>>(nu, alpha, ph, omega, sh, sv, t, x, r);
-      RS_LAUNCHED(1);
-      rn = rs_norm2(r, nu, st);
+      const double omega = hp[4];
+      rn = std::sqrt((double)hp[4 + 1]);
       if (!std::isfinite(rn)) { *its_out = its; *relres = NAN; return 2; }
       if (rn <= tol * bn) { done = true; break; }
       if (omega == 0.0) { broke = true; break; }
-      rho_prev = rho;
     }
     // true residual r = b - A x
     spmv<double, double, double, double>(ls, ls->val.p, x, ls->b.p, r, st);
@@ -1276,25 +1424,10 @@ __global__ void k_loop_cond(cudaGraphConditionalHandle h, const int *jd, const d
 }
 __global__ void k_loop_params(double *lp, double thr, double cap) { lp[0] = thr; lp[1] = cap; lp[2] = 0.0; lp[3] = 0.0; }
 
-// Wait until the device has completed a step's pinned slot.  The Givens column
-// is written while the step's last kernel is still scaling the next basis
-// vector, so the decision is taken and the next step queued before the GPU
-// runs dry (a stream synchronisation left it idle for some 8 us per step).
-// The stream is asked now and then, so that a failed launch ends the wait.
-static void wait_slot(const volatile double *done, cudaStream_t s) {
-  for (unsigned it = 1; *done == 0.0; it++) {
-    if (it % 64 == 0) std::this_thread::yield();
-    if (it % 4096 == 0) {
-      const cudaError_t e = cudaStreamQuery(s);
-      if (e == cudaSuccess) break;
-      if (e != cudaErrorNotReady) RS_CUDA(e);
-    }
-  }
-  std::atomic_thread_fence(std::memory_order_acquire);
-}
-
 int ls_solve(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
-  if (ls->o.krylov == SIM_KRYLOV_BICGSTAB) return ls_solve_bicgstab(ls, tol, its_out, relres, x0);
+  if (ls->o.krylov == SIM_KRYLOV_BICGSTAB)
+    return ls->o.precision == SIM_PREC_FP64 ? ls_solve_bicgstab<double>(ls, tol, its_out, relres, x0)
+                                            : ls_solve_bicgstab<float>(ls, tol, its_out, relres, x0);
   cudaStream_t s = ls->st;
   int nu = 2 * ls->nb, m = std::min(ls->o.restart, ORTHO_MAXV - 1), maxit = ls->o.max_lin;
   // df: double-float Arnoldi basis (its kernels use 32-bit offsets into the
