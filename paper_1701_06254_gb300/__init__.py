@@ -609,7 +609,7 @@ class WarmStart:
         _check(self._L.sim_ws_zero_grad(self.h))
 
     def use_tcgen05(self, on=True):
-        """tcgen05 or mma.sync (default) kernels for the forward / data-gradient convolutions."""
+        """tcgen05 (default) or mma.sync kernels for the forward / data-gradient convolutions (same bits)."""
         _check(self._L.sim_ws_use_tcgen05(self.h, 1 if on else 0))
 
     def adam(self, lr):

@@ -982,7 +982,10 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update_df(int nu, int ch,
 // hnorm[0]; previous Givens rotations, a new one, and the residual estimate
 // |g_{j+1}| (host: the step's pinned slot).  One warp; the rotations are a
 // serial recurrence of four FP64 operations a step, which two lanes share
-// (each operation holds the FP64 pipe for 64 cycles).
+// (each operation holds the FP64 pipe for 64 cycles).  The roundings are
+// written out: in mixed precision a difference in the last bit reaches the
+// next cycle's residual and its FP32 copy, and a system that needs several
+// cycles then takes another path (155k cells, 92 against 95 iterations).
 // G layout: [0..m*(m+1)) H column-major (m+1 per column), cs[m], sn[m], g[m+1]
 __device__ __forceinline__ void arnoldi_col(int j, int m, const double *h1, const double *h2, const int *flag,
                                             const double *hnorm, double *G, volatile double *host) {
@@ -997,12 +1000,12 @@ __device__ __forceinline__ void arnoldi_col(int j, int m, const double *h1, cons
   const double hn = hnorm[0];
   double a = sc[0];
   for (int k = 0; k < j; k++) {                  // lane 0: the rotated entry k, lane 1: what goes on to k + 1
-    const double x = (lane & 1) ? -ssn[k] : scs[k], y = (lane & 1) ? scs[k] : ssn[k];
-    const double t = x * a + y * sc[k + 1];
+    const double b = sc[k + 1], t = (lane & 1) ? __fma_rn(scs[k], b, -__dmul_rn(ssn[k], a))
+                                               : __fma_rn(scs[k], a, __dmul_rn(ssn[k], b));
     a = __shfl_sync(0xffffffffu, t, 1);
     if (lane == 0) col[k] = t;
   }
-  const double rr = sqrt(a * a + hn * hn), q = ((lane & 1) ? hn : a) / rr;
+  const double rr = sqrt(__fma_rn(hn, hn, __dmul_rn(a, a))), q = ((lane & 1) ? hn : a) / rr;
   const double sj = __shfl_sync(0xffffffffu, q, 1);
   if (lane != 0) return;
   cs[j] = q; sn[j] = sj;

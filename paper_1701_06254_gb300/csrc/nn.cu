@@ -15,19 +15,18 @@
 // contiguous ([v][C], v = i + nx (j + ny k), the simulator's cell order).
 // The network input has 16 channels (8 used; the rest stay zero so every
 // contraction is a whole number of 16-wide MMA steps).  Weights: FP32 master
-// copy [27][Co][Ci] (+ Adam moments), and two BF16 copies made after every
+// copy [27][Co][Ci] (+ Adam moments), and two BF16 copies made with every
 // update: [27][Co][Ci] for the forward pass and the tap-flipped transpose
-// [26-t][Ci][Co] for the data gradient, which is then the same kernel.
+// [26-t][Ci][Co] for the data gradient, which is then the same kernel; both
+// stored as the core matrices of the MMAs' descriptors (woffs).
 //
-// Every contraction runs on the tensor cores: mma.sync m16n8k16 BF16 with
-// FP32 accumulation.  The forward/data-gradient kernel is an implicit GEMM
-// (M = voxels, N = output channels, K = 27 taps x input channels): each tap's
-// shifted input rows and weight slice are staged in shared memory with
-// cp.async (zero-fill outside the grid), double buffered across taps, and
-// fed to the MMAs with ldmatrix.  The weight-gradient kernel contracts over
-// voxels (M = output channels, N = input channels) with ldmatrix.trans from
-// the voxel-major tiles, one CTA per (voxel chunk, tap), partials reduced in
-// a fixed order so results do not depend on scheduling.
+// Every contraction runs on the tensor cores, BF16 with FP32 accumulation.
+// The forward / data-gradient kernel is an implicit GEMM (M = voxels, N =
+// output channels, K = 27 taps x input channels) on tcgen05, fed from one
+// halo copy per tile (k_conv_tc); k_conv and k_conv_halo are the same
+// contraction with mma.sync m16n8k16, in the same order.  The weight-gradient
+// kernel contracts over voxels for all layers in one launch, partials reduced
+// in a fixed order so results do not depend on scheduling.
 #include "common.cuh"
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
@@ -351,7 +350,11 @@ __global__ void __launch_bounds__(128) k_conv_halo(int nx, int ny, int nz, const
 
 // ------------------------------------------ implicit-GEMM conv, tcgen05 ---
 // The same contraction on the 5th-generation tensor cores, the operands of
-// all 27 taps taken from one copy of the input halo in shared memory.
+// all 27 taps taken from one copy of the input halo in shared memory.  Bound
+// by the MMAs' shared-memory reads (M = 128, N = 32, K = 16: 5 KB, 40 cycles
+// measured) and, on small grids, by the chain copy -> MMAs -> store.  Under
+// ncu with cold caches, 32 -> 32 channels: 65,536 voxels 11.3 us (28 with
+// k_conv_halo), 128 voxels 5.9; 64 -> 32 at 136,091 voxels 39 us.
 //
 // A CTA owns an 8 x 16 x NZ box of output voxels; each z slice is one M = 128
 // accumulator of CO columns in TMEM (row r = x + 8 y).  The halo lies in
@@ -362,10 +365,11 @@ __global__ void __launch_bounds__(128) k_conv_halo(int nx, int ny, int nz, const
 // shifted start address, and nothing is gathered per tap; a plane's pad
 // keeps the copies' writes free of bank conflicts.  The weights of all taps
 // come by one bulk copy (they are stored as core matrices), issued before
-// the wait for the kernel that makes X.  One thread issues the 27 x CI / 16
-// x NZ MMAs, K ascending within each tap as in k_conv, slices innermost; the
-// results are the same bits as with mma.sync.  Epilogue: tcgen05.ld, thread
-// = voxel row, bias / ReLU or the data-gradient mask.  Every wait is
+// the wait for the kernel that makes X.  The ninth warp
+// issues a slice's 27 x CI / 16 MMAs, K ascending within each tap as in
+// k_conv, once its three halo slices are there; the results are the same bits
+// as with mma.sync.  Epilogue, while the next slice is contracted: tcgen05.ld,
+// thread = voxel row, bias / ReLU or the data-gradient mask.  Every wait is
 // bounded; on a timeout the kernel records an error and writes nothing.
 __device__ __forceinline__ uint64_t tc_desc(unsigned saddr, unsigned lbo, unsigned sbo) {
   uint64_t d = 0;
@@ -645,7 +649,9 @@ __global__ void __launch_bounds__(TC_T) k_conv_tc(int nx, int ny, int nz, int NZ
 // start of a column only load.  Eight warps copy two steps ahead, the ninth
 // issues the MMAs; after WFL slices (64 MMAs on an accumulator) all twelve
 // move the sums to FP32 registers, one z shift per four warps, so that the
-// tensor cores' accumulation chains stay short.
+// tensor cores' accumulation chains stay short.  One CTA per SM (TMEM and
+// registers).  All 15 layers of a 64x64x16 grid: 59 us, where a launch per
+// layer with mma.sync and its reduction took 507.
 constexpr int WYP = THY + 1, WYB = TBY + 1;                      // y pitches, odd: copies free of bank conflicts
 constexpr int WR = 6, WSLOT = WR + 2;                            // dZ ring: slots, with the two copies
 constexpr int WA_BYTES = 11 * 4 * WYP * 16 + 64, WNS = 4, WLA = 2, WFL = 8;
