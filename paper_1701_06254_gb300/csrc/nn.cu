@@ -32,6 +32,7 @@
 #include <cuda_bf16.h>
 #include <algorithm>
 #include <cmath>
+#include <utility>
 #include <memory>
 #include <mutex>
 
@@ -1749,13 +1750,17 @@ __global__ void k_ws_target(int n, const double *y, const double *sc, float *T) 
 // rms over the n cells of the two interleaved components of v -> out[0], out[1].
 // One cluster of eight CTAs, whose partial sums the first adds through
 // distributed shared memory: no workspace and a fixed order.  With a single
-// CTA its SM's FP64 pipe and latency bounded the sum.
+// CTA its SM's FP64 pipe and latency bounded the sum.  Another CTA's shared
+// memory may be written only once that CTA runs: every thread arrives on the
+// cluster's barrier at the start and waits for it before the store, so that
+// the summation hides the barrier; the second barrier ends the stores.
 constexpr int RMS_C = 8, RMS_U = 4;
 __global__ void __cluster_dims__(RMS_C, 1, 1) __launch_bounds__(1024) k_rms2(int n, const double *v, double *out) {
   __shared__ double sh[2][32];
   __shared__ double all[2][RMS_C];
   cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
   const int t = threadIdx.x, rank = (int)cl.block_rank(), step = RMS_C * 1024;
+  auto running = cl.barrier_arrive();
   double s0 = 0.0, s1 = 0.0;
   for (int c0 = rank * 1024 + t; c0 < n; c0 += RMS_U * step) {
     double2 a[RMS_U];
@@ -1772,6 +1777,7 @@ __global__ void __cluster_dims__(RMS_C, 1, 1) __launch_bounds__(1024) k_rms2(int
   s0 = warp_sum(s0); s1 = warp_sum(s1);
   if ((t & 31) == 0) { sh[0][t >> 5] = s0; sh[1][t >> 5] = s1; }
   __syncthreads();
+  cl.barrier_wait(std::move(running));                 // all eight CTAs run
   if (t < 64) {
     const double x = warp_sum(sh[t >> 5][t & 31]);
     if ((t & 31) == 0) *cl.map_shared_rank(&all[t >> 5][rank], 0) = x;
