@@ -1127,14 +1127,25 @@ struct sim_ws_s {
   std::vector<std::unique_ptr<sample>> data;
   size_t max_samples = 1u << 30;
   unsigned long long seed = 0;
-  std::mutex use;                         // one caller at a time (activations are shared)
+  std::mutex use;                         // one caller at a time (activations are shared): see ws_turn
+  cudaEvent_t last = nullptr;             // the last simulator's reads of the output, on its own stream
   bool tc = true;                         // tcgen05 convolutions (else mma.sync)
   int *err = nullptr, *err_dev = nullptr; // host-mapped: set by a kernel whose bounded wait gave up
   pack_table tab;
   ~sim_ws_s() {
     if (st) cudaStreamDestroy(st);
+    if (last) cudaEventDestroy(last);
     if (err) cudaFreeHost(err);
   }
+};
+
+// A caller's turn on the handle: the host lock, and stream s (the stream of
+// its first access to the activations) behind the last simulator's reads of
+// them.  ws_predict returns with its GPU work queued on two streams, so the
+// lock alone would let the next caller write what that work still reads.
+struct ws_turn {
+  std::lock_guard<std::mutex> guard;
+  ws_turn(sim_ws_s *w, cudaStream_t s) : guard(w->use) { RS_CUDA(cudaStreamWaitEvent(s, w->last, 0)); }
 };
 
 namespace nn {
@@ -1488,6 +1499,7 @@ extern "C" sim_status sim_ws_create(sim_ws_t *out, unsigned long long seed) {
   *out = nullptr;
   std::unique_ptr<sim_ws_s> w(new sim_ws_s());
   RS_CUDA(cudaStreamCreateWithFlags(&w->st, cudaStreamNonBlocking));
+  RS_CUDA(cudaEventCreateWithFlags(&w->last, cudaEventDisableTiming));
   ws_layout(w.get());
   w->seed = seed;
   // He-normal weights (std sqrt(2 / (27 ci))), zero biases; padding channels
@@ -1538,6 +1550,7 @@ extern "C" sim_status sim_ws_params(sim_ws_t w, int which, float *dst, size_t n,
   if (needed) *needed = ne;
   if (!dst) return SIM_OK;
   if (n < ne) RS_FAIL(SIM_ERR_ARG, "sim_ws_params: buffer holds %zu of %zu values", n, ne);
+  ws_turn turn(w, w->st);
   w->E.ensure(ne);
   k_export<<<grid_for(ne, 256), 256, 0, w->st>>>((int)ne, which == 0 ? w->P.p : w->G.p,
                                                 which == 1 && w->accum > 0 ? (float)w->accum : 1.f, w->E.p);
@@ -1561,6 +1574,7 @@ extern "C" sim_status sim_ws_set_params(sim_ws_t w, const float *src, size_t n) 
         for (int c = 0; c < ct; c++) h[w->woff[l] + ((size_t)t * co + o) * ci + c] = src[q++];
     for (int o = 0; o < co; o++) h[w->boff[l] + o] = src[q++];
   }
+  ws_turn turn(w, w->st);
   RS_CUDA(cudaMemcpyAsync(w->P.p, h.data(), w->np * sizeof(float), cudaMemcpyHostToDevice, w->st));
   RS_CUDA(cudaMemsetAsync(w->M.p, 0, w->np * sizeof(float), w->st));
   RS_CUDA(cudaMemsetAsync(w->Vm.p, 0, w->np * sizeof(float), w->st));
@@ -1583,6 +1597,7 @@ static void load_features(sim_ws_s *w, dims d, const float *feat) {
 extern "C" sim_status sim_ws_forward(sim_ws_t w, int nx, int ny, int nz, const float *feat, float *y) {
   ABI_BEGIN
   if (!w || !feat || !y || nx < 1 || ny < 1 || nz < 1) RS_FAIL(SIM_ERR_ARG, "sim_ws_forward: bad argument");
+  ws_turn turn(w, w->st);
   dims d = {nx, ny, nz};
   load_features(w, d, feat);
   forward(w);
@@ -1599,6 +1614,7 @@ extern "C" sim_status sim_ws_backward(sim_ws_t w, int nx, int ny, int nz, const 
                                       double *loss) {
   ABI_BEGIN
   if (!w || !feat || !target || nx < 1 || ny < 1 || nz < 1) RS_FAIL(SIM_ERR_ARG, "sim_ws_backward: bad argument");
+  ws_turn turn(w, w->st);
   dims d = {nx, ny, nz};
   load_features(w, d, feat);
   size_t V = d.V();
@@ -1618,6 +1634,7 @@ extern "C" sim_status sim_ws_backward(sim_ws_t w, int nx, int ny, int nz, const 
 extern "C" sim_status sim_ws_zero_grad(sim_ws_t w) {
   ABI_BEGIN
   if (!w) RS_FAIL(SIM_ERR_ARG, "NULL handle");
+  ws_turn turn(w, w->st);
   zero_grad(w);
   RS_CUDA(cudaStreamSynchronize(w->st));
   ABI_END
@@ -1626,6 +1643,7 @@ extern "C" sim_status sim_ws_zero_grad(sim_ws_t w) {
 extern "C" sim_status sim_ws_adam(sim_ws_t w, double lr) {
   ABI_BEGIN
   if (!w || !(lr > 0)) RS_FAIL(SIM_ERR_ARG, "sim_ws_adam: bad argument");
+  ws_turn turn(w, w->st);
   adam(w, lr);
   RS_CUDA(cudaStreamSynchronize(w->st));
   ABI_END
@@ -1634,6 +1652,7 @@ extern "C" sim_status sim_ws_adam(sim_ws_t w, double lr) {
 extern "C" sim_status sim_ws_dataset(sim_ws_t w, int *n_samples) {
   ABI_BEGIN
   if (!w || !n_samples) RS_FAIL(SIM_ERR_ARG, "NULL argument");
+  std::lock_guard<std::mutex> guard(w->use);
   *n_samples = (int)w->data.size();
   ABI_END
 }
@@ -1644,6 +1663,7 @@ extern "C" sim_status sim_ws_train(sim_ws_t w, int epochs, int batch, double lr,
                                    double *mean_loss) {
   ABI_BEGIN
   if (!w || epochs < 0 || batch < 1 || !(lr > 0)) RS_FAIL(SIM_ERR_ARG, "sim_ws_train: bad argument");
+  ws_turn turn(w, w->st);
   int n = (int)w->data.size();
   if (n == 0) RS_FAIL(SIM_ERR_STATE, "sim_ws_train: no recorded samples");
   std::vector<int> order(n);
@@ -1676,6 +1696,7 @@ extern "C" sim_status sim_ws_train(sim_ws_t w, int epochs, int batch, double lr,
 extern "C" sim_status sim_ws_eval(sim_ws_t w, double *mean_loss) {
   ABI_BEGIN
   if (!w || !mean_loss) RS_FAIL(SIM_ERR_ARG, "NULL argument");
+  ws_turn turn(w, w->st);
   int n = (int)w->data.size();
   if (n == 0) RS_FAIL(SIM_ERR_STATE, "sim_ws_eval: no recorded samples");
   RS_CUDA(cudaMemsetAsync(w->lsum.p, 0, sizeof(double), w->st));
@@ -1800,7 +1821,7 @@ void ws_rms2(int n, const double *v, double *out, cudaStream_t s) {
 // is b; yp, sc as above (device)
 void ws_predict(sim_ws_s *w, int nx, int ny, int nz, int nb, const double *b, const double *kx, const double *sw,
                 const double *yp, const double *sc, double *y, cudaStream_t s) {
-  std::lock_guard<std::mutex> guard(w->use);
+  ws_turn turn(w, s);
   dims d = {nx, ny, nz};
   ensure_dims(w, d);
   int n = d.V();
@@ -1817,6 +1838,7 @@ void ws_predict(sim_ws_s *w, int nx, int ny, int nz, int nb, const double *b, co
   RS_CUDA(cudaEventDestroy(ev));
   k_ws_predict<<<grid_for(2 * nb, 256), 256, 0, s>>>(n, nb, w->Y.p, y, y + 2 * (size_t)nb);
   RS_LAUNCHED(1);
+  RS_CUDA(cudaEventRecord(w->last, s));
 }
 
 // append (features, target) of a solved system to the dataset
