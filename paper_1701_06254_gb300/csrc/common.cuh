@@ -315,7 +315,7 @@ struct sim_ls_s {
     gev.clear(); gev_fam.clear();
   }
   void graph_timers();          // after a replay has completed
-  int *errw = nullptr, *errw_dev = nullptr;   // device error word (host-mapped)
+  int *errw = nullptr, *errw_dev = nullptr;   // device error words (host-mapped): [0] RAS setup, [1] the network's kernels
   bool have_setup = false;
   double *noalloc_scratch = nullptr;   // device address of the allocation-free norm's array (noalloc.cu)
   // timing: events in pairs, the family of each pair in ev_fam
@@ -362,8 +362,8 @@ int sim_history(sim_t h, double *y, double *sc, int have, bool save);   // y: 2 
 // learned warm start (nn.cu)
 struct sim_ws_s;
 void ws_rms2(int n, const double *v, double *out, cudaStream_t s);
-void ws_check(sim_ws_s *w);   // fails if one of the network's kernels gave up (after a synchronisation)
+void ws_check(volatile int *err);   // fails if one of the network's kernels gave up (after a synchronisation)
 void ws_predict(sim_ws_s *w, int nx, int ny, int nz, int nb, const double *b, const double *kx, const double *sw,
-                const double *yp, const double *sc, double *y, cudaStream_t s);
+                const double *yp, const double *sc, double *y, int *err, cudaStream_t s);
 void ws_record(sim_ws_s *w, int nx, int ny, int nz, const double *b, const double *kx, const double *sw,
                const double *yp, const double *sc, const double *y, cudaStream_t s);

@@ -1131,6 +1131,7 @@ struct sim_ws_s {
   cudaEvent_t last = nullptr;             // the last simulator's reads of the output, on its own stream
   bool tc = true;                         // tcgen05 convolutions (else mma.sync)
   int *err = nullptr, *err_dev = nullptr; // host-mapped: set by a kernel whose bounded wait gave up
+  int *err_turn = nullptr;                // where the kernels of the present turn set it: err_dev, or a simulator's own word
   pack_table tab;
   ~sim_ws_s() {
     if (st) cudaStreamDestroy(st);
@@ -1143,9 +1144,14 @@ struct sim_ws_s {
 // its first access to the activations) behind the last simulator's reads of
 // them.  ws_predict returns with its GPU work queued on two streams, so the
 // lock alone would let the next caller write what that work still reads.
+// The kernels report to err: the handle's own word, or a simulator's, which
+// reads it after its own synchronisation, when the next turn may have begun.
 struct ws_turn {
   std::lock_guard<std::mutex> guard;
-  ws_turn(sim_ws_s *w, cudaStream_t s) : guard(w->use) { RS_CUDA(cudaStreamWaitEvent(s, w->last, 0)); }
+  ws_turn(sim_ws_s *w, cudaStream_t s, int *err = nullptr) : guard(w->use) {
+    RS_CUDA(cudaStreamWaitEvent(s, w->last, 0));
+    w->err_turn = err ? err : w->err_dev;
+  }
 };
 
 namespace nn {
@@ -1237,7 +1243,7 @@ static void conv_tc_launch(sim_ws_s *w, dims d, const bf16 *X, int ldx, int offx
   }
   const unsigned tiles = (unsigned)(txy * ((d.nz + NZ - 1) / NZ));
   launch_pdl(k_conv_tc<CI, CO, MODE>, tiles, TC_T, (size_t)tc_bytes(CI, CO, NZ), w->st, d.nx, d.ny, d.nz, NZ, X, ldx, offx,
-             Wt, bias, relu, out, ldo, offo, mask, ldm, offm, w->err_dev);
+             Wt, bias, relu, out, ldo, offo, mask, ldm, offm, w->err_turn);
   RS_LAUNCHED(1);
 }
 
@@ -1335,7 +1341,7 @@ static void wgrad(sim_ws_s *w, const wg_in in[NLAYER], int nl, double lscale) {
     L.part = p; p += (size_t)L.nchunk * 27 * L.co * L.ci;
     L.bpart = p; p += (size_t)L.nchunk * L.co;
   }
-  launch_pdl(k_conv_wgrad, (unsigned)block, WG_T, (size_t)WG_BYTES, w->st, tab, w->err_dev);
+  launch_pdl(k_conv_wgrad, (unsigned)block, WG_T, (size_t)WG_BYTES, w->st, tab, w->err_turn);
   launch_pdl(k_wgrad_reduce, grid_for(w->np, 256) + 1, 256, 0, w->st, tab, (int)w->np, w->G.p, nl, w->lpart.p, lscale,
              w->lsum.p);
   RS_LAUNCHED(2);
@@ -1482,16 +1488,15 @@ static size_t export_count() {
   return n;
 }
 
-// a tensor-core kernel whose bounded wait gave up leaves a flag; report it
-// (the caller has synchronised with the kernels)
-static void check_err(sim_ws_s *w) {
-  volatile int *e = w->err;
+// a tensor-core kernel whose bounded wait gave up leaves a flag in the
+// turn's error word; report it (the caller has synchronised with the kernels)
+void ws_check(volatile int *e) {
   if (*e) {
     *e = 0;
     RS_FAIL(SIM_ERR_TIMEOUT, "warm-start network: a tensor-core pipeline wait gave up");
   }
 }
-void ws_check(sim_ws_s *w) { check_err(w); }
+static void check_err(sim_ws_s *w) { ws_check(w->err); }
 
 extern "C" sim_status sim_ws_create(sim_ws_t *out, unsigned long long seed) {
   ABI_BEGIN
@@ -1818,10 +1823,11 @@ void ws_rms2(int n, const double *v, double *out, cudaStream_t s) {
 
 // predicted update as two candidates in y (2 x 2 nb, FP64, device: pressure
 // part, then saturation part) for the system whose decoupled right-hand side
-// is b; yp, sc as above (device)
+// is b; yp, sc as above (device).  err (device address of a host-mapped word):
+// set by a kernel that gave up, for ws_check after a synchronisation with s
 void ws_predict(sim_ws_s *w, int nx, int ny, int nz, int nb, const double *b, const double *kx, const double *sw,
-                const double *yp, const double *sc, double *y, cudaStream_t s) {
-  ws_turn turn(w, s);
+                const double *yp, const double *sc, double *y, int *err, cudaStream_t s) {
+  ws_turn turn(w, s, err);
   dims d = {nx, ny, nz};
   ensure_dims(w, d);
   int n = d.V();

@@ -573,7 +573,8 @@ static int s_solve(sim_s *h, double eta, double bn, int *its, double *rel) {
     h->dws.ensure(2 * (size_t)nu); h->u.ensure(3 * (size_t)nu);
     {
       rs_timed tm_net(ls, SIM_T_NETWORK);
-      ws_predict(h->ws, h->nx, h->ny, h->nz, nb, ls->b.p, h->kx.p, h->s.p, h->yprev.p, h->wsc.p, h->dws.p, st);
+      ws_predict(h->ws, h->nx, h->ny, h->nz, nb, ls->b.p, h->kx.p, h->s.p, h->yprev.p, h->wsc.p, h->dws.p,
+                 ls->errw_dev + 1, st);
     }
     // candidates: the previous step's first update (if any), then the
     // network's pressure and saturation parts
@@ -591,7 +592,7 @@ static int s_solve(sim_s *h, double eta, double bn, int *its, double *rel) {
     for (int i = 0; i < m; i++) { xs[q] = u[i]; ys[q] = ls->b.p; q++; }
     double dv[9];
     rs_dots(xs, ys, q, nu, dv, st);
-    ws_check(h->ws);                                   // (rs_dots has synchronised)
+    ws_check(ls->errw + 1);                            // (rs_dots has synchronised)
     double G[3][3] = {{0}}, r[3] = {0};
     q = 0;
     for (int i = 0; i < m; i++) for (int j = 0; j <= i; j++) { G[i][j] = G[j][i] = dv[q]; q++; }
