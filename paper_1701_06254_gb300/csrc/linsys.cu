@@ -1314,7 +1314,10 @@ static void wait_slot(const volatile double *done, cudaStream_t s) {
 // when the recursive residual meets tol ||b||, then checks the true residual
 // b - A x; when that misses the tolerance, or on a breakdown (rho, (rh, v)
 // or omega zero), it restarts from the true residual with rh = r.  At most
-// max_lin iterations.  0 = converged, 1 = iteration cap, 2 = non-finite.
+// max_lin iterations; a breakdown in the first iteration after a restart,
+// which the next restart would only repeat (a right-hand side below the FP32
+// range, whose preconditioned vector is zero), ends the solve.  0 =
+// converged, 1 = iteration cap or such a breakdown, 2 = non-finite.
 template <class Tz>
 static int ls_solve_bicgstab(sim_ls_s *ls, double tol, int *its_out, double *relres, bool x0) {
   cudaStream_t st = ls->st;
@@ -1361,6 +1364,7 @@ static int ls_solve_bicgstab(sim_ls_s *ls, double tol, int *its_out, double *rel
     RS_CHECK_LAUNCH();
     wait(1);
     bool broke = false, done = false;
+    const int its0 = its;
     while (its < maxit) {
       const double rho = hp[4 + 2];
       if (!std::isfinite(rho)) { *its_out = its; *relres = NAN; return 2; }
@@ -1404,7 +1408,7 @@ static int ls_solve_bicgstab(sim_ls_s *ls, double tol, int *its_out, double *rel
     if (!std::isfinite(rn)) { rc = 2; break; }
     if (rn <= tol * bn) { rc = 0; break; }
     if (its >= maxit) { rc = 1; break; }
-    if (!done && !broke) { rc = 1; break; }
+    if (!done && (!broke || its == its0)) { rc = 1; break; }
   }
   *its_out = its;
   *relres = rc == 2 ? NAN : rn / bn;
