@@ -583,7 +583,9 @@ void ls_setup(sim_ls_s *ls) {
 #define ORTHO_BS 256
 // Each block owns a fixed chunk of at most ORTHO_CH rows and keeps its slice
 // of w in shared memory.  Basis vectors are streamed vector-outer, rows-inner,
-// so loads are coalesced and independent.
+// so loads are coalesced and independent.  V, w and h carry no __restrict__: a
+// programmatic launch starts while the kernels that write them still run, and
+// no read-only load may move above pdl_wait (as in k_bsr_spmv).
 #define ORTHO_CH 8192
 
 __device__ __forceinline__ double warp_sum_d(double v) {
@@ -752,10 +754,9 @@ __device__ __forceinline__ void norm_tail(int nv, const double *part, double *nr
 }
 
 // part[k][b] = V_k . w over the block's rows (k < nv); with_norm: part[nv][b] = w . w
-__global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots(int nu, int ch, int nv, const double *__restrict__ V,
-                                                            const double *__restrict__ w, double *part, int with_norm,
-                                                            const int *cond, const int *jd, int *ticket, double *out,
-                                                            int pdl) {
+__global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots(int nu, int ch, int nv, const double *V, const double *w,
+                                                            double *part, int with_norm, const int *cond, const int *jd,
+                                                            int *ticket, double *out, int pdl) {
   if (pdl) { pdl_trigger(); pdl_wait(); }
   if (cond && *cond == 0) return;
   if (jd) nv = *jd + 1;                        // graph replay: the step index lives on the device
@@ -794,10 +795,10 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots(int nu, int ch, int 
 }
 
 // w -= sum_k h_k V_k over the block's rows, then part[0][b] = ||w||^2
-__global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update(int nu, int ch, int nv, const double *__restrict__ V,
-                                                              double *w, const double *__restrict__ h, double *part,
-                                                              const int *cond, int *jd, int *ticket, double *nrm,
-                                                              int *flag, const double *h1, double *hnorm, int pdl) {
+__global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update(int nu, int ch, int nv, const double *V, double *w,
+                                                              const double *h, double *part, const int *cond, int *jd,
+                                                              int *ticket, double *nrm, int *flag, const double *h1,
+                                                              double *hnorm, int pdl) {
   if (pdl) { pdl_trigger(); pdl_wait(); }
   if (cond && *cond == 0) return;
   if (jd) nv = *jd + 1;
@@ -842,10 +843,9 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update(int nu, int ch, in
 // (lo), w at w (hi) and w + nu (lo).  Vector offsets are 32-bit (the basis
 // holds at most 2 (ORTHO_MAXV + 1) nu < 2^31 floats) and each thread takes
 // two rows per iteration, so that 32 loads are in flight together.
-__global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots_df(int nu, int ch, int nv, const float *__restrict__ V,
-                                                               const float *__restrict__ w, double *part,
-                                                               int with_norm, const int *cond, const int *jd,
-                                                               int *ticket, double *out, int pdl) {
+__global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots_df(int nu, int ch, int nv, const float *V, const float *w,
+                                                               double *part, int with_norm, const int *cond,
+                                                               const int *jd, int *ticket, double *out, int pdl) {
   if (pdl) { pdl_trigger(); pdl_wait(); }
   if (cond && *cond == 0) return;
   if (jd) nv = *jd + 1;
@@ -906,11 +906,10 @@ __global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_dots_df(int nu, int ch, i
 // k_ortho_update on pair planes: w -= sum_k h_k V_k (h FP64, split once per
 // block), then part[0][b] = ||w||^2 over the block's rows; two rows per
 // thread per iteration
-__global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update_df(int nu, int ch, int nv, const float *__restrict__ V,
-                                                                 float *w, const double *__restrict__ h, double *part,
-                                                                 const int *cond, int *jd, int *ticket, double *nrm,
-                                                                 int *flag, const double *h1, double *hnorm,
-                                                                 float *isp, int pdl) {
+__global__ void __launch_bounds__(ORTHO_BS, 4) k_ortho_update_df(int nu, int ch, int nv, const float *V, float *w,
+                                                                 const double *h, double *part, const int *cond,
+                                                                 int *jd, int *ticket, double *nrm, int *flag,
+                                                                 const double *h1, double *hnorm, float *isp, int pdl) {
   if (pdl) { pdl_trigger(); pdl_wait(); }
   if (cond && *cond == 0) return;
   if (jd) nv = *jd + 1;

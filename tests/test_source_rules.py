@@ -24,3 +24,34 @@ def test_a_solve_reads_the_error_word_it_gave_to_the_network():
     given = re.search(r"ws_predict\([^;]*ls->errw_dev \+ (\d+)", body)
     read = re.search(r"ws_check\(ls->errw \+ (\d+)\)", body)
     assert given and read and given.group(1) == read.group(1) != "0"
+
+
+# What a kernel may declare __restrict__ although it starts while the kernels
+# before it still run: data fixed between setups (patterns, matrix values,
+# level operators, inverse diagonals, the coarsest inverse).
+FIXED = {"rp", "ci", "val", "vh", "vl", "v", "dinv", "invT"}
+
+
+def _kernels(src):
+    """(parameter list, body) of every __global__ function."""
+    for m in re.finditer(r"__global__", src):
+        j = src.index("{", m.start())
+        if ";" in src[m.start():j]:
+            continue
+        depth, k = 0, j
+        while True:
+            depth += {"{": 1, "}": -1}.get(src[k], 0)
+            if depth == 0:
+                break
+            k += 1
+        yield src[m.start():j], src[j:k]
+
+
+@pytest.mark.parametrize("name", sorted(f for f in os.listdir(CSRC) if f.endswith(".cu")))
+def test_programmatic_kernels_restrict_fixed_data_only(name):
+    """A const __restrict__ pointer lets the compiler use read-only loads and
+    move them above the wait for the kernel that writes the data."""
+    for head, body in _kernels(_source(name)):
+        if "pdl_wait" in body:
+            names = set(re.findall(r"\*\s*__restrict__\s*(\w+)", head))
+            assert names <= FIXED, (" ".join(head.split())[:120], names - FIXED)
