@@ -251,6 +251,7 @@ struct ras_data {
   dbuf<unsigned char> blob;     // the streams
   size_t lvl_smem[2] = {0, 0};  // k_ras_levels' shared memory, without and with the pruned lists
   size_t pack_smem = 0;         // k_ras_pack's tables
+  dbuf<int> pack_lv, pack_gr;   // the same in global memory, where they do not fit
   bool symmetric = false;       // the pattern has (c, i) for every (i, c)
   bool pruned = false;          // the last setup left unneeded rows out of the apply's lists
   dbuf<int> gidx, gord;         // gather order (owned rows first): global row, ext index

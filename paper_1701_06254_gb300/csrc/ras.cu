@@ -160,7 +160,7 @@ void ras_build_static(sim_ls_s *ls) {
     R.smem_bytes = ((size_t)mmax + 2) * yb;
     // k_ras_pack's tables: groups per level, then the groups' sizes
     R.pack_smem = (4 * (size_t)mmax + (size_t)R.max_nnz / RAS_K + 24) * sizeof(int);
-    R.smem_path = fits && R.smem_bytes <= RAS_SMEM_BUDGET && R.pack_smem <= RAS_SMEM_BUDGET;
+    R.smem_path = fits && R.smem_bytes <= RAS_SMEM_BUDGET;
     if (R.smem_path) {
       // gather / scatter order: the owned rows first, each part in natural
       // order (runs of neighbouring cells share their sectors)
@@ -184,6 +184,7 @@ void ras_build_static(sim_ls_s *ls) {
       R.symmetric = d2h(asym.p, 1, st)[0] == 0;
       R.alvl_rows.alloc(2 * next_tot); R.alvl_ptr.alloc(2 * (next_tot + nsub));
       R.gdesc.alloc(2 * ext.size() + 8 * (size_t)nsub + nnz_tot / RAS_K + 1);
+      if (R.pack_smem > RAS_SMEM_BUDGET) { R.pack_lv.alloc(2 * ext.size() + nsub); R.pack_gr.alloc(R.gdesc.n); }
       RS_CUDA(cudaStreamSynchronize(st));                  // the host vectors above go out of scope
     }
   }
@@ -781,13 +782,16 @@ __device__ __forceinline__ size_t ras_group0(int s, int base, int pbase) {
 // groups are counted, numbered, sized and placed, then filled one warp each.
 // (The first version split each level with one thread walking its rows: 0.47
 // ms per setup on the 1M-cell case, bound by that thread's dependent loads.)
-template <class T, class TB>
+// The groups' tables lie in shared memory, or for subdomains of more than some
+// 10,000 rows (GT) in global memory: the setup alone reads them, so they must
+// not decide where the streamed apply ends.
+template <class T, class TB, bool GT>
 __global__ void __launch_bounds__(128) k_ras_pack(const int *sub_ptr, const int *lrp_ptr, const int *frp,
                                                   const int *fci, const int *fdiag, const int *ipos, const int *gord,
                                                   uint16_t *gpos, const T *fv, const T *dinv, const int *lvl_rows,
                                                   const int *nlev, const int *lvl_ptr, const long long *blob_off,
                                                   unsigned char *blobs, uint2 *gdesc, int *ngrp, const int *order,
-                                                  int *err) {
+                                                  int *err, int *lv_tab, int *gr_tab) {
   const int s = order[blockIdx.x], base = sub_ptr[s], m = sub_ptr[s + 1] - base, pbase = lrp_ptr[s], fbase = base + s;
   const int *pL = lvl_ptr + 2 * (base + s), *pU = pL + (m + 1);
   const int *rL = lvl_rows + 2 * base, *rU = rL + m;
@@ -799,11 +803,11 @@ __global__ void __launch_bounds__(128) k_ras_pack(const int *sub_ptr, const int 
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   constexpr int AH = ras_ahead<TB>();
   __shared__ int ngr, ngl, pad0, pad1;                      // groups, those of the L sweep, the empty ones' starts
-  // dynamic shared memory: per level its group count (then the first group's
-  // index), per group its bytes (then its start)
+  // per level its group count (then the first group's index), per group its
+  // bytes (then its start); at most 2 m levels
   extern __shared__ int psm[];
   const int nLw = nL > 1 ? nL - 1 : 0, nlevels = nLw + nU;
-  int *lgc = psm, *gby = psm + nlevels + 1;
+  int *lgc = GT ? lv_tab + 2 * (size_t)base + s : psm, *gby = GT ? gr_tab + ras_group0(s, base, pbase) : psm + nlevels + 1;
   // positions in gather order
   for (int k = threadIdx.x; k < m; k += blockDim.x) gpos[base + k] = (uint16_t)ipos[base + gord[base + k]];
   // groups of one level of the sweep order (L levels 1..nL-1, then U levels):
@@ -1183,26 +1187,31 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
   }
 }
 
+template <class T, class TB> static void ras_pack_go(sim_ls_s *ls, const T *fv, const T *dinv) {
+  ras_data &R = ls->ras;
+  auto go = [&](auto kern, size_t smem) {
+    kern<<<R.nsub, 128, smem, ls->st>>>(R.sub_ptr.p, R.lrp_ptr.p, R.frp.p, R.fci.p, R.fdiag.p, R.ipos.p, R.gord.p,
+                                        R.gpos.p, fv, dinv, R.pruned ? R.alvl_rows.p : R.lvl_rows.p, R.nlev.p,
+                                        R.pruned ? R.alvl_ptr.p : R.lvl_ptr.p, R.blob_off.p, R.blob.p, R.gdesc.p,
+                                        R.ngrp.p, R.order.p, ls->errw_dev, R.pack_lv.p, R.pack_gr.p);
+  };
+  if (R.pack_smem > RAS_SMEM_BUDGET) go(k_ras_pack<T, TB, true>, 0);
+  else {
+    static bool attr = false;
+    if (!attr) {
+      RS_CUDA(cudaFuncSetAttribute(k_ras_pack<T, TB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RAS_SMEM_BUDGET));
+      attr = true;
+    }
+    go(k_ras_pack<T, TB, false>, R.pack_smem);
+  }
+  RS_LAUNCHED(1);
+}
 void ras_pack(sim_ls_s *ls) {
   ras_data &R = ls->ras;
   if (!R.smem_path) return;
-  static bool pattr = false;
-  if (!pattr) {
-    RS_CUDA(cudaFuncSetAttribute(k_ras_pack<float, __nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, RAS_SMEM_BUDGET));
-    RS_CUDA(cudaFuncSetAttribute(k_ras_pack<float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, RAS_SMEM_BUDGET));
-    RS_CUDA(cudaFuncSetAttribute(k_ras_pack<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, RAS_SMEM_BUDGET));
-    pattr = true;
-  }
-#define RAS_PACK(T, TB, FV, DI)                                                                                      \
-  k_ras_pack<T, TB><<<R.nsub, 128, R.pack_smem, ls->st>>>(                                                           \
-      R.sub_ptr.p, R.lrp_ptr.p, R.frp.p, R.fci.p, R.fdiag.p, R.ipos.p, R.gord.p, R.gpos.p, FV, DI,                  \
-      R.pruned ? R.alvl_rows.p : R.lvl_rows.p, R.nlev.p, R.pruned ? R.alvl_ptr.p : R.lvl_ptr.p, R.blob_off.p,       \
-      R.blob.p, R.gdesc.p, R.ngrp.p, R.order.p, ls->errw_dev)
-  if (ls->o.precision == SIM_PREC_MIXED_BF16) RAS_PACK(float, __nv_bfloat16, R.fval32.p, R.dinv32.p);
-  else if (ls->o.precision != SIM_PREC_FP64) RAS_PACK(float, float, R.fval32.p, R.dinv32.p);
-  else RAS_PACK(double, double, R.fval.p, R.dinv.p);
-#undef RAS_PACK
-  RS_LAUNCHED(1);
+  if (ls->o.precision == SIM_PREC_MIXED_BF16) ras_pack_go<float, __nv_bfloat16>(ls, R.fval32.p, R.dinv32.p);
+  else if (ls->o.precision != SIM_PREC_FP64) ras_pack_go<float, float>(ls, R.fval32.p, R.dinv32.p);
+  else ras_pack_go<double, double>(ls, R.fval.p, R.dinv.p);
 }
 
 template <class T, class Tin>
