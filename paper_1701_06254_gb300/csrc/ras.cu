@@ -41,6 +41,7 @@
 #define RAS_SMEM_BUDGET (200 * 1024)
 #define RAS_K 6                                  // entries of a row per group
 #define RAS_START_MAX (1LL << 24)                // a stream's bytes: 20-bit starts in units of 16
+#define RAS_NONFINITE (1 << 30)                  // with a subdomain's group count: its stream has Inf or NaN
 // groups held in registers ahead of the sweep
 template <class TB> __host__ __device__ constexpr int ras_ahead() { return sizeof(TB) == 2 ? 3 : 2; }
 // stored bytes per 2x2 block
@@ -897,6 +898,7 @@ __global__ void __launch_bounds__(128) k_ras_pack(const int *sub_ptr, const int 
       gd[g] = make_uint2((unsigned)(gby[g] >> 4) | 1u << 20, 0);
     }
   }
+  bool bad = false;                                                  // a stored value is not finite
   for (int lv = wid; lv < nlevels; lv += nwarps) {
     int g = lgc[lv];
     split(lv, [&](bool up, int i, int ne, int q0, int p) {
@@ -938,7 +940,11 @@ __global__ void __launch_bounds__(128) k_ras_pack(const int *sub_ptr, const int 
             } else if (k < n) {
               for (int w = 0; w < 4; w++) v[w] = fv[4 * (size_t)(qe + k) + w];
             }
-            for (int w = 0; w < 4; w++) dst[4 * u + w] = to_blob_d<TB>(v[w]);
+            for (int w = 0; w < 4; w++) {
+              const TB z = to_blob_d<TB>(v[w]);
+              dst[4 * u + w] = z;
+              bad |= !isfinite((T)z);
+            }
           }
         }
         at += PB * cnt;
@@ -949,6 +955,7 @@ __global__ void __launch_bounds__(128) k_ras_pack(const int *sub_ptr, const int 
       g++;
     });
   }
+  if (bad) atomicOr(&ngrp[2 * s + 1], RAS_NONFINITE);
 }
 
 template <class T> struct v2_t;
@@ -968,7 +975,9 @@ template <> struct v2_t<double> { typedef double2 type; };
 // ras_ahead groups early (every lane its own row; no ring, no waits), missing
 // entries multiply the zero element, and what a lane or a group does not
 // have keeps an earlier group's values, which only ever multiply that zero
-// or are not stored.  A bulk prefetch into L2 runs RAS_PF_BYTES ahead of the
+// or are not stored.  A subdomain with a value that is not finite (a singular
+// block) takes a copy of the sweeps that clears them, so that Inf or NaN stays
+// in the rows that depend on it.  A bulk prefetch into L2 runs RAS_PF_BYTES ahead of the
 // loads.  20 blocks per SM (at most 96 registers): with 113 the 2500
 // subdomains of the 1M-cell case needed a second wave.
 //
@@ -1005,7 +1014,7 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
   T2 *y = reinterpret_cast<T2 *>(sm4);
   const int tid = threadIdx.x, row_of = tid / LPR, comp = tid & 1;
   const int s = order[blockIdx.x], base = sub_ptr[s], m = sub_ptr[s + 1] - base, no = nown[s];
-  const int ngl = ngrp[2 * s], ng = ngrp[2 * s + 1];
+  const int ngl = ngrp[2 * s], ngw = ngrp[2 * s + 1], ng = ngw & ~RAS_NONFINITE;
   const int *gidx = gidx_all + base;
   const uint16_t *gpos = gpos_all + base;
   const unsigned char *st = blobs + blob_off[s];
@@ -1029,8 +1038,10 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
   int gq = 0;
   auto fetch_desc = [&]() { const uint2 d = __ldg(gd + min(gq, glast)); gq++; return d; };
   uint2 dq0 = fetch_desc(), dq1 = fetch_desc();
-  // the next group into a register set
-  auto load = [&](ras_group<NP> &G) {
+  // the next group into a register set; CLEAR: what the lane's row does not
+  // have becomes zero
+  auto load = [&](ras_group<NP> &G, auto clear_) {
+    constexpr bool CLEAR = decltype(clear_)::value;
     const uint2 d = dq0;
     dq0 = dq1;
     dq1 = fetch_desc();
@@ -1045,6 +1056,7 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
     for (int k = 1; k < NP; k++) {
       const int n = k < 6 ? (d.y >> (6 * (k - 1))) & 63 : d.x >> 26;
       if (row_of < n) G.p[k] = __ldg(st_b + q);
+      else if (CLEAR) G.p[k] = make_uint4(0, 0, 0, 0);
       q += (D ? 2 : 1) * n;
     }
     // prefetch (thread 0) when the loads come within RAS_PF_BYTES of it
@@ -1076,7 +1088,7 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
       if (p0 + u * BS < m) { T2 t; t.x = (T)v[u].x; t.y = (T)v[u].y; y[pos[u]] = t; }
   }
 #pragma unroll
-  for (int k = 0; k < AHEAD; k++) load(S[k]);
+  for (int k = 0; k < AHEAD; k++) load(S[k], std::false_type());      // (the sets are zero)
   if (tid < 2) { T2 z; z.x = 0; z.y = 0; y[m + tid] = z; }
   sync();
   // one group: blocks of piece k are k BPP .. ; in a U group block 0 is the
@@ -1161,14 +1173,18 @@ k_ras_apply_stream(const long long *blob_off, const unsigned char *blobs, const 
       else { T2 t; t.x = a0; t.y = a1; y[row] = t; }
     }
   };
-  auto sweep = [&](int n, auto up_) {                    // n groups, a multiple of AHEAD
+  auto sweep = [&](int n, auto up_, auto clear_) {       // n groups, a multiple of AHEAD
     for (int g = 0; g < n; g += AHEAD) {
 #pragma unroll
-      for (int k = 0; k < AHEAD; k++) { solve(S[k], up_); load(S[k]); sync(); }
+      for (int k = 0; k < AHEAD; k++) { solve(S[k], up_); load(S[k], clear_); sync(); }
     }
   };
-  sweep(ngl, std::integral_constant<int, 0>());
-  sweep(ng - ngl, std::integral_constant<int, 1>());
+  auto sweeps = [&](auto clear_) {
+    sweep(ngl, std::integral_constant<int, 0>(), clear_);
+    sweep(ng - ngl, std::integral_constant<int, 1>(), clear_);
+  };
+  if (ngw & RAS_NONFINITE) sweeps(std::true_type());
+  else sweeps(std::false_type());
   for (int p0 = tid; p0 < no; p0 += 8 * BS) {            // the owned rows come first in gather order
     T2 v[8], w[8];
 #pragma unroll
