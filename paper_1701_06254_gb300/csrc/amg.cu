@@ -20,12 +20,13 @@
 // ------------------------------------------------------------ pattern -----
 // tpos[q]: the position of (j, i) in row j for entry q = (i, j), by binary
 // search; L lanes per row (one for short rows, a warp for long ones: a thread
-// walking 40 searches one after another was latency-bound)
+// walking 40 searches one after another was latency-bound).  g, the thread's
+// number, is unsigned: with 32 lanes per row it passes 2^31 at 2^26 rows.
 template <int L>
-__device__ __forceinline__ void tpos_row(int g, int n, const int *rp, const int *ci, int *tpos, int *err) {
-  const int i = g / L;
+__device__ __forceinline__ void tpos_row(unsigned g, int n, const int *rp, const int *ci, int *tpos, int *err) {
+  const int i = (int)(g / L);
   if (i >= n) return;
-  for (int q = rp[i] + g % L; q < rp[i + 1]; q += L) {
+  for (int q = rp[i] + (int)(g % L); q < rp[i + 1]; q += L) {
     int j = ci[q], lo = rp[j], hi = rp[j + 1] - 1, pos = -1;
     while (lo <= hi) {
       int mid = (lo + hi) >> 1, c = ci[mid];
