@@ -404,9 +404,9 @@ sim_status sim_batch_autotune(sim_batch_t b, const int *candidates, int n_candid
  * (3x3x3 convolutions, 32 channels, ReLU, average-pool down, nearest up,
  * skip concatenation) on the simulator's grid; all its contractions run
  * as BF16 tensor-core MMAs with FP32 accumulation (tcgen05 with TMEM
- * accumulators; mma.sync convolutions behind sim_ws_use_tcgen05), for inference and for training (Adam with FP32 master
- * weights).  It is grid-size agnostic: weights trained on one grid apply to
- * any other.  Inputs per cell (8 channels): the Newton residual, i.e. the
+ * accumulators; mma.sync convolutions behind sim_ws_use_tcgen05), for
+ * inference and for training (Adam with FP32 master weights).  It is
+ * grid-size agnostic: weights trained on one grid apply to any other.  Inputs per cell (8 channels): the Newton residual, i.e. the
  * decoupled right-hand side b (pressure and saturation rows, each over its
  * rms over the cells), (ln k - 4) / 2, 4 (s_w - 0.5), the previous solve's
  * update (each component over its rms; zero before the first solve) and two
@@ -414,8 +414,9 @@ sim_status sim_batch_autotune(sim_batch_t b, const int *candidates, int n_candid
  * saturation) with unit rms over the cells; well rows are not predicted (0).
  * The two components enter the initial guess as separate candidates whose
  * scales a least-squares fit sets (sim_ws_attach).  The head layer starts at
- * zero: an untrained network predicts nothing.  A handle is used by one caller at a time (calls
- * on it are serialised internally). */
+ * zero: an untrained network predicts nothing.  A handle may be shared by
+ * simulators and callers in several threads: calls on it take turns, on the
+ * host and on the GPU. */
 typedef struct sim_ws_s *sim_ws_t;
 sim_status sim_ws_create(sim_ws_t *out, unsigned long long seed);   /* He-normal weights from seed, zero head */
 void sim_ws_destroy(sim_ws_t ws);

@@ -21,7 +21,8 @@
 // tpos[q]: the position of (j, i) in row j for entry q = (i, j), by binary
 // search; L lanes per row (one for short rows, a warp for long ones: a thread
 // walking 40 searches one after another was latency-bound).  g, the thread's
-// number, is unsigned: with 32 lanes per row it passes 2^31 at 2^26 rows.
+// number, is unsigned: with 32 lanes per row it would pass 2^31 at 2^26 rows,
+// not far above the largest grid that is accepted (50M cells).
 template <int L>
 __device__ __forceinline__ void tpos_row(unsigned g, int n, const int *rp, const int *ci, int *tpos, int *err) {
   const int i = (int)(g / L);

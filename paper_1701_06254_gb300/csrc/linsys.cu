@@ -255,8 +255,9 @@ template <> struct vec2_t<float> { typedef float2 type; };
 // ascending block order.
 #define SPMV_WARPS 8
 #define SPMV_CHUNK 256
-// (The FP32 kernel of large systems stays at 32 registers, 8 blocks per SM,
-// only without the wait and without jd: 40 registers cost it 8%.)
+// (jd is read with an FP64 matrix only: the FP32 kernels need 32 registers, 8
+// blocks per SM, without it and 40 with it, which cost them 7% on 1M cells.
+// PDL is a template argument so that large systems run without the wait.)
 template <class Tv, class Tx, class Tf, class Ty, bool PDL>
 __global__ void __launch_bounds__(SPMV_WARPS * 32)
 k_bsr_spmv(int nb, const int *__restrict__ rp, const int *__restrict__ ci, const Tv *__restrict__ val,

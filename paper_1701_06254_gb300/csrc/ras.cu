@@ -785,7 +785,8 @@ __device__ __forceinline__ size_t ras_group0(int s, int base, int pbase) {
 // ms per setup on the 1M-cell case, bound by that thread's dependent loads.)
 // The groups' tables lie in shared memory, or for subdomains of more than some
 // 10,000 rows (GT) in global memory: the setup alone reads them, so they must
-// not decide where the streamed apply ends.
+// not decide where the streamed apply ends (24x24x360 cells, BF16, 208
+// iterations: 380 ms per step, RAS 244 us per launch).
 template <class T, class TB, bool GT>
 __global__ void __launch_bounds__(128) k_ras_pack(const int *sub_ptr, const int *lrp_ptr, const int *frp,
                                                   const int *fci, const int *fdiag, const int *ipos, const int *gord,
@@ -971,15 +972,19 @@ template <> struct v2_t<double> { typedef double2 type; };
 // mostly one warp's own instructions.  They are kept few and free of
 // branches, so that the loads of a later group fill the waits of the current
 // one (a uniform branch costs about as much as a block's product; the same
-// sweep with a test per entry took 108 us per launch on the 1M-cell case): a group's pieces come straight from global memory into registers,
-// ras_ahead groups early (every lane its own row; no ring, no waits), missing
-// entries multiply the zero element, and what a lane or a group does not
-// have keeps an earlier group's values, which only ever multiply that zero
-// or are not stored.  A subdomain with a value that is not finite (a singular
-// block) takes a copy of the sweeps that clears them, so that Inf or NaN stays
-// in the rows that depend on it.  A bulk prefetch into L2 runs RAS_PF_BYTES ahead of the
-// loads.  20 blocks per SM (at most 96 registers): with 113 the 2500
-// subdomains of the 1M-cell case needed a second wave.
+// sweep with a test per entry took 108 us per launch on the 1M-cell case): a
+// group's pieces come straight from global memory into registers, ras_ahead
+// groups early (every lane its own row; no ring, no waits), missing entries
+// multiply the zero element, and what a lane or a group does not have keeps an
+// earlier group's values, which only ever multiply that zero or are not
+// stored.  A subdomain with a value that is not finite (a singular block)
+// takes a copy of the sweeps that clears them, so that Inf and NaN stay in the
+// rows that depend on it.  A bulk prefetch into L2 runs RAS_PF_BYTES ahead of
+// the loads.  One lane per row, BF16: 20 blocks per SM (at most 96 registers),
+// since with 113 the 2500 subdomains of the 1M-cell case needed a second wave
+// (111 us); FP64 input spills 120 bytes at that limit and takes the same 85
+// us.  FP32 factors take 124 registers, 16 blocks per SM; the 68 subdomains
+// that then start late are the shortest (longest first): 84 us.
 //
 // Per launch in the solver, against the sweep it replaces (factors through a
 // shared-memory ring, products by entry, then sums by row): 1M cells, BF16,
@@ -996,7 +1001,10 @@ template <> struct v2_t<double> { typedef double2 type; };
 // Per launch, one against two lanes: 200k, FP32, 43 -> 37 us; 65k, BF16, 36 ->
 // 28 us; 150k with overlap 2, 44 -> 39 us; 155k, 33 -> 29 us.  Beyond one wave
 // the second warp's instructions compete with the other blocks' (1M cells:
-// one lane, 84 us).
+// one lane, 84 us).  The rule counts subdomains only, since two lanes also win
+// where the vectors of thick models leave fewer blocks resident (BF16, one
+// against two lanes: 256 subdomains of 360 layers, two per SM, 381 -> 281 us;
+// 576 of them 683 -> 498; 900 of 200 layers, four per SM, 396 -> 318).
 #define RAS_PF_BYTES 8192
 #define RAS_PF_STEP 2048
 #define RAS_W2_MAX (152 * 8)

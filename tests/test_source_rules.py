@@ -58,9 +58,9 @@ def test_programmatic_kernels_restrict_fixed_data_only(name):
 
 
 def test_lane_numbers_of_wide_rows_are_unsigned():
-    """32 lanes per row: the thread's number passes 2^31 at 2^26 rows, before
-    the row's number does; as an int it would name a negative row.  (A system
-    of that size does not belong in a test.)"""
+    """32 lanes per row: the thread's number would pass 2^31 at 2^26 rows, not
+    far above the 50M cells that are accepted; as an int it would then name a
+    negative row."""
     s = _source("amg.cu")
     m = re.search(r"void tpos_row\((\w+) g,", s)
     assert m and m.group(1) == "unsigned"
