@@ -1129,6 +1129,7 @@ struct sim_ws_s {
   unsigned long long seed = 0;
   std::mutex use;                         // one caller at a time (activations are shared): see ws_turn
   cudaEvent_t last = nullptr;             // the last simulator's reads of the output, on its own stream
+  bool recorded = false;                  // last has been recorded (never for a network that no simulator uses)
   bool tc = true;                         // tcgen05 convolutions (else mma.sync)
   int *err = nullptr, *err_dev = nullptr; // host-mapped: set by a kernel whose bounded wait gave up
   int *err_turn = nullptr;                // where the kernels of the present turn set it: err_dev, or a simulator's own word
@@ -1149,7 +1150,7 @@ struct sim_ws_s {
 struct ws_turn {
   std::lock_guard<std::mutex> guard;
   ws_turn(sim_ws_s *w, cudaStream_t s, int *err = nullptr) : guard(w->use) {
-    RS_CUDA(cudaStreamWaitEvent(s, w->last, 0));
+    if (w->recorded) RS_CUDA(cudaStreamWaitEvent(s, w->last, 0));
     w->err_turn = err ? err : w->err_dev;
   }
 };
@@ -1845,6 +1846,7 @@ void ws_predict(sim_ws_s *w, int nx, int ny, int nz, int nb, const double *b, co
   k_ws_predict<<<grid_for(2 * nb, 256), 256, 0, s>>>(n, nb, w->Y.p, y, y + 2 * (size_t)nb);
   RS_LAUNCHED(1);
   RS_CUDA(cudaEventRecord(w->last, s));
+  w->recorded = true;
 }
 
 // append (features, target) of a solved system to the dataset
