@@ -141,8 +141,8 @@ def ras_bytes(ls, precision):
 # ncu captures of the benchmark's own command (profiles/dram_traffic_channelised_1m.md),
 # keyed on (kernel family, precision, decoupling); a configuration without a
 # capture of the current kernels reports null
-NCU_TRAFFIC = {("ras", "mixed_bf16", "qi"): 217.0e6, ("spmv_prec", "mixed_bf16", "qi"): 165.7e6,
-               ("spmv64", "mixed_bf16", "qi"): 271.3e6, ("vcycle", "mixed_bf16", "qi"): 353.6e6}
+NCU_TRAFFIC = {("ras", "mixed_bf16", "qi"): 217.0e6, ("spmv_prec", "mixed_bf16", "qi"): 166.1e6,
+               ("spmv64", "mixed_bf16", "qi"): 275.4e6, ("vcycle", "mixed_bf16", "qi"): 353.6e6}
 
 
 def ncu_traffic(kernel, args):
