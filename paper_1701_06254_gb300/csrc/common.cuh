@@ -67,9 +67,10 @@ inline unsigned grid_for(size_t n, int bs) { size_t g = (n + bs - 1) / bs; retur
 // Programmatic dependent launch: a kernel launched with launch_pdl may be
 // scheduled while the kernel before it in the stream is still running, so
 // its launch latency overlaps that kernel's last wave.  Such a kernel calls
-// pdl_wait() before it touches memory: the wait returns once the previous
-// kernel has completed and its writes are visible (at once when there is no
-// such kernel).  pdl_trigger() lets the next kernel be scheduled early.
+// pdl_wait() before it touches what earlier kernels of the chain read or write
+// (it may fetch data fixed between setups before): the wait returns once the
+// previous kernel has completed and its writes are visible (at once when there
+// is no such kernel).  pdl_trigger() lets the next kernel be scheduled early.
 // rs_pdl_off (per host thread) makes launch_pdl an ordinary launch: used
 // while recording a graph body that cannot hold programmatic edges.
 inline thread_local bool rs_pdl_off = false;
